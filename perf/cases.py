@@ -36,32 +36,32 @@ def listed():
     return [
         # The smallest call: a book of pensions in payment at one flat rate, exact; what a pricing
         # or a reporting program asks for many times over (configuration 1).
-        reserves("flat rate, exact", "annuities", "f64", 1000, 1, n_steps=720, out="f64", flat=True),
+        reserves("flat rate exact", "annuities", "f64", 1000, 1, n_steps=720, out="f64", flat=True),
         # A small book with an odd number of scenarios, results to ordinary host arrays: the
         # interactive call in the default form.
-        reserves("small mixed book, host", "mix", "comp", 1537, 157, out="f64", place="host"),
+        reserves("small mixed book host", "mix", "comp", 1537, 157, out="f64", place="host"),
         # A whole office's in-force book under the 1,000 scenarios of Solvency II, default form
         # (configuration 2).
         reserves("mixed book", "mix", "comp", 100_000, 1000),
         # The same in the form that is fastest within 1e-6.
-        reserves("mixed book, deflated", "mix", "deflated", 100_000, 1000),
+        reserves("mixed book deflated", "mix", "deflated", 100_000, 1000),
         # The largest: a million annuities, 50 years (configuration 5, the benchmark's headline).
-        reserves("million annuities, deflated", "annuities", "deflated", 1_000_000, 1000, n_steps=600, horizon=600),
+        reserves("million annuities deflated", "annuities", "deflated", 1_000_000, 1000, n_steps=600, horizon=600),
         # End to end: records and scenarios reloaded from host memory in the call, reserves
         # delivered into page-locked host memory.
-        reserves("book reloaded, deflated", "annuities", "deflated", 100_000, 1000, n_steps=600, horizon=600,
+        reserves("book reloaded deflated", "annuities", "deflated", 100_000, 1000, n_steps=600, horizon=600,
                  place="reload"),
         # Escalating and annual payments (the paper's cohort, Section 5) as cash-flow schedules.
         reserves("scheduled payments", "mix", "comp", 20_000, 1000, schedules=True),
         # Two-life products in full precision: the run that others are checked against.
-        reserves("two lives, exact", "two_life", "f64", 3000, 333, out="f64"),
+        reserves("two lives exact", "two_life", "f64", 3000, 333, out="f64"),
         # Contracts on up to four lives (Section 4.3).
         dict(name="up to four lives", family="mlife", form="comp", n_pol=5000, n_scen=1000, n_steps=1200),
         # Nested valuation by brute force, at full size (configuration 3).
-        dict(name="nested, deflated", family="nested", book="annuities", form="deflated", n_pol=2000, n_outer=100,
+        dict(name="nested deflated", family="nested", book="annuities", form="deflated", n_pol=2000, n_outer=100,
              n_nodes=40, n_inner=1000),
         # A few outer paths of a mixed book in the default form: what an outer path costs.
-        dict(name="nested, mixed book", family="nested", book="mix", form="comp", n_pol=331, n_outer=8, n_nodes=25,
+        dict(name="nested mixed book", family="nested", book="mix", form="comp", n_pol=331, n_outer=8, n_nodes=25,
              n_inner=1000),
         # One training step of the surrogate: forward and backward at the batch that it trains with.
         dict(name="surrogate gradient", family="network", rows=8192),
