@@ -393,7 +393,7 @@ typedef struct {
     double a, b, sigma;   /* Vasicek dr = a (b - r) dt + sigma dW; a > 0, sigma >= 0    */
     double r0;            /* short rate at month 0                                     */
     int32_t mode;         /* RSV_NESTED_MC or RSV_NESTED_CURVE                         */
-    int32_t batch_outer;  /* outer paths per inner-path batch; 0 = fit 4 GiB           */
+    int32_t batch_outer;  /* >= 0; without effect: the inner paths are not stored     */
     int32_t outer_first;  /* global index of the first outer path: the call values the
                              paths outer_first .. outer_first + n_outer - 1, whose random
                              streams are keyed by that index (below 2^24), so that the
@@ -418,14 +418,13 @@ typedef struct {
 } rsv_nested_out;
 
 /* Nested valuation of the loaded portfolio (tables and portfolio needed, no
- * scenario set).  opts->form selects the arithmetic, opts->outputs and
- * opts->horizon must be 0.  With RSV_FORM_F32_DEFLATED the brute-force mode
- * runs in deflated units (products 0-5): each inner path's deflators are the
- * FP64 running products of its discount factors from the node, and
- * L_{o,n,i} = sum_p scale_p sum_{t >= m} D_i(m, t+1) E_p(t) with the policies'
- * expected cash flows E_p of rsv_compute_reserves' deflated form (the in-force
- * weighting at the node is part of them); the curve and surrogate modes then
- * run compensated.  Blocking unless opts->on_device.
+ * scenario set); opts->outputs and opts->horizon must be 0.  The brute-force and
+ * curve modes value the portfolio's expected cash flows from the node on, E(t) =
+ * sum_p amount_p E_p(t) (the in-force weighting at the node is part of them), on
+ * each inner path: L_{o,n,i} = sum_{t >= m} D_i(m, t+1) E(t) plus what matures at
+ * the node, in FP64 in every form.
+ * opts->form selects what is accepted (RSV_FORM_F32_DEFLATED: products 0-5 and the
+ * tables of that form).  Blocking unless opts->on_device.
  * Errors: RSV_E_STATE, RSV_E_ARG (bad spec, NULL L_mean/L_q995, a record as
  * in rsv_compute_reserves), RSV_E_ASSUMPTION, RSV_E_CUDA, RSV_E_NOMEM. */
 rsv_status rsv_compute_nested(rsv_ctx *ctx, const rsv_opts *opts, const rsv_nested_spec *spec,

@@ -220,15 +220,16 @@ struct rsv_ctx {
     DevBuf d_ctl;       // [0] queue head, [1] status
     DevBuf d_partial, d_part2;
     DevBuf d_o_v0f, d_o_v0d, d_o_tot, d_o_pt, d_o_traj;   // staging for host outputs
-    DevBuf d_nest_w, d_nest_ln, d_nest_rn, d_nest_d0, d_nest_plane, d_nest_mean, d_nest_kth, d_nest_all;
-    DevBuf d_nest_bm;            // Box-Muller tables of the inner-path generator (staged once)
+    DevBuf d_nest_rn, d_nest_d0, d_nest_plane, d_nest_mean, d_nest_kth, d_nest_all;
+    DevBuf d_nest_bm;            // tables of the inner-path generators (staged once)
     bool nest_bm_ready = false;
+    // expected cash flows: survivor columns of the tables, policy records, portfolio sums
+    DevBuf d_cf_tab, d_cf_pol, d_cf_sum;
+    std::vector<double> h_cf_tab;   // the columns on the host, kept: the upload may still read them
+    unsigned long long cf_tab_gen = 0;
+    int cf_tab_rows = 0, cf_tab_n = 0, cf_tab_scaled = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     cudaStream_t copy_stream = nullptr;   // device-to-host copies of V0 column blocks
-    // the deflated brute force's two pipelines: valuation (high priority) and the
-    // FP64 inner-path generator (low priority), with their ordering events
-    cudaStream_t nest_val = nullptr, nest_gen = nullptr;
-    cudaEvent_t nest_ev[5] = {};   // start, generated[2], valued[2]
     cudaEvent_t ev_block = nullptr;
     bool ev_recorded = false;
     int tuned[4] = {-1, -1, -1, -1};
@@ -271,6 +272,11 @@ rsv_status build_layout(rsv_ctx* c, int P, int horizon, int max_steps, int P_gen
 // call this; the deflated form builds its own records from the host copy).
 rsv_status layout_to_device(rsv_ctx* c);
 rsv_status build_tables(rsv_ctx* c, int form, size_t& smem);
+// Bytes of n_tab tables of pad entries in a form's entry format; RSV_E_ARG above kMaxSmem.
+rsv_status table_bytes(rsv_ctx* c, int form, int pad, int n_tab, size_t& smem);
+struct CfTables;
+// The survivor columns of the layout's tables on the device (cashflow.cu).
+rsv_status cf_tables(rsv_ctx* c, CfTables& T);
 // The first n_tab loaded tables, pad entries each, in a form's entry format
 // on the device (cached by shape and table generation); smem = their bytes.
 rsv_status stage_tables(rsv_ctx* c, int form, int pad, int n_tab, size_t& smem);
@@ -286,6 +292,7 @@ struct DeflTabs {
     std::vector<std::vector<double>> ell;
 };
 rsv_status defl_table_shape(rsv_ctx* c, const Layout& L, DeflTabs& T);
+rsv_status defl_table_range(rsv_ctx* c, DeflTabs& T);
 rsv_status defl_table_stage(rsv_ctx* c, DeflTabs& T);
 // Per-scenario totals from per-tile (row) partial sums [n_rows][s_pad], in a
 // fixed order (rsv_abi.cu).

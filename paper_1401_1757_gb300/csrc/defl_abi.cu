@@ -61,10 +61,9 @@ rsv_status defl_table_shape(rsv_ctx* c, const Layout& L, DeflTabs& T) {
     return RSV_OK;
 }
 
-rsv_status defl_table_stage(rsv_ctx* c, DeflTabs& T) {
-    const int n_tab = T.n_tab, dpad = T.dpad, arr_d = T.arr_d;
-    const bool use_a = T.use_a, use_d = T.use_d;
-    // life tables: [A | deaths][table][4 copies shifted by c][dpad], A_k = l_{k+1}, deaths_k = l_k q_k
+// The FP64 life tables T.ell; a table out of the form's range is refused.
+rsv_status defl_table_range(rsv_ctx* c, DeflTabs& T) {
+    const int n_tab = T.n_tab, dpad = T.dpad;
     T.ell.assign(n_tab, {});
     for (int t = 0; t < n_tab; ++t) {
         T.ell[t] = life_table(c->tab[t], dpad + 4);
@@ -73,6 +72,15 @@ rsv_status defl_table_stage(rsv_ctx* c, DeflTabs& T) {
                 return fail(c, RSV_E_ARG, "table %d: survival to age %d months is below 2^-220, out of the "
                                           "deflated form's range", t, k + 1);
     }
+    return RSV_OK;
+}
+
+rsv_status defl_table_stage(rsv_ctx* c, DeflTabs& T) {
+    const int n_tab = T.n_tab, dpad = T.dpad, arr_d = T.arr_d;
+    const bool use_a = T.use_a, use_d = T.use_d;
+    const rsv_status st = defl_table_range(c, T);
+    if (st != RSV_OK) return st;
+    // life tables: [A | deaths][table][4 copies shifted by c][dpad], A_k = l_{k+1}, deaths_k = l_k q_k
     const unsigned long long tkey = c->tab_gen * 1000003ull + (unsigned)dpad * 131ull + (unsigned)n_tab * 7ull +
                                     (use_a ? 1ull : 0ull) + (use_d ? 2ull : 0ull);
     if (c->defl_tab_key != tkey) {

@@ -9,10 +9,10 @@
 //   L_{o,n,i} = sum_p amount_p sum_j pi_{p,n,j} r_{p,j}(node; inner path i)
 //
 // where pi_{p,n,j} is the probability that policy p is in reduced state j at
-// the node (deterministic mortality, FP64 on the host) and r_{p,j} is the
-// reserve at the node by the backward recurrence (Eq. generalForm) on the
-// inner path's discount factors -- the same tile kernels as the valuation
-// run, started t_off = m_n steps later.
+// the node (deterministic mortality) and r_{p,j} the reserve at the node on the
+// inner path's discount factors.  The reserve is linear in the discount products
+// (Eq. basicReserveSummation), so this is the value at the node of the
+// portfolio's expected cash flows after it (cashflow.cuh).
 //
 // Random numbers: Philox4x32-10 (Salmon et al., SC'11), counter (k, c1, c2,
 // c3), key (seed lo, seed hi); step 2k takes words 0,1 and step 2k+1 words
@@ -29,8 +29,8 @@
 
 #include "fp64_series.cuh"
 #include "nested.cuh"
-#include "defl_kernel.cuh"
 #include "philox.cuh"
+#include "rsv_device.cuh"
 #include "rsv.h"
 #include "abi_guard.cuh"
 
@@ -215,151 +215,87 @@ __global__ void outer_paths_kernel(VasStep s, uint64_t seed, int o_first, int n_
     }
 }
 
-template <class VE>
-__device__ __forceinline__ VE to_plane(double x);
-template <>
-__device__ __forceinline__ double to_plane<double>(double x) { return x; }
-template <>
-__device__ __forceinline__ float to_plane<float>(double x) { return __double2float_rn(x); }
-template <>
-__device__ __forceinline__ float2 to_plane<float2>(double x) {
-    const float h = __double2float_rn(x);
-    return make_float2(h, __double2float_rn(x - (double)h));
+// ------------------------------------------------------------ inner paths ----
+// One thread values one inner path while it generates it:
+//   L_{o,n,i} = due[m] + sum_tau D(tau + 1) flow[m + tau],   m = n node_step,
+// with the discount product D carried along the path and the portfolio's
+// expected cash flows from cashflow.cuh.  The sum over the policies is inside
+// flow: with deterministic mortality the pi-weighted reserve at the node is the
+// value of the expected cash flows after it, so a path costs its random walk and one
+// multiply-add per month however large the book is, and no discount factor is
+// written to memory.  Paths of a node are packed into blocks over the outer
+// paths, the blocks run node-major, longest remaining projections first.
+constexpr int kPathNT = 128;
+
+struct PathArgs {
+    uint64_t seed;
+    int32_t o_first, n_outer, n_nodes, node_step, n_inner, n_steps;   // n_steps: the portfolio's longest projection
+    const double* r_node;
+    const void* tables;    // Box-Muller tables of the generator
+    const double* flow;
+    const double* due;
+    double* L_all;
+};
+
+template <class Path>
+__device__ __forceinline__ void for_each_path(const PathArgs& a, Path path) {
+    const long long per_node = (long long)a.n_outer * a.n_inner, blocks = (per_node + kPathNT - 1) / kPathNT;
+    for (long long b = blockIdx.x; b < blocks * a.n_nodes; b += gridDim.x) {
+        const int n = (int)(b / blocks);
+        const long long k = (b - n * blocks) * kPathNT + threadIdx.x;
+        if (k >= per_node) continue;
+        const int o = (int)(k / a.n_inner), i = (int)(k - (long long)o * a.n_inner);
+        const int m = n * a.node_step, left = max(0, a.n_steps - m);
+        const double r = a.r_node[(size_t)o * a.n_nodes + n];
+        const double now = m <= a.n_steps ? a.due[m] : 0.0;
+        a.L_all[((size_t)o * a.n_nodes + n) * a.n_inner + i] =
+            now + path((uint32_t)i, (uint32_t)n, (3u << 24) | (uint32_t)(a.o_first + o), r, m, left);
+    }
 }
 
-// Inner paths of outer paths [o0, o0 + B), every node: one thread per path.
-// Plane layout [B][n_nodes][Lmax][i_pad]; node n fills rows 0 .. Ln[n]-1.
-template <class VE>
-__global__ void inner_paths_kernel(VasStep s, uint64_t seed, int o_first, int o0, int B, int n_nodes, int n_inner, int i_pad,
-                                   int Lmax, const int* __restrict__ Ln, const double* __restrict__ r_node,
-                                   const double2* __restrict__ bm_g, VE* __restrict__ plane) {
+// FP64 throughout: bound by the FP64 pipe, about 55 operations a month.  Before,
+// the discount factors went through a plane in memory to a valuation kernel that
+// ran every policy on them: 2,000 annuities x 100 outer paths x 40 nodes x 1,000
+// inner paths 311 ms deflated (the generator on a second stream), now 203 ms;
+// 331 mixed policies x 8 x 25 x 1,000, compensated, 60.4 ms, now 23.4 ms.
+__global__ void __launch_bounds__(kPathNT) inner_paths_kernel(const VasStep s, const PathArgs a) {
     __shared__ double2 bm[BM_SC + BM_LG];   // 18 KiB: the Box-Muller tables
-    for (int k = threadIdx.x; k < BM_SC + BM_LG; k += blockDim.x) bm[k] = bm_g[k];
+    for (int k = threadIdx.x; k < BM_SC + BM_LG; k += blockDim.x) bm[k] = static_cast<const double2*>(a.tables)[k];
     __syncthreads();
-    const size_t total = (size_t)B * n_nodes * i_pad;
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(idx % i_pad);
-        const int n = (int)((idx / i_pad) % n_nodes);
-        const int ol = (int)(idx / ((size_t)i_pad * n_nodes));
-        const int o = o0 + ol;
-        VE* base = plane + ((size_t)ol * n_nodes + n) * Lmax * i_pad + i;
-        const int L = Ln[n];
-        if (i >= n_inner) {   // padding lanes read finite factors
-            for (int t = 0; t < L; ++t) base[(size_t)t * i_pad] = to_plane<VE>(1.0);
-            continue;
-        }
-        vasicek_path(s, seed, (uint32_t)i, (uint32_t)n, (3u << 24) | (uint32_t)(o_first + o),
-                     r_node[(size_t)o * n_nodes + n], L, bm,
-                     [&](int t, double v, double) { base[(size_t)t * i_pad] = to_plane<VE>(v); });
-    }
+    for_each_path(a, [&](uint32_t c1, uint32_t c2, uint32_t c3, double r, int m, int left) {
+        const double* __restrict__ flow = a.flow + m;
+        double D = 1.0, L = 0.0;
+        vasicek_path(s, a.seed, c1, c2, c3, r, left, bm, [&](int t, double v, double) {
+            D = __dmul_rn(D, v);
+            L = __fma_rn(D, __ldg(flow + t), L);
+        });
+        return L;
+    });
 }
 
-// The curve mode with the outer paths on the lanes: every outer path's node
-// rate gives one curve, and all outer paths share the in-force weights, so
-// plane[n][t][o] holds outer path o's curve at node n (one virtual outer
-// path whose "inner paths" are the real outer paths).  Padding lanes get 1.
-template <class VE>
-__global__ void curve_planes_lanes_kernel(double a, double b, double sigma, double dt, int n_outer, int n_nodes,
-                                          int o_pad, int Lmax, const int* __restrict__ Ln,
-                                          const double* __restrict__ r_node, VE* __restrict__ plane) {
-    const size_t total = (size_t)n_nodes * Lmax * o_pad;
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const int o = (int)(idx % o_pad);
-        const int t = (int)((idx / o_pad) % Lmax);
-        const int n = (int)(idx / ((size_t)o_pad * Lmax));
-        double v = 1.0;
-        if (o < n_outer && t < Ln[n]) {
-            const double r = r_node[(size_t)o * n_nodes + n];
-            v = exp(vasicek_lnP((t + 1) * dt, r, a, b, sigma) - vasicek_lnP(t * dt, r, a, b, sigma));
-        }
-        plane[idx] = to_plane<VE>(v);
-    }
+// The curve mode: L_{o,n} on the Vasicek forward curve of the node's rate, whose
+// discount products are the zero-coupon prices P(tau + 1 | r) = exp(A - B r); A and B
+// depend on the maturity alone (curve_ab), so a month costs one exponential.
+// One warp a (node, outer path), the lanes over the months, a fixed-order sum.
+__global__ void curve_ab_kernel(double a, double b, double sigma, double dt, int n_steps, double2* __restrict__ ab) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n_steps) return;
+    const double T = (t + 1) * dt;
+    ab[t] = make_double2(vasicek_lnP(T, 0.0, a, b, sigma), -expm1(-a * T) / a);
 }
 
-// L[o][n] = Lt[n][o] (the curve mode's node liabilities back to outer-major)
-__global__ void transpose_on_kernel(const double* __restrict__ Lt, int n_outer, int n_nodes, double* __restrict__ L) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_outer * n_nodes) return;
-    const int o = i / n_nodes, n = i - o * n_nodes;
-    L[i] = Lt[(size_t)n * n_outer + o];
-}
-
-// ------------------------------------------------------- nested recurrence ----
-// One CTA per item (o, n, chunk of 32 inner paths); its warps share the
-// policy tiles, each lane accumulates the pi-weighted reserves of its path,
-// and the CTA adds the warps' sums in a fixed order (deterministic).
-template <int FORM, int P, int NT>
-__global__ void __launch_bounds__(NT, NT == 128 ? 3 : 1) nested_kernel(const NestedArgs a) {
-    using TabE = typename Tr<FORM>::TabE;
-    using VE = typename Tr<FORM>::VE;
-    constexpr int NW = NT / 32;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ uint64_t bar;
-    __shared__ int s_item;
-    __shared__ double red[NW][32];
-    TabE* tab = reinterpret_cast<TabE*>(smem_raw);
-    if (!stage_to_smem(tab, a.tab, (uint32_t)a.tab_bytes, &bar, a.status)) return;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
-    for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(a.counter, 1);
-        __syncthreads();
-        const int item = s_item;
-        __syncthreads();
-        if (item >= a.n_items) break;
-        // items run node-major: early nodes (longest projections) first
-        const int chunk = item % a.n_chunks;
-        const int ol = (item / a.n_chunks) % a.B;
-        const int n = item / (a.n_chunks * a.B);
-        const int m = n * a.node_step;
-        const VE* plane = static_cast<const VE*>(a.v) + ((size_t)ol * a.n_nodes + n) * a.Lmax * a.i_pad;
-        const TileEnv env{a.slots, plane, a.i_pad, a.n_inner, 0, nullptr, nullptr, nullptr, a.n_inner};
-        const double* wts = a.wts + (size_t)n * 3;
-        const size_t wstride = (size_t)a.n_nodes * 3;
-        double acc[1] = {0.0};
-        for (int tile = warp; tile < a.n_tiles; tile += NW) {
-            if (a.slots[(size_t)tile * P].S < m) continue;   // whole tile ended before the node
-            const int kind = a.tile_kind[tile];
-            if (kind == K_JL) {
-                Tile<FORM, P, 1, K_JL, false> w(env, tab, tile, chunk, lane, m);
-                w.run_steps();
-                w.epilogue_weighted(acc, wts, wstride);
-            } else if (kind == K_ANN) {
-                Tile<FORM, P, 1, K_ANN, false> w(env, tab, tile, chunk, lane, m);
-                w.run_steps();
-                w.epilogue_weighted(acc, wts, wstride);
-            } else if (kind == K_ANN2) {
-                Tile<FORM, P, 1, K_ANN2, false> w(env, tab, tile, chunk, lane, m);
-                w.run_steps();
-                w.epilogue_weighted(acc, wts, wstride);
-            } else if (kind == K_ASS2) {
-                Tile<FORM, P, 1, K_ASS2, false> w(env, tab, tile, chunk, lane, m);
-                w.run_steps();
-                w.epilogue_weighted(acc, wts, wstride);
-            } else if (kind == K_LS2) {
-                Tile<FORM, P, 1, K_LS2, false> w(env, tab, tile, chunk, lane, m);
-                w.run_steps();
-                w.epilogue_weighted(acc, wts, wstride);
-            } else {
-                Tile<FORM, P, 1, K_ASS, false> w(env, tab, tile, chunk, lane, m);
-                w.run_steps();
-                w.epilogue_weighted(acc, wts, wstride);
-            }
-        }
-        red[warp][lane] = acc[0];
-        __syncthreads();
-        if (warp == 0) {
-            double sum = 0.0;
+__global__ void curve_value_kernel(const PathArgs a, const double2* __restrict__ ab) {
+    const int lane = threadIdx.x & 31;
+    const long long k = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;   // node-major
+    if (k >= (long long)a.n_outer * a.n_nodes) return;                            // whole warps leave together
+    const int n = (int)(k / a.n_outer), o = (int)(k - (long long)n * a.n_outer);
+    const int m = n * a.node_step, left = max(0, a.n_steps - m);
+    const double r = a.r_node[(size_t)o * a.n_nodes + n];
+    double L = 0.0;
+    for (int t = lane; t < left; t += 32) L = __fma_rn(exp(__fma_rn(-ab[t].y, r, ab[t].x)), a.flow[m + t], L);
 #pragma unroll
-            for (int w = 0; w < NW; ++w) sum += red[w][lane];
-            const int i = chunk * 32 + lane;
-            if (i < a.n_inner)
-                a.L_all[((size_t)(a.o0 + ol) * a.n_nodes + n) * a.n_inner + i] = sum;
-        }
-        __syncthreads();
-    }
+    for (int d = 16; d > 0; d >>= 1) L += __shfl_xor_sync(0xffffffffu, L, d);
+    if (lane == 0) a.L_all[(size_t)o * a.n_nodes + n] = (m <= a.n_steps ? a.due[m] : 0.0) + L;
 }
 
 // Mean and k-th largest over the inner paths of each (o, n), one CTA each.
@@ -415,282 +351,31 @@ __global__ void node_stats_kernel(const double* __restrict__ L_all, int n_inner,
     }
 }
 
-// ------------------------------------------- deflated brute-force mode ----
-// Inner paths as deflator planes: D_i(m, m+tau+1), the FP64 running product
-// of the path's monthly discount factors from the node, rounded to FP32, in
-// rows of four steps [B][n_nodes][G4][i_pad]; zeros from the node's remaining
-// length to the end of its last group of four.  One thread per path.
-__global__ void inner_paths_defl_kernel(VasStep s, uint64_t seed, int o_first, int o0, int B, int n_nodes, int n_inner, int i_pad,
-                                        int G4, const int* __restrict__ Ln, const double* __restrict__ r_node,
-                                        const double2* __restrict__ bm_g, float* __restrict__ plane) {
-    __shared__ double2 bm[BM_SC + BM_LG];   // 18 KiB: the Box-Muller tables
-    for (int k = threadIdx.x; k < BM_SC + BM_LG; k += blockDim.x) bm[k] = bm_g[k];
-    __syncthreads();
-    const size_t total = (size_t)B * n_nodes * i_pad;
-    for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total;
-         idx += (size_t)gridDim.x * blockDim.x) {
-        const int i = (int)(idx % i_pad);
-        const int n = (int)((idx / i_pad) % n_nodes);
-        const int ol = (int)(idx / ((size_t)i_pad * n_nodes));
-        const int o = o0 + ol;
-        // element (tau, i) at ((ol n_nodes + n) G4 + tau / 4) i_pad 4 + 4 i + tau % 4
-        float* base = plane + ((size_t)ol * n_nodes + n) * G4 * i_pad * 4 + 4 * (size_t)i;
-        const int L = Ln[n], Lr = (L + 3) / 4 * 4;
-        auto at = [&](int tau) -> float& { return base[(size_t)(tau >> 2) * i_pad * 4 + (tau & 3)]; };
-        if (i >= n_inner) {   // padding lanes: finite factors, never written out
-            for (int tau = 0; tau < Lr; ++tau) at(tau) = 1.0f;
-            continue;
-        }
-        double D = 1.0;
-        vasicek_path(s, seed, (uint32_t)i, (uint32_t)n, (3u << 24) | (uint32_t)(o_first + o),
-                     r_node[(size_t)o * n_nodes + n], L, bm, [&](int t, double v, double) {
-                         D = __dmul_rn(D, v);
-                         at(t) = __double2float_rn(D);
-                     });
-        for (int tau = L; tau < Lr; ++tau) at(tau) = 0.0f;
-    }
-}
-
-// Node liabilities by the deflated recurrence.  One CTA per item (node n,
-// outer path of the batch, chunk of 32 M inner paths); its NW warps share the
-// policy tiles, lane l holds inner paths chunk + m 32 + l of every policy of
-// its tile (P x M chains).  Per chain-step one FP32 fused multiply-add of the
-// path's deflator and the policy's expected cash flow (two accumulators on
-// alternate steps, folded into a double-float every 16 steps); per tile the
-// scaled sums are added into each path's double-float liability, and the
-// CTA adds its warps' liabilities in a fixed order in FP64.
-// One whole 16-step span from the node, groups g0 .. g0 - 3 (g0 = 3 mod 4),
-// the inner paths' deflator rows read from the plane (row stride i_pad).
-template <int KIND, int P, int M, bool CHECK, class Lane>
-__device__ __forceinline__ void nest_span(Lane& st, const DeflPol<P>& pp, const float4* __restrict__ tab,
-                                          const float4* __restrict__ plane, int i_pad, int g0) {
-    const float4* row = plane + (size_t)g0 * i_pad;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        float4 d[M];
-#pragma unroll
-        for (int q = 0; q < M; ++q) d[q] = row[q * 32];
-        row -= i_pad;
-        if (u == 0) defl_group<KIND, P, M, true>(st, pp, tab, d, g0 - u, CHECK);
-        else defl_group<KIND, P, M, false>(st, pp, tab, d, g0 - u, CHECK);
-    }
-    defl_fold_all(st);
-}
-
-template <int P, int M, int NW>
-__global__ void __launch_bounds__(NW * 32, 2) nested_defl_kernel(const NestDeflArgs a) {
-    using Lane = DeflLaneX2<P, M>;   // packed pairs, as the valuation kernel
-    constexpr int CH = 32 * M;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ uint64_t bar;
-    __shared__ int s_item;
-    __shared__ float2 red[NW][CH];
-    if (!stage_to_smem(smem_raw, a.tab, (uint32_t)a.tab_bytes, &bar, a.status)) return;
-    const float4* tab = reinterpret_cast<const float4*>(smem_raw);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int dpad4 = a.dpad / 4;
-
-    for (;;) {
-        if (threadIdx.x == 0) s_item = atomicAdd(a.counter, 1);
-        __syncthreads();
-        const int item = s_item;
-        __syncthreads();
-        if (item >= a.n_items) break;
-        // node-major: the early nodes (longest projections) first
-        const int chunk = item % a.n_chunks;
-        const int ol = (item / a.n_chunks) % a.B;
-        const int n = item / (a.n_chunks * a.B);
-        const int m = n * a.node_step;
-        const float4* plane = a.D + ((size_t)ol * a.n_nodes + n) * a.G4 * a.i_pad + (size_t)chunk * CH + lane;
-        float acc_h[M], acc_l[M];
-#pragma unroll
-        for (int q = 0; q < M; ++q) acc_h[q] = acc_l[q] = 0.0f;
-        for (int tile = warp; tile < a.n_tiles; tile += NW) {
-            const NestSlot* rec = a.slots + (size_t)tile * P;
-            if (rec[0].S < m) continue;   // the tile's longest policy ended before the node
-            const int kind = a.tile_kind[tile];
-            // the runs of the tile's policies from the node
-            DeflPol<P> pp;
-            int smin = 1 << 30, smax = 0;
-            Lane st;
-            float h0s[P][M];
-#pragma unroll
-            for (int i = 0; i < P; ++i) {
-                const NestSlot r = rec[i];
-                int S = r.S - m;
-                const bool live = r.pol >= 0 && S >= 0 && !(r.unit && m > 0);
-                if (!live) S = 0;
-                pp.S[i] = S;
-                smin = min(smin, S);
-                smax = max(smax, S);
-                pp.ix[i] = r.ix;
-                pp.iy[i] = r.iy;
-                // life 1: aligned run at age + m, or a zero group; the unit group at node 0
-                const int a1 = r.age1 + m;
-                if (r.unit) {
-                    pp.off1[i] = r.base1 + (a.dpad - 8) / 4;
-                    pp.gz1[i] = 1;
-                } else if (a1 >= r.z1) {
-                    pp.off1[i] = r.base1 + (r.z1 + 3) / 4;
-                    pp.gz1[i] = 0;
-                } else {
-                    pp.off1[i] = r.base1 + (a1 & 3) * dpad4 + (a1 >> 2);
-                    pp.gz1[i] = (r.z1 - a1 + 3) / 4;
-                }
-                const int a2 = r.age2 + m;
-                if (a2 >= r.z2) {
-                    pp.off2[i] = r.base2 + (r.z2 + 3) / 4;
-                    pp.gz2[i] = 0;
-                } else {
-                    pp.off2[i] = r.base2 + (a2 & 3) * dpad4 + (a2 >> 2);
-                    pp.gz2[i] = (r.z2 - a2 + 3) / 4;
-                }
-#pragma unroll
-                for (int q = 0; q < M; ++q) {   // the boundary D(m, S) mat
-                    float h0 = 0.0f;
-                    if (live && r.mat != 0.0f) {
-                        float dS = 1.0f;
-                        if (S > 0) dS = reinterpret_cast<const float*>(plane + (size_t)((S - 1) >> 2) * a.i_pad + q * 32)[(S - 1) & 3];
-                        h0 = __fmul_rn(dS, r.mat);
-                    }
-                    h0s[i][q] = h0;
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < P; ++i) st.start(i, h0s[i]);
-            st.clear_acc();
-            if (smax > 0) {
-                // groups of four steps from the node, descending; 16-step spans
-                // aligned at the node (a span opens at g = 3 mod 4 and is folded at
-                // g = 0 mod 4; the top span may be partial and starts from zero)
-                const int g_top = (smax - 1) >> 2;
-                auto run = [&](auto kind_c) {
-                    constexpr int KIND = decltype(kind_c)::value;
-                    int g = g_top;
-#pragma unroll 1
-                    for (; g >= 0 && (g & 3) != 3; --g) {   // the partial top span
-                        float4 d[M];
-#pragma unroll
-                        for (int q = 0; q < M; ++q) d[q] = plane[(size_t)g * a.i_pad + q * 32];
-                        defl_group<KIND, P, M, false>(st, pp, tab, d, g, true);
-                        if ((g & 3) == 0) defl_fold_all(st);
-                    }
-                    // whole spans g .. g - 3; only those reaching a policy's end check
-#pragma unroll 1
-                    for (; g >= 3; g -= 4) {
-                        if (4 * g + 3 >= smin) nest_span<KIND, P, M, true>(st, pp, tab, plane, a.i_pad, g);
-                        else nest_span<KIND, P, M, false>(st, pp, tab, plane, a.i_pad, g);
-                    }
-                };
-                if (kind == K_ANN) run(std::integral_constant<int, K_ANN>{});
-                else if (kind == K_ASS) run(std::integral_constant<int, K_ASS>{});
-                else if (kind == K_JL) run(std::integral_constant<int, K_JL>{});
-                else run(std::integral_constant<int, K_ANN2>{});
-            }
-            // this tile's scaled sums into the paths' liabilities
-#pragma unroll
-            for (int i = 0; i < P; ++i) {
-                const float sh = rec[i].sc_h, sl = rec[i].sc_l;
-                float Hs[M], Ls[M];
-                st.sum(i, Hs, Ls);
-#pragma unroll
-                for (int q = 0; q < M; ++q) {
-                    const float H = Hs[q], L = Ls[q];
-                    const float p = __fmul_rn(H, sh);
-                    float e = __fmaf_rn(H, sh, -p);
-                    e = __fmaf_rn(H, sl, e);
-                    e = __fmaf_rn(L, sh, e);
-                    defl_fold(acc_h[q], acc_l[q], p);
-                    acc_l[q] = __fadd_rn(acc_l[q], e);
-                }
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < M; ++q) red[warp][q * 32 + lane] = make_float2(acc_h[q], acc_l[q]);
-        __syncthreads();
-        if (warp == 0) {
-#pragma unroll
-            for (int q = 0; q < M; ++q) {
-                double x = 0.0;
-                for (int w = 0; w < NW; ++w) {
-                    const float2 v = red[w][q * 32 + lane];
-                    x += (double)v.x + (double)v.y;
-                }
-                const int i = chunk * CH + q * 32 + lane;
-                if (i < a.n_inner) a.L_all[((size_t)(a.o0 + ol) * a.n_nodes + n) * a.n_inner + i] = x;
-            }
-        }
-        __syncthreads();
-    }
-}
-
 // ------------------------------------------------------------- launchers ----
-cudaError_t launch_inner_paths_defl(const VasStep& s, uint64_t seed, int o_first, int o0, int B, int n_nodes, int n_inner,
-                                    int i_pad, int G4, const int* Ln, const double* r_node, const double2* bm,
-                                    float4* plane, int sm_count, int ctas_per_sm, cudaStream_t st) {
-    inner_paths_defl_kernel<<<sm_count * ctas_per_sm, 128, 0, st>>>(s, seed, o_first, o0, B, n_nodes, n_inner, i_pad, G4, Ln, r_node, bm,
-                                                          reinterpret_cast<float*>(plane));
+cudaError_t launch_nested_paths(const VasStep& s, const NestedRun& q, cudaStream_t st) {
+    const long long per_node = (long long)q.n_outer * q.n_inner;
+    const long long blocks = (per_node + kPathNT - 1) / kPathNT * q.n_nodes;
+    const int grid = (int)std::min<long long>(blocks, 0x7fffffffLL);
+    PathArgs a{q.seed, q.o_first, q.n_outer, q.n_nodes, q.node_step, q.n_inner, q.n_steps,
+               q.r_node, q.tables, q.flow, q.due, q.L_all};
+    inner_paths_kernel<<<grid, kPathNT, 0, st>>>(s, a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_nested_defl(const NestDeflArgs& a, int sm_count, int max_per_sm, cudaStream_t st) {
-    constexpr int P = kNestDeflP, M = 2, NW = 8;
-    auto k = nested_defl_kernel<P, M, NW>;
-    const size_t smem = (size_t)a.tab_bytes;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+cudaError_t launch_nested_curve(const NestedRun& q, double2* ab, cudaStream_t st) {
+    PathArgs a{q.seed, q.o_first, q.n_outer, q.n_nodes, q.node_step, 1, q.n_steps,
+               q.r_node, nullptr, q.flow, q.due, q.L_all};
+    if (q.n_steps > 0) curve_ab_kernel<<<(q.n_steps + 127) / 128, 128, 0, st>>>(q.a, q.b, q.sigma, 1.0 / 12.0, q.n_steps, ab);
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    int bps = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k, NW * 32, smem);
-    if (e != cudaSuccess) return e;
-    if (bps < 1) return cudaErrorInvalidConfiguration;
-    const long long grid = std::min<long long>((long long)sm_count * std::min(bps, max_per_sm), std::max(1, a.n_items));
-    k<<<(int)grid, NW * 32, smem, st>>>(a);
+    const long long warps = (long long)q.n_outer * q.n_nodes;
+    curve_value_kernel<<<(unsigned)((warps + 3) / 4), 128, 0, st>>>(a, ab);
     return cudaGetLastError();
-}
-
-template <int FORM, int P, int NT>
-cudaError_t launch_nested_t(const NestedArgs& a, int sm_count, size_t smem, cudaStream_t st) {
-    auto k = nested_kernel<FORM, P, NT>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    int bps = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k, NT, smem);
-    if (e != cudaSuccess) return e;
-    if (bps < 1) return cudaErrorInvalidConfiguration;
-    const long long grid = std::min<long long>((long long)sm_count * bps, std::max(1, a.n_items));
-    k<<<(int)grid, NT, smem, st>>>(a);
-    return cudaGetLastError();
-}
-
-int nested_tile_width(int form) { return form == F_F32 ? 4 : (form == F_COMP ? 6 : 2); }
-
-cudaError_t launch_nested(int form, const NestedArgs& a, int sm_count, size_t smem, cudaStream_t st) {
-    switch (form) {
-    case F_F64: return launch_nested_t<F_F64, 2, 256>(a, sm_count, smem, st);
-    case F_F32: return launch_nested_t<F_F32, 4, 256>(a, sm_count, smem, st);
-    default: return launch_nested_t<F_COMP, 6, 128>(a, sm_count, smem, st);
-    }
 }
 
 cudaError_t launch_outer_paths(const VasStep& s, uint64_t seed, int o_first, int n_outer, int n_nodes, int node_step, double r0,
                                double* r_node, double* d0, cudaStream_t st) {
     outer_paths_kernel<<<(n_outer + 3) / 4, 128, 0, st>>>(s, seed, o_first, n_outer, n_nodes, node_step, r0, r_node, d0);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_inner_paths(int form, const VasStep& s, uint64_t seed, int o_first, int o0, int B, int n_nodes, int n_inner,
-                               int i_pad, int Lmax, const int* Ln, const double* r_node, const double2* bm,
-                               void* plane, int sm_count, cudaStream_t st) {
-    const int grid = sm_count * 8;
-    if (form == F_F64)
-        inner_paths_kernel<double><<<grid, 128, 0, st>>>(s, seed, o_first, o0, B, n_nodes, n_inner, i_pad, Lmax, Ln, r_node,
-                                                          bm, static_cast<double*>(plane));
-    else if (form == F_F32)
-        inner_paths_kernel<float><<<grid, 128, 0, st>>>(s, seed, o_first, o0, B, n_nodes, n_inner, i_pad, Lmax, Ln, r_node,
-                                                         bm, static_cast<float*>(plane));
-    else
-        inner_paths_kernel<float2><<<grid, 128, 0, st>>>(s, seed, o_first, o0, B, n_nodes, n_inner, i_pad, Lmax, Ln, r_node,
-                                                          bm, static_cast<float2*>(plane));
     return cudaGetLastError();
 }
 
@@ -708,30 +393,6 @@ __global__ void generator_math_kernel(const uint32_t* __restrict__ w, const doub
         out[4 * i + 2] = cs;
         out[4 * i + 3] = exp_small(x[i]);
     }
-}
-
-cudaError_t launch_curve_planes_lanes(int form, double a, double b, double sigma, int n_outer, int n_nodes, int o_pad,
-                                      int Lmax, const int* Ln, const double* r_node, void* plane, int sm_count,
-                                      cudaStream_t st) {
-    const int grid = sm_count * 8;
-    const double dt = 1.0 / 12.0;
-    if (form == F_F64)
-        curve_planes_lanes_kernel<double><<<grid, 128, 0, st>>>(a, b, sigma, dt, n_outer, n_nodes, o_pad, Lmax, Ln,
-                                                                 r_node, static_cast<double*>(plane));
-    else if (form == F_F32)
-        curve_planes_lanes_kernel<float><<<grid, 128, 0, st>>>(a, b, sigma, dt, n_outer, n_nodes, o_pad, Lmax, Ln,
-                                                                r_node, static_cast<float*>(plane));
-    else
-        curve_planes_lanes_kernel<float2><<<grid, 128, 0, st>>>(a, b, sigma, dt, n_outer, n_nodes, o_pad, Lmax, Ln,
-                                                                 r_node, static_cast<float2*>(plane));
-    return cudaGetLastError();
-}
-
-cudaError_t launch_transpose_on(const double* Lt, int n_outer, int n_nodes, double* L, cudaStream_t st) {
-    const int n = n_outer * n_nodes;
-    if (n <= 0) return cudaSuccess;
-    transpose_on_kernel<<<(n + 255) / 256, 256, 0, st>>>(Lt, n_outer, n_nodes, L);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_node_stats(const double* L_all, int n_on, int n_inner, int k, double* mean, double* kth,

@@ -18,6 +18,7 @@
 #include "rsv.h"
 #include "abi_guard.cuh"
 #include "ctx.cuh"
+#include "cashflow.cuh"
 #include "nested.cuh"
 #include "scan.cuh"
 #include "summation.cuh"
@@ -531,11 +532,17 @@ rsv_status rsv::build_tables(rsv_ctx* c, int form, size_t& smem) {
     return stage_tables(c, form, c->lay.tab_pad, c->lay.n_tab, smem);
 }
 
-rsv_status rsv::stage_tables(rsv_ctx* c, int form, int pad, int n_tab, size_t& smem) {
+rsv_status rsv::table_bytes(rsv_ctx* c, int form, int pad, int n_tab, size_t& smem) {
     const size_t esz = form == F_F32 ? sizeof(float2) : 16;
     smem = (size_t)n_tab * pad * esz;
     if (smem > kMaxSmem)
         return fail(c, RSV_E_ARG, "decrement tables need %zu bytes of shared memory (max %zu)", smem, kMaxSmem);
+    return RSV_OK;
+}
+
+rsv_status rsv::stage_tables(rsv_ctx* c, int form, int pad, int n_tab, size_t& smem) {
+    const rsv_status st = table_bytes(c, form, pad, n_tab, smem);
+    if (st != RSV_OK) return st;
     if (c->tab_pad_of[form] == pad && c->n_tab_of[form] == n_tab && c->tab_gen_of[form] == c->tab_gen)
         return RSV_OK;
     std::vector<unsigned char> h(smem);
@@ -831,8 +838,7 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     return RSV_OK;
 }
 
-// In-force weights amount x Pr[reduced state j at node n] (FP64), the
-// remaining projection length per node, and the nested launch sequence.
+// The nested run: outer paths, then every (node, outer path, inner path) by its mode.
 rsv_status compute_nested(rsv_ctx* c, const rsv_opts* o, const rsv_nested_spec* sp, rsv_nested_out* out) {
     if (!o || !sp || !out) return fail(c, RSV_E_ARG, "opts, spec and out must not be NULL");
     if (o->form < F_F64 || o->form > F_DEFL) return fail(c, RSV_E_ARG, "bad form %d", o->form);
@@ -861,86 +867,29 @@ rsv_status compute_nested(rsv_ctx* c, const rsv_opts* o, const rsv_nested_spec* 
     for (auto& t : c->tab) any_tab |= !t.empty();
     if (!any_tab) return fail(c, RSV_E_STATE, "no decrement table loaded");
 
-    // The deflated form values the brute-force mode in deflated units; the
-    // curve and surrogate modes run it compensated.
-    const bool mc = sp->mode == RSV_NESTED_MC;
+    // The brute-force and curve modes value the portfolio's expected cash flows
+    // (one policy per layout tile); what the forms refuse of products and tables
+    // stays refused.
+    const bool mc = sp->mode == RSV_NESTED_MC, sur = sp->mode == RSV_NESTED_SURROGATE;
+    const bool curve = sp->mode == RSV_NESTED_CURVE;
     const bool defl = o->form == F_DEFL && mc;
     const int form = o->form == F_DEFL && !mc ? F_COMP : o->form;
-    const int P = defl ? kNestDeflP : nested_tile_width(form);
-    rsv_status st = build_layout(c, P, 0, kMaxAgeSteps);
-    if (st == RSV_OK) st = layout_to_device(c);
+    rsv_status st = build_layout(c, 1, 0, kMaxAgeSteps);
     if (st != RSV_OK) return st;
+    const Layout& L = c->lay;
     size_t smem = 0;
-    DeflTabs T;
     if (defl) {
-        if ((st = defl_table_shape(c, c->lay, T)) != RSV_OK) return st;
-        if ((st = defl_table_stage(c, T)) != RSV_OK) return st;
-        smem = T.bytes;
-    } else if ((st = build_tables(c, form, smem)) != RSV_OK) {
+        DeflTabs T;
+        if ((st = defl_table_shape(c, L, T)) != RSV_OK) return st;
+        if ((st = defl_table_range(c, T)) != RSV_OK) return st;
+    } else if ((st = table_bytes(c, form, L.tab_pad, L.n_tab, smem)) != RSV_OK) {
         return st;
     }
-    const Layout& L = c->lay;
     const int n_pol = (int)c->pols.size(), NN = sp->n_nodes, NO = sp->n_outer, step = sp->node_step_m;
-    const bool sur = sp->mode == RSV_NESTED_SURROGATE;
     const int n_inner = mc ? sp->n_inner : 1;
-    const int i_pad = defl ? (n_inner + 63) / 64 * 64 : (n_inner + 31) / 32 * 32;
 
-    // weights and remaining lengths
-    std::vector<double> w((size_t)std::max(1, n_pol) * NN * 3, 0.0);
-    std::vector<int> Ln(NN, 0), Sp(std::max(1, n_pol), 0);
-    for (int p = 0; p < n_pol; ++p) {
-        const rsv_policy& r = c->pols[p];
-        ProductModel pm;
-        product_model(r.product, pm);   // validated by build_layout
-        const bool jl = pm.multi_state, two = pm.two_life, ann = pm.annuity;
-        const int S = product_steps(r, table_len(c, r.table1), two ? table_len(c, r.table2) : 0);
-        Sp[p] = S;
-        const std::vector<double>& tx = c->tab[r.table1];
-        const std::vector<double>& ty = c->tab[two ? r.table2 : r.table1];
-        double Px = 1.0, Py = 1.0;
-        int u = 0;
-        for (int n = 0; n < NN; ++n) {
-            const int m = n * step;
-            for (; u < m; ++u) {
-                Px *= (r.age1_m + u < (int)tx.size()) ? tx[r.age1_m + u] : 0.0;
-                if (two) Py *= (r.age2_m + u < (int)ty.size()) ? ty[r.age2_m + u] : 0.0;
-            }
-            if (S < m || (ann && r.term_m > 0 && r.term_m <= m)) continue;   // ended before the node
-            Ln[n] = std::max(Ln[n], S - m);
-            double* wp = &w[((size_t)p * NN + n) * 3];
-            if (!jl) {
-                wp[0] = two ? r.amount * Px * Py : r.amount * Px;   // joint products: both alive
-            } else if (r.state0 == 0) {
-                wp[0] = r.amount * Px * Py;
-                wp[1] = r.amount * Px * (1.0 - Py);
-                wp[2] = r.amount * (1.0 - Px) * Py;
-            } else if (r.state0 == 1) {
-                wp[1] = r.amount * Px;
-            } else {
-                wp[2] = r.amount * Py;
-            }
-        }
-    }
-    const int Lmax = std::max(1, *std::max_element(Ln.begin(), Ln.end()));
-    const int G4 = (Lmax + 3) / 4;   // the deflated planes' rows of four steps
-    const size_t esz = form == F_F32 ? sizeof(float) : 8;
-    const size_t per_outer = defl ? (size_t)NN * G4 * i_pad * sizeof(float4) : (size_t)NN * Lmax * i_pad * esz;
-    int B = sp->batch_outer > 0 ? sp->batch_outer : (int)std::max<size_t>(1, (size_t(4) << 30) / per_outer);
-    // the deflated brute force pipelines the generator of batch i + 1 with the
-    // valuation of batch i: two plane buffers, and at least eight batches so
-    // that the first and last stages are short
-    if (defl && sp->batch_outer <= 0) B = std::max(1, std::min(B / 2, (NO + 7) / 8));
-    B = std::min(B, NO);
-
-    CU(c->d_nest_w.ensure(w.size() * sizeof(double)));
-    CU(c->d_nest_ln.ensure(NN * sizeof(int)));
     CU(c->d_nest_rn.ensure((size_t)NO * NN * sizeof(double)));
     CU(c->d_nest_d0.ensure((size_t)NO * NN * sizeof(double)));
-    const bool curve = sp->mode == RSV_NESTED_CURVE;
-    const int o_pad = (NO + 31) / 32 * 32;   // the curve mode: outer paths on the lanes
-    const size_t curve_plane = (size_t)NN * Lmax * o_pad * esz;
-    if (curve) CU(c->d_nest_plane.ensure(curve_plane + (size_t)NN * NO * sizeof(double)));
-    else if (!sur) CU(c->d_nest_plane.ensure((size_t)(defl ? 2 : 1) * B * per_outer));
     CU(c->d_nest_mean.ensure((size_t)NO * NN * sizeof(double)));
     CU(c->d_nest_kth.ensure((size_t)NO * NN * sizeof(double)));
     double* Lall = (o->on_device && out->L_all) ? out->L_all : nullptr;
@@ -949,55 +898,116 @@ rsv_status compute_nested(rsv_ctx* c, const rsv_opts* o, const rsv_nested_spec* 
         Lall = c->d_nest_all.as<double>();
     }
     CU(c->d_ctl.ensure(2 * sizeof(int32_t)));
-    CU(cudaMemcpyAsync(c->d_nest_w.p, w.data(), w.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-    CU(cudaMemcpyAsync(c->d_nest_ln.p, Ln.data(), NN * sizeof(int), cudaMemcpyHostToDevice, c->stream));
     CU(cudaMemsetAsync(c->d_ctl.p, 0, 2 * sizeof(int32_t), c->stream));
 
     const VasStep vs = vasicek_step_constants(sp->a, sp->b, sp->sigma, 1.0 / 12.0);
+    CfTables T;
+    const int T_max = L.max_S;
+    if (!sur) {   // uploads before the timed kernels
+        if ((st = layout_to_device(c)) != RSV_OK || (st = upload_amounts(c)) != RSV_OK || (st = cf_tables(c, T)) != RSV_OK)
+            return st;
+        if (mc && !c->nest_bm_ready) {
+            CU(c->d_nest_bm.ensure((size_t)(BM_SC + BM_LG) * sizeof(double2)));
+            CU(cudaMemcpyAsync(c->d_nest_bm.p, bm_tables_host(), (size_t)(BM_SC + BM_LG) * sizeof(double2),
+                               cudaMemcpyHostToDevice, c->stream));
+            c->nest_bm_ready = true;
+        }
+        CU(c->d_cf_pol.ensure((size_t)std::max(1, n_pol) * sizeof(CfPol)));
+        // scratch of the splits | curve's A, B | flow | due
+        CU(c->d_cf_sum.ensure(((size_t)2 * kCfSplits + 4) * (T_max + 1) * sizeof(double)));
+    }
     CU(cudaEventRecord(c->ev0, c->stream));
     CU(launch_outer_paths(vs, sp->seed, sp->outer_first, NO, NN, step, sp->r0, c->d_nest_rn.as<double>(), c->d_nest_d0.as<double>(),
                           c->stream));
-    NestedArgs a{};
-    a.tab = c->d_tab[form].p;
-    a.tab_bytes = (int32_t)smem;
-    a.v = c->d_nest_plane.p;
-    a.i_pad = i_pad;
-    a.n_inner = n_inner;
-    a.Lmax = Lmax;
-    a.n_nodes = NN;
-    a.node_step = step;
-    a.slots = L.slots.as<SlotRec>();
-    a.tile_kind = L.kinds.as<int32_t>();
-    a.n_tiles = L.n_tiles;
-    a.wts = c->d_nest_w.as<double>();
-    a.n_chunks = i_pad / 32;
-    a.counter = c->d_ctl.as<int32_t>();
-    a.status = c->d_ctl.as<int32_t>() + 1;
-    a.L_all = Lall;
+    if (!sur) {
+        double* part = c->d_cf_sum.as<double>();
+        double* ab = part + (size_t)2 * kCfSplits * (T_max + 1);   // first: 16-byte aligned
+        double* flow = ab + 2 * (size_t)(T_max + 1);
+        double* due = flow + (T_max + 1);
+        CfPol* recs = c->d_cf_pol.as<CfPol>();
+        CU(launch_cf_records(T, L.slots.as<SlotRec>(), L.kinds.as<int32_t>(), c->d_amount.as<double>(), L.n_tiles, L.tab_pad,
+                             recs, c->stream));
+        CU(launch_cf_portfolio(T, recs, L.n_tiles, T_max, part, flow, due, c->stream));
+        const NestedRun run{sp->seed, sp->a, sp->b, sp->sigma, sp->r0, sp->outer_first, NO, NN, step, n_inner, T_max,
+                            c->d_nest_rn.as<double>(), c->d_nest_bm.p, flow, due, Lall};
+        if (curve) {
+            CU(launch_nested_curve(run, reinterpret_cast<double2*>(ab), c->stream));
+        } else {
+            CU(launch_nested_paths(vs, run, c->stream));
+        }
+    }
     if (sur) {
-        // one query per in-force (policy, state) and (outer path, node), at the
+        // One query per in-force (policy, state) and (outer path, node), at the
         // node's rate; the lists depend on the node only and are expanded over
-        // the outer paths on the device
-        const size_t on_n = (size_t)NO * NN;
+        // the outer paths on the device.  The weights are amount x Pr[reduced
+        // state j at node n] (FP64), in closed form from the survivor columns, a
+        // node to a host part.
+        if ((st = cf_tables(c, T)) != RSV_OK) return st;
+        const size_t cols = (size_t)L.n_tab * T.rows;
+        const double* hm = c->h_cf_tab.data();
+        const int32_t* hz = reinterpret_cast<const int32_t*>(hm + 2 * cols);
+        const int32_t* hex = hz + cols;
+        auto alive = [&](int table, int age, int m) {
+            const size_t i = (size_t)table * T.rows + age;
+            if (m > hz[i] - age) return 0.0;
+            const int d = hex[i + m] - hex[i];
+            return d > 1 ? 0.0 : hm[i + m] / hm[i] * (d ? 0x1p-512 : 1.0);
+        };
+        struct Node {
+            std::vector<rsv_query> q;
+            std::vector<double> w;
+            double base = 0.0;
+            int left = 0;
+        };
+        std::vector<Node> nodes(NN);
+        const int parts = std::max(1, std::min(std::min(NN, 16), (int)((long long)n_pol * NN / 4096)));
+        run_parts(parts, [&](int part) {
+            for (int n = part; n < NN; n += parts) {
+                Node& nd = nodes[n];
+                const int m = n * step;
+                nd.q.reserve(n_pol);
+                nd.w.reserve(n_pol);
+                for (int p = 0; p < n_pol; ++p) {
+                    const rsv_policy& r = c->pols[p];
+                    ProductModel pm;
+                    product_model(r.product, pm);   // validated by build_layout
+                    const int S = product_steps(r, table_len(c, r.table1), pm.two_life ? table_len(c, r.table2) : 0);
+                    if (S < m || (pm.annuity && r.term_m > 0 && r.term_m <= m)) continue;   // ended before the node
+                    nd.left = std::max(nd.left, S - m);
+                    const double Px = alive(r.table1, r.age1_m, m);
+                    const double Py = pm.two_life ? alive(r.table2, r.age2_m, m) : 1.0;
+                    double w[3] = {0.0, 0.0, 0.0};
+                    if (!pm.multi_state) {
+                        w[0] = r.amount * Px * Py;   // joint products: both alive
+                    } else if (r.state0 == 0) {
+                        w[0] = r.amount * Px * Py;
+                        w[1] = r.amount * Px * (1.0 - Py);
+                        w[2] = r.amount * (1.0 - Px) * Py;
+                    } else {
+                        w[r.state0] = r.amount * (r.state0 == 1 ? Px : Py);
+                    }
+                    for (int j = 0; j < 3; ++j) {
+                        if (w[j] == 0.0) continue;
+                        if (S == m) {   // matures at the node: its boundary value, no projection
+                            nd.base += pm.bnd * w[j];
+                            continue;
+                        }
+                        nd.q.push_back(rsv_query{p, m, j, 0, 0.0});
+                        nd.w.push_back(w[j]);
+                    }
+                }
+            }
+        });
+        int Lmax = 1;
         std::vector<rsv_query> nq;
         std::vector<double> nw, nbase(NN, 0.0);
         std::vector<long long> noff(NN + 1, 0);
         for (int n = 0; n < NN; ++n) {
             noff[n] = (long long)nq.size();
-            const int m = n * step;
-            for (int p = 0; p < n_pol; ++p)
-                for (int j = 0; j < 3; ++j) {
-                    const double wj = w[((size_t)p * NN + n) * 3 + j];
-                    if (wj == 0.0) continue;
-                    if (Sp[p] == m) {   // matures at the node: its boundary value, no projection
-                        ProductModel pm;
-                        product_model(c->pols[p].product, pm);
-                        nbase[n] += pm.bnd * wj;
-                        continue;
-                    }
-                    nq.push_back(rsv_query{p, m, j, 0, 0.0});
-                    nw.push_back(wj);
-                }
+            nq.insert(nq.end(), nodes[n].q.begin(), nodes[n].q.end());
+            nw.insert(nw.end(), nodes[n].w.begin(), nodes[n].w.end());
+            nbase[n] = nodes[n].base;
+            Lmax = std::max(Lmax, nodes[n].left);
         }
         noff[NN] = (long long)nq.size();
         const long long Qn = (long long)nq.size();
@@ -1048,175 +1058,6 @@ rsv_status compute_nested(rsv_ctx* c, const rsv_opts* o, const rsv_nested_spec* 
         }
         if (out->n_fallback) *out->n_fallback = nfb;
     }
-    if (curve) {
-        // one virtual outer path whose "inner paths" are the outer paths: every
-        // lane carries a different outer path's curve, all sharing the weights
-        double* Lt = reinterpret_cast<double*>(static_cast<char*>(c->d_nest_plane.p) + curve_plane);
-        CU(launch_curve_planes_lanes(form, sp->a, sp->b, sp->sigma, NO, NN, o_pad, Lmax, c->d_nest_ln.as<int>(),
-                                     c->d_nest_rn.as<double>(), c->d_nest_plane.p, c->sm_count, c->stream));
-        NestedArgs ac = a;
-        ac.i_pad = o_pad;
-        ac.n_inner = NO;
-        ac.n_chunks = o_pad / 32;
-        ac.B = 1;
-        ac.o0 = 0;
-        ac.n_items = NN * ac.n_chunks;
-        ac.L_all = Lt;
-        CU(cudaMemsetAsync(c->d_ctl.p, 0, sizeof(int32_t), c->stream));
-        if (L.n_tiles > 0) CU(launch_nested(form, ac, c->sm_count, smem, c->stream));
-        else CU(cudaMemsetAsync(Lt, 0, (size_t)NN * NO * sizeof(double), c->stream));
-        CU(launch_transpose_on(Lt, NO, NN, Lall, c->stream));
-    }
-    if (!sur && !curve && !c->nest_bm_ready) {   // the generator's tables: once per context (static host copy)
-        CU(c->d_nest_bm.ensure((size_t)(BM_SC + BM_LG) * sizeof(double2)));
-        CU(cudaMemcpyAsync(c->d_nest_bm.p, bm_tables_host(), (size_t)(BM_SC + BM_LG) * sizeof(double2),
-                           cudaMemcpyHostToDevice, c->stream));
-        c->nest_bm_ready = true;
-    }
-    NestDeflArgs da{};
-    if (defl) {   // policy slots of the deflated tiles: runs, scales, boundary weights
-        std::vector<NestSlot> ns(L.h_s2.size());
-        for (int f = 0; f < L.n_tiles; ++f) {
-            const int kind = L.h_k2[f];
-            for (int k = 0; k < P; ++k) {
-                const SlotRec& r = L.h_s2[(size_t)f * P + k];
-                NestSlot d{};
-                const int tb1 = r.idx1 / L.tab_pad, a1 = r.idx1 % L.tab_pad;
-                const int tb2 = r.idx2 / L.tab_pad, a2 = r.idx2 % L.tab_pad;
-                const int arr1 = kind == K_ASS ? T.arr_d : 0;
-                d.base1 = (arr1 * T.n_tab + tb1) * T.dpad;   // float4 index of copy 0: 4 dpad floats per copy
-                d.base2 = (0 * T.n_tab + tb2) * T.dpad;
-                d.age1 = a1;
-                d.age2 = a2;
-                d.z1 = (int)c->tab[tb1].size() + (kind == K_ASS ? 1 : 0);
-                d.z2 = (int)c->tab[tb2].size();
-                d.S = r.S;
-                d.pol = r.pol;
-                d.kind = kind;
-                auto ell_at = [&](int tb, int a) { return a < (int)T.ell[tb].size() ? T.ell[tb][a] : 0.0; };
-                const double lx = ell_at(tb1, a1), ly = ell_at(tb2, a2);
-                const double amount = r.pol >= 0 ? c->pols[r.pol].amount : 0.0;
-                const double rho = (double)r.rho_h + (double)r.rho_l;
-                double scale = 0.0;
-                if (kind == K_ANN || kind == K_ASS) {
-                    scale = lx > 0.0 ? amount / lx : 0.0;
-                    if (kind == K_ASS && r.bnd != 0.0f) d.mat = (float)((double)r.bnd * ell_at(tb1, a1 + r.S));
-                    if (kind == K_ASS && r.S == 0) {
-                        scale = amount;
-                        d.mat = r.bnd;
-                    } else if (kind == K_ASS && !(lx > 0.0)) {
-                        scale = amount;
-                        d.mat = 0.0f;
-                        d.unit = 1;
-                    }
-                } else {
-                    scale = amount;
-                    const double ix = lx > 0.0 ? 1.0 / lx : 0.0, iy = ly > 0.0 ? 1.0 / ly : 0.0;
-                    if (kind == K_ANN2) {
-                        d.ix = (float)ix;
-                        d.iy = (float)iy;
-                    } else {
-                        d.ix = r.state0 == 2 ? 0.0f : (float)ix;
-                        d.iy = r.state0 == 1 ? 0.0f : (float)(rho * iy);
-                    }
-                }
-                d.sc_h = (float)scale;
-                d.sc_l = (float)(scale - (double)d.sc_h);
-                ns[(size_t)f * P + k] = d;
-            }
-        }
-        CU(c->d_defl_slots.ensure(std::max<size_t>(1, ns.size()) * sizeof(NestSlot)));
-        CU(c->d_defl_kinds.ensure(std::max<size_t>(1, L.h_k2.size()) * sizeof(int32_t)));
-        if (!ns.empty()) {
-            CU(cudaMemcpyAsync(c->d_defl_slots.p, ns.data(), ns.size() * sizeof(NestSlot), cudaMemcpyHostToDevice,
-                               c->stream));
-            CU(cudaMemcpyAsync(c->d_defl_kinds.p, L.h_k2.data(), L.h_k2.size() * sizeof(int32_t),
-                               cudaMemcpyHostToDevice, c->stream));
-        }
-        c->defl_lay_key = 0;   // the valuation's slot records were overwritten
-        da.tab = c->d_defl_tab.as<float>();
-        da.tab_bytes = (int32_t)T.bytes;
-        da.dpad = T.dpad;
-        da.D = c->d_nest_plane.as<float4>();
-        da.i_pad = i_pad;
-        da.n_inner = n_inner;
-        da.G4 = G4;
-        da.n_nodes = NN;
-        da.node_step = step;
-        da.slots = c->d_defl_slots.as<NestSlot>();
-        da.tile_kind = c->d_defl_kinds.as<int32_t>();
-        da.n_tiles = L.n_tiles;
-        da.n_chunks = i_pad / 64;
-        da.counter = c->d_ctl.as<int32_t>();
-        da.status = c->d_ctl.as<int32_t>() + 1;
-        da.L_all = Lall;
-    }
-    if (defl && !sur && !curve) {
-        // generator (FP64 pipe) and valuation (FP32 pipes) of consecutive batches
-        // run concurrently: the generator of batch i + 1 on a low-priority stream
-        // into the other plane buffer, the valuation of batch i on a
-        // high-priority stream at one CTA per SM, so that both fit on every SM
-        if (!c->nest_val) {
-            int lo = 0, hi = 0;
-            CU(cudaDeviceGetStreamPriorityRange(&lo, &hi));
-            CU(cudaStreamCreateWithPriority(&c->nest_val, cudaStreamNonBlocking, hi));
-            CU(cudaStreamCreateWithPriority(&c->nest_gen, cudaStreamNonBlocking, lo));
-            for (cudaEvent_t& e : c->nest_ev) CU(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-        }
-        cudaEvent_t ev_start = c->nest_ev[0], *ev_gen = c->nest_ev + 1, *ev_val = c->nest_ev + 3;
-        CU(cudaEventRecord(ev_start, c->stream));   // the outer paths, weights and queue word are ready
-        CU(cudaStreamWaitEvent(c->nest_gen, ev_start, 0));
-        CU(cudaStreamWaitEvent(c->nest_val, ev_start, 0));
-        const size_t buf4 = (size_t)B * per_outer / sizeof(float4);
-        int i = 0;
-        for (int o0 = 0; o0 < NO; o0 += B, ++i) {
-            const int Bc = std::min(B, NO - o0), bi = i & 1;
-            float4* plane = c->d_nest_plane.as<float4>() + bi * buf4;
-            if (i >= 2) CU(cudaStreamWaitEvent(c->nest_gen, ev_val[bi], 0));   // the buffer's last reader
-            CU(launch_inner_paths_defl(vs, sp->seed, sp->outer_first, o0, Bc, NN, n_inner, i_pad, G4, c->d_nest_ln.as<int>(),
-                                       c->d_nest_rn.as<double>(), c->d_nest_bm.as<double2>(), plane, c->sm_count, 4,
-                                       c->nest_gen));
-            CU(cudaEventRecord(ev_gen[bi], c->nest_gen));
-            CU(cudaStreamWaitEvent(c->nest_val, ev_gen[bi], 0));
-            const long long items = (long long)NN * Bc * da.n_chunks;
-            if (items > 0x7fffffffLL) return fail(c, RSV_E_ARG, "too many nested work items");
-            da.D = plane;
-            da.B = Bc;
-            da.o0 = o0;
-            da.n_items = (int32_t)items;
-            CU(cudaMemsetAsync(c->d_ctl.p, 0, sizeof(int32_t), c->nest_val));
-            if (L.n_tiles > 0) {
-                CU(launch_nested_defl(da, c->sm_count, 1, c->nest_val));
-            } else {
-                CU(cudaMemsetAsync(Lall + (size_t)o0 * NN * n_inner, 0, (size_t)Bc * NN * n_inner * sizeof(double),
-                                   c->nest_val));
-            }
-            CU(cudaEventRecord(ev_val[bi], c->nest_val));
-        }
-        // the call's stream continues once both pipelines are done
-        CU(cudaEventRecord(ev_gen[0], c->nest_gen));
-        CU(cudaStreamWaitEvent(c->stream, ev_gen[0], 0));
-        CU(cudaEventRecord(ev_val[0], c->nest_val));
-        CU(cudaStreamWaitEvent(c->stream, ev_val[0], 0));
-    }
-    for (int o0 = 0; o0 < NO && !sur && !curve && !defl; o0 += B) {
-        const int Bc = std::min(B, NO - o0);
-        CU(launch_inner_paths(form, vs, sp->seed, sp->outer_first, o0, Bc, NN, n_inner, i_pad, Lmax, c->d_nest_ln.as<int>(),
-                              c->d_nest_rn.as<double>(), c->d_nest_bm.as<double2>(), c->d_nest_plane.p, c->sm_count,
-                              c->stream));
-        const long long items = (long long)NN * Bc * a.n_chunks;
-        if (items > 0x7fffffffLL) return fail(c, RSV_E_ARG, "too many nested work items");
-        a.B = Bc;
-        a.o0 = o0;
-        a.n_items = (int32_t)items;
-        CU(cudaMemsetAsync(c->d_ctl.p, 0, sizeof(int32_t), c->stream));
-        if (L.n_tiles > 0) {
-            CU(launch_nested(form, a, c->sm_count, smem, c->stream));
-        } else {
-            CU(cudaMemsetAsync(Lall + (size_t)o0 * NN * n_inner, 0, (size_t)Bc * NN * n_inner * sizeof(double),
-                               c->stream));
-        }
-    }
     const int k = mc ? std::max(1, (int)std::ceil(0.005 * n_inner - 1e-9)) : 1;
     CU(launch_node_stats(Lall, NO * NN, n_inner, k, c->d_nest_mean.as<double>(), c->d_nest_kth.as<double>(),
                          c->stream));
@@ -1266,8 +1107,8 @@ rsv_status rsv_destroy(rsv_ctx* c) try {
     cudaStreamSynchronize(c->stream);
     for (DevBuf* b : {&c->d_amount, &c->d_vstage, &c->d_v64, &c->d_v32, &c->d_v2, &c->d_tab[0], &c->d_tab[1],
                       &c->d_tab[2], &c->lay.slots, &c->lay.kinds, &c->d_ctl, &c->d_partial, &c->d_part2,
-                      &c->d_o_v0f, &c->d_o_v0d, &c->d_o_tot, &c->d_o_pt, &c->d_o_traj, &c->d_nest_w,
-                      &c->d_nest_ln, &c->d_nest_rn, &c->d_nest_d0, &c->d_nest_plane, &c->d_nest_mean,
+                      &c->d_o_v0f, &c->d_o_v0d, &c->d_o_tot, &c->d_o_pt, &c->d_o_traj, &c->d_cf_tab,
+                      &c->d_cf_pol, &c->d_cf_sum, &c->d_nest_rn, &c->d_nest_d0, &c->d_nest_plane, &c->d_nest_mean,
                       &c->d_nest_kth, &c->d_nest_all, &c->d_pols, &c->sur.d_flag, &c->sur.d_q, &c->sur.d_lab,
                       &c->sur.d_y, &c->sur.d_X, &c->sur.d_pred, &c->sur.d_err, &c->sur.d_aux, &c->sur.d_curve,
                       &c->sur.d_comm, &c->sur.d_lnb, &c->d_tabf[0], &c->d_tabf[1], &c->d_tabf[2], &c->d_vf64,
@@ -1279,10 +1120,6 @@ rsv_status rsv_destroy(rsv_ctx* c) try {
     if (c->ev0) cudaEventDestroy(c->ev0);
     if (c->ev1) cudaEventDestroy(c->ev1);
     c->h_defl_stage.release();
-    for (cudaEvent_t& e : c->nest_ev)
-        if (e) cudaEventDestroy(e);
-    if (c->nest_val) cudaStreamDestroy(c->nest_val);
-    if (c->nest_gen) cudaStreamDestroy(c->nest_gen);
     if (c->ev_block) cudaEventDestroy(c->ev_block);
     if (c->copy_stream) {
         cudaStreamSynchronize(c->copy_stream);
