@@ -422,7 +422,7 @@ typedef struct {
  * curve modes value the portfolio's expected cash flows from the node on, E(t) =
  * sum_p amount_p E_p(t) (the in-force weighting at the node is part of them), on
  * each inner path: L_{o,n,i} = sum_{t >= m} D_i(m, t+1) E(t) plus what matures at
- * the node, in FP64 in every form.
+ * the node, in FP64 in every form (to 4e-10 of that with RSV_FORM_F32_DEFLATED).
  * opts->form selects what is accepted (RSV_FORM_F32_DEFLATED: products 0-5 and the
  * tables of that form).  Blocking unless opts->on_device.
  * Errors: RSV_E_STATE, RSV_E_ARG (bad spec, NULL L_mean/L_q995, a record as

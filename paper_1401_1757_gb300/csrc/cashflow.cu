@@ -57,7 +57,9 @@ __global__ void cf_sum_kernel(const CfTables T, const CfPol* __restrict__ pols, 
 }
 
 __global__ void __launch_bounds__(1024) cf_finish_kernel(const double* __restrict__ part, int n_steps,
-                                                         double* __restrict__ flow, double* __restrict__ due) {
+                                                         double* __restrict__ flow, double* __restrict__ due,
+                                                         float2* __restrict__ flow2, double* __restrict__ scale) {
+    __shared__ double top[1024];
     const int rows = n_steps + 1;
     for (int t = threadIdx.x; t < rows; t += blockDim.x) {
         double M = 0.0;
@@ -65,10 +67,28 @@ __global__ void __launch_bounds__(1024) cf_finish_kernel(const double* __restric
         due[t] = M;
     }
     __syncthreads();
+    double mx = 0.0;
     for (int t = threadIdx.x; t < n_steps; t += blockDim.x) {
         double A = due[t + 1];
         for (int k = 0; k < kCfSplits; ++k) A += part[(size_t)k * 2 * rows + t];
         flow[t] = A;
+        mx = fmax(mx, fabs(A));
+    }
+    top[threadIdx.x] = mx;
+    __syncthreads();
+    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+        if (threadIdx.x < w) top[threadIdx.x] = fmax(top[threadIdx.x], top[threadIdx.x + w]);
+        __syncthreads();
+    }
+    int ex = 0;
+    if (top[0] > 0.0 && top[0] < INFINITY) frexp(top[0], &ex);
+    ex = max(-1000, min(1000, ex));   // both scalings finite
+    const double s = ldexp(1.0, ex), r = ldexp(1.0, -ex);
+    if (threadIdx.x == 0) scale[0] = s;
+    for (int t = threadIdx.x; t < n_steps; t += blockDim.x) {
+        const double c = flow[t] * r;
+        const float h = __double2float_rn(c);
+        flow2[t] = make_float2(h, __double2float_rn(c - (double)h));
     }
 }
 
@@ -82,12 +102,12 @@ cudaError_t launch_cf_records(const CfTables& T, const SlotRec* slots, const int
 }
 
 cudaError_t launch_cf_portfolio(const CfTables& T, const CfPol* pols, int n, int n_steps, double* part, double* flow,
-                                double* due, cudaStream_t st) {
+                                double* due, float2* flow2, double* scale, cudaStream_t st) {
     const dim3 grid((n_steps + 1 + 127) / 128, kCfSplits);
     cf_sum_kernel<<<grid, 128, 0, st>>>(T, pols, n, n_steps, part);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    cf_finish_kernel<<<1, 1024, 0, st>>>(part, n_steps, flow, due);
+    cf_finish_kernel<<<1, 1024, 0, st>>>(part, n_steps, flow, due, flow2, scale);
     return cudaGetLastError();
 }
 

@@ -100,10 +100,11 @@ cudaError_t launch_cf_records(const CfTables& T, const SlotRec* slots, const int
 // The portfolio's cash flows: with A(t) = sum_p amount_p E_p(t) and M(t) the sum of
 // amount_p B_p over the policies with S = t,
 //   flow[t] = A(t) + M(t + 1), t < n_steps;   due[t] = M(t), t <= n_steps
-// in FP64, in a fixed order.
+// in FP64, in a fixed order; flow2 is flow / scale[0] as FP32 head and tail, scale[0] the
+// power of two that makes the largest of them less than 1 (1 if all are zero).
 // part: scratch of 2 * kCfSplits * (n_steps + 1) doubles.
 constexpr int kCfSplits = 64;
 cudaError_t launch_cf_portfolio(const CfTables& T, const CfPol* pols, int n, int n_steps, double* part, double* flow,
-                                double* due, cudaStream_t st);
+                                double* due, float2* flow2, double* scale, cudaStream_t st);
 
 }  // namespace rsv

@@ -233,6 +233,8 @@ struct PathArgs {
     const double* r_node;
     const void* tables;    // Box-Muller tables of the generator
     const double* flow;
+    const float2* flow2;   // flow / scale[0], FP32 head and tail
+    const double* scale;
     const double* due;
     double* L_all;
 };
@@ -253,11 +255,11 @@ __device__ __forceinline__ void for_each_path(const PathArgs& a, Path path) {
     }
 }
 
-// FP64 throughout: bound by the FP64 pipe, about 55 operations a month.  Before,
-// the discount factors went through a plane in memory to a valuation kernel that
-// ran every policy on them: 2,000 annuities x 100 outer paths x 40 nodes x 1,000
-// inner paths 311 ms deflated (the generator on a second stream), now 203 ms;
-// 331 mixed policies x 8 x 25 x 1,000, compensated, 60.4 ms, now 23.4 ms.
+// FP64 throughout (all forms but the deflated one, and model parameters outside
+// the double-float generator's range): bound by the FP64 pipe, about 55
+// operations a month.  Before, the discount factors went through a plane in memory to a
+// valuation kernel that ran every policy on them: 331 mixed policies x 8 outer
+// paths x 25 nodes x 1,000 inner paths, compensated, 60.4 ms, now 23.4 ms.
 __global__ void __launch_bounds__(kPathNT) inner_paths_kernel(const VasStep s, const PathArgs a) {
     __shared__ double2 bm[BM_SC + BM_LG];   // 18 KiB: the Box-Muller tables
     for (int k = threadIdx.x; k < BM_SC + BM_LG; k += blockDim.x) bm[k] = static_cast<const double2*>(a.tables)[k];
@@ -270,6 +272,191 @@ __global__ void __launch_bounds__(kPathNT) inner_paths_kernel(const VasStep s, c
             L = __fma_rn(D, __ldg(flow + t), L);
         });
         return L;
+    });
+}
+
+// ---- the generator in double-float FP32 -------------------------------------
+// GB300 issues 64 FP32 operations in the time of one FP64 operation, so the
+// walk runs in double-floats (about 2^-46 a step), with the random words and the
+// argument reductions in integers, which keeps them exact:
+//   ln u:  u = (2 w + 1) 2^-33 = 2^(-1-lz) y, y in [1, 2) with 32 fraction bits;
+//          r = y inv_j - 1 exactly as an integer (inv_j: 18 bits), split into two
+//          exact floats; log1p(r) = r - r^2/2 + r^3 (1/3 - r/4 + r^2/5), the square as a
+//          double-float (|r| < 2^-8: the next term is below 2^-50);
+//   R = sqrt(-2 ln u): the hardware reciprocal square root and one Newton step
+//          with the exact residual;
+//   sin, cos of 2 pi u: the nearest of 1,024 table angles (at the intervals'
+//          middles) and the addition theorems with |b| < pi/1024;
+//   x' = e x + l11 z1 (x = r - b), and 1 - I = (1 - b dt) - k1 x - l21 z1 - l22 z2
+//          by fused multiply-adds onto a head near 1, whose rounding errors a second
+//          fused multiply-add recovers exactly; exp(-I) from 1 - I by its series
+//          to I^6;
+//   D *= exp(-I);  L += D flow (product and sum error-free).
+// The deflated form takes it: its liabilities are within 1.2e-11 of 64 bits (its own
+// bound is 9e-7; its planes gave 1.6e-8).  2,000 annuities x 100 outer paths x 40
+// nodes x 1,000 inner paths: 203 ms by the FP64 walk, 12.9 ms so; about 220
+// instructions a month, issue 80% busy, FMA pipe 63%.
+struct NzStep {
+    float2 e, l11, k1, l21, l22, q0;   // constants as FP32 head and tail; q0 = 1 - b dt
+};
+
+constexpr int NZ_SC = 1024, NZ_LG = 128;   // float4 entries: (sin, cos) pairs, then (inv_j, L_j, k_j - 1)
+constexpr float kLn2Head = 0.693145751953125f;          // ln 2 to 18 bits, so that small integers times it are exact
+constexpr float kLn2Tail = 1.42860682030941723e-6f;
+constexpr float kPi32Head = 7.314590396335798e-10f, kPi32Tail = -2.035470213827790e-17f;   // pi 2^-32
+
+__device__ __forceinline__ void fast_two_sum(float a, float b, float& s, float& e) {
+    s = __fadd_rn(a, b);
+    e = __fsub_rn(b, __fsub_rn(s, a));
+}
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+    s = __fadd_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+// s = c + a b rounded, e its rounding error (|c| >= |a b|: c - s is exact)
+__device__ __forceinline__ void fma_err(float a, float b, float c, float& s, float& e) {
+    s = __fmaf_rn(a, b, c);
+    e = __fmaf_rn(a, b, __fsub_rn(c, s));
+}
+__device__ __forceinline__ uint32_t shl_clamped(uint32_t x, uint32_t n) {   // 0 for n >= 32
+    uint32_t r;
+    asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(n));
+    return r;
+}
+__device__ __forceinline__ float rsqrt_hw(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// R = sqrt(-2 ln u), u = (w + 1/2) 2^-32
+__device__ __forceinline__ df nz_radius(uint32_t w, const float4* __restrict__ lg) {
+    const uint32_t lz = (uint32_t)__clz((int)w);   // 32 for w = 0
+    const uint32_t y = (shl_clamped(w, lz) << 1) + shl_clamped(1u, lz);   // fraction bits of 2 w + 1, normalised
+    const float4 t = lg[y >> 25];
+    const uint32_t inv = __float_as_uint(t.x);
+    const uint64_t prod = (uint64_t)y * inv;
+    const int hi = (int)(uint32_t)(prod >> 32) + (int)inv - (1 << 18);
+    const uint32_t lo = (uint32_t)prod;               // r = (hi 2^32 + lo) 2^-50
+    const int a = (hi << 12) | (int)(lo >> 20);       // |a| < 2^22
+    const float rh = __fmaf_rn(__int_as_float(0x4B400000 + a), 0x1p-30f, -12582912.0f * 0x1p-30f);
+    const float rl = __fmaf_rn(__uint_as_float(0x4B000000u | (lo & 0xFFFFFu)), 0x1p-50f, -8388608.0f * 0x1p-50f);
+    const float p = __fmul_rn(rh, rh);
+    const float pe = __fmaf_rn(rh, __fadd_rn(rl, rl), __fmaf_rn(rh, rh, -p));
+    const float c3 = __fmul_rn(__fmul_rn(p, rh), __fmaf_rn(rh, __fmaf_rn(rh, 0.2f, -0.25f), 0.333333343f));
+    const float E = __fsub_rn(t.w, __int2float_rn((int)lz));   // k_j - 1 - lz
+    float s1, e1, s2, e2, s3, e3;
+    fast_two_sum(__fmul_rn(E, kLn2Head), t.y, s1, e1);
+    fast_two_sum(s1, rh, s2, e2);
+    two_sum(s2, __fmul_rn(-0.5f, p), s3, e3);
+    float tail = __fadd_rn(__fmaf_rn(E, kLn2Tail, t.z), rl);
+    tail = __fadd_rn(__fadd_rn(tail, __fadd_rn(e1, e2)), __fadd_rn(e3, c3));
+    tail = __fmaf_rn(-0.5f, pe, tail);
+    const float lh = __fadd_rn(s3, tail);
+    const float ll = __fsub_rn(tail, __fsub_rn(lh, s3));
+    const float ah = __fmul_rn(-2.0f, lh);
+    const float q = rsqrt_hw(ah), s = __fmul_rn(ah, q);
+    const float res = __fmaf_rn(-2.0f, ll, __fmaf_rn(-s, s, ah));
+    return df{s, __fmul_rn(res, __fmul_rn(0.5f, q))};
+}
+
+// (sin, cos)(2 pi u), u = (w + 1/2) 2^-32
+__device__ __forceinline__ void nz_sincos(uint32_t w, const float4* __restrict__ sc, df& sn, df& cs) {
+    const float4 t = sc[w >> 22];   // sin and cos of 2 pi (j + 1/2) / 1024, head and tail
+    const float F = __fsub_rn(__uint_as_float(0x4B000001u | ((w << 1) & 0x7FFFFEu)), 12582912.0f);
+    const float b = __fmul_rn(F, kPi32Head);
+    float bl = __fmaf_rn(F, kPi32Tail, __fmaf_rn(F, kPi32Head, -b));
+    const float b2 = __fmul_rn(b, b);
+    bl = __fmaf_rn(__fmul_rn(b2, b), -0.166666672f, bl);                          // sin b = b + bl
+    const float cm = __fmul_rn(b2, __fmaf_rn(b2, 0.0416666679f, -0.5f));          // cos b - 1
+    float p = __fmul_rn(t.z, b), e = __fmaf_rn(t.z, b, -p), s, es;
+    fast_two_sum(t.x, p, s, es);
+    e = __fadd_rn(__fadd_rn(e, es), t.y);
+    e = __fmaf_rn(t.z, bl, e);
+    e = __fmaf_rn(t.w, b, e);
+    sn = df{s, __fmaf_rn(t.x, cm, e)};
+    p = __fmul_rn(-t.x, b), e = __fmaf_rn(-t.x, b, -p);
+    fast_two_sum(t.z, p, s, es);
+    e = __fadd_rn(__fadd_rn(e, es), t.w);
+    e = __fmaf_rn(-t.x, bl, e);
+    e = __fmaf_rn(-t.y, b, e);
+    cs = df{s, __fmaf_rn(t.z, cm, e)};
+}
+
+struct NzState {
+    df x, D, L;   // r - b, the discount product from the node, the liability / scale
+};
+
+__device__ __forceinline__ void nz_step(NzState& q, const NzStep& s, uint32_t w0, uint32_t w1, float2 c,
+                                        const float4* __restrict__ tb) {
+    const df R = nz_radius(w0, tb + NZ_SC);
+    df sn, cs;
+    nz_sincos(w1, tb, sn, cs);
+    const df z1 = df_mul(R, cs), z2 = df_mul(R, sn);
+    // 1 - I
+    float r1, r2, r3, t1, t2, t3;
+    fma_err(-s.k1.x, q.x.h, s.q0.x, r1, t1);
+    fma_err(-s.l21.x, z1.h, r1, r2, t2);
+    fma_err(-s.l22.x, z2.h, r2, r3, t3);
+    float tl = __fadd_rn(__fadd_rn(t1, s.q0.y), __fadd_rn(t2, t3));
+    tl = __fmaf_rn(-s.k1.x, q.x.l, tl);
+    tl = __fmaf_rn(-s.k1.y, q.x.h, tl);
+    tl = __fmaf_rn(-s.l21.x, z1.l, tl);
+    tl = __fmaf_rn(-s.l21.y, z1.h, tl);
+    tl = __fmaf_rn(-s.l22.x, z2.l, tl);
+    tl = __fmaf_rn(-s.l22.y, z2.h, tl);
+    // x' = e x + l11 z1
+    const float ph = __fmul_rn(s.e.x, q.x.h), zh = __fmul_rn(s.l11.x, z1.h);
+    float pe = __fmaf_rn(s.e.x, q.x.h, -ph), ze = __fmaf_rn(s.l11.x, z1.h, -zh), xh, xe;
+    pe = __fmaf_rn(s.e.y, q.x.h, __fmaf_rn(s.e.x, q.x.l, pe));
+    ze = __fmaf_rn(s.l11.y, z1.h, __fmaf_rn(s.l11.x, z1.l, ze));
+    two_sum(ph, zh, xh, xe);
+    const float xl = __fadd_rn(xe, __fadd_rn(pe, ze));
+    q.x.h = __fadd_rn(xh, xl);
+    q.x.l = __fsub_rn(xl, __fsub_rn(q.x.h, xh));
+    // v = exp(-I) = (1 - I) + I^2/2 - I^3/6 + ..., I = i - tl with i = 1 - r3 exact
+    const float i = __fsub_rn(1.0f, r3);
+    const float i2 = __fmul_rn(i, i), i2e = __fmaf_rn(i, i, -i2);
+    const float poly = __fmaf_rn(i, __fmaf_rn(i, __fmaf_rn(i, 1.0f / 720.0f, -1.0f / 120.0f), 1.0f / 24.0f), -1.0f / 6.0f);
+    float vh, ve;
+    fast_two_sum(r3, __fmul_rn(0.5f, i2), vh, ve);
+    const float vl = __fadd_rn(__fmaf_rn(-i, tl, __fadd_rn(tl, ve)),
+                               __fmaf_rn(0.5f, i2e, __fmul_rn(__fmul_rn(i2, i), poly)));
+    const df D = df_mul(q.D, df{vh, vl});
+    q.D.h = __fadd_rn(D.h, D.l);
+    q.D.l = __fsub_rn(D.l, __fsub_rn(q.D.h, D.h));
+    // L += D c
+    const float g = __fmul_rn(c.x, q.D.h);
+    float ge = __fmaf_rn(c.x, q.D.h, -g), lh, le;
+    ge = __fmaf_rn(c.y, q.D.h, __fmaf_rn(c.x, q.D.l, ge));
+    two_sum(q.L.h, g, lh, le);
+    le = __fadd_rn(__fadd_rn(q.L.l, ge), le);
+    q.L.h = __fadd_rn(lh, le);
+    q.L.l = __fsub_rn(le, __fsub_rn(q.L.h, lh));
+}
+
+__global__ void __launch_bounds__(kPathNT) inner_paths_df_kernel(const NzStep s, double b, const PathArgs a) {
+    __shared__ float4 tb[NZ_SC + NZ_LG];   // 18 KiB
+    for (int k = threadIdx.x; k < NZ_SC + NZ_LG; k += blockDim.x) tb[k] = static_cast<const float4*>(a.tables)[k];
+    __syncthreads();
+    const uint32_t k0 = (uint32_t)a.seed, k1 = (uint32_t)(a.seed >> 32);
+    const double scale = a.scale[0];
+    for_each_path(a, [&](uint32_t c1, uint32_t c2, uint32_t c3, double r, int m, int left) {
+        const float2* __restrict__ flow = a.flow2 + m;
+        const double x = r - b;
+        NzState q;
+        q.x.h = __double2float_rn(x);
+        q.x.l = __double2float_rn(x - (double)q.x.h);
+        q.D = df{1.0f, 0.0f};
+        q.L = df{0.0f, 0.0f};
+        for (int t = 0; t < left; t += 2) {
+            uint32_t w[4];
+            philox4x32_10((uint32_t)(t >> 1), c1, c2, c3, k0, k1, w);
+            nz_step(q, s, w[0], w[1], __ldg(flow + t), tb);
+            if (t + 1 < left) nz_step(q, s, w[2], w[3], __ldg(flow + t + 1), tb);
+        }
+        return ((double)q.L.h + (double)q.L.l) * scale;
     });
 }
 
@@ -352,19 +539,75 @@ __global__ void node_stats_kernel(const double* __restrict__ L_all, int n_inner,
 }
 
 // ------------------------------------------------------------- launchers ----
-cudaError_t launch_nested_paths(const VasStep& s, const NestedRun& q, cudaStream_t st) {
+// Host tables of the double-float generator, as float4 (see nz_radius, nz_sincos).
+static const float4* nz_tables_host() {
+    static const std::vector<float4> t = [] {
+        std::vector<float4> v(NZ_SC + NZ_LG);
+        const long double two_pi = 6.283185307179586476925286766559005768L;
+        auto split = [](long double x, float& h, float& l) {
+            h = (float)x;
+            l = (float)(x - (long double)h);
+        };
+        for (int j = 0; j < NZ_SC; ++j) {
+            const long double x = two_pi * (2 * j + 1) / (2 * NZ_SC);
+            split(std::sin(x), v[j].x, v[j].y);
+            split(std::cos(x), v[j].z, v[j].w);
+        }
+        for (int j = 0; j < NZ_LG; ++j) {
+            const double c = 1.0 + (j + 0.5) / NZ_LG;
+            const uint32_t inv = (uint32_t)std::nearbyint(std::ldexp(1.0 / c, 18));
+            const int k = j >= BM_LG_K0 ? 1 : 0;
+            float4& e = v[NZ_SC + j];
+            memcpy(&e.x, &inv, sizeof inv);
+            split(-std::log(std::ldexp((long double)inv, k - 18)), e.y, e.z);
+            e.w = (float)(k - 1);
+        }
+        return v;
+    }();
+    return t.data();
+}
+
+// Tables of both generators, once per context: [FP64 | double-float].
+size_t nested_table_bytes() { return (size_t)(BM_SC + BM_LG) * sizeof(double2) + (size_t)(NZ_SC + NZ_LG) * sizeof(float4); }
+cudaError_t upload_nested_tables(void* dst, cudaStream_t st) {
+    const size_t a = (size_t)(BM_SC + BM_LG) * sizeof(double2);
+    cudaError_t e = cudaMemcpyAsync(dst, bm_tables_host(), a, cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) return e;
+    return cudaMemcpyAsync(static_cast<char*>(dst) + a, nz_tables_host(), (size_t)(NZ_SC + NZ_LG) * sizeof(float4),
+                           cudaMemcpyHostToDevice, st);
+}
+
+// The double-float generator holds rates as offsets from b and 1 - I near 1: the rates
+// must stay within about 0.25 of b (ten standard deviations, so never seen) and
+// b itself be moderate, so that a month's I stays below 0.05.
+bool nested_df_range(const NestedRun& q) {
+    const double sd = q.sigma * std::sqrt(std::min(1.0 / (2.0 * q.a), 800.0));
+    return std::fabs(q.b) <= 0.25 && std::fabs(q.r0 - q.b) + 10.0 * sd <= 0.25;
+}
+
+cudaError_t launch_nested_paths(const VasStep& s, const NestedRun& q, bool use_df, cudaStream_t st) {
     const long long per_node = (long long)q.n_outer * q.n_inner;
     const long long blocks = (per_node + kPathNT - 1) / kPathNT * q.n_nodes;
     const int grid = (int)std::min<long long>(blocks, 0x7fffffffLL);
     PathArgs a{q.seed, q.o_first, q.n_outer, q.n_nodes, q.node_step, q.n_inner, q.n_steps,
-               q.r_node, q.tables, q.flow, q.due, q.L_all};
-    inner_paths_kernel<<<grid, kPathNT, 0, st>>>(s, a);
+               q.r_node, q.tables, q.flow, q.flow2, q.scale, q.due, q.L_all};
+    if (!use_df) {
+        inner_paths_kernel<<<grid, kPathNT, 0, st>>>(s, a);
+    } else {
+        auto two = [](double x) {
+            const float h = (float)x;
+            return make_float2(h, (float)(x - (double)h));
+        };
+        const NzStep z{two(s.e), two(s.l11), two(s.k1), two(s.l21), two(s.l22), two(1.0 - s.b * s.dt)};
+        a.tables = static_cast<const char*>(q.tables) + (size_t)(BM_SC + BM_LG) * sizeof(double2);
+        inner_paths_df_kernel<<<grid, kPathNT, 0, st>>>(z, s.b, a);
+    }
     return cudaGetLastError();
 }
 
 cudaError_t launch_nested_curve(const NestedRun& q, double2* ab, cudaStream_t st) {
     PathArgs a{q.seed, q.o_first, q.n_outer, q.n_nodes, q.node_step, 1, q.n_steps,
-               q.r_node, nullptr, q.flow, q.due, q.L_all};
+               q.r_node, nullptr, q.flow, q.flow2, q.scale, q.due, q.L_all};
     if (q.n_steps > 0) curve_ab_kernel<<<(q.n_steps + 127) / 128, 128, 0, st>>>(q.a, q.b, q.sigma, 1.0 / 12.0, q.n_steps, ab);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;

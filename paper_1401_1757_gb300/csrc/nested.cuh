@@ -33,12 +33,18 @@ struct NestedRun {
     int32_t o_first, n_outer, n_nodes, node_step, n_inner;
     int32_t n_steps;          // the portfolio's longest projection from valuation
     const double* r_node;     // [n_outer][n_nodes]
-    const void* tables;       // bm_tables_host
+    const void* tables;       // upload_nested_tables
     const double* flow;       // launch_cf_portfolio's outputs
+    const float2* flow2;
+    const double* scale;
     const double* due;
     double* L_all;            // [n_outer][n_nodes][n_inner]
 };
-cudaError_t launch_nested_paths(const VasStep& s, const NestedRun& q, cudaStream_t st);
+size_t nested_table_bytes();
+cudaError_t upload_nested_tables(void* dst, cudaStream_t st);
+// Whether the double-float generator covers the run's model.
+bool nested_df_range(const NestedRun& q);
+cudaError_t launch_nested_paths(const VasStep& s, const NestedRun& q, bool use_df, cudaStream_t st);
 // The curve mode; ab: n_steps entries of scratch.
 cudaError_t launch_nested_curve(const NestedRun& q, double2* ab, cudaStream_t st);
 cudaError_t launch_node_stats(const double* L_all, int n_on, int n_inner, int k, double* mean, double* kth,

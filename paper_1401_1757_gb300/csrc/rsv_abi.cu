@@ -907,14 +907,13 @@ rsv_status compute_nested(rsv_ctx* c, const rsv_opts* o, const rsv_nested_spec* 
         if ((st = layout_to_device(c)) != RSV_OK || (st = upload_amounts(c)) != RSV_OK || (st = cf_tables(c, T)) != RSV_OK)
             return st;
         if (mc && !c->nest_bm_ready) {
-            CU(c->d_nest_bm.ensure((size_t)(BM_SC + BM_LG) * sizeof(double2)));
-            CU(cudaMemcpyAsync(c->d_nest_bm.p, bm_tables_host(), (size_t)(BM_SC + BM_LG) * sizeof(double2),
-                               cudaMemcpyHostToDevice, c->stream));
+            CU(c->d_nest_bm.ensure(nested_table_bytes()));
+            CU(upload_nested_tables(c->d_nest_bm.p, c->stream));
             c->nest_bm_ready = true;
         }
         CU(c->d_cf_pol.ensure((size_t)std::max(1, n_pol) * sizeof(CfPol)));
-        // scratch of the splits | curve's A, B | flow | due
-        CU(c->d_cf_sum.ensure(((size_t)2 * kCfSplits + 4) * (T_max + 1) * sizeof(double)));
+        // scratch of the splits | flow | due | flow2 | scale | curve's A, B
+        CU(c->d_cf_sum.ensure(((size_t)2 * kCfSplits + 5) * (T_max + 1) * sizeof(double) + sizeof(double)));
     }
     CU(cudaEventRecord(c->ev0, c->stream));
     CU(launch_outer_paths(vs, sp->seed, sp->outer_first, NO, NN, step, sp->r0, c->d_nest_rn.as<double>(), c->d_nest_d0.as<double>(),
@@ -922,18 +921,21 @@ rsv_status compute_nested(rsv_ctx* c, const rsv_opts* o, const rsv_nested_spec* 
     if (!sur) {
         double* part = c->d_cf_sum.as<double>();
         double* ab = part + (size_t)2 * kCfSplits * (T_max + 1);   // first: 16-byte aligned
-        double* flow = ab + 2 * (size_t)(T_max + 1);
+        double* flow2 = ab + 2 * (size_t)(T_max + 1);
+        double* flow = flow2 + (T_max + 1);
         double* due = flow + (T_max + 1);
+        double* scale = due + (T_max + 1);
         CfPol* recs = c->d_cf_pol.as<CfPol>();
         CU(launch_cf_records(T, L.slots.as<SlotRec>(), L.kinds.as<int32_t>(), c->d_amount.as<double>(), L.n_tiles, L.tab_pad,
                              recs, c->stream));
-        CU(launch_cf_portfolio(T, recs, L.n_tiles, T_max, part, flow, due, c->stream));
+        CU(launch_cf_portfolio(T, recs, L.n_tiles, T_max, part, flow, due, reinterpret_cast<float2*>(flow2), scale, c->stream));
         const NestedRun run{sp->seed, sp->a, sp->b, sp->sigma, sp->r0, sp->outer_first, NO, NN, step, n_inner, T_max,
-                            c->d_nest_rn.as<double>(), c->d_nest_bm.p, flow, due, Lall};
+                            c->d_nest_rn.as<double>(), c->d_nest_bm.p, flow, reinterpret_cast<const float2*>(flow2), scale,
+                            due, Lall};
         if (curve) {
             CU(launch_nested_curve(run, reinterpret_cast<double2*>(ab), c->stream));
         } else {
-            CU(launch_nested_paths(vs, run, c->stream));
+            CU(launch_nested_paths(vs, run, o->form == F_DEFL && nested_df_range(run), c->stream));
         }
     }
     if (sur) {
