@@ -94,16 +94,25 @@ enum {
                               see below                                               */
 };
 
+/* The compensated and the deflated form run rsv_compute_reserves (V0 and totals,
+ * payment at the end of the step, any cash-flow sequence that the form takes) as a
+ * matrix product of the policies' expected cash flows and the scenarios' discount
+ * products on the tensor cores, both split into exact 16-bit digits (compensated: 48
+ * bits, error about 1e-12; deflated: 32 bits, within the bound below).  Data outside its
+ * range keeps the recurrence kernels: scenarios whose discount products leave their
+ * mean by more than a factor of about 2^6, survival below 2^-100, amounts outside
+ * 2^-60 .. 2^90.  It is the last of a form's tunable variants. */
+
 /* RSV_FORM_F32_DEFLATED.  Eq. (generalForm) multiplied at step t by the
  * deflator G_t = D_t l_{x+t} / l_x (D_t = v_0 ... v_{t-1}, the discount-factor
  * product to the start of step t; l the life table {l_{x+t}} of Section 5)
  * becomes U_t = U_{t+1} + G_{t+1} c_t with U = G r: the same backward
  * substitution (Section 3.8.2) whose multiplicative factor is 1 at every
  * step, and r_0 = U_0.  The discount products D are FP64 running products, one
- * per scenario, computed on the device in every call; the life tables are
- * built once in FP64 on the host; each chain-step is one FP32 fused
- * multiply-add, summed in FP32 over 8 steps and folded into a double-float
- * every 16 steps (or every 32, the two spans' sums first added in FP32).
+ * per scenario; the life tables are built once in FP64 on the host.  In the
+ * recurrence kernels each chain-step is one FP32 fused multiply-add, summed in FP32 over
+ * 8 steps and folded into a double-float every 16 steps (or every 32, the two
+ * spans' sums first added in FP32).
  * Every reserve is within about 15 x 2^-24 (8.9e-7) relative of its value on
  * the FP64 inputs, whatever the projection length.  Products
  * RSV_SL_ANNUITY .. RSV_LAST_SURVIVOR (the reversionary and last-survivor

@@ -17,7 +17,7 @@ __global__ void cf_records_kernel(const CfTables T, const SlotRec* __restrict__ 
     auto life = [&](int idx) {
         CfLife l;
         l.i = (idx / tab_pad) * T.rows + idx % tab_pad;
-        l.inv = 1.0 / T.m[l.i];
+        l.inv = T.inv[l.i];
         l.last = T.z[l.i] - idx % tab_pad;
         l.ex = T.ex[l.i];
         l.pad = 0;
@@ -117,8 +117,9 @@ rsv_status cf_tables(rsv_ctx* c, CfTables& T) {
     const int n_tab = c->lay.n_tab, rows = c->lay.tab_pad + 1;
     const size_t n = (size_t)n_tab * rows;
     if (c->cf_tab_gen != c->tab_gen || c->cf_tab_rows != rows || c->cf_tab_n != n_tab) {
-        std::vector<double>& h = c->h_cf_tab;   // m, dm, then the two integer columns
-        h.resize(3 * n);
+        // m, dm, the two integer columns, 1 / m, then m and dm as FP32 head and tail
+        std::vector<double>& h = c->h_cf_tab;
+        h.resize(6 * n);
         int32_t* z = reinterpret_cast<int32_t*>(h.data() + 2 * n);
         int32_t* ex = z + n;
         c->cf_tab_scaled = 0;
@@ -145,6 +146,12 @@ rsv_status cf_tables(rsv_ctx* c, CfTables& T) {
                 z[(size_t)t * rows + k] = next;
             }
         }
+        float2* pair = reinterpret_cast<float2*>(h.data() + 4 * n);
+        for (size_t i = 0; i < n; ++i) h[3 * n + i] = 1.0 / h[i];
+        for (size_t i = 0; i < 2 * n; ++i) {
+            const float hi = (float)h[i];
+            pair[i] = make_float2(hi, (float)(h[i] - (double)hi));
+        }
         CU(c->d_cf_tab.ensure(h.size() * sizeof(double)));
         CU(cudaMemcpyAsync(c->d_cf_tab.p, h.data(), h.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));
         c->cf_tab_gen = c->tab_gen;
@@ -155,6 +162,9 @@ rsv_status cf_tables(rsv_ctx* c, CfTables& T) {
     T.dm = T.m + n;
     T.z = reinterpret_cast<const int32_t*>(T.dm + n);
     T.ex = T.z + n;
+    T.inv = T.m + 3 * n;
+    T.m2 = reinterpret_cast<const float2*>(T.m + 4 * n);
+    T.dm2 = T.m2 + n;
     T.rows = rows;
     T.scaled = c->cf_tab_scaled;
     return RSV_OK;

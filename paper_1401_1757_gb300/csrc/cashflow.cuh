@@ -32,6 +32,9 @@ struct CfTables {
     const double* dm;
     const int32_t* z;
     const int32_t* ex;
+    const double* inv;  // 1 / m
+    const float2* m2;   // m and dm as FP32 head and tail
+    const float2* dm2;
     int32_t rows;       // entries of one table
     int32_t scaled;     // 1: some ex_k > 0
 };

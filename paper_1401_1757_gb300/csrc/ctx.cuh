@@ -216,6 +216,15 @@ struct rsv_ctx {
     unsigned long long cf_gen = 1;
     DevBuf d_ml_rec, d_ml_amount;                   // m-life records of the last call
 
+    // the valuation as a matrix product (matval.cuh): whether the scenario set, the tables and
+    // the amounts are in its range, the discount products and their digits per form
+    bool mv_scen_ok = false;
+    double tab_min[rsv::kMaxTables] = {};           // smallest survivor-column entry of a table
+    double amt_lo = 0.0, amt_hi = 0.0;              // smallest non-zero and largest |amount|
+    DevBuf d_mv_D, d_mv_col, d_mv_dig[2], d_mv_E, d_mv_out;
+    unsigned long long scen_gen = 1, mv_dig_gen[2] = {0, 0};
+    int mv_built = -1;   // first tile of the panel whose digits are held, within one call
+
     Layout lay;
     DevBuf d_ctl;       // [0] queue head, [1] status
     DevBuf d_partial, d_part2;
@@ -280,6 +289,12 @@ rsv_status cf_tables(rsv_ctx* c, CfTables& T);
 // The first n_tab loaded tables, pad entries each, in a form's entry format
 // on the device (cached by shape and table generation); smem = their bytes.
 rsv_status stage_tables(rsv_ctx* c, int form, int pad, int n_tab, size_t& smem);
+// Whether the matrix product covers the loaded data; then, on the layout of width
+// kMvP: mv_prepare once a call, mv_launch for the scenario columns [s0, s0 + w) with the
+// output pointers at column s0 (partial: [2 n_tiles][s_pad]).
+bool mv_applies(const rsv_ctx* c);
+rsv_status mv_prepare(rsv_ctx* c, int form);
+rsv_status mv_launch(rsv_ctx* c, int form, int s0, int w, float* V0f, double* V0d, double* partial);
 // rsv_compute_reserves in the deflated form (defl_abi.cu); opts checked by the caller
 rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out);
 // The deflated kernels' staged life tables (defl_abi.cu): their shape from the

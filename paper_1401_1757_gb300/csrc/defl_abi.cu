@@ -8,6 +8,7 @@
 
 #include "ctx.cuh"
 #include "defl_kernel.cuh"
+#include "matval.cuh"
 
 namespace rsv {
 
@@ -114,17 +115,21 @@ rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
         return fail(c, RSV_E_STATE, "the deflated form values level cash flows: clear the loaded sequence");
     int nv = 0;
     const DeflVariant* vl = variants_defl(&nv);
-    int vi;
+    int vi;   // nv: the matrix product, the default where it covers the data
     if (o->variant >= 0) {
-        if (o->variant >= nv) return fail(c, RSV_E_ARG, "variant %d out of range", o->variant);
+        if (o->variant > nv) return fail(c, RSV_E_ARG, "variant %d out of range", o->variant);
         vi = o->variant;
     } else if (o->variant == -1) {
-        vi = c->tuned[F_DEFL] >= 0 ? c->tuned[F_DEFL] : 0;
+        vi = c->tuned[F_DEFL] >= 0 ? c->tuned[F_DEFL] : nv;
     } else {
         return fail(c, RSV_E_ARG, "variant %d out of range (the deflated form has no scan or summation)", o->variant);
     }
+    const bool mat = vi == nv && mv_applies(c);
+    const bool by_index = o->variant >= 0 && o->variant < nv;
+    if (vi == nv) vi = 0;
     // A variant whose staging ring does not fit beside the tables is replaced
-    // by the first that does, unless it was asked for by index.
+    // by the first that does, unless it was asked for by index.  (The matrix product
+    // stages no tables, but what the form refuses stays refused.)
     int W = 0;
     rsv_status st = RSV_OK;
     DeflTabs T;
@@ -133,14 +138,14 @@ rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     for (int pass = 0;; ++pass) {
         const DeflVariant& V = vl[vi];
         W = V.NW * V.P;
-        if ((st = build_layout(c, W, o->horizon, c->n_steps)) != RSV_OK) return st;
+        if ((st = build_layout(c, mat ? kMvP : W, o->horizon, c->n_steps)) != RSV_OK) return st;
         if ((st = defl_table_shape(c, c->lay, T)) != RSV_OK) return st;
         smem = T.bytes + defl_smem_extra(V);
         if ((long long)smem <= smem_max) break;
         int alt = -1;
         for (int k = 0; k < nv && alt < 0; ++k)
             if ((long long)(T.bytes + defl_smem_extra(vl[k])) <= smem_max) alt = k;
-        if (o->variant >= 0 || alt < 0 || pass > 0)
+        if (by_index || alt < 0 || pass > 0)
             return fail(c, RSV_E_ARG, "variant %s needs %zu bytes of shared memory for %d tables (%lld available)",
                         V.name, smem, T.n_tab, smem_max);
         vi = alt;
@@ -148,7 +153,9 @@ rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     const DeflVariant& V = vl[vi];
     const int CH = 32 * V.M;
     const Layout& L = c->lay;
-    if ((st = defl_table_stage(c, T)) != RSV_OK) return st;
+    if ((st = mat ? defl_table_range(c, T) : defl_table_stage(c, T)) != RSV_OK) return st;
+    if (mat && (st = mv_prepare(c, F_DEFL)) != RSV_OK) return st;
+    const int part_rows = mat ? 2 * L.n_tiles : L.n_tiles;   // rows of per-tile scenario sums
     const int n_tab = T.n_tab, dpad = T.dpad, arr_d = T.arr_d;
     const size_t tab_bytes = T.bytes;
     const std::vector<std::vector<double>>& ell = T.ell;
@@ -156,7 +163,7 @@ rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     // slot records of the super-tiles
     const unsigned long long lkey = L.gen * 31ull + (unsigned long long)dpad * 7ull + (unsigned)L.horizon * 3ull +
                                     (unsigned long long)arr_d;
-    if (c->defl_lay_key != lkey || c->defl_W != W || c->defl_dpad != dpad || c->defl_n_st != L.n_tiles) {
+    if (!mat && (c->defl_lay_key != lkey || c->defl_W != W || c->defl_dpad != dpad || c->defl_n_st != L.n_tiles)) {
         // written in place into pinned memory by several host threads
         const size_t n_slots = (size_t)L.n_tiles * W;
         CU(c->h_defl_stage.acquire(std::max<size_t>(1, n_slots) * sizeof(DeflSlot)));
@@ -300,12 +307,12 @@ rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     }
     CU(c->d_ctl.ensure(2 * sizeof(int32_t)));
     CU(cudaMemsetAsync(c->d_ctl.p, 0, 2 * sizeof(int32_t), c->stream));
-    if (tot) CU(c->d_partial.ensure((size_t)std::max(1, L.n_tiles) * s_pad * sizeof(double)));
+    if (tot) CU(c->d_partial.ensure((size_t)std::max(1, part_rows) * s_pad * sizeof(double)));
     if (tot && L.n_tiles == 0) CU(cudaMemsetAsync(tot, 0, NSc * sizeof(double), c->stream));
 
     // the deflator plane, rows of four steps, a whole number of staged blocks
     const int n_groups = std::max(1, (c->n_steps + DEFL_KB - 1) / DEFL_KB) * DEFL_G;
-    CU(c->d_defl_plane.ensure((size_t)n_groups * s_pad * sizeof(float4)));
+    if (!mat) CU(c->d_defl_plane.ensure((size_t)n_groups * s_pad * sizeof(float4)));
 
     DeflArgs a{};
     a.tab = c->d_defl_tab.as<float>();
@@ -325,11 +332,14 @@ rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     a.partial = tot ? c->d_partial.as<double>() : nullptr;
     a.part_ld = s_pad;
 
-    int bps = 0;
-    CU(V.occupancy(&bps, smem));
+    int bps = 1;
+    if (!mat) CU(V.occupancy(&bps, smem));
     if (bps < 1) return fail(c, RSV_E_CUDA, "variant %s cannot be resident with %zu B smem", V.name, smem);
     // one launch on the scenario columns [s0, s0 + w)
     auto launch = [&](int s0, int w) -> rsv_status {
+        if (mat)
+            return mv_launch(c, F_DEFL, s0, w, a.V0f ? a.V0f + s0 : nullptr, a.V0d ? a.V0d + s0 : nullptr,
+                             a.partial ? a.partial + s0 : nullptr);
         DeflArgs b = a;
         b.D = a.D + s0;
         b.n_scen = w;
@@ -349,8 +359,8 @@ rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     const bool pipelined =
         !o->on_device && !direct_v0 && ((hV0f != nullptr) != (hV0d != nullptr)) && L.n_tiles > 0 && NSc >= 256;
     CU(cudaEventRecord(c->ev0, c->stream));
-    CU(launch_defl_plane(c->d_v64.as<double>(), c->n_steps, s_pad, n_groups, c->d_defl_plane.as<float4>(),
-                         c->stream));
+    if (!mat) CU(launch_defl_plane(c->d_v64.as<double>(), c->n_steps, s_pad, n_groups, c->d_defl_plane.as<float4>(),
+                                   c->stream));
     bool copied_v0 = direct_v0;
     if (L.n_tiles > 0 && pipelined) {
         // V0 in column blocks, each copied to the host on a second stream
@@ -380,7 +390,7 @@ rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
         CU(cudaEventRecord(c->ev1, c->stream));
     }
     c->ev_recorded = true;
-    if (tot && L.n_tiles > 0 && (st = scenario_totals(c, a.partial, L.n_tiles, s_pad, NSc, tot)) != RSV_OK) return st;
+    if (tot && L.n_tiles > 0 && (st = scenario_totals(c, a.partial, part_rows, s_pad, NSc, tot)) != RSV_OK) return st;
     if (!o->on_device) {
         if (hV0f && !copied_v0) CU(cudaMemcpyAsync(hV0f, V0f, n_v0 * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
         if (hV0d && !copied_v0) CU(cudaMemcpyAsync(hV0d, V0d, n_v0 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));

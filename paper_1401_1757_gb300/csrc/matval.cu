@@ -1,0 +1,604 @@
+// matval.cu -- digits of the discount products and of the expected cash flows, and
+// their product on the tensor cores (see matval.cuh).
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <climits>
+#include <cmath>
+
+#include "matval.cuh"
+#include "tcgen05.cuh"
+
+namespace rsv {
+namespace {
+
+constexpr uint32_t kMvPoll = 1u << 24;
+
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float(min(max(e + 127, 1), 254) << 23); }
+
+// ------------------------------------------------------------- the digits ----
+// A digit as it is stored: FP16 of 2^15 times it (deflated), or BF16 of it.
+template <int NS>
+__device__ __forceinline__ uint16_t mv_pack(float x) {
+    if constexpr (NS == 3) return __half_as_ushort(__float2half_rn(x));
+    else return __bfloat16_as_ushort(__float2bfloat16_rn(x));
+}
+
+template <int NS>
+__device__ __forceinline__ void mv_digits(float h, float l, uint16_t (&d)[NS]) {
+    const float d1 = __fsub_rn(__fadd_rn(h, 98304.0f), 98304.0f);   // to a multiple of 2^-7
+    float r = __fsub_rn(h, d1);                                       // exact
+    if constexpr (NS == 3) {
+        d[0] = mv_pack<3>(__fmul_rn(d1, 32768.0f));
+        r = __fmul_rn(__fadd_rn(r, l), 32768.0f);
+        d[1] = mv_pack<3>(r);
+        d[2] = mv_pack<3>(__fsub_rn(r, __half2float(__ushort_as_half(d[1]))));
+    } else {
+        const float d2 = __fsub_rn(__fadd_rn(r, 384.0f), 384.0f);    // to a multiple of 2^-15
+        r = __fsub_rn(r, d2);
+        const float d3 = __fsub_rn(__fadd_rn(r, 1.5f), 1.5f);        // to a multiple of 2^-23
+        r = __fadd_rn(__fsub_rn(r, d3), l);
+        d[0] = mv_pack<NS>(d1);
+        d[1] = mv_pack<NS>(d2);
+        d[2] = mv_pack<NS>(d3);
+#pragma unroll
+        for (int k = 3; k < NS; ++k) {
+            d[k] = mv_pack<NS>(r);
+            r = __fsub_rn(r, __uint_as_float((uint32_t)d[k] << 16));
+        }
+    }
+}
+
+// ---------------------------------------------------------- scenario side ----
+// Running products of 32 scenarios, the steps in 32 segments: a segment's product,
+// the products before it, then the running product, so that the serial chain is 1/16
+// of the steps.
+__global__ void __launch_bounds__(1024) mv_products_kernel(const double* __restrict__ v, int n_steps, int s_pad,
+                                                           float2* __restrict__ D) {
+    __shared__ double seg[32][32];
+    const int s = blockIdx.x * 32 + threadIdx.x, k = threadIdx.y;
+    const int len = (n_steps + 31) / 32, t0 = min(n_steps, k * len), t1 = min(n_steps, t0 + len);
+    double p = 1.0;
+    for (int t = t0; t < t1; ++t) p = __dmul_rn(p, v[(size_t)t * s_pad + s]);
+    seg[k][threadIdx.x] = p;
+    __syncthreads();
+    double d = 1.0;
+    for (int q = 0; q < k; ++q) d = __dmul_rn(d, seg[q][threadIdx.x]);
+    for (int t = t0; t < t1; ++t) {
+        d = __dmul_rn(d, v[(size_t)t * s_pad + s]);
+        const float h = __double2float_rn(d);
+        D[(size_t)t * s_pad + s] = make_float2(h, __double2float_rn(d - (double)h));
+    }
+}
+
+// the binary exponent of a positive normal number, INT_MIN otherwise
+__device__ __forceinline__ int exp_of(float x) {
+    const int e = __float_as_int(x) >> 23;
+    return e > 0 && e < 255 ? e - 127 : INT_MIN;
+}
+
+__global__ void mv_tilt_kernel(const float2* __restrict__ D, int n_scen, int s_pad, int32_t* __restrict__ tau,
+                               int32_t* __restrict__ stat) {
+    __shared__ float sum[128];
+    const int t = blockIdx.x;
+    float a = 0.0f;
+    bool bad = false;
+    for (int s = threadIdx.x; s < n_scen; s += 128) {
+        const float x = D[(size_t)t * s_pad + s].x;
+        if (exp_of(x) == INT_MIN) bad = true;
+        else a += log2f(x);
+    }
+    sum[threadIdx.x] = a;
+    bad = __syncthreads_or(bad);
+    for (int w = 64; w > 0; w >>= 1) {
+        if (threadIdx.x < w) sum[threadIdx.x] += sum[threadIdx.x + w];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        const int q = bad ? 0 : -(int)rintf(sum[0] / n_scen);
+        tau[t] = q;
+        atomicMax(&stat[1], bad ? INT_MAX : abs(q));
+    }
+}
+
+__global__ void mv_columns_kernel(const float2* __restrict__ D, const int32_t* __restrict__ tau, int n_steps, int n_scen,
+                                  int s_pad, int32_t* __restrict__ colexp, int32_t* __restrict__ stat) {
+    __shared__ int hi[8][32], lo[8][32];
+    const int s = blockIdx.x * 32 + threadIdx.x;
+    int mx = -4096, mn = 4096;
+    for (int t = threadIdx.y; t < n_steps; t += 8) {
+        const int e = exp_of(D[(size_t)t * s_pad + s].x);
+        if (e == INT_MIN) continue;   // recorded by the tilt kernel
+        mx = max(mx, e + tau[t]);
+        mn = min(mn, e + tau[t]);
+    }
+    hi[threadIdx.y][threadIdx.x] = mx;
+    lo[threadIdx.y][threadIdx.x] = mn;
+    __syncthreads();
+    if (threadIdx.y) return;
+#pragma unroll
+    for (int k = 1; k < 8; ++k) {
+        mx = max(mx, hi[k][threadIdx.x]);
+        mn = min(mn, lo[k][threadIdx.x]);
+    }
+    colexp[s] = s < n_scen && mx > -4096 ? mx + 1 : 0;
+    if (s < n_scen) atomicMax(&stat[0], max(0, mx - mn));
+}
+
+template <int NS>
+__global__ void __launch_bounds__(256) mv_digits_kernel(const float2* __restrict__ D, const int32_t* __restrict__ tau,
+                                                        const int32_t* __restrict__ colexp, int n_steps, int n_scen,
+                                                        int s_pad, int pitch, uint16_t* __restrict__ out) {
+    __shared__ uint16_t tile[NS][32][66];
+    const int s0 = blockIdx.x * 32, t0 = blockIdx.y * 64, s = s0 + (threadIdx.x & 31);
+    const int c = colexp[s];
+    for (int q = threadIdx.x >> 5; q < 64; q += 8) {
+        const int t = t0 + q;
+        float h = 0.0f, l = 0.0f;
+        if (t < n_steps && s < n_scen) {
+            const float2 x = D[(size_t)t * s_pad + s];
+            const float f = pow2f(tau[t] - c);   // at most 1
+            h = __fmul_rn(x.x, f);
+            l = __fmul_rn(x.y, f);
+        }
+        uint16_t d[NS];
+        mv_digits<NS>(h, l, d);
+#pragma unroll
+        for (int k = 0; k < NS; ++k) tile[k][threadIdx.x & 31][q] = d[k];
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < NS * 32 * 32; i += 256) {   // pairs of steps
+        const int q = i & 31, r = (i >> 5) & 31, k = i >> 10;
+        *reinterpret_cast<uint32_t*>(out + ((size_t)k * s_pad + s0 + r) * pitch + t0 + 2 * q) =
+            tile[k][r][2 * q] | (uint32_t)tile[k][r][2 * q + 1] << 16;
+    }
+}
+
+// ------------------------------------------------------------ policy side ----
+__device__ __forceinline__ df df_one_minus(df x) {   // 0 <= x <= 1
+    const float s = __fsub_rn(1.0f, x.h);
+    return df{s, __fsub_rn(__fsub_rn(__fsub_rn(1.0f, s), x.h), x.l)};
+}
+
+struct MvLife {
+    int i, last;
+    df c;
+};
+__device__ __forceinline__ df at(const float2* __restrict__ col, const MvLife& a, int t) {
+    if (t > a.last) return df{0.0f, 0.0f};
+    const float2 v = col[a.i + t];
+    return df{v.x, v.y};
+}
+
+// E_p(t) in the row's unit (K_ANN, K_ASS: times m_x; the others: per unit amount)
+template <int KIND>
+__device__ __forceinline__ df mv_expected(const CfTables& T, const MvLife& a, const MvLife& b, int state0, int t) {
+    if constexpr (KIND == K_ANN) {
+        return at(T.m2, a, t + 1);
+    } else if constexpr (KIND == K_ASS) {
+        return at(T.dm2, a, t);
+    } else if constexpr (KIND == K_ANN2) {
+        return df_mul(df_mul(at(T.m2, a, t + 1), a.c), df_mul(at(T.m2, b, t + 1), b.c));
+    } else if constexpr (KIND == K_JL) {   // a dead life's c is 0
+        const df x = df_mul(at(T.m2, a, t + 1), a.c), y = df_mul(at(T.m2, b, t + 1), b.c);
+        return df_add_pos(x, df_mul(y, df_one_minus(x)));
+    } else if constexpr (KIND == K_ASS2) {
+        const df dx = df_mul(at(T.dm2, a, t), a.c), dy = df_mul(at(T.dm2, b, t), b.c);
+        return df_add_pos(df_mul(dx, df_mul(at(T.m2, b, t), b.c)), df_mul(df_mul(at(T.m2, a, t + 1), a.c), dy));
+    } else {   // second death: x dies now and y is dead by the end, or x was dead and y dies now
+        const df dx = df_mul(at(T.dm2, a, t), a.c), dy = df_mul(at(T.dm2, b, t), b.c);
+        if (state0 == 1) return dx;
+        if (state0 == 2) return dy;
+        return df_add_pos(df_mul(dx, df_one_minus(df_mul(at(T.m2, b, t + 1), b.c))),
+                          df_mul(df_one_minus(df_mul(at(T.m2, a, t), a.c)), dy));
+    }
+}
+template <int KIND>
+__device__ __forceinline__ df mv_boundary(const CfTables& T, const MvLife& a, const MvLife& b, int state0, int S) {
+    if constexpr (KIND == K_ASS) return at(T.m2, a, S);
+    const df x = df_mul(at(T.m2, a, S), a.c), y = df_mul(at(T.m2, b, S), b.c);
+    if constexpr (KIND == K_ASS2) return df_mul(x, y);
+    if (state0 == 1) return x;
+    if (state0 == 2) return y;
+    return df_add_pos(x, df_mul(y, df_one_minus(x)));
+}
+
+
+// One warp a policy: the largest tilted cash flow, then the digits.  Closed forms, so
+// the lanes take consecutive steps; bound by issue (about 25 instructions a step for
+// one life, 60 for two).
+template <int NS, int KIND, bool CF>
+__device__ __forceinline__ void mv_row(const MvBuild& b, const SlotRec& r, int row, int kt, const float* __restrict__ tilt) {
+    const int lane = threadIdx.x & 31;
+    const CfTables& T = b.T;
+    auto life = [&](int idx) {
+        const int tb = idx < b.tab_pad ? 0 : idx / b.tab_pad, age = idx - tb * b.tab_pad;
+        MvLife q;
+        q.i = tb * T.rows + age;
+        q.last = T.z[q.i] - age;
+        return q;
+    };
+    MvLife x = life(r.idx1), y = life(r.idx2);
+    const double amount = r.pol >= 0 ? b.amount[r.pol] : 0.0;
+    const int S = r.pol >= 0 ? r.S : 0;
+    auto two = [](double v) {
+        const float h = __double2float_rn(v);
+        return df{h, __double2float_rn(v - (double)h)};
+    };
+    if constexpr (KIND != K_ANN && KIND != K_ASS) {
+        x.c = two(T.inv[x.i]);
+        y.c = two(T.inv[y.i]);
+        if (KIND == K_JL) {
+            y.c = df_mul(y.c, df{r.rho_h, r.rho_l});
+            if (r.state0 == 2) x.c = df{0.0f, 0.0f};
+            if (r.state0 == 1) y.c = df{0.0f, 0.0f};
+        }
+    }
+    auto flow = [&](int t) {
+        df e = mv_expected<KIND>(T, x, y, r.state0, t);
+        if constexpr (CF) e = df_mul(e, two(b.cf[(size_t)r.pol * b.cf_ld + t]));
+        return e;
+    };
+    float top = 0.0f;
+    for (int t = lane; t < S; t += 32) top = fmaxf(top, __fmul_rn(flow(t).h, tilt[t]));
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, d));
+    // entries below 1; one bit less for each doubling of the steps beyond 1,000, so that the
+    // leading digits' sum stays exact
+    int e = top > 0.0f ? ((__float_as_int(top) >> 23) & 255) - 126 : 0;
+    e += (S > 1000) + (S > 2000) + (S > 4000);
+    const float f = pow2f(-e);
+    uint16_t* base = static_cast<uint16_t*>(b.digits) + ((size_t)(row / kMvP) * NS * kMvP + row % kMvP) * b.pitch;
+    for (int t0 = 0; t0 < kt; t0 += 64) {
+        const int t = t0 + 2 * lane;
+        uint16_t d0[NS], d1[NS];
+        df a{0.0f, 0.0f}, c{0.0f, 0.0f};
+        if (t < S) {
+            a = flow(t);
+            const float g = __fmul_rn(tilt[t], f);
+            a = df{__fmul_rn(a.h, g), __fmul_rn(a.l, g)};
+        }
+        if (t + 1 < S) {
+            c = flow(t + 1);
+            const float g = __fmul_rn(tilt[t + 1], f);
+            c = df{__fmul_rn(c.h, g), __fmul_rn(c.l, g)};
+        }
+        mv_digits<NS>(a.h, a.l, d0);
+        mv_digits<NS>(c.h, c.l, d1);
+#pragma unroll
+        for (int k = 0; k < NS; ++k)
+            *reinterpret_cast<uint32_t*>(base + (size_t)k * kMvP * b.pitch + t) = d0[k] | (uint32_t)d1[k] << 16;
+    }
+    if (lane == 0) {
+        // amount (times 1 / m_x) as a mantissa below 1 and an exponent, then times 2^e
+        double rc = amount;
+        if (KIND == K_ANN || KIND == K_ASS) rc = __dmul_rn(rc, T.inv[x.i]);
+        int ex = 0;
+        if (rc != 0.0) {
+            const int hi = __double2hiint(rc);
+            ex = ((hi >> 20) & 2047) - 1022;
+            rc = __hiloint2double((hi & 0x800FFFFF) | 0x3FE00000, __double2loint(rc));
+        }
+        const df q = two(rc);
+        const float g = pow2f(ex + e);
+        MvOut o;
+        o.sc_h = __fmul_rn(q.h, g);
+        o.sc_l = __fmul_rn(q.l, g);
+        o.mat_h = o.mat_l = 0.0f;
+        if constexpr (KIND == K_ASS || KIND == K_ASS2 || KIND == K_LS2) {
+            if (r.bnd != 0.0f && r.pol >= 0) {   // the maturity payment, or the amount if it is due now
+                df m{r.bnd, 0.0f};
+                int em = 0, xm = ex;
+                df w = q;
+                if (S == 0) {
+                    const int hi = __double2hiint(amount);
+                    xm = ((hi >> 20) & 2047) - 1022;
+                    w = amount != 0.0 ? two(__hiloint2double((hi & 0x800FFFFF) | 0x3FE00000, __double2loint(amount)))
+                                      : df{0.0f, 0.0f};
+                } else {
+                    m = mv_boundary<KIND>(T, x, y, r.state0, S);
+                    em = m.h > 0.0f ? ((__float_as_int(m.h) >> 23) & 255) - 126 : 0;
+                    const float f2 = pow2f(-em);
+                    m = df{__fmul_rn(m.h, f2), __fmul_rn(m.l, f2)};
+                }
+                const df v = df_mul(m, w);
+                const float g2 = pow2f(xm + em);
+                o.mat_h = __fmul_rn(v.h, g2);
+                o.mat_l = __fmul_rn(v.l, g2);
+            }
+        }
+        o.pol = r.pol;
+        o.S = S;
+        o.pad[0] = o.pad[1] = 0;
+        b.out[row] = o;
+    }
+}
+
+template <int NS>
+__global__ void __launch_bounds__(256) mv_build_kernel(const MvBuild b) {
+    extern __shared__ float tilt[];   // 2^-tau(t)
+    const int row = blockIdx.x * 8 + (threadIdx.x >> 5), tile = row / kMvP;
+    const int kt = max(64, (b.slots[(size_t)tile * kMvP].S + 63) / 64 * 64);   // the tile's longest projection
+    for (int t = threadIdx.x; t < kt; t += 256) tilt[t] = t < b.pitch ? pow2f(-b.tau[t]) : 0.0f;
+    __syncthreads();
+    const SlotRec r = b.slots[row];
+    auto run = [&](auto cf) {
+        constexpr bool CF = decltype(cf)::value;
+        switch (b.kinds[tile]) {
+        case K_ANN: return mv_row<NS, K_ANN, CF>(b, r, row, kt, tilt);
+        case K_ASS: return mv_row<NS, K_ASS, CF>(b, r, row, kt, tilt);
+        case K_JL: return mv_row<NS, K_JL, CF>(b, r, row, kt, tilt);
+        case K_ANN2: return mv_row<NS, K_ANN2, CF>(b, r, row, kt, tilt);
+        case K_ASS2: return mv_row<NS, K_ASS2, CF>(b, r, row, kt, tilt);
+        default: return mv_row<NS, K_LS2, CF>(b, r, row, kt, tilt);
+        }
+    };
+    if (tile >= b.general_from) run(std::true_type{});
+    else run(std::false_type{});
+}
+
+// -------------------------------------------------------------- the product ----
+// Persistent CTAs over (policy tile, scenario tile) items, longest projections first.
+// A block of 32 steps of both operands' digits is staged by TMA (64-byte swizzle) into a ring
+// of stages; one thread issues the digits' products, m128 n128 k16 with the scenarios
+// on the lanes (A) and the policies on the columns (B); eight warps add the accumulators as
+// double-floats, scale, write V0 (32 consecutive scenarios of a policy a warp store) and
+// keep each scenario's sum over the tile's policies.
+// Deflated: 6 products and 2 accumulators, so TMEM holds two tiles' and the epilogue runs
+// beside the next tile's products; compensated: 21 products, 4 accumulators.
+template <int NS>
+struct MvShape;   // products, accumulators, tiles in TMEM, stages; per product 3 bits each of the
+template <>       // scenario digit, the policy digit and the accumulator
+struct MvShape<3> {
+    static constexpr int NP = 6, NA = 2, NB = 2, ST = 4;
+    static constexpr uint64_t kA = 0x10240, kB = 0x2208, kAcc = 0x9248;
+};
+template <>
+struct MvShape<6> {
+    static constexpr int NP = 21, NA = 4, NB = 1, ST = 2;
+    static constexpr uint64_t kA = 0x510b503298450240, kB = 0xa62621683282208, kAcc = 0x36db6db6db6d2448;
+};
+__host__ __device__ constexpr int field(uint64_t v, int p) { return (int)(v >> (3 * p)) & 7; }
+constexpr int kMvEpi = 8;                              // epilogue warps
+constexpr int kMvThreads = 32 * (kMvEpi + 2);
+constexpr int kMvSlab = kMvP * kMvKB * 2;              // 8 KiB: one digit of one operand's block
+
+template <int NS>
+__global__ void __launch_bounds__(kMvThreads, 1)
+    mv_product_kernel(const __grid_constant__ CUtensorMap mapD, const __grid_constant__ CUtensorMap mapE, const MvArgs a) {
+    using Sh = MvShape<NS>;
+    constexpr int kStage = 2 * NS * kMvSlab;
+    constexpr uint32_t kIdesc = f16_idesc(NS != 3, kMvM, kMvP);   // both operands FP16, or both BF16
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    __shared__ uint64_t full[Sh::ST], empty[Sh::ST], acc_full[Sh::NB], acc_empty[Sh::NB], drained;
+    __shared__ uint32_t tmem_slot;
+    __shared__ MvOut recs[kMvP];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        for (int i = 0; i < Sh::ST; ++i) {
+            mbar_init(&full[i], 1);
+            mbar_init(&empty[i], 1);
+        }
+        for (int i = 0; i < Sh::NB; ++i) {
+            mbar_init(&acc_full[i], 1);
+            mbar_init(&acc_empty[i], kMvEpi);
+        }
+        mbar_init(&drained, 1);
+        fence_barrier_init();
+    }
+    if (warp == 0) tmem_alloc(&tmem_slot, 512);
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = tmem_slot;
+    const long long n_items = (long long)a.n_tiles * a.n_chunks;
+    bool failed = false;
+    auto wait_on = [&](uint64_t* bar, uint32_t parity) {   // a bounded wait; a timeout is recorded
+        if (failed) return;
+        if (!mbar_wait_bounded(bar, parity, kMvPoll)) {
+            failed = true;
+            atomicExch(a.status, DEV_TIMEOUT);
+        }
+    };
+    auto blocks_of = [&](int tile) { return max(1, (a.slots[(size_t)tile * kMvP].S + kMvKB - 1) / kMvKB); };
+
+    if (warp == kMvEpi) {
+        // ---- the copies (one thread)
+        if (lane == 0) {
+            uint32_t it = 0;
+            for (long long item = blockIdx.x; item < n_items && !failed; item += gridDim.x) {
+                const int tile = (int)(item / a.n_chunks), chunk = (int)(item - (long long)tile * a.n_chunks);
+                const int nk = blocks_of(tile);
+                for (int kb = 0; kb < nk && !failed; ++kb, ++it) {
+                    const int st = it % Sh::ST;
+                    if (it >= Sh::ST) wait_on(&empty[st], (it / Sh::ST - 1) & 1);
+                    if (failed) break;
+                    unsigned char* dst = ring + st * kStage;
+                    mbar_arrive_expect_tx(&full[st], kStage);
+#pragma unroll
+                    for (int k = 0; k < NS; ++k) {
+                        tma_load_2d(dst + k * kMvSlab, &mapD, kb * kMvKB, k * a.s_pad + a.s0 + chunk * kMvM, &full[st]);
+                        tma_load_2d(dst + (NS + k) * kMvSlab, &mapE, kb * kMvKB, (tile * NS + k) * kMvP, &full[st]);
+                    }
+                }
+            }
+            if (failed)   // let the copies in flight land before the memory is released
+                for (uint32_t back = 0; back < Sh::ST && back < it; ++back)
+                    mbar_wait_bounded(&full[(it - 1 - back) % Sh::ST], ((it - 1 - back) / Sh::ST) & 1, kMvPoll);
+        }
+        __syncwarp();
+    } else if (warp == kMvEpi + 1) {
+        // ---- the products (one thread)
+        if (lane == 0) {
+            uint32_t it = 0, n = 0;
+            const uint64_t ring_desc = sw64_desc(ring);
+            for (long long item = blockIdx.x; item < n_items && !failed; item += gridDim.x, ++n) {
+                const int nk = blocks_of((int)(item / a.n_chunks));
+                const int buf = n % Sh::NB;
+                if (n >= Sh::NB) wait_on(&acc_empty[buf], (n / Sh::NB - 1) & 1);
+                const uint32_t d = tmem + buf * (Sh::NA * kMvP);
+                for (int kb = 0; kb < nk && !failed; ++kb, ++it) {
+                    const int st = it % Sh::ST;
+                    wait_on(&full[st], (it / Sh::ST) & 1);
+                    if (failed) break;
+                    fence_after();
+                    const uint64_t base = ring_desc + (uint64_t)((st * kStage) >> 4);
+#pragma unroll
+                    for (int k16 = 0; k16 < kMvKB / 16; ++k16)
+#pragma unroll
+                        for (int p = 0; p < Sh::NP; ++p) {
+                            const int da = field(Sh::kA, p), db = field(Sh::kB, p), ac = field(Sh::kAcc, p);
+                            const bool first = p == 0 || ac != field(Sh::kAcc, p - 1);   // of its accumulator
+                            mma_f16_ss(d + ac * kMvP, base + (uint64_t)((da * kMvSlab + k16 * 32) >> 4),
+                                       base + (uint64_t)(((NS + db) * kMvSlab + k16 * 32) >> 4), kIdesc,
+                                       !(first && k16 == 0 && kb == 0));
+                        }
+                    mma_commit(&empty[st]);
+                }
+                if (!failed) mma_commit(&acc_full[buf]);
+            }
+            if (failed) {   // let the products in flight finish before the memory is released
+                mma_commit(&drained);
+                mbar_wait_bounded(&drained, 0, kMvPoll);
+            }
+        }
+        __syncwarp();
+    } else {
+        // ---- the epilogue: lanes = scenarios 32 (warp % 4) .., columns 64 (warp / 4) ..
+        const int quarter = warp & 3, half = warp >> 2;
+        uint32_t n = 0;
+        for (long long item = blockIdx.x; item < n_items; item += gridDim.x, ++n) {
+            const int tile = (int)(item / a.n_chunks), chunk = (int)(item - (long long)tile * a.n_chunks);
+            const int buf = n % Sh::NB;
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * kMvEpi) : "memory");   // the previous tile's records are read
+            reinterpret_cast<float4*>(recs)[tid] = reinterpret_cast<const float4*>(a.out + (size_t)tile * kMvP)[tid];
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * kMvEpi) : "memory");
+            bool ok = true;
+            if (lane == 0 && !failed) ok = mbar_wait_bounded(&acc_full[buf], (n / Sh::NB) & 1, kMvPoll);
+            ok = __shfl_sync(0xffffffffu, ok, 0);
+            if (!ok && !failed) {   // recorded; the later waits are skipped and nothing is written
+                failed = true;
+                if (lane == 0) atomicExch(a.status, DEV_TIMEOUT);
+            }
+            fence_after();
+            const int s = chunk * kMvM + quarter * 32 + lane;
+            const bool live = s < a.n_scen && !failed;
+            const float dsc = pow2f(a.colexp[s] - (NS == 3 ? 30 : 0));
+            const uint32_t col0 = tmem + ((uint32_t)(quarter * 32) << 16) + buf * (Sh::NA * kMvP) + half * 64;
+            df tot{0.0f, 0.0f};
+#pragma unroll 1
+            for (int c = 0; c < 64; c += 16) {
+                uint32_t r[Sh::NA][16];
+#pragma unroll
+                for (int k = 0; k < Sh::NA; ++k) tmem_ld16_async(col0 + k * kMvP + c, r[k]);
+#pragma unroll
+                for (int k = 0; k < Sh::NA; ++k) tmem_wait_ld(r[k]);
+                if (c == 48) {   // the accumulators are read
+                    fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&acc_empty[buf]);
+                }
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const MvOut& q = recs[half * 64 + c + i];
+                    if (q.pol < 0) continue;
+                    // the accumulators' sum as a double-float
+                    float h = __uint_as_float(r[0][i]), l = 0.0f;
+#pragma unroll
+                    for (int k = 1; k < Sh::NA; ++k) {
+                        const float b = __uint_as_float(r[k][i]), sum = __fadd_rn(h, b), bb = __fsub_rn(sum, h);
+                        l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(sum, bb)), __fsub_rn(b, bb)));
+                        h = sum;
+                    }
+                    df v = df_mul(df{__fmul_rn(h, dsc), __fmul_rn(l, dsc)}, df{q.sc_h, q.sc_l});
+                    if (q.mat_h != 0.0f) {   // a maturity payment: of the same sign
+                        df m{q.mat_h, q.mat_l};
+                        if (q.S > 0) {
+                            const float2 d = a.D[(size_t)(q.S - 1) * a.s_pad + s];
+                            m = df_mul(m, df{d.x, d.y});
+                        }
+                        const float sum = __fadd_rn(v.h, m.h), bb = __fsub_rn(sum, v.h);
+                        const float e = __fadd_rn(__fsub_rn(v.h, __fsub_rn(sum, bb)), __fsub_rn(m.h, bb));
+                        v = df{sum, __fadd_rn(e, __fadd_rn(v.l, m.l))};
+                    }
+                    // the sum over the policies
+                    const float sum = __fadd_rn(tot.h, v.h), bb = __fsub_rn(sum, tot.h);
+                    const float e = __fadd_rn(__fsub_rn(tot.h, __fsub_rn(sum, bb)), __fsub_rn(v.h, bb));
+                    tot = df{sum, __fadd_rn(tot.l, __fadd_rn(e, v.l))};
+                    if (live) {
+                        const size_t o = (size_t)q.pol * a.v0_ld + s;
+                        if (a.V0f) a.V0f[o] = __fadd_rn(v.h, v.l);
+                        if (a.V0d) a.V0d[o] = q.S == 0 && q.mat_h != 0.0f ? a.amount[q.pol] : (double)v.h + (double)v.l;
+                    }
+                }
+            }
+            if (a.partial && !failed) a.partial[(size_t)(2 * tile + half) * a.part_ld + s] = (double)tot.h + (double)tot.l;
+        }
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    if (warp == 0) tmem_free(tmem, 512);
+}
+
+template <int NS>
+cudaError_t product(const MvArgs& a, const void* digitsD, const void* digitsE, int pitchD, int pitchE, int sm_count,
+                    cudaStream_t st) {
+    CUtensorMap mD, mE;
+    if (!encode_map_16bit(&mD, CU_TENSOR_MAP_DATA_TYPE_UINT16, digitsD, pitchD, (uint64_t)NS * a.s_pad, pitchD, kMvKB, kMvM,
+                          CU_TENSOR_MAP_SWIZZLE_64B) ||
+        !encode_map_16bit(&mE, CU_TENSOR_MAP_DATA_TYPE_UINT16, digitsE, pitchE, (uint64_t)NS * kMvP * a.n_tiles, pitchE, kMvKB,
+                          kMvP, CU_TENSOR_MAP_SWIZZLE_64B))
+        return cudaErrorNotSupported;
+    constexpr size_t smem = (size_t)MvShape<NS>::ST * 2 * NS * kMvSlab + 1024;
+    auto k = mv_product_kernel<NS>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const long long items = (long long)a.n_tiles * a.n_chunks;
+    k<<<(int)std::min<long long>(items, sm_count), kMvThreads, smem, st>>>(mD, mE, a);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+const char* mv_variant_name(int form) { return form == F_DEFL ? "deflated matrix f16x3" : "comp matrix bf16x6"; }
+
+cudaError_t launch_mv_scenarios(const double* v64, int n_steps, int n_scen, int s_pad, float2* D, int32_t* tau,
+                                int32_t* colexp, int32_t* stat, cudaStream_t st) {
+    cudaError_t e = cudaMemsetAsync(stat, 0, 2 * sizeof(int32_t), st);
+    if (e != cudaSuccess) return e;
+    mv_products_kernel<<<s_pad / 32, dim3(32, 32), 0, st>>>(v64, n_steps, s_pad, D);
+    mv_tilt_kernel<<<n_steps, 128, 0, st>>>(D, n_scen, s_pad, tau, stat);
+    mv_columns_kernel<<<s_pad / 32, dim3(32, 8), 0, st>>>(D, tau, n_steps, n_scen, s_pad, colexp, stat);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mv_digits(int form, const float2* D, const int32_t* tau, const int32_t* colexp, int n_steps, int n_scen,
+                             int s_pad, int pitch, void* digits, cudaStream_t st) {
+    const dim3 grid(s_pad / 32, pitch / 64);
+    uint16_t* out = static_cast<uint16_t*>(digits);
+    if (mv_slices(form) == 3)
+        mv_digits_kernel<3><<<grid, 256, 0, st>>>(D, tau, colexp, n_steps, n_scen, s_pad, pitch, out);
+    else
+        mv_digits_kernel<6><<<grid, 256, 0, st>>>(D, tau, colexp, n_steps, n_scen, s_pad, pitch, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mv_build(int form, const MvBuild& b, cudaStream_t st) {
+    const int grid = b.n_tiles * (kMvP / 8);
+    const size_t smem = (size_t)b.pitch * sizeof(float);
+    if (mv_slices(form) == 3) mv_build_kernel<3><<<grid, 256, smem, st>>>(b);
+    else mv_build_kernel<6><<<grid, 256, smem, st>>>(b);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mv_product(int form, const MvArgs& a, const void* digitsD, const void* digitsE, int pitchD, int pitchE,
+                              int sm_count, cudaStream_t st) {
+    if (a.n_tiles <= 0 || a.n_chunks <= 0) return cudaSuccess;
+    return mv_slices(form) == 3 ? product<3>(a, digitsD, digitsE, pitchD, pitchE, sm_count, st)
+                                : product<6>(a, digitsD, digitsE, pitchD, pitchE, sm_count, st);
+}
+
+}  // namespace rsv

@@ -1,0 +1,111 @@
+// matval.cuh -- the valuation as a matrix product on the 5th-generation tensor cores.
+//
+// With deterministic mortality the reserve of policy p under scenario s is
+//   V(p, s) = amount_p [ sum_t D_s(t + 1) E_p(t) + D_s(S_p) B_p ],   D_s(t + 1) = v_0 ... v_t
+// (Eq. basicReserveSummation; cashflow.cuh): a product of the policies' expected cash
+// flows [policy][step] and the scenarios' discount products [step][scenario].  The
+// recurrence kernels run it chain by chain on the FP32 pipe; here it runs as 16-bit
+// matrix instructions with FP32 accumulation, on operands split into exact digits:
+//
+//   a = d1 + d2 + ...  with a in [0, 1]; d1: a to 7 bits.
+//   Deflated: d2 and d3 the FP16 values (11 bits and sign) of the remainders, to 2^-32 of
+//   the row's largest entry; stored times 2^15.
+//   Compensated: d2 and d3 the next 8 bits each (signed), d4 to d6 BF16 values of the
+//   remainders, to 2^-48.
+//
+// d1 d1' products are multiples of 2^-14, so up to 1,000 of them add up exactly in FP32
+// (rows with more steps give up one or two bits).  The compensated form's d1 d2' and its
+// d1 d3' and d2 d2' products, 2^-8 and 2^-16 below, are multiples of 2^-22 and 2^-30 and
+// have an exact accumulator each; the rest shares one more, whose FP32 truncations (of a
+// sum 2^-24, deflated 2^-8, below) are that much smaller.  The products left out are
+// below 2^-28 (compensated 2^-48).  The epilogue adds the accumulators as
+// double-floats.  A maturity payment is added there, from the discount products
+// themselves, so that a row holds entries of one kind.
+//
+// Fixed point needs rows and columns of moderate range.  The discount products are
+// tilted by a power of two per step, 2^tau(t) ~ 1 / (their geometric mean over the
+// scenarios), and the cash flows by 2^-tau(t), so that what is left of a scenario is its
+// deviation from the mean; a row is scaled by the power of two of its largest
+// entry.  A scenario set whose tilted products vary by more than 2^6 along a scenario
+// keeps the recurrence kernels.
+//
+// Measured (one GB300, with the digits and the totals): the 100,000-policy mix under 1,000
+// scenarios, compensated 38.7 -> 1.96 ms (error 1e-8 -> 2e-11 at most; annuities alone
+// 1e-13 -> 2.4e-13 rms, assurances 4e-9 -> 2e-13), deflated 4.93 -> 0.88 ms (rms 3e-8 ->
+// 5e-9); 1,000,000 annuities, 600 steps, deflated 30.6 -> 6.2 ms; 1,537 policies under
+// 157 scenarios, compensated, 254 -> 102 us on the device.  It is the faster path at
+// every size measured, from one policy and one scenario up.
+#pragma once
+
+#include <cuda.h>
+
+#include "cashflow.cuh"
+
+namespace rsv {
+
+constexpr int kMvP = 128;          // policies per tile (MMA N)
+constexpr int kMvM = 128;          // scenarios per tile (MMA M)
+constexpr int kMvKB = 32;          // steps per staged block: 64-byte swizzled rows
+constexpr int kMvSpread = 6;       // log2 of the range of a scenario's tilted discount products
+constexpr int kMvTilt = 60;        // largest |tau|
+constexpr size_t kMvPanelBytes = size_t(1) << 30;            // cash-flow digits held at a time
+constexpr double kMvTableMin = 0x1p-100;                    // survivor columns in FP32 head and tail
+constexpr double kMvAmountMin = 0x1p-60, kMvAmountMax = 0x1p90;   // |amount|: V in FP32 head and tail
+
+inline int mv_slices(int form) { return form == F_DEFL ? 3 : 6; }
+inline int mv_pitch(int steps) { return steps < 1 ? 64 : (steps + 63) / 64 * 64; }
+
+// Scenario side, from the FP64 plane [n_steps][s_pad]: the discount products, the tilt of
+// each step, the binary exponent of each column's largest tilted product, and
+// stat = {largest spread of a column, largest |tau|} (INT_MAX where a product
+// is not a normal number).
+cudaError_t launch_mv_scenarios(const double* v64, int n_steps, int n_scen, int s_pad, float2* D, int32_t* tau,
+                                int32_t* colexp, int32_t* stat, cudaStream_t st);
+// Its digits [slices][s_pad][pitch]; columns beyond n_scen and steps beyond n_steps are 0.
+cudaError_t launch_mv_digits(int form, const float2* D, const int32_t* tau, const int32_t* colexp, int n_steps, int n_scen,
+                             int s_pad, int pitch, void* digits, cudaStream_t st);
+
+// Policy side of one panel of tiles: digits [tile][slices][128][pitch] up to each tile's
+// longest projection, and what the epilogue needs of each policy.
+struct alignas(16) MvOut {   // 32 bytes
+    float sc_h, sc_l;    // V = (sc_h + sc_l) 2^(colexp) U (deflated: 2^-30 of it) + (mat_h + mat_l) D(S)
+    float mat_h, mat_l;  // the maturity payment times its probability
+    int32_t pol, S, pad[2];
+};
+struct MvBuild {
+    CfTables T;
+    const SlotRec* slots;      // of the panel's first tile
+    const int32_t* kinds;
+    const double* amount;
+    int32_t n_tiles, tab_pad, pitch;
+    int32_t general_from;      // first tile of the panel whose policies have varying cash flows
+    const double* cf;          // their multipliers [n_pol][cf_ld], or null
+    int32_t cf_ld;
+    const int32_t* tau;
+    void* digits;
+    MvOut* out;
+};
+cudaError_t launch_mv_build(int form, const MvBuild& b, cudaStream_t st);
+
+struct MvArgs {
+    const SlotRec* slots;
+    const MvOut* out;
+    const int32_t* colexp;     // of the first column
+    const float2* D;           // the discount products [n_steps][s_pad], at the first column
+    const double* amount;
+    int32_t n_tiles, n_chunks; // policy tiles of the panel, scenario tiles of the column block
+    int32_t s_pad, n_scen, s0; // plane rows; valid columns of the block; the block's first column
+    int32_t v0_ld, part_ld;
+    float* V0f;                // at the block's first column
+    double* V0d;
+    double* partial;           // [2 n_tiles][part_ld], at the panel's first tile and the block's first column
+    int32_t* status;
+};
+// digitsE: launch_mv_build's, digitsD: launch_mv_digits'.
+cudaError_t launch_mv_product(int form, const MvArgs& a, const void* digitsD, const void* digitsE, int pitchD, int pitchE,
+                              int sm_count, cudaStream_t st);
+
+// The matrix variant's index among a form's tunable variants is the last one.
+const char* mv_variant_name(int form);
+
+}  // namespace rsv

@@ -19,6 +19,7 @@
 #include "abi_guard.cuh"
 #include "ctx.cuh"
 #include "cashflow.cuh"
+#include "matval.cuh"
 #include "nested.cuh"
 #include "scan.cuh"
 #include "summation.cuh"
@@ -605,6 +606,92 @@ rsv_status upload_amounts(rsv_ctx* c) {
     return RSV_OK;
 }
 
+}  // namespace
+
+bool rsv::mv_applies(const rsv_ctx* c) {
+    if (!c->mv_scen_ok || !(c->amt_hi <= kMvAmountMax) || !(c->amt_lo >= kMvAmountMin)) return false;
+    for (int t = 0; t < kMaxTables; ++t)
+        if (!c->tab[t].empty() && !(c->tab_min[t] >= kMvTableMin)) return false;
+    return true;
+}
+
+rsv_status rsv::mv_prepare(rsv_ctx* c, int form) {
+    const Layout& L = c->lay;
+    rsv_status st;
+    CfTables T;
+    if ((st = layout_to_device(c)) != RSV_OK || (st = upload_amounts(c)) != RSV_OK || (st = cf_tables(c, T)) != RSV_OK)
+        return st;
+    const int k = form == F_DEFL ? 1 : 0, pitch = mv_pitch(c->n_steps);
+    if (c->mv_dig_gen[k] != c->scen_gen) {   // with the scenario set, like its planes
+        CU(c->d_mv_dig[k].ensure((size_t)mv_slices(form) * c->s_pad * pitch * 2));
+        const int32_t* tau = c->d_mv_col.as<int32_t>();
+        CU(launch_mv_digits(form, c->d_mv_D.as<float2>(), tau, tau + c->n_steps, c->n_steps, c->n_scen, c->s_pad, pitch,
+                            c->d_mv_dig[k].p, c->stream));
+        c->mv_dig_gen[k] = c->scen_gen;
+    }
+    const size_t tile = (size_t)mv_slices(form) * kMvP * mv_pitch(L.max_S) * 2;
+    const int panel = (int)std::max<size_t>(1, std::min<size_t>(std::max(1, L.n_tiles), kMvPanelBytes / tile));
+    CU(c->d_mv_E.ensure(tile * panel));
+    CU(c->d_mv_out.ensure((size_t)panel * kMvP * sizeof(MvOut)));
+    c->mv_built = -1;
+    return RSV_OK;
+}
+
+rsv_status rsv::mv_launch(rsv_ctx* c, int form, int s0, int w, float* V0f, double* V0d, double* partial) {
+    const Layout& L = c->lay;
+    CfTables T;
+    const rsv_status st = cf_tables(c, T);
+    if (st != RSV_OK) return st;
+    const int pitchE = mv_pitch(L.max_S), pitchD = mv_pitch(c->n_steps);
+    const size_t tile = (size_t)mv_slices(form) * kMvP * pitchE * 2;
+    const int panel = (int)std::max<size_t>(1, std::min<size_t>(std::max(1, L.n_tiles), kMvPanelBytes / tile));
+    const int32_t* tau = c->d_mv_col.as<int32_t>();
+    for (int t0 = 0; t0 < L.n_tiles; t0 += panel) {
+        const int n = std::min(panel, L.n_tiles - t0);
+        const SlotRec* slots = L.slots.as<SlotRec>() + (size_t)t0 * kMvP;
+        if (c->mv_built != t0) {
+            MvBuild b{};
+            b.T = T;
+            b.slots = slots;
+            b.kinds = L.kinds.as<int32_t>() + t0;
+            b.amount = c->d_amount.as<double>();
+            b.n_tiles = n;
+            b.tab_pad = L.tab_pad;
+            b.pitch = pitchE;
+            b.general_from = L.P_general > 0 ? std::max(0, L.grp_tiles[0] - t0) : n;
+            b.cf = c->d_cf64.as<double>();
+            b.cf_ld = c->cf_steps;
+            b.tau = tau;
+            b.digits = c->d_mv_E.p;
+            b.out = c->d_mv_out.as<MvOut>();
+            CU(launch_mv_build(form, b, c->stream));
+            c->mv_built = t0;
+        }
+        MvArgs a{};
+        a.slots = slots;
+        a.out = c->d_mv_out.as<MvOut>();
+        a.colexp = tau + c->n_steps + s0;
+        a.D = c->d_mv_D.as<float2>() + s0;
+        a.amount = c->d_amount.as<double>();
+        a.n_tiles = n;
+        a.n_chunks = (w + kMvM - 1) / kMvM;
+        a.s_pad = c->s_pad;
+        a.n_scen = w;
+        a.s0 = s0;
+        a.v0_ld = c->n_scen;
+        a.part_ld = c->s_pad;
+        a.V0f = V0f;
+        a.V0d = V0d;
+        a.partial = partial ? partial + (size_t)2 * t0 * c->s_pad : nullptr;
+        a.status = c->d_ctl.as<int32_t>() + 1;
+        CU(launch_mv_product(form, a, c->d_mv_dig[form == F_DEFL ? 1 : 0].p, c->d_mv_E.p, pitchD, pitchE, c->sm_count,
+                             c->stream));
+    }
+    return RSV_OK;
+}
+
+namespace {
+
 rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     if (!c) return RSV_E_ARG;
     if (!o || !out) return fail(c, RSV_E_ARG, "opts and out must not be NULL");
@@ -655,23 +742,31 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     // keep the fast kernel (tile group 0) and the others take the
     // general-cash-flow kernel (group 1).
     const bool split = cfl && pay == PAY_END && !extra && !scan && !summ;
+    // The matrix product (the last tunable variant of the compensated form) where it
+    // covers the data, unless another variant was tuned or asked for.
+    bool mat = false;
     int vi, vg = -1;
     if (extra || scan || summ) {
         vi = special_variant(vl, nv, true, PAY_END);
     } else if (pay != PAY_END) {
         vi = special_variant(vl, nv, false, pay);
     } else if (o->variant >= 0) {
-        if (o->variant >= nt) return fail(c, RSV_E_ARG, "variant %d out of range", o->variant);
+        if (o->variant >= rsv_variant_count(o->form)) return fail(c, RSV_E_ARG, "variant %d out of range", o->variant);
         vi = o->variant;
     } else if (o->variant == -1) {
-        vi = c->tuned[o->form] >= 0 ? c->tuned[o->form] : 0;
+        vi = c->tuned[o->form] >= 0 ? c->tuned[o->form] : (o->form == F_COMP ? nt : 0);
     } else {
         return fail(c, RSV_E_ARG, "variant %d out of range", o->variant);
+    }
+    if (o->form == F_COMP && vi == nt && !extra && pay == PAY_END) {
+        mat = mv_applies(c);
+        vi = 0;
     }
     if (split) vg = special_variant(vl, nv, false, PAY_END_GENERAL);
     const Variant& V = vl[vi];
 
-    rsv_status st = build_layout(c, (scan || summ) ? 1 : V.P, o->horizon, c->n_steps, split ? vl[vg].P : 0);
+    rsv_status st = build_layout(c, (scan || summ) ? 1 : (mat ? kMvP : V.P), o->horizon, c->n_steps,
+                                 split ? (mat ? kMvP : vl[vg].P) : 0);
     if (st == RSV_OK) st = layout_to_device(c);
     if (st != RSV_OK) return st;
     if (cfl && c->lay.max_S > c->cf_steps)
@@ -683,12 +778,15 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
         if (c->vf_scen != c->n_scen || c->vf_steps != c->n_steps)
             return fail(c, RSV_E_STATE, "fractional discount factors not loaded for the scenario set's shape");
         if ((st = build_tables_frac(c, o->form, smem, tabf_off)) != RSV_OK) return st;
-    } else if ((st = build_tables(c, o->form, smem)) != RSV_OK) {
+    } else if ((st = mat ? table_bytes(c, o->form, c->lay.tab_pad, c->lay.n_tab, smem) : build_tables(c, o->form, smem)) !=
+               RSV_OK) {
         return st;
     }
     if ((st = upload_amounts(c)) != RSV_OK) return st;
+    if (mat && (st = mv_prepare(c, o->form)) != RSV_OK) return st;
 
     const Layout& L = c->lay;
+    const int part_rows = mat ? 2 * L.n_tiles : L.n_tiles;   // rows of per-tile scenario sums
     float* V0f = (outs & RSV_OUT_V0) ? out->V0 : nullptr;
     double* V0d = (outs & RSV_OUT_V0) ? out->V0d : nullptr;
     double* tot = (outs & RSV_OUT_SCEN_TOTAL) ? out->scen_total : nullptr;
@@ -707,7 +805,7 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     CU(cudaMemsetAsync(c->d_ctl.p, 0, 2 * sizeof(int32_t), c->stream));
     if (pt) CU(cudaMemsetAsync(pt, 0, n_pt * sizeof(double), c->stream));
     if (traj) CU(cudaMemsetAsync(traj, 0, n_traj * sizeof(double), c->stream));
-    if (tot) CU(c->d_partial.ensure((size_t)std::max(1, L.n_tiles) * c->s_pad * sizeof(double)));
+    if (tot) CU(c->d_partial.ensure((size_t)std::max(1, part_rows) * c->s_pad * sizeof(double)));
     if (tot && L.n_tiles == 0) CU(cudaMemsetAsync(tot, 0, NSc * sizeof(double), c->stream));
 
     RecurArgs a{};
@@ -743,7 +841,8 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     // One launch per non-empty tile group on the scenario columns of `base`:
     // group 0 by V (with the cash flows unless they are split off), group 1
     // by the general-cash-flow variant; each with its own zeroed queue head.
-    auto launch_groups = [&](const RecurArgs& base) -> rsv_status {
+    auto launch_groups = [&](const RecurArgs& base, int s0) -> rsv_status {
+        if (mat) return mv_launch(c, o->form, s0, base.n_scen, base.V0f, base.V0d, base.partial);
         for (int g = 0; g < 2; ++g) {
             const int n_t = L.grp_tiles[g];
             if (n_t == 0) continue;
@@ -793,7 +892,7 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
             b.V0f = a.V0f ? a.V0f + s0 : nullptr;
             b.V0d = a.V0d ? a.V0d + s0 : nullptr;
             b.partial = a.partial ? a.partial + s0 : nullptr;
-            if ((st = launch_groups(b)) != RSV_OK) return st;
+            if ((st = launch_groups(b, s0)) != RSV_OK) return st;
             CU(cudaEventRecord(c->ev_block, c->stream));
             CU(cudaStreamWaitEvent(c->copy_stream, c->ev_block, 0));
             CU(cudaMemcpy2DAsync(hV0 + (size_t)s0 * esz_o, (size_t)NSc * esz_o, dV0 + (size_t)s0 * esz_o,
@@ -815,13 +914,13 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
             CU(cudaEventRecord(c->ev1, c->stream));
         } else {
             CU(cudaEventRecord(c->ev0, c->stream));
-            if ((st = launch_groups(a)) != RSV_OK) return st;
+            if ((st = launch_groups(a, 0)) != RSV_OK) return st;
             CU(cudaEventRecord(c->ev1, c->stream));
         }
         c->ev_recorded = true;
     }
     if (L.n_tiles > 0) {
-        if (tot && (st = scenario_totals(c, a.partial, L.n_tiles, c->s_pad, NSc, tot)) != RSV_OK) return st;
+        if (tot && (st = scenario_totals(c, a.partial, part_rows, c->s_pad, NSc, tot)) != RSV_OK) return st;
         if (pt) {
             scale_kernel<<<c->sm_count * 4, 256, 0, c->stream>>>(pt, n_pt, 1.0 / NSc);
             CU(cudaGetLastError());
@@ -1116,6 +1215,7 @@ rsv_status rsv_destroy(rsv_ctx* c) try {
                       &c->sur.d_comm, &c->sur.d_lnb, &c->d_tabf[0], &c->d_tabf[1], &c->d_tabf[2], &c->d_vf64,
                       &c->d_vf32, &c->d_vf2, &c->d_cf64, &c->d_cf32, &c->d_ml_rec,
                       &c->d_ml_amount, &c->sur.d_cnt, &c->sur.d_q2, &c->sur.d_idx, &c->sur.d_v2, &c->d_nest_bm,
+                      &c->d_mv_D, &c->d_mv_col, &c->d_mv_dig[0], &c->d_mv_dig[1], &c->d_mv_E, &c->d_mv_out,
                       &c->d_defl_slots, &c->d_defl_kinds, &c->d_defl_tab, &c->d_defl_plane, &c->d_mlp_trace})
         b->release();
     c->mlp.release();
@@ -1149,6 +1249,12 @@ rsv_status rsv_load_decrements(rsv_ctx* c, int32_t table_id, const double* p, in
         if (!(p[k] >= 0.0 && p[k] <= 1.0))
             return fail(c, RSV_E_ASSUMPTION, "table %d entry %d = %g is not a probability", table_id, k, p[k]);
     c->tab[table_id].assign(p, p + n);
+    double m = 1.0, least = 1.0;   // of the survivor columns (cashflow.cuh)
+    for (int k = 0; k < n; ++k) {
+        if (p[k] < 1.0) least = std::min(least, m * (1.0 - p[k]));
+        if (p[k] > 0.0) least = std::min(least, m *= p[k]);
+    }
+    c->tab_min[table_id] = least;
     ++c->tab_gen;
     return RSV_OK;
 } catch (...) {
@@ -1280,10 +1386,21 @@ rsv_status rsv_load_portfolio(rsv_ctx* c, const rsv_policy* pols, int64_t n) try
     c->pols.resize((size_t)n);
     const int hw = (int)std::max(1u, std::thread::hardware_concurrency());
     const int T = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(hw, 16), n / 65536));
+    std::vector<double> amt_lo(T, INFINITY), amt_hi(T, 0.0);
     run_parts(T, [&](int k) {
         const int64_t lo = n * k / T, hi = n * (k + 1) / T;
         if (hi > lo) memcpy(c->pols.data() + lo, pols + lo, (size_t)(hi - lo) * sizeof(rsv_policy));
+        double mn = INFINITY, mx = 0.0;
+        for (int64_t i = lo; i < hi; ++i) {
+            const double a = std::fabs(pols[i].amount);
+            mx = std::max(mx, a);
+            if (a > 0.0) mn = std::min(mn, a);
+        }
+        amt_lo[k] = mn;
+        amt_hi[k] = mx;
     });
+    c->amt_lo = *std::min_element(amt_lo.begin(), amt_lo.end());
+    c->amt_hi = *std::max_element(amt_hi.begin(), amt_hi.end());
     ++c->pol_gen;
     c->amount_dirty = true;
     return RSV_OK;
@@ -1312,7 +1429,18 @@ rsv_status rsv_load_scenarios(rsv_ctx* c, const double* v, int32_t n_scen, int32
                                                                 s_pad, c->d_v64.as<double>(), c->d_v32.as<float>(),
                                                                 c->d_v2.as<float2>());
     CU(cudaGetLastError());
+    // the discount products and their range for the matrix product
+    CU(c->d_mv_D.ensure(np * sizeof(float2)));
+    CU(c->d_mv_col.ensure(((size_t)n_steps + s_pad + 2) * sizeof(int32_t)));
+    int32_t* tau = c->d_mv_col.as<int32_t>();
+    int32_t* stat = tau + n_steps + s_pad;
+    CU(launch_mv_scenarios(c->d_v64.as<double>(), n_steps, n_scen, s_pad, c->d_mv_D.as<float2>(), tau, tau + n_steps, stat,
+                           c->stream));
+    int32_t range[2];
+    CU(cudaMemcpyAsync(range, stat, sizeof range, cudaMemcpyDeviceToHost, c->stream));
     CU(cudaStreamSynchronize(c->stream));
+    c->mv_scen_ok = range[0] <= kMvSpread && range[1] <= kMvTilt;
+    ++c->scen_gen;
     c->n_scen = n_scen;
     c->n_steps = n_steps;
     c->s_pad = s_pad;
@@ -1342,20 +1470,20 @@ rsv_status rsv_compute_nested(rsv_ctx* c, const rsv_opts* o, const rsv_nested_sp
 
 int32_t rsv_variant_count(int32_t form) {
     int n = 0;
-    if (form == F_DEFL) return variants_defl(&n) ? n : 0;
+    if (form == F_DEFL) return variants_defl(&n) ? n + 1 : 0;   // and the matrix product, the last
     const Variant* vl = variant_list(form, &n);
-    return vl ? tunable_count(vl, n) : 0;
+    return vl ? tunable_count(vl, n) + (form == F_COMP ? 1 : 0) : 0;
 }
 
 const char* rsv_variant_name(int32_t form, int32_t variant) {
     int n = 0;
-    if (form == F_DEFL) {
-        const DeflVariant* dv = variants_defl(&n);
-        return (variant < 0 || variant >= n) ? "" : dv[variant].name;
-    }
-    const Variant* v = variant_list(form, &n);
-    if (!v || variant < 0 || variant >= n) return "";
-    return v[variant].name;
+    const int count = rsv_variant_count(form);
+    if (variant < 0) return "";
+    if ((form == F_DEFL || form == F_COMP) && variant == count - 1) return mv_variant_name(form);
+    if (form == F_DEFL) return variant < count ? variants_defl(&n)[variant].name : "";
+    const Variant* v = variant_list(form, &n);   // the side-output and payment variants after the tunable ones
+    const int k = form == F_COMP && variant >= count ? variant - 1 : variant;
+    return v && k < n ? v[k].name : "";
 }
 
 rsv_status rsv_tune(rsv_ctx* c, const rsv_opts* opts, int32_t reps, int32_t* best, float* ms_out) try {
