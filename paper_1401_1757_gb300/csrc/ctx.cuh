@@ -291,7 +291,7 @@ rsv_status cf_tables(rsv_ctx* c, CfTables& T);
 rsv_status stage_tables(rsv_ctx* c, int form, int pad, int n_tab, size_t& smem);
 // Whether the matrix product covers the loaded data; then, on the layout of width
 // kMvP: mv_prepare once a call, mv_launch for the scenario columns [s0, s0 + w) with the
-// output pointers at column s0 (partial: [2 n_tiles][s_pad]).
+// output pointers at column s0 (partial: [n_tiles][s_pad]).
 bool mv_applies(const rsv_ctx* c);
 rsv_status mv_prepare(rsv_ctx* c, int form);
 rsv_status mv_launch(rsv_ctx* c, int form, int s0, int w, float* V0f, double* V0d, double* partial);

@@ -155,7 +155,6 @@ rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     const Layout& L = c->lay;
     if ((st = mat ? defl_table_range(c, T) : defl_table_stage(c, T)) != RSV_OK) return st;
     if (mat && (st = mv_prepare(c, F_DEFL)) != RSV_OK) return st;
-    const int part_rows = mat ? 2 * L.n_tiles : L.n_tiles;   // rows of per-tile scenario sums
     const int n_tab = T.n_tab, dpad = T.dpad, arr_d = T.arr_d;
     const size_t tab_bytes = T.bytes;
     const std::vector<std::vector<double>>& ell = T.ell;
@@ -307,7 +306,7 @@ rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     }
     CU(c->d_ctl.ensure(2 * sizeof(int32_t)));
     CU(cudaMemsetAsync(c->d_ctl.p, 0, 2 * sizeof(int32_t), c->stream));
-    if (tot) CU(c->d_partial.ensure((size_t)std::max(1, part_rows) * s_pad * sizeof(double)));
+    if (tot) CU(c->d_partial.ensure((size_t)std::max(1, L.n_tiles) * s_pad * sizeof(double)));
     if (tot && L.n_tiles == 0) CU(cudaMemsetAsync(tot, 0, NSc * sizeof(double), c->stream));
 
     // the deflator plane, rows of four steps, a whole number of staged blocks
@@ -390,7 +389,7 @@ rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
         CU(cudaEventRecord(c->ev1, c->stream));
     }
     c->ev_recorded = true;
-    if (tot && L.n_tiles > 0 && (st = scenario_totals(c, a.partial, part_rows, s_pad, NSc, tot)) != RSV_OK) return st;
+    if (tot && L.n_tiles > 0 && (st = scenario_totals(c, a.partial, L.n_tiles, s_pad, NSc, tot)) != RSV_OK) return st;
     if (!o->on_device) {
         if (hV0f && !copied_v0) CU(cudaMemcpyAsync(hV0f, V0f, n_v0 * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
         if (hV0d && !copied_v0) CU(cudaMemcpyAsync(hV0d, V0d, n_v0 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));

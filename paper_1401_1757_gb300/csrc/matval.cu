@@ -339,43 +339,67 @@ __global__ void __launch_bounds__(256) mv_build_kernel(const MvBuild b) {
 }
 
 // -------------------------------------------------------------- the product ----
-// Persistent CTAs over (policy tile, scenario tile) items, longest projections first.
-// A block of 32 steps of both operands' digits is staged by TMA (64-byte swizzle) into a ring
-// of stages; one thread issues the digits' products, m128 n128 k16 with the scenarios
-// on the lanes (A) and the policies on the columns (B); eight warps add the accumulators as
+// Persistent pairs of CTAs over (policy tile, pair of scenario tiles) items.  A block of
+// steps of the digits is staged by TMA into a ring of stages: each CTA its 128 scenarios'
+// (A) and half of the tile's 128 policies' (B); one thread of rank 0 issues the digits'
+// products, m256 n128 k16 over both CTAs (cta_group::2).  In each CTA the scenarios are
+// on the lanes and the policies on the columns; sixteen warps add the accumulators as
 // double-floats, scale, write V0 (32 consecutive scenarios of a policy a warp store) and
-// keep each scenario's sum over the tile's policies.
+// sum each scenario over the tile's policies.
 // Deflated: 6 products and 2 accumulators, so TMEM holds two tiles' and the epilogue runs
 // beside the next tile's products; compensated: 21 products, 4 accumulators.
 template <int NS>
-struct MvShape;   // products, accumulators, tiles in TMEM, stages; per product 3 bits each of the
-template <>       // scenario digit, the policy digit and the accumulator
-struct MvShape<3> {
-    static constexpr int NP = 6, NA = 2, NB = 2, ST = 4;
-    static constexpr uint64_t kA = 0x10240, kB = 0x2208, kAcc = 0x9248;
+struct MvShape;   // accumulators, tiles in TMEM, stages, steps of a block (64: 128-byte swizzled
+template <>       // rows); the products are (i, j), i + j < NS, of scenario digit i and policy
+struct MvShape<3> {   // digit j, in accumulator min(i + j, NA - 1)
+    static constexpr int NA = 2, NB = 2, ST = 3, KB = 64;
 };
 template <>
 struct MvShape<6> {
-    static constexpr int NP = 21, NA = 4, NB = 1, ST = 2;
-    static constexpr uint64_t kA = 0x510b503298450240, kB = 0xa62621683282208, kAcc = 0x36db6db6db6d2448;
+    static constexpr int NA = 4, NB = 1, ST = 3, KB = 32;
 };
-__host__ __device__ constexpr int field(uint64_t v, int p) { return (int)(v >> (3 * p)) & 7; }
-constexpr int kMvEpi = 8;                              // epilogue warps
+constexpr int kMvEpi = 4 * kMvParts;                   // epilogue warps
 constexpr int kMvThreads = 32 * (kMvEpi + 2);
-constexpr int kMvSlab = kMvP * kMvKB * 2;              // 8 KiB: one digit of one operand's block
+constexpr int kMvHalf = kMvP / 2;                      // policies staged by one CTA of a pair
+
+// shared memory of a stage: NS slabs of scenario digits, then NS of policy digits
+template <int NS>
+struct MvStage {
+    static constexpr int kA = kMvM * MvShape<NS>::KB * 2, kB = kMvHalf * MvShape<NS>::KB * 2;
+    static constexpr int kBytes = NS * (kA + kB);
+};
+
+// The products of scenario digit I and policy digits J .., then of digits I + 1 ..; more: the
+// accumulators hold earlier blocks' sums.
+template <int NS, int I, int J>
+__device__ __forceinline__ void mv_products(uint32_t d, uint64_t base, int off, uint32_t idesc, bool more) {
+    using G = MvStage<NS>;
+    constexpr int acc = I + J < MvShape<NS>::NA ? I + J : MvShape<NS>::NA - 1;
+    constexpr bool first = I == 0 && J == acc;   // of its accumulator
+    mma_f16_ss_pair(d + acc * kMvP, base + (uint64_t)((I * G::kA + off) >> 4),
+                    base + (uint64_t)((NS * G::kA + J * G::kB + off) >> 4), idesc, !first || more);
+    if constexpr (I + J + 1 < NS) mv_products<NS, I, J + 1>(d, base, off, idesc, more);
+    else if constexpr (I + 1 < NS) mv_products<NS, I + 1, 0>(d, base, off, idesc, more);
+}
 
 template <int NS>
-__global__ void __launch_bounds__(kMvThreads, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
     mv_product_kernel(const __grid_constant__ CUtensorMap mapD, const __grid_constant__ CUtensorMap mapE, const MvArgs a) {
     using Sh = MvShape<NS>;
-    constexpr int kStage = 2 * NS * kMvSlab;
-    constexpr uint32_t kIdesc = f16_idesc(NS != 3, kMvM, kMvP);   // both operands FP16, or both BF16
+    using G = MvStage<NS>;
+    constexpr int KB = Sh::KB;
+    constexpr uint32_t kIdesc = f16_idesc(NS != 3, 2 * kMvM, kMvP);   // both operands FP16, or both BF16
     extern __shared__ __align__(1024) unsigned char smem_raw[];
+    // (both CTAs of a pair place everything alike)
     unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    // rank 0's full[st]: both CTAs' copies of a stage; empty[st]: its products are done;
+    // acc_full: a tile's products are done; rank 0's acc_empty: both epilogues have read it
     __shared__ uint64_t full[Sh::ST], empty[Sh::ST], acc_full[Sh::NB], acc_empty[Sh::NB], drained;
     __shared__ uint32_t tmem_slot;
     __shared__ MvOut recs[kMvP];
+    __shared__ float2 sums[kMvParts][kMvM];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = (int)cluster_rank();
     if (tid == 0) {
         for (int i = 0; i < Sh::ST; ++i) {
             mbar_init(&full[i], 1);
@@ -383,17 +407,18 @@ __global__ void __launch_bounds__(kMvThreads, 1)
         }
         for (int i = 0; i < Sh::NB; ++i) {
             mbar_init(&acc_full[i], 1);
-            mbar_init(&acc_empty[i], kMvEpi);
+            mbar_init(&acc_empty[i], 2 * kMvEpi);
         }
         mbar_init(&drained, 1);
         fence_barrier_init();
     }
-    if (warp == 0) tmem_alloc(&tmem_slot, 512);
+    if (warp == 0) tmem_alloc_pair(&tmem_slot, 512);
     fence_before();
-    __syncthreads();
+    cluster_sync();
     fence_after();
     const uint32_t tmem = tmem_slot;
-    const long long n_items = (long long)a.n_tiles * a.n_chunks;
+    const int n_pairs = (a.n_chunks + 1) / 2, n_clusters = (int)gridDim.x / 2, cluster = (int)blockIdx.x / 2;
+    const long long n_items = (long long)a.n_tiles * n_pairs;
     bool failed = false;
     auto wait_on = [&](uint64_t* bar, uint32_t parity) {   // a bounded wait; a timeout is recorded
         if (failed) return;
@@ -402,40 +427,44 @@ __global__ void __launch_bounds__(kMvThreads, 1)
             atomicExch(a.status, DEV_TIMEOUT);
         }
     };
-    auto blocks_of = [&](int tile) { return max(1, (a.slots[(size_t)tile * kMvP].S + kMvKB - 1) / kMvKB); };
+    auto blocks_of = [&](int tile) { return max(1, (a.slots[(size_t)tile * kMvP].S + KB - 1) / KB); };
 
     if (warp == kMvEpi) {
-        // ---- the copies (one thread)
-        if (lane == 0) {
+        // ---- the copies (one thread of each CTA)
+        if (elect_one()) {
             uint32_t it = 0;
-            for (long long item = blockIdx.x; item < n_items && !failed; item += gridDim.x) {
-                const int tile = (int)(item / a.n_chunks), chunk = (int)(item - (long long)tile * a.n_chunks);
+            for (long long item = cluster; item < n_items && !failed; item += n_clusters) {
+                const int tile = (int)(item / n_pairs), chunk = 2 * (int)(item - (long long)tile * n_pairs) + rank;
                 const int nk = blocks_of(tile);
                 for (int kb = 0; kb < nk && !failed; ++kb, ++it) {
                     const int st = it % Sh::ST;
                     if (it >= Sh::ST) wait_on(&empty[st], (it / Sh::ST - 1) & 1);
                     if (failed) break;
-                    unsigned char* dst = ring + st * kStage;
-                    mbar_arrive_expect_tx(&full[st], kStage);
+                    unsigned char* dst = ring + st * G::kBytes;
+                    const uint32_t bar = of_rank0(&full[st]);
+                    if (rank == 0) mbar_arrive_expect_tx(&full[st], 2 * G::kBytes);
 #pragma unroll
                     for (int k = 0; k < NS; ++k) {
-                        tma_load_2d(dst + k * kMvSlab, &mapD, kb * kMvKB, k * a.s_pad + a.s0 + chunk * kMvM, &full[st]);
-                        tma_load_2d(dst + (NS + k) * kMvSlab, &mapE, kb * kMvKB, (tile * NS + k) * kMvP, &full[st]);
+                        tma_load_2d_pair(dst + k * G::kA, &mapD, kb * KB, k * a.s_pad + a.s0 + chunk * kMvM, bar);
+                        tma_load_2d_pair(dst + NS * G::kA + k * G::kB, &mapE, kb * KB, (tile * NS + k) * kMvP + rank * kMvHalf,
+                                         bar);
                     }
                 }
             }
-            if (failed)   // let the copies in flight land before the memory is released
+            // let the copies in flight land before the memory is released (rank 1's complete on
+            // rank 0's barriers, and rank 1 stays until rank 0 has come to the end)
+            if (failed && rank == 0)
                 for (uint32_t back = 0; back < Sh::ST && back < it; ++back)
                     mbar_wait_bounded(&full[(it - 1 - back) % Sh::ST], ((it - 1 - back) / Sh::ST) & 1, kMvPoll);
         }
         __syncwarp();
     } else if (warp == kMvEpi + 1) {
-        // ---- the products (one thread)
-        if (lane == 0) {
+        // ---- the products (one thread of rank 0)
+        if (rank == 0 && elect_one()) {
             uint32_t it = 0, n = 0;
-            const uint64_t ring_desc = sw64_desc(ring);
-            for (long long item = blockIdx.x; item < n_items && !failed; item += gridDim.x, ++n) {
-                const int nk = blocks_of((int)(item / a.n_chunks));
+            const uint64_t ring_desc = KB == 64 ? sw128_desc(ring) : sw64_desc(ring);
+            for (long long item = cluster; item < n_items && !failed; item += n_clusters, ++n) {
+                const int nk = blocks_of((int)(item / n_pairs));
                 const int buf = n % Sh::NB;
                 if (n >= Sh::NB) wait_on(&acc_empty[buf], (n / Sh::NB - 1) & 1);
                 const uint32_t d = tmem + buf * (Sh::NA * kMvP);
@@ -444,36 +473,30 @@ __global__ void __launch_bounds__(kMvThreads, 1)
                     wait_on(&full[st], (it / Sh::ST) & 1);
                     if (failed) break;
                     fence_after();
-                    const uint64_t base = ring_desc + (uint64_t)((st * kStage) >> 4);
+                    const uint64_t base = ring_desc + (uint64_t)((st * G::kBytes) >> 4);
 #pragma unroll
-                    for (int k16 = 0; k16 < kMvKB / 16; ++k16)
-#pragma unroll
-                        for (int p = 0; p < Sh::NP; ++p) {
-                            const int da = field(Sh::kA, p), db = field(Sh::kB, p), ac = field(Sh::kAcc, p);
-                            const bool first = p == 0 || ac != field(Sh::kAcc, p - 1);   // of its accumulator
-                            mma_f16_ss(d + ac * kMvP, base + (uint64_t)((da * kMvSlab + k16 * 32) >> 4),
-                                       base + (uint64_t)(((NS + db) * kMvSlab + k16 * 32) >> 4), kIdesc,
-                                       !(first && k16 == 0 && kb == 0));
-                        }
-                    mma_commit(&empty[st]);
+                    for (int k16 = 0; k16 < KB / 16; ++k16) mv_products<NS, 0, 0>(d, base, k16 * 32, kIdesc, kb + k16 > 0);
+                    mma_commit_pair(&empty[st]);
                 }
-                if (!failed) mma_commit(&acc_full[buf]);
+                if (!failed) mma_commit_pair(&acc_full[buf]);
             }
             if (failed) {   // let the products in flight finish before the memory is released
-                mma_commit(&drained);
+                mma_commit_pair(&drained);
                 mbar_wait_bounded(&drained, 0, kMvPoll);
             }
         }
         __syncwarp();
     } else {
-        // ---- the epilogue: lanes = scenarios 32 (warp % 4) .., columns 64 (warp / 4) ..
-        const int quarter = warp & 3, half = warp >> 2;
+        // ---- the epilogue: lanes = scenarios 32 (warp % 4) .., columns kCols (warp / 4) ..
+        constexpr int kCols = kMvP / (kMvEpi / 4);
+        const int quarter = warp & 3, part = warp >> 2;
         uint32_t n = 0;
-        for (long long item = blockIdx.x; item < n_items; item += gridDim.x, ++n) {
-            const int tile = (int)(item / a.n_chunks), chunk = (int)(item - (long long)tile * a.n_chunks);
+        uint32_t acc_free[Sh::NB];
+        for (int i = 0; i < Sh::NB; ++i) acc_free[i] = of_rank0(&acc_empty[i]);
+        for (long long item = cluster; item < n_items; item += n_clusters, ++n) {
+            const int tile = (int)(item / n_pairs), chunk = 2 * (int)(item - (long long)tile * n_pairs) + rank;
             const int buf = n % Sh::NB;
-            asm volatile("bar.sync 1, %0;" ::"n"(32 * kMvEpi) : "memory");   // the previous tile's records are read
-            reinterpret_cast<float4*>(recs)[tid] = reinterpret_cast<const float4*>(a.out + (size_t)tile * kMvP)[tid];
+            if (tid < kMvP * 2) reinterpret_cast<float4*>(recs)[tid] = reinterpret_cast<const float4*>(a.out + (size_t)tile * kMvP)[tid];
             asm volatile("bar.sync 1, %0;" ::"n"(32 * kMvEpi) : "memory");
             bool ok = true;
             if (lane == 0 && !failed) ok = mbar_wait_bounded(&acc_full[buf], (n / Sh::NB) & 1, kMvPoll);
@@ -484,80 +507,102 @@ __global__ void __launch_bounds__(kMvThreads, 1)
             }
             fence_after();
             const int s = chunk * kMvM + quarter * 32 + lane;
-            const bool live = s < a.n_scen && !failed;
-            const float dsc = pow2f(a.colexp[s] - (NS == 3 ? 30 : 0));
-            const uint32_t col0 = tmem + ((uint32_t)(quarter * 32) << 16) + buf * (Sh::NA * kMvP) + half * 64;
+            const bool inside = chunk < a.n_chunks, live = s < a.n_scen && !failed;   // an odd last pair's second tile is empty
+            const int sl = inside ? s : 0;
+            const float dsc = pow2f(a.colexp[sl] - (NS == 3 ? 30 : 0));
+            const uint32_t col0 = tmem + ((uint32_t)(quarter * 32) << 16) + buf * (Sh::NA * kMvP) + part * kCols;
             df tot{0.0f, 0.0f};
+            // the columns of this warp, 16 at a time and without branches over them (padding
+            // rows are 0), so that their chains overlap; MAT: maturity payments
+            auto columns = [&](auto with_maturity) {
+                constexpr bool MAT = decltype(with_maturity)::value;
 #pragma unroll 1
-            for (int c = 0; c < 64; c += 16) {
-                uint32_t r[Sh::NA][16];
+                for (int c = 0; c < kCols; c += 16) {
+                    uint32_t r[Sh::NA][16];
 #pragma unroll
-                for (int k = 0; k < Sh::NA; ++k) tmem_ld16_async(col0 + k * kMvP + c, r[k]);
+                    for (int k = 0; k < Sh::NA; ++k) tmem_ld16_async(col0 + k * kMvP + c, r[k]);
 #pragma unroll
-                for (int k = 0; k < Sh::NA; ++k) tmem_wait_ld(r[k]);
-                if (c == 48) {   // the accumulators are read
-                    fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&acc_empty[buf]);
-                }
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const MvOut& q = recs[half * 64 + c + i];
-                    if (q.pol < 0) continue;
-                    // the accumulators' sum as a double-float
-                    float h = __uint_as_float(r[0][i]), l = 0.0f;
-#pragma unroll
-                    for (int k = 1; k < Sh::NA; ++k) {
-                        const float b = __uint_as_float(r[k][i]), sum = __fadd_rn(h, b), bb = __fsub_rn(sum, h);
-                        l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(sum, bb)), __fsub_rn(b, bb)));
-                        h = sum;
+                    for (int k = 0; k < Sh::NA; ++k) tmem_wait_ld(r[k]);
+                    if (c == kCols - 16) {   // the accumulators are read
+                        fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive_remote(acc_free[buf]);
                     }
-                    df v = df_mul(df{__fmul_rn(h, dsc), __fmul_rn(l, dsc)}, df{q.sc_h, q.sc_l});
-                    if (q.mat_h != 0.0f) {   // a maturity payment: of the same sign
-                        df m{q.mat_h, q.mat_l};
-                        if (q.S > 0) {
-                            const float2 d = a.D[(size_t)(q.S - 1) * a.s_pad + s];
-                            m = df_mul(m, df{d.x, d.y});
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const MvOut& q = recs[part * kCols + c + i];
+                        // the accumulators' sum as a double-float
+                        float h = __uint_as_float(r[0][i]), l = 0.0f;
+#pragma unroll
+                        for (int k = 1; k < Sh::NA; ++k) {
+                            const float b = __uint_as_float(r[k][i]), sum = __fadd_rn(h, b), bb = __fsub_rn(sum, h);
+                            l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(sum, bb)), __fsub_rn(b, bb)));
+                            h = sum;
                         }
-                        const float sum = __fadd_rn(v.h, m.h), bb = __fsub_rn(sum, v.h);
-                        const float e = __fadd_rn(__fsub_rn(v.h, __fsub_rn(sum, bb)), __fsub_rn(m.h, bb));
-                        v = df{sum, __fadd_rn(e, __fadd_rn(v.l, m.l))};
-                    }
-                    // the sum over the policies
-                    const float sum = __fadd_rn(tot.h, v.h), bb = __fsub_rn(sum, tot.h);
-                    const float e = __fadd_rn(__fsub_rn(tot.h, __fsub_rn(sum, bb)), __fsub_rn(v.h, bb));
-                    tot = df{sum, __fadd_rn(tot.l, __fadd_rn(e, v.l))};
-                    if (live) {
-                        const size_t o = (size_t)q.pol * a.v0_ld + s;
-                        if (a.V0f) a.V0f[o] = __fadd_rn(v.h, v.l);
-                        if (a.V0d) a.V0d[o] = q.S == 0 && q.mat_h != 0.0f ? a.amount[q.pol] : (double)v.h + (double)v.l;
+                        df v = df_mul(df{__fmul_rn(h, dsc), __fmul_rn(l, dsc)}, df{q.sc_h, q.sc_l});
+                        const int pol = q.pol;
+                        bool due = false;
+                        if constexpr (MAT) {   // a maturity payment, of the same sign, or 0
+                            const float2 d = a.D[(size_t)max(q.S - 1, 0) * a.s_pad + sl];
+                            due = q.S == 0;
+                            const df m = df_mul(df{q.mat_h, q.mat_l}, due ? df{1.0f, 0.0f} : df{d.x, d.y});
+                            const float sum = __fadd_rn(v.h, m.h), bb = __fsub_rn(sum, v.h);
+                            const float e = __fadd_rn(__fsub_rn(v.h, __fsub_rn(sum, bb)), __fsub_rn(m.h, bb));
+                            v = df{sum, __fadd_rn(e, __fadd_rn(v.l, m.l))};
+                            due = due && q.mat_h != 0.0f;
+                        }
+                        // the sum over the policies
+                        const float sum = __fadd_rn(tot.h, v.h), bb = __fsub_rn(sum, tot.h);
+                        const float e = __fadd_rn(__fsub_rn(tot.h, __fsub_rn(sum, bb)), __fsub_rn(v.h, bb));
+                        tot = df{sum, __fadd_rn(tot.l, __fadd_rn(e, v.l))};
+                        const size_t o = (size_t)pol * a.v0_ld + s;
+                        if (live && pol >= 0) {
+                            if (a.V0f) a.V0f[o] = __fadd_rn(v.h, v.l);
+                            if (a.V0d) a.V0d[o] = due ? a.amount[pol] : (double)v.h + (double)v.l;
+                        }
                     }
                 }
+            };
+            const int kind = a.kinds[tile];
+            if (kind == K_ASS || kind == K_ASS2 || kind == K_LS2) columns(std::true_type{});
+            else columns(std::false_type{});
+            // the parts' sums in part order; then the records and sums may be overwritten
+            sums[part][quarter * 32 + lane] = make_float2(tot.h, tot.l);
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * kMvEpi) : "memory");
+            if (part == 0 && a.partial && inside && !failed) {
+                double x = 0.0;
+#pragma unroll
+                for (int k = 0; k < kMvParts; ++k) {
+                    const float2 v = sums[k][quarter * 32 + lane];
+                    x += (double)v.x + (double)v.y;
+                }
+                a.partial[(size_t)tile * a.part_ld + s] = x;
             }
-            if (a.partial && !failed) a.partial[(size_t)(2 * tile + half) * a.part_ld + s] = (double)tot.h + (double)tot.l;
         }
     }
     fence_before();
-    __syncthreads();
+    cluster_sync();   // neither CTA leaves while the other may reach into it
     fence_after();
-    if (warp == 0) tmem_free(tmem, 512);
+    if (warp == 0) tmem_free_pair(tmem, 512);
 }
 
 template <int NS>
 cudaError_t product(const MvArgs& a, const void* digitsD, const void* digitsE, int pitchD, int pitchE, int sm_count,
                     cudaStream_t st) {
+    using Sh = MvShape<NS>;
+    constexpr auto swz = Sh::KB == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
     CUtensorMap mD, mE;
-    if (!encode_map_16bit(&mD, CU_TENSOR_MAP_DATA_TYPE_UINT16, digitsD, pitchD, (uint64_t)NS * a.s_pad, pitchD, kMvKB, kMvM,
-                          CU_TENSOR_MAP_SWIZZLE_64B) ||
-        !encode_map_16bit(&mE, CU_TENSOR_MAP_DATA_TYPE_UINT16, digitsE, pitchE, (uint64_t)NS * kMvP * a.n_tiles, pitchE, kMvKB,
-                          kMvP, CU_TENSOR_MAP_SWIZZLE_64B))
+    if (!encode_map_16bit(&mD, CU_TENSOR_MAP_DATA_TYPE_UINT16, digitsD, pitchD, (uint64_t)NS * a.s_pad, pitchD, Sh::KB, kMvM,
+                          swz) ||
+        !encode_map_16bit(&mE, CU_TENSOR_MAP_DATA_TYPE_UINT16, digitsE, pitchE, (uint64_t)NS * kMvP * a.n_tiles, pitchE, Sh::KB,
+                          kMvHalf, swz))
         return cudaErrorNotSupported;
-    constexpr size_t smem = (size_t)MvShape<NS>::ST * 2 * NS * kMvSlab + 1024;
+    constexpr size_t smem = (size_t)Sh::ST * MvStage<NS>::kBytes + 1024;
     auto k = mv_product_kernel<NS>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const long long items = (long long)a.n_tiles * a.n_chunks;
-    k<<<(int)std::min<long long>(items, sm_count), kMvThreads, smem, st>>>(mD, mE, a);
+    const long long items = (long long)a.n_tiles * ((a.n_chunks + 1) / 2);
+    k<<<2 * (int)std::min<long long>(items, sm_count / 2), kMvThreads, smem, st>>>(mD, mE, a);
     return cudaGetLastError();
 }
 

@@ -45,7 +45,7 @@ namespace rsv {
 
 constexpr int kMvP = 128;          // policies per tile (MMA N)
 constexpr int kMvM = 128;          // scenarios per tile (MMA M)
-constexpr int kMvKB = 32;          // steps per staged block: 64-byte swizzled rows
+constexpr int kMvParts = 4;        // column groups of the epilogue
 constexpr int kMvSpread = 6;       // log2 of the range of a scenario's tilted discount products
 constexpr int kMvTilt = 60;        // largest |tau|
 constexpr size_t kMvPanelBytes = size_t(1) << 30;            // cash-flow digits held at a time
@@ -89,6 +89,7 @@ cudaError_t launch_mv_build(int form, const MvBuild& b, cudaStream_t st);
 
 struct MvArgs {
     const SlotRec* slots;
+    const int32_t* kinds;
     const MvOut* out;
     const int32_t* colexp;     // of the first column
     const float2* D;           // the discount products [n_steps][s_pad], at the first column
@@ -98,7 +99,7 @@ struct MvArgs {
     int32_t v0_ld, part_ld;
     float* V0f;                // at the block's first column
     double* V0d;
-    double* partial;           // [2 n_tiles][part_ld], at the panel's first tile and the block's first column
+    double* partial;           // [n_tiles][part_ld], at the panel's first tile and the block's first column
     int32_t* status;
 };
 // digitsE: launch_mv_build's, digitsD: launch_mv_digits'.

@@ -669,6 +669,7 @@ rsv_status rsv::mv_launch(rsv_ctx* c, int form, int s0, int w, float* V0f, doubl
         }
         MvArgs a{};
         a.slots = slots;
+        a.kinds = L.kinds.as<int32_t>() + t0;
         a.out = c->d_mv_out.as<MvOut>();
         a.colexp = tau + c->n_steps + s0;
         a.D = c->d_mv_D.as<float2>() + s0;
@@ -682,7 +683,7 @@ rsv_status rsv::mv_launch(rsv_ctx* c, int form, int s0, int w, float* V0f, doubl
         a.part_ld = c->s_pad;
         a.V0f = V0f;
         a.V0d = V0d;
-        a.partial = partial ? partial + (size_t)2 * t0 * c->s_pad : nullptr;
+        a.partial = partial ? partial + (size_t)t0 * c->s_pad : nullptr;
         a.status = c->d_ctl.as<int32_t>() + 1;
         CU(launch_mv_product(form, a, c->d_mv_dig[form == F_DEFL ? 1 : 0].p, c->d_mv_E.p, pitchD, pitchE, c->sm_count,
                              c->stream));
@@ -786,7 +787,6 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     if (mat && (st = mv_prepare(c, o->form)) != RSV_OK) return st;
 
     const Layout& L = c->lay;
-    const int part_rows = mat ? 2 * L.n_tiles : L.n_tiles;   // rows of per-tile scenario sums
     float* V0f = (outs & RSV_OUT_V0) ? out->V0 : nullptr;
     double* V0d = (outs & RSV_OUT_V0) ? out->V0d : nullptr;
     double* tot = (outs & RSV_OUT_SCEN_TOTAL) ? out->scen_total : nullptr;
@@ -805,7 +805,7 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     CU(cudaMemsetAsync(c->d_ctl.p, 0, 2 * sizeof(int32_t), c->stream));
     if (pt) CU(cudaMemsetAsync(pt, 0, n_pt * sizeof(double), c->stream));
     if (traj) CU(cudaMemsetAsync(traj, 0, n_traj * sizeof(double), c->stream));
-    if (tot) CU(c->d_partial.ensure((size_t)std::max(1, part_rows) * c->s_pad * sizeof(double)));
+    if (tot) CU(c->d_partial.ensure((size_t)std::max(1, L.n_tiles) * c->s_pad * sizeof(double)));
     if (tot && L.n_tiles == 0) CU(cudaMemsetAsync(tot, 0, NSc * sizeof(double), c->stream));
 
     RecurArgs a{};
@@ -920,7 +920,7 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
         c->ev_recorded = true;
     }
     if (L.n_tiles > 0) {
-        if (tot && (st = scenario_totals(c, a.partial, part_rows, c->s_pad, NSc, tot)) != RSV_OK) return st;
+        if (tot && (st = scenario_totals(c, a.partial, L.n_tiles, c->s_pad, NSc, tot)) != RSV_OK) return st;
         if (pt) {
             scale_kernel<<<c->sm_count * 4, 256, 0, c->stream>>>(pt, n_pt, 1.0 / NSc);
             CU(cudaGetLastError());
