@@ -30,11 +30,12 @@
 // keeps the recurrence kernels.
 //
 // Measured (one GB300, with the digits and the totals): the 100,000-policy mix under 1,000
-// scenarios, compensated 38.7 -> 1.96 ms (error 1e-8 -> 2e-11 at most; annuities alone
-// 1e-13 -> 2.4e-13 rms, assurances 4e-9 -> 2e-13), deflated 4.93 -> 0.88 ms (rms 3e-8 ->
-// 5e-9); 1,000,000 annuities, 600 steps, deflated 30.6 -> 6.2 ms; 1,537 policies under
-// 157 scenarios, compensated, 254 -> 102 us on the device.  It is the faster path at
-// every size measured, from one policy and one scenario up.
+// scenarios, compensated 38.7 -> 1.56 ms (error 1e-8 -> 2e-11 at most; annuities alone
+// 1e-13 -> 2.4e-13 rms, assurances 4e-9 -> 2e-13), deflated 4.93 -> 0.62 ms (rms 3e-8 ->
+// 5e-9); 1,000,000 annuities, 600 steps, deflated 30.6 -> 4.3 ms.  It is the faster path
+// at every size measured: one policy and one scenario 53 -> 49 us compensated and
+// 158 -> 37 us deflated (host call included), 1,000 policies under 157 scenarios of the
+// mix 276 -> 102 us and 282 -> 63 us.
 #pragma once
 
 #include <cuda.h>
@@ -55,12 +56,25 @@ constexpr double kMvAmountMin = 0x1p-60, kMvAmountMax = 0x1p90;   // |amount|: V
 inline int mv_slices(int form) { return form == F_DEFL ? 3 : 6; }
 inline int mv_pitch(int steps) { return steps < 1 ? 64 : (steps + 63) / 64 * 64; }
 
-// Scenario side, from the FP64 plane [n_steps][s_pad]: the discount products, the tilt of
-// each step, the binary exponent of each column's largest tilted product, and
-// stat = {largest spread of a column, largest |tau|} (INT_MAX where a product
-// is not a normal number).
-cudaError_t launch_mv_scenarios(const double* v64, int n_steps, int n_scen, int s_pad, float2* D, int32_t* tau,
-                                int32_t* colexp, int32_t* stat, cudaStream_t st);
+// Scenario side, from the FP64 plane [n_steps][s_pad]: the discount products, and
+struct MvScen {
+    int32_t* tau;       // [n_steps] tilt of each step
+    float* tilt;        // [n_steps] 2^-tau and
+    float* tilt_top;    // [n_steps] its running maximum
+    int32_t* colexp;    // [s_pad] binary exponent of each column's largest tilted product
+    int32_t* colmin;    // [s_pad] scratch
+    int32_t* stat;      // largest spread of a column, largest |tau| (INT_MAX where a product is
+                        // not a normal number)
+    static size_t words(int n_steps, int s_pad) { return 3 * (size_t)n_steps + 2 * (size_t)s_pad + 2; }
+    static MvScen at(void* p, int n_steps, int s_pad) {
+        int32_t* w = static_cast<int32_t*>(p);
+        float* t = reinterpret_cast<float*>(w + n_steps);
+        int32_t* c = w + 3 * (size_t)n_steps;
+        return MvScen{w, t, t + n_steps, c, c + s_pad, c + 2 * (size_t)s_pad};
+    }
+};
+cudaError_t launch_mv_scenarios(const double* v64, int n_steps, int n_scen, int s_pad, float2* D, const MvScen& c,
+                                cudaStream_t st);
 // Its digits [slices][s_pad][pitch]; columns beyond n_scen and steps beyond n_steps are 0.
 cudaError_t launch_mv_digits(int form, const float2* D, const int32_t* tau, const int32_t* colexp, int n_steps, int n_scen,
                              int s_pad, int pitch, void* digits, cudaStream_t st);
@@ -81,7 +95,10 @@ struct MvBuild {
     int32_t general_from;      // first tile of the panel whose policies have varying cash flows
     const double* cf;          // their multipliers [n_pol][cf_ld], or null
     int32_t cf_ld;
-    const int32_t* tau;
+    int32_t n_steps;           // of the scenario set
+    int32_t rows_per_warp;     // 1 to 16: more once there are tiles enough to fill the chip
+    const float* tilt;
+    const float* tilt_top;
     void* digits;
     MvOut* out;
 };
