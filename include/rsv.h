@@ -100,7 +100,7 @@ enum {
  * products on the tensor cores, both split into exact 16-bit digits (compensated: 48
  * bits, error about 1e-12; deflated: 32 bits, within the bound below).  Data outside its
  * range keeps the recurrence kernels: scenarios whose discount products leave their
- * mean by more than a factor of about 2^6, survival below 2^-100, amounts outside
+ * mean by more than a factor of about 2^10 (deflated 2^8), survival below 2^-100, amounts outside
  * 2^-60 .. 2^90.  It is the last of a form's tunable variants. */
 
 /* RSV_FORM_F32_DEFLATED.  Eq. (generalForm) multiplied at step t by the
@@ -361,7 +361,7 @@ typedef struct {     /* 64 bytes */
  * tables loaded by rsv_load_decrements.  opts: form (any), outputs RSV_OUT_V0
  * and/or RSV_OUT_SCEN_TOTAL, on_device; horizon, payment and variant 0 / -1.
  * out->V0 / V0d: [n][n_scen]; out->scen_total: [n_scen], summed over the
- * policies in order.  The records are copied.
+ * policies in a fixed order.  The records are copied.
  * Errors: RSV_E_STATE (tables or scenarios missing), RSV_E_ARG (bad opts or
  * record, a table not loaded, ages plus steps above 4096), RSV_E_ASSUMPTION
  * (amount not finite, a projection longer than the scenarios), RSV_E_CUDA,

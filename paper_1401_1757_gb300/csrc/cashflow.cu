@@ -111,12 +111,15 @@ cudaError_t launch_cf_portfolio(const CfTables& T, const CfPol* pols, int n, int
     return cudaGetLastError();
 }
 
-// The survivor columns of the layout's tables, on the device (once per change of
-// the tables or of the projections' reach).
+// The survivor columns of every loaded table, on the device (once per change of the
+// tables): kMaxAgeSteps + 1 entries each, the reach of any projection.
 rsv_status cf_tables(rsv_ctx* c, CfTables& T) {
-    const int n_tab = c->lay.n_tab, rows = c->lay.tab_pad + 1;
+    int n_tab = 0;
+    for (int t = 0; t < kMaxTables; ++t)
+        if (!c->tab[t].empty()) n_tab = t + 1;
+    const int rows = kMaxAgeSteps + 1;
     const size_t n = (size_t)n_tab * rows;
-    if (c->cf_tab_gen != c->tab_gen || c->cf_tab_rows != rows || c->cf_tab_n != n_tab) {
+    if (c->cf_tab_gen != c->tab_gen) {
         // m, dm, the two integer columns, 1 / m, then m and dm as FP32 head and tail
         std::vector<double>& h = c->h_cf_tab;
         h.resize(6 * n);
@@ -155,8 +158,6 @@ rsv_status cf_tables(rsv_ctx* c, CfTables& T) {
         CU(c->d_cf_tab.ensure(h.size() * sizeof(double)));
         CU(cudaMemcpyAsync(c->d_cf_tab.p, h.data(), h.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));
         c->cf_tab_gen = c->tab_gen;
-        c->cf_tab_rows = rows;
-        c->cf_tab_n = n_tab;
     }
     T.m = c->d_cf_tab.as<double>();
     T.dm = T.m + n;

@@ -11,6 +11,7 @@
 
 #include "host_parts.h"
 #include "rsv.h"
+#include "matval.cuh"
 #include "mlp.cuh"
 #include "recur_kernel.cuh"
 #include "surrogate.cuh"
@@ -217,12 +218,12 @@ struct rsv_ctx {
     DevBuf d_ml_rec, d_ml_amount;                   // m-life records of the last call
 
     // the valuation as a matrix product (matval.cuh): whether the scenario set, the tables and
-    // the amounts are in its range, the discount products and their digits per form
-    bool mv_scen_ok = false;
+    // the amounts are in its range, the discount products and their digits per digit count
+    int mv_spread = 0x7fffffff;   // of the scenario set (mv_max_spread)
     double tab_min[rsv::kMaxTables] = {};           // smallest survivor-column entry of a table
     double amt_lo = 0.0, amt_hi = 0.0;              // smallest non-zero and largest |amount|
-    DevBuf d_mv_D, d_mv_col, d_mv_dig[2], d_mv_E, d_mv_out;
-    unsigned long long scen_gen = 1, mv_dig_gen[2] = {0, 0};
+    DevBuf d_mv_D, d_mv_col, d_mv_dig[3], d_mv_E, d_mv_out;
+    unsigned long long scen_gen = 1, mv_dig_gen[3] = {0, 0, 0};
     int mv_built = -1;   // first tile of the panel whose digits are held, within one call
 
     Layout lay;
@@ -236,7 +237,7 @@ struct rsv_ctx {
     DevBuf d_cf_tab, d_cf_pol, d_cf_sum;
     std::vector<double> h_cf_tab;   // the columns on the host, kept: the upload may still read them
     unsigned long long cf_tab_gen = 0;
-    int cf_tab_rows = 0, cf_tab_n = 0, cf_tab_scaled = 0;
+    int cf_tab_scaled = 0;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     cudaStream_t copy_stream = nullptr;   // device-to-host copies of V0 column blocks
     cudaEvent_t ev_block = nullptr;
@@ -283,8 +284,7 @@ rsv_status layout_to_device(rsv_ctx* c);
 rsv_status build_tables(rsv_ctx* c, int form, size_t& smem);
 // Bytes of n_tab tables of pad entries in a form's entry format; RSV_E_ARG above kMaxSmem.
 rsv_status table_bytes(rsv_ctx* c, int form, int pad, int n_tab, size_t& smem);
-struct CfTables;
-// The survivor columns of the layout's tables on the device (cashflow.cu).
+// The survivor columns of the loaded tables on the device (cashflow.cu).
 rsv_status cf_tables(rsv_ctx* c, CfTables& T);
 // The first n_tab loaded tables, pad entries each, in a form's entry format
 // on the device (cached by shape and table generation); smem = their bytes.
@@ -292,8 +292,15 @@ rsv_status stage_tables(rsv_ctx* c, int form, int pad, int n_tab, size_t& smem);
 // Whether the matrix product covers the loaded data; then, on the layout of width
 // kMvP: mv_prepare once a call, mv_launch for the scenario columns [s0, s0 + w) with the
 // output pointers at column s0 (partial: [n_tiles][s_pad]).
-bool mv_applies(const rsv_ctx* c);
+bool mv_applies(const rsv_ctx* c, int form, double amt_lo, double amt_hi);
 rsv_status mv_prepare(rsv_ctx* c, int form);
+// Its parts, for rows that come from elsewhere (m lives): the scenario set's digits, the tiles
+// of a panel and their buffers (d_mv_E, d_mv_out), and the product of a built panel
+// (a: steps, kinds, amount, n_tiles and the outputs set).
+rsv_status mv_scenario_digits(rsv_ctx* c, int form);
+int mv_panel_tiles(const rsv_ctx* c, int form, int max_S, int n_tiles);
+rsv_status mv_panel_buffers(rsv_ctx* c, int form, int max_S, int tiles);
+rsv_status mv_multiply(rsv_ctx* c, int form, MvArgs a, int max_S, int s0, int w);
 rsv_status mv_launch(rsv_ctx* c, int form, int s0, int w, float* V0f, double* V0d, double* partial);
 // rsv_compute_reserves in the deflated form (defl_abi.cu); opts checked by the caller
 rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out);

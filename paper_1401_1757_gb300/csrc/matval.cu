@@ -46,7 +46,7 @@ __device__ __forceinline__ void mv_digits(float h0, float l0, float h1, float l1
     float a = __fsub_rn(__fadd_rn(h0, M1), M1), b = __fsub_rn(__fadd_rn(h1, M1), M1);
     float r = __fsub_rn(h0, a), s = __fsub_rn(h1, b);               // exact
     d[0] = mv_pack<NS>(a, b);
-    if constexpr (NS == 6) {
+    if constexpr (NS != 3) {
 #pragma unroll
         for (int k = 1; k < 3; ++k) {   // to a multiple of 2^-15, then of 2^-23
             const float M = k == 1 ? 384.0f : 1.5f;
@@ -248,14 +248,75 @@ __device__ __forceinline__ df mv_boundary(const CfTables& T, const MvLife& a, co
 }
 
 
-// One warp a policy: the scale of the row, then the digits, four consecutive steps a lane.
-// Closed forms, so no chain over the steps.  200,000 annuities x 520 steps: 248 -> 166 us
-// deflated (0.64 GB, past the L2: bound by the memory's write rate), 290 -> 231 us
+// ---- one row by one warp: the scale of the row, then the digits, four consecutive steps a
+// lane.  Closed forms, so no chain over the steps.  200,000 annuities x 520 steps: 248 ->
+// 166 us deflated (0.64 GB, past the L2: bound by the memory's write rate), 290 -> 231 us
 // compensated, when the lanes took four steps, packed conversions and no pass for the
 // largest entry of a level annuity.
+__device__ __forceinline__ df df_of(double v) {
+    const float h = __double2float_rn(v);
+    return df{h, __double2float_rn(v - (double)h)};
+}
+
+// the largest tilted head of flow(t), t < S
+template <class Flow>
+__device__ __forceinline__ float mv_top(const Flow& flow, int S, const float* __restrict__ tilt) {
+    float top = 0.0f;
+    for (int t = threadIdx.x & 31; t < S; t += 32) top = fmaxf(top, __fmul_rn(flow(t).h, tilt[t]));
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, d));
+    return top;
+}
+// the row's binary exponent: entries below 1; one bit less for each doubling of the steps
+// beyond 1,000, so that the leading digits' sum stays exact
+__device__ __forceinline__ int mv_row_exp(float top, int S) {
+    const int e = top > 0.0f ? ((__float_as_int(top) >> 23) & 255) - 126 : 0;
+    return e + (S > 1000) + (S > 2000) + (S > 4000);
+}
+// digits of flow(t) tilted and times 2^-e, t < live, and zeros up to kt
+template <int NS, class Flow>
+__device__ __forceinline__ void mv_write_row(const Flow& flow, int live, int e, int kt, const float* __restrict__ tilt,
+                                             void* digits, int row, int pitch) {
+    const float f = pow2f(kMvLog<NS> - e);
+    uint16_t* base = static_cast<uint16_t*>(digits) + ((size_t)(row / kMvP) * NS * kMvP + row % kMvP) * pitch;
+    for (int t = 4 * (threadIdx.x & 31); t < kt; t += 128) {
+        df v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = t + k < live ? flow(t + k) : df{0.0f, 0.0f};
+        const float4 w = *reinterpret_cast<const float4*>(tilt + t);
+        const float g[4] = {__fmul_rn(w.x, f), __fmul_rn(w.y, f), __fmul_rn(w.z, f), __fmul_rn(w.w, f)};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = df{__fmul_rn(v[k].h, g[k]), __fmul_rn(v[k].l, g[k])};
+        uint32_t d0[NS], d1[NS];
+        mv_digits<NS>(v[0].h, v[0].l, v[1].h, v[1].l, d0);
+        mv_digits<NS>(v[2].h, v[2].l, v[3].h, v[3].l, d1);
+#pragma unroll
+        for (int k = 0; k < NS; ++k)
+            *reinterpret_cast<uint2*>(base + (size_t)k * kMvP * pitch + t) = make_uint2(d0[k], d1[k]);
+    }
+}
+// a normal FP64 number as a double-float below 1 in magnitude and a binary exponent (0: 0)
+__device__ __forceinline__ df df_mantissa(double v, int& ex) {
+    ex = 0;
+    if (v == 0.0) return df{0.0f, 0.0f};
+    const int hi = __double2hiint(v);
+    ex = ((hi >> 20) & 2047) - 1022;
+    return df_of(__hiloint2double((hi & 0x800FFFFF) | 0x3FE00000, __double2loint(v)));
+}
+__device__ __forceinline__ MvOut mv_out(df unit, int ex, int e, int pol, int S) {
+    const float g = pow2f(ex + e);
+    MvOut o;
+    o.sc_h = __fmul_rn(unit.h, g);
+    o.sc_l = __fmul_rn(unit.l, g);
+    o.mat_h = o.mat_l = 0.0f;
+    o.pol = pol;
+    o.S = S;
+    o.pad[0] = o.pad[1] = 0;
+    return o;
+}
+
 template <int NS, int KIND, bool CF>
 __device__ __forceinline__ void mv_row(const MvBuild& b, const SlotRec& r, int row, int kt, const float* __restrict__ tilt) {
-    const int lane = threadIdx.x & 31;
     const CfTables& T = b.T;
     auto life = [&](int idx) {
         const int tb = idx < b.tab_pad ? 0 : idx / b.tab_pad, age = idx - tb * b.tab_pad;
@@ -267,13 +328,9 @@ __device__ __forceinline__ void mv_row(const MvBuild& b, const SlotRec& r, int r
     MvLife x = life(r.idx1), y = life(r.idx2);
     const double amount = r.pol >= 0 ? b.amount[r.pol] : 0.0;
     const int S = r.pol >= 0 ? r.S : 0;
-    auto two = [](double v) {
-        const float h = __double2float_rn(v);
-        return df{h, __double2float_rn(v - (double)h)};
-    };
     if constexpr (KIND != K_ANN && KIND != K_ASS) {
-        x.c = two(T.inv[x.i]);
-        y.c = two(T.inv[y.i]);
+        x.c = df_of(T.inv[x.i]);
+        y.c = df_of(T.inv[y.i]);
         if (KIND == K_JL) {
             y.c = df_mul(y.c, df{r.rho_h, r.rho_l});
             if (r.state0 == 2) x.c = df{0.0f, 0.0f};
@@ -282,83 +339,36 @@ __device__ __forceinline__ void mv_row(const MvBuild& b, const SlotRec& r, int r
     }
     auto flow = [&](int t) {
         df e = mv_expected<KIND>(T, x, y, r.state0, t);
-        if constexpr (CF) e = df_mul(e, two(b.cf[(size_t)r.pol * b.cf_ld + t]));
+        if constexpr (CF) e = df_mul(e, df_of(b.cf[(size_t)r.pol * b.cf_ld + t]));
         return e;
     };
-    // The largest entry.  A level annuity's cash flows do not increase, so its first one
-    // times the largest tilt bounds them (it is the largest unless the tilt increases
-    // later, by negative rates); the others are looked through.
-    constexpr bool LEVEL_ANNUITY = !CF && (KIND == K_ANN || KIND == K_ANN2 || KIND == K_JL);
-    float top = 0.0f;
-    if constexpr (LEVEL_ANNUITY) {
-        if (S > 0) top = __fmul_rn(flow(0).h, b.tilt_top[S - 1]);
+    int e;
+    if constexpr (!CF && (KIND == K_ANN || KIND == K_ANN2 || KIND == K_JL)) {
+        // A level annuity's cash flows do not increase, so its first one times the largest
+        // tilt bounds them (it is the largest unless the tilt increases later, by
+        // negative rates); the others are looked through.
+        e = mv_row_exp(S > 0 ? __fmul_rn(flow(0).h, b.tilt_top[S - 1]) : 0.0f, S);
     } else {
-        for (int t = lane; t < S; t += 32) top = fmaxf(top, __fmul_rn(flow(t).h, tilt[t]));
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, d));
+        e = mv_row_exp(mv_top(flow, S, tilt), S);
     }
-    // entries below 1; one bit less for each doubling of the steps beyond 1,000, so that the
-    // leading digits' sum stays exact
-    int e = top > 0.0f ? ((__float_as_int(top) >> 23) & 255) - 126 : 0;
-    e += (S > 1000) + (S > 2000) + (S > 4000);
-    const float f = pow2f(kMvLog<NS> - e);
-    uint16_t* base = static_cast<uint16_t*>(b.digits) + ((size_t)(row / kMvP) * NS * kMvP + row % kMvP) * b.pitch;
-    // the steps with a cash flow: for one life also those it can live through
-    int live = S;
-    if (KIND == K_ANN) live = min(S, x.last);
-    if (KIND == K_ASS) live = min(S, x.last + 1);
-    const float2* col = KIND == K_ASS ? T.dm2 + x.i : T.m2 + x.i + 1;
-    for (int t = 4 * lane; t < kt; t += 128) {
-        df v[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            v[k] = df{0.0f, 0.0f};
-            if (t + k < live) {
-                if constexpr (!CF && (KIND == K_ANN || KIND == K_ASS)) {
-                    const float2 w = __ldg(col + t + k);
-                    v[k] = df{w.x, w.y};
-                } else {
-                    v[k] = flow(t + k);
-                }
-            }
-        }
-        const float4 w = *reinterpret_cast<const float4*>(tilt + t);
-        const float g[4] = {__fmul_rn(w.x, f), __fmul_rn(w.y, f), __fmul_rn(w.z, f), __fmul_rn(w.w, f)};
-#pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = df{__fmul_rn(v[k].h, g[k]), __fmul_rn(v[k].l, g[k])};
-        uint32_t d0[NS], d1[NS];
-        mv_digits<NS>(v[0].h, v[0].l, v[1].h, v[1].l, d0);
-        mv_digits<NS>(v[2].h, v[2].l, v[3].h, v[3].l, d1);
-#pragma unroll
-        for (int k = 0; k < NS; ++k)
-            *reinterpret_cast<uint2*>(base + (size_t)k * kMvP * b.pitch + t) = make_uint2(d0[k], d1[k]);
+    if constexpr (!CF && (KIND == K_ANN || KIND == K_ASS)) {   // straight from the column
+        const int live = KIND == K_ANN ? min(S, x.last) : min(S, x.last + 1);
+        const float2* col = KIND == K_ASS ? T.dm2 + x.i : T.m2 + x.i + 1;
+        mv_write_row<NS>([&](int t) { const float2 w = __ldg(col + t); return df{w.x, w.y}; }, live, e, kt, tilt, b.digits, row,
+                         b.pitch);
+    } else {
+        mv_write_row<NS>(flow, S, e, kt, tilt, b.digits, row, b.pitch);
     }
-    if (lane == 0) {
-        // amount (times 1 / m_x) as a mantissa below 1 and an exponent, then times 2^e
-        double rc = amount;
-        if (KIND == K_ANN || KIND == K_ASS) rc = __dmul_rn(rc, T.inv[x.i]);
-        int ex = 0;
-        if (rc != 0.0) {
-            const int hi = __double2hiint(rc);
-            ex = ((hi >> 20) & 2047) - 1022;
-            rc = __hiloint2double((hi & 0x800FFFFF) | 0x3FE00000, __double2loint(rc));
-        }
-        const df q = two(rc);
-        const float g = pow2f(ex + e);
-        MvOut o;
-        o.sc_h = __fmul_rn(q.h, g);
-        o.sc_l = __fmul_rn(q.l, g);
-        o.mat_h = o.mat_l = 0.0f;
+    if ((threadIdx.x & 31) == 0) {
+        int ex;
+        const df q = df_mantissa(KIND == K_ANN || KIND == K_ASS ? __dmul_rn(amount, T.inv[x.i]) : amount, ex);
+        MvOut o = mv_out(q, ex, e, r.pol, S);
         if constexpr (KIND == K_ASS || KIND == K_ASS2 || KIND == K_LS2) {
             if (r.bnd != 0.0f && r.pol >= 0) {   // the maturity payment, or the amount if it is due now
-                df m{r.bnd, 0.0f};
+                df m{r.bnd, 0.0f}, w = q;
                 int em = 0, xm = ex;
-                df w = q;
                 if (S == 0) {
-                    const int hi = __double2hiint(amount);
-                    xm = ((hi >> 20) & 2047) - 1022;
-                    w = amount != 0.0 ? two(__hiloint2double((hi & 0x800FFFFF) | 0x3FE00000, __double2loint(amount)))
-                                      : df{0.0f, 0.0f};
+                    w = df_mantissa(amount, xm);
                 } else {
                     m = mv_boundary<KIND>(T, x, y, r.state0, S);
                     em = m.h > 0.0f ? ((__float_as_int(m.h) >> 23) & 255) - 126 : 0;
@@ -371,10 +381,99 @@ __device__ __forceinline__ void mv_row(const MvBuild& b, const SlotRec& r, int r
                 o.mat_l = __fmul_rn(v.l, g2);
             }
         }
-        o.pol = r.pol;
-        o.S = S;
-        o.pad[0] = o.pad[1] = 0;
         b.out[row] = o;
+    }
+}
+
+// ---- contracts on up to four lives (MvLives): the lives are independent, so a step's
+// expected cash flow is a polynomial in their survival and death probabilities.  A life
+// that is absent counts for nothing (an annuity counts it as dead, an assurance as alive).
+//   annuity:    Pr[k or more alive at the end of step t]
+//   assurance:  the k-th death in step t: Pr[k or more dead] is linear in each life, so its
+//               growth is the sum, over the lives moved one by one to the step's end, of the
+//               life's deaths times Pr[exactly k - 1 of the others are dead]
+__device__ __forceinline__ df mv_lives_flow(const CfTables& T, const MvLives& r, const MvLife (&l)[4], const df (&one)[4], int t) {
+    const bool ass = r.flags & 1;
+    df p[4], q[4];   // alive and dead at the end of the step
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        p[i] = l[i].last < 0 ? one[i] : df_mul(at(T.m2, l[i], t + 1), l[i].c);
+        q[i] = df_one_minus(p[i]);
+    }
+    if (!ass) {
+        df c[5] = {q[0], p[0], df{0.0f, 0.0f}, df{0.0f, 0.0f}, df{0.0f, 0.0f}};   // Pr[j alive]
+#pragma unroll
+        for (int i = 1; i < 4; ++i) {
+            c[i + 1] = df_mul(c[i], p[i]);
+#pragma unroll
+            for (int j = i; j > 0; --j) c[j] = df_add_pos(df_mul(c[j], q[i]), df_mul(c[j - 1], p[i]));
+            c[0] = df_mul(c[0], q[i]);
+        }
+        df e = c[4];
+#pragma unroll
+        for (int j = 3; j > 0; --j)
+            if (j >= r.k) e = df_add_pos(e, c[j]);
+        return e;
+    }
+    df e{0.0f, 0.0f};
+    df a[4], b[4];   // the lives not yet moved: alive and dead at the start
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        a[i] = l[i].last < 0 ? one[i] : df_mul(at(T.m2, l[i], t), l[i].c);
+        b[i] = df_one_minus(a[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (l[i].last < 0) continue;
+        df c[4] = {df{1.0f, 0.0f}, df{0.0f, 0.0f}, df{0.0f, 0.0f}, df{0.0f, 0.0f}};   // Pr[j of the others dead]
+        int n = 0;
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+            if (o == i) continue;
+            const df al = o < i ? p[o] : a[o], de = o < i ? q[o] : b[o];
+            ++n;
+            c[n] = df_mul(c[n - 1], de);
+#pragma unroll
+            for (int j = n - 1; j > 0; --j) c[j] = df_add_pos(df_mul(c[j], al), df_mul(c[j - 1], de));
+            c[0] = df_mul(c[0], al);
+        }
+        const df w = r.k == 1 ? c[0] : (r.k == 2 ? c[1] : (r.k == 3 ? c[2] : c[3]));
+        e = df_add_pos(e, df_mul(df_mul(at(T.dm2, l[i], t), l[i].c), w));
+    }
+    return e;
+}
+
+template <int NS>
+__global__ void __launch_bounds__(256) mv_build_lives_kernel(const CfTables T, const MvLives* __restrict__ recs,
+                                                             const double* __restrict__ amount, int pitch, int n_steps,
+                                                             const float* __restrict__ tilt_g, void* digits,
+                                                             MvOut* __restrict__ out) {
+    extern __shared__ float4 tilt4[];
+    float* tilt = reinterpret_cast<float*>(tilt4);
+    const int row = blockIdx.x * 8 + (threadIdx.x >> 5), tile = row / kMvP;
+    const int kt = max(64, (recs[(size_t)tile * kMvP].S + 63) / 64 * 64);
+    for (int t = threadIdx.x; t < kt; t += 256) tilt[t] = t < n_steps ? tilt_g[t] : 0.0f;
+    __syncthreads();
+    const MvLives r = recs[row];
+    const bool ass = r.flags & 1;
+    MvLife l[4];
+    df one[4];   // of a life that takes no part: 1 alive for ever, 0 dead
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const bool dead = r.flags >> (8 + i) & 1, absent = r.idx[i] < 0;
+        one[i] = df{absent && ass ? 1.0f : 0.0f, 0.0f};
+        l[i].i = absent ? 0 : r.idx[i];
+        l[i].last = absent || dead ? -1 : T.z[l[i].i] - l[i].i % T.rows;
+        l[i].c = df_of(T.inv[l[i].i]);
+    }
+    const int S = r.pol >= 0 ? r.S : 0;
+    auto flow = [&](int t) { return mv_lives_flow(T, r, l, one, t); };
+    const int e = mv_row_exp(mv_top(flow, S, tilt), S);
+    mv_write_row<NS>(flow, S, e, kt, tilt, digits, row, pitch);
+    if ((threadIdx.x & 31) == 0) {
+        int ex;
+        const df q = df_mantissa(r.pol >= 0 ? amount[r.pol] : 0.0, ex);
+        out[row] = mv_out(q, ex, e, r.pol, S);
     }
 }
 
@@ -412,13 +511,17 @@ __global__ void __launch_bounds__(256) mv_build_kernel(const MvBuild b) {
 // on the lanes and the policies on the columns; sixteen warps add the accumulators as
 // double-floats, scale, write V0 (32 consecutive scenarios of a policy a warp store) and
 // sum each scenario over the tile's policies.
-// Deflated: 6 products and 2 accumulators, so TMEM holds two tiles' and the epilogue runs
-// beside the next tile's products; compensated: 21 products, 4 accumulators.
+// Three digits: 6 products and 2 accumulators, so TMEM holds two tiles' and the epilogue
+// runs beside the next tile's products; four and six: 10 and 21 products, 4 accumulators.
 template <int NS>
 struct MvShape;   // accumulators, tiles in TMEM, stages, steps of a block (64: 128-byte swizzled
 template <>       // rows); the products are (i, j), i + j < NS, of scenario digit i and policy
 struct MvShape<3> {   // digit j, in accumulator min(i + j, NA - 1)
     static constexpr int NA = 2, NB = 2, ST = 3, KB = 64;
+};
+template <>
+struct MvShape<4> {
+    static constexpr int NA = 4, NB = 1, ST = 4, KB = 32;
 };
 template <>
 struct MvShape<6> {
@@ -493,7 +596,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
             atomicExch(a.status, DEV_TIMEOUT);
         }
     };
-    auto blocks_of = [&](int tile) { return max(1, (a.slots[(size_t)tile * kMvP].S + KB - 1) / KB); };
+    auto blocks_of = [&](int tile) { return max(1, (a.steps[(size_t)tile * kMvP * kMvRecWords] + KB - 1) / KB); };
 
     if (warp == kMvEpi) {
         // ---- the copies (one thread of each CTA)
@@ -629,7 +732,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
                     }
                 }
             };
-            const int kind = a.kinds[tile];
+            const int kind = a.kinds ? a.kinds[tile] : K_ANN;
             if (kind == K_ASS || kind == K_ASS2 || kind == K_LS2) columns(std::true_type{});
             else columns(std::false_type{});
             // the parts' sums in part order; then the records and sums may be overwritten
@@ -674,7 +777,7 @@ cudaError_t product(const MvArgs& a, const void* digitsD, const void* digitsE, i
 
 }  // namespace
 
-const char* mv_variant_name(int form) { return form == F_DEFL ? "deflated matrix f16x3" : "comp matrix bf16x6"; }
+const char* mv_variant_name(int form) { return form == F_DEFL ? "deflated matrix f16x3 bf16x4" : "comp matrix bf16x6"; }
 
 cudaError_t launch_mv_scenarios(const double* v64, int n_steps, int n_scen, int s_pad, float2* D, const MvScen& c,
                                 cudaStream_t st) {
@@ -691,30 +794,36 @@ cudaError_t launch_mv_scenarios(const double* v64, int n_steps, int n_scen, int 
     return cudaGetLastError();
 }
 
-cudaError_t launch_mv_digits(int form, const float2* D, const int32_t* tau, const int32_t* colexp, int n_steps, int n_scen,
+cudaError_t launch_mv_digits(int ns, const float2* D, const int32_t* tau, const int32_t* colexp, int n_steps, int n_scen,
                              int s_pad, int pitch, void* digits, cudaStream_t st) {
     const dim3 grid(s_pad / 32, pitch / 64);
     uint32_t* out = static_cast<uint32_t*>(digits);
-    if (mv_slices(form) == 3)
-        mv_digits_kernel<3><<<grid, 256, 0, st>>>(D, tau, colexp, n_steps, n_scen, s_pad, pitch, out);
-    else
-        mv_digits_kernel<6><<<grid, 256, 0, st>>>(D, tau, colexp, n_steps, n_scen, s_pad, pitch, out);
+    auto k = ns == 3 ? mv_digits_kernel<3> : (ns == 4 ? mv_digits_kernel<4> : mv_digits_kernel<6>);
+    k<<<grid, 256, 0, st>>>(D, tau, colexp, n_steps, n_scen, s_pad, pitch, out);
     return cudaGetLastError();
 }
 
-cudaError_t launch_mv_build(int form, const MvBuild& b, cudaStream_t st) {
+cudaError_t launch_mv_build(int ns, const MvBuild& b, cudaStream_t st) {
     const int grid = b.n_tiles * (kMvP / (8 * b.rows_per_warp));
     const size_t smem = (size_t)b.pitch * sizeof(float);
-    if (mv_slices(form) == 3) mv_build_kernel<3><<<grid, 256, smem, st>>>(b);
-    else mv_build_kernel<6><<<grid, 256, smem, st>>>(b);
+    auto k = ns == 3 ? mv_build_kernel<3> : (ns == 4 ? mv_build_kernel<4> : mv_build_kernel<6>);
+    k<<<grid, 256, smem, st>>>(b);
     return cudaGetLastError();
 }
 
-cudaError_t launch_mv_product(int form, const MvArgs& a, const void* digitsD, const void* digitsE, int pitchD, int pitchE,
+cudaError_t launch_mv_build_lives(const CfTables& T, const MvLives* recs, const double* amount, int n_tiles, int pitch,
+                                  int n_steps, const float* tilt, void* digits, MvOut* out, cudaStream_t st) {
+    mv_build_lives_kernel<6><<<n_tiles * (kMvP / 8), 256, (size_t)pitch * sizeof(float), st>>>(T, recs, amount, pitch, n_steps,
+                                                                                            tilt, digits, out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mv_product(int ns, const MvArgs& a, const void* digitsD, const void* digitsE, int pitchD, int pitchE,
                               int sm_count, cudaStream_t st) {
     if (a.n_tiles <= 0 || a.n_chunks <= 0) return cudaSuccess;
-    return mv_slices(form) == 3 ? product<3>(a, digitsD, digitsE, pitchD, pitchE, sm_count, st)
-                                : product<6>(a, digitsD, digitsE, pitchD, pitchE, sm_count, st);
+    if (ns == 3) return product<3>(a, digitsD, digitsE, pitchD, pitchE, sm_count, st);
+    if (ns == 4) return product<4>(a, digitsD, digitsE, pitchD, pitchE, sm_count, st);
+    return product<6>(a, digitsD, digitsE, pitchD, pitchE, sm_count, st);
 }
 
 }  // namespace rsv

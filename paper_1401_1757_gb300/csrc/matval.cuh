@@ -8,26 +8,26 @@
 // matrix instructions with FP32 accumulation, on operands split into exact digits:
 //
 //   a = d1 + d2 + ...  with a in [0, 1]; d1: a to 7 bits.
-//   Deflated: d2 and d3 the FP16 values (11 bits and sign) of the remainders, to 2^-32 of
-//   the row's largest entry; stored times 2^15.
-//   Compensated: d2 and d3 the next 8 bits each (signed), d4 to d6 BF16 values of the
-//   remainders, to 2^-48.
+//   Three digits: d2 and d3 the FP16 values (11 bits and sign) of the remainders, to 2^-32
+//   of the row's largest entry; stored times 2^15.
+//   Four and six: d2 and d3 the next 8 bits each (signed), the others BF16 values of the
+//   remainders, to 2^-33 and 2^-48.
 //
-// d1 d1' products are multiples of 2^-14, so up to 1,000 of them add up exactly in FP32
-// (rows with more steps give up one or two bits).  The compensated form's d1 d2' and its
-// d1 d3' and d2 d2' products, 2^-8 and 2^-16 below, are multiples of 2^-22 and 2^-30 and
-// have an exact accumulator each; the rest shares one more, whose FP32 truncations (of a
-// sum 2^-24, deflated 2^-8, below) are that much smaller.  The products left out are
-// below 2^-28 (compensated 2^-48).  The epilogue adds the accumulators as
-// double-floats.  A maturity payment is added there, from the discount products
-// themselves, so that a row holds entries of one kind.
+// The products of digits i and j, i + j at most the last digit's number, are taken.  d1 d1'
+// products are multiples of 2^-14, so up to 1,000 of them add up exactly in FP32 (rows with
+// more steps give up one or two bits).  With four and six digits d1 d2', and d1 d3' and
+// d2 d2', 2^-8 and 2^-16 below, are multiples of 2^-22 and 2^-30 and have an exact
+// accumulator each; the rest shares one more, whose FP32 truncations (of a sum 2^-24,
+// with three digits 2^-8, below) are that much smaller.  The epilogue adds the
+// accumulators as double-floats.  A maturity payment is added there, from the discount
+// products themselves, so that a row holds entries of one kind.
 //
 // Fixed point needs rows and columns of moderate range.  The discount products are
 // tilted by a power of two per step, 2^tau(t) ~ 1 / (their geometric mean over the
 // scenarios), and the cash flows by 2^-tau(t), so that what is left of a scenario is its
 // deviation from the mean; a row is scaled by the power of two of its largest
-// entry.  A scenario set whose tilted products vary by more than 2^6 along a scenario
-// keeps the recurrence kernels.
+// entry.  A scenario set whose tilted products vary by too much along a scenario (see
+// mv_max_spread) keeps the recurrence kernels.
 //
 // Measured (one GB300, with the digits and the totals): the 100,000-policy mix under 1,000
 // scenarios, compensated 38.7 -> 1.56 ms (error 1e-8 -> 2e-11 at most; annuities alone
@@ -47,13 +47,23 @@ namespace rsv {
 constexpr int kMvP = 128;          // policies per tile (MMA N)
 constexpr int kMvM = 128;          // scenarios per tile (MMA M)
 constexpr int kMvParts = 4;        // column groups of the epilogue
-constexpr int kMvSpread = 6;       // log2 of the range of a scenario's tilted discount products
 constexpr int kMvTilt = 60;        // largest |tau|
 constexpr size_t kMvPanelBytes = size_t(1) << 30;            // cash-flow digits held at a time
 constexpr double kMvTableMin = 0x1p-100;                    // survivor columns in FP32 head and tail
 constexpr double kMvAmountMin = 0x1p-60, kMvAmountMax = 0x1p90;   // |amount|: V in FP32 head and tail
 
-inline int mv_slices(int form) { return form == F_DEFL ? 3 : 6; }
+// The spread of a scenario set: the largest difference of the binary exponents of a scenario's
+// tilted discount products (Vasicek paths, sd of the rate 2.2%: 3 to 5 over 50 years, 5 to 7
+// over 100).  The worst error is that of a single payment at the smallest, row entry
+// >= 1/2 and column entry >= 2^-(spread + 1):
+//   three digits (deflated, spread to 4): 2^-27 left out, 2^(spread - 25) of the payment,
+//     within the form's bound of 15 x 2^-24; at larger spreads the truncations of the low
+//     accumulator also grow past it (2e-6 measured at 7);
+//   four (deflated, to 8): below 2^-30 left out, 2^(spread - 28);
+//   six (compensated, to 10): about 2^-46 left out, 2^(spread - 44).
+inline int mv_max_spread(int form) { return form == F_DEFL ? 8 : 10; }
+inline int mv_digits_of(int form, int spread) { return form == F_DEFL ? (spread <= 4 ? 3 : 4) : 6; }
+inline int mv_digit_set(int ns) { return ns == 3 ? 0 : (ns == 4 ? 1 : 2); }   // index of a digit count
 inline int mv_pitch(int steps) { return steps < 1 ? 64 : (steps + 63) / 64 * 64; }
 
 // Scenario side, from the FP64 plane [n_steps][s_pad]: the discount products, and
@@ -76,13 +86,13 @@ struct MvScen {
 cudaError_t launch_mv_scenarios(const double* v64, int n_steps, int n_scen, int s_pad, float2* D, const MvScen& c,
                                 cudaStream_t st);
 // Its digits [slices][s_pad][pitch]; columns beyond n_scen and steps beyond n_steps are 0.
-cudaError_t launch_mv_digits(int form, const float2* D, const int32_t* tau, const int32_t* colexp, int n_steps, int n_scen,
+cudaError_t launch_mv_digits(int ns, const float2* D, const int32_t* tau, const int32_t* colexp, int n_steps, int n_scen,
                              int s_pad, int pitch, void* digits, cudaStream_t st);
 
 // Policy side of one panel of tiles: digits [tile][slices][128][pitch] up to each tile's
 // longest projection, and what the epilogue needs of each policy.
 struct alignas(16) MvOut {   // 32 bytes
-    float sc_h, sc_l;    // V = (sc_h + sc_l) 2^(colexp) U (deflated: 2^-30 of it) + (mat_h + mat_l) D(S)
+    float sc_h, sc_l;    // V = (sc_h + sc_l) 2^(colexp) U (three digits: 2^-30 of it) + (mat_h + mat_l) D(S)
     float mat_h, mat_l;  // the maturity payment times its probability
     int32_t pol, S, pad[2];
 };
@@ -102,11 +112,25 @@ struct MvBuild {
     void* digits;
     MvOut* out;
 };
-cudaError_t launch_mv_build(int form, const MvBuild& b, cudaStream_t st);
+cudaError_t launch_mv_build(int ns, const MvBuild& b, cudaStream_t st);
+
+// A contract on up to four lives (32 bytes; records of one tile in decreasing steps).
+struct MvLives {
+    int32_t idx[4];  // survivor-column index of each life at valuation, -1: no such life
+    int32_t S;
+    int32_t pol;     // -1: padding
+    int32_t k;       // 1 .. 4
+    int32_t flags;   // bit 0: assurance (on the k-th death), else annuity (k or more alive);
+                     // bits 8..11: dead at valuation
+};
+static_assert(sizeof(MvLives) == sizeof(SlotRec), "record strides");
+constexpr int kMvRecWords = sizeof(SlotRec) / 4;
+cudaError_t launch_mv_build_lives(const CfTables& T, const MvLives* recs, const double* amount, int n_tiles, int pitch,
+                                  int n_steps, const float* tilt, void* digits, MvOut* out, cudaStream_t st);
 
 struct MvArgs {
-    const SlotRec* slots;
-    const int32_t* kinds;
+    const int32_t* steps;      // the steps of the panel's first record; one record is kMvRecWords
+    const int32_t* kinds;      // of the tiles, or null: no maturity payments
     const MvOut* out;
     const int32_t* colexp;     // of the first column
     const float2* D;           // the discount products [n_steps][s_pad], at the first column
@@ -119,8 +143,8 @@ struct MvArgs {
     double* partial;           // [n_tiles][part_ld], at the panel's first tile and the block's first column
     int32_t* status;
 };
-// digitsE: launch_mv_build's, digitsD: launch_mv_digits'.
-cudaError_t launch_mv_product(int form, const MvArgs& a, const void* digitsD, const void* digitsE, int pitchD, int pitchE,
+// digitsE: launch_mv_build's, digitsD: launch_mv_digits', both of ns digits.
+cudaError_t launch_mv_product(int ns, const MvArgs& a, const void* digitsD, const void* digitsE, int pitchD, int pitchE,
                               int sm_count, cudaStream_t st);
 
 // The matrix variant's index among a form's tunable variants is the last one.

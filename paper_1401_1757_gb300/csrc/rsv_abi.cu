@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <thread>
 #include <cmath>
+#include <climits>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -615,31 +616,60 @@ rsv_status upload_amounts(rsv_ctx* c) {
 
 }  // namespace
 
-bool rsv::mv_applies(const rsv_ctx* c) {
-    if (!c->mv_scen_ok || !(c->amt_hi <= kMvAmountMax) || !(c->amt_lo >= kMvAmountMin)) return false;
+bool rsv::mv_applies(const rsv_ctx* c, int form, double amt_lo, double amt_hi) {
+    if (c->mv_spread > mv_max_spread(form) || !(amt_hi <= kMvAmountMax) || !(amt_lo >= kMvAmountMin)) return false;
     for (int t = 0; t < kMaxTables; ++t)
         if (!c->tab[t].empty() && !(c->tab_min[t] >= kMvTableMin)) return false;
     return true;
+}
+
+rsv_status rsv::mv_scenario_digits(rsv_ctx* c, int form) {
+    const int ns = mv_digits_of(form, c->mv_spread), k = mv_digit_set(ns), pitch = mv_pitch(c->n_steps);
+    if (c->mv_dig_gen[k] == c->scen_gen) return RSV_OK;   // with the scenario set, like its planes
+    CU(c->d_mv_dig[k].ensure((size_t)ns * c->s_pad * pitch * 2));
+    const MvScen mv = MvScen::at(c->d_mv_col.p, c->n_steps, c->s_pad);
+    CU(launch_mv_digits(ns, c->d_mv_D.as<float2>(), mv.tau, mv.colexp, c->n_steps, c->n_scen, c->s_pad, pitch,
+                        c->d_mv_dig[k].p, c->stream));
+    c->mv_dig_gen[k] = c->scen_gen;
+    return RSV_OK;
+}
+
+int rsv::mv_panel_tiles(const rsv_ctx* c, int form, int max_S, int n_tiles) {
+    const size_t tile = (size_t)mv_digits_of(form, c->mv_spread) * kMvP * mv_pitch(max_S) * 2;
+    return (int)std::max<size_t>(1, std::min<size_t>(std::max(1, n_tiles), kMvPanelBytes / tile));
+}
+
+rsv_status rsv::mv_panel_buffers(rsv_ctx* c, int form, int max_S, int tiles) {
+    CU(c->d_mv_E.ensure((size_t)mv_digits_of(form, c->mv_spread) * kMvP * mv_pitch(max_S) * 2 * tiles));
+    CU(c->d_mv_out.ensure((size_t)tiles * kMvP * sizeof(MvOut)));
+    return RSV_OK;
+}
+
+rsv_status rsv::mv_multiply(rsv_ctx* c, int form, MvArgs a, int max_S, int s0, int w) {
+    a.out = c->d_mv_out.as<MvOut>();
+    a.colexp = MvScen::at(c->d_mv_col.p, c->n_steps, c->s_pad).colexp + s0;
+    a.D = c->d_mv_D.as<float2>() + s0;
+    a.n_chunks = (w + kMvM - 1) / kMvM;
+    a.s_pad = c->s_pad;
+    a.n_scen = w;
+    a.s0 = s0;
+    a.v0_ld = c->n_scen;
+    a.part_ld = c->s_pad;
+    a.status = c->d_ctl.as<int32_t>() + 1;
+    const int ns = mv_digits_of(form, c->mv_spread);
+    CU(launch_mv_product(ns, a, c->d_mv_dig[mv_digit_set(ns)].p, c->d_mv_E.p, mv_pitch(c->n_steps), mv_pitch(max_S),
+                         c->sm_count, c->stream));
+    return RSV_OK;
 }
 
 rsv_status rsv::mv_prepare(rsv_ctx* c, int form) {
     const Layout& L = c->lay;
     rsv_status st;
     CfTables T;
-    if ((st = layout_to_device(c)) != RSV_OK || (st = upload_amounts(c)) != RSV_OK || (st = cf_tables(c, T)) != RSV_OK)
+    if ((st = layout_to_device(c)) != RSV_OK || (st = upload_amounts(c)) != RSV_OK || (st = cf_tables(c, T)) != RSV_OK ||
+        (st = mv_scenario_digits(c, form)) != RSV_OK ||
+        (st = mv_panel_buffers(c, form, L.max_S, mv_panel_tiles(c, form, L.max_S, L.n_tiles))) != RSV_OK)
         return st;
-    const int k = form == F_DEFL ? 1 : 0, pitch = mv_pitch(c->n_steps);
-    if (c->mv_dig_gen[k] != c->scen_gen) {   // with the scenario set, like its planes
-        CU(c->d_mv_dig[k].ensure((size_t)mv_slices(form) * c->s_pad * pitch * 2));
-        const MvScen mv = MvScen::at(c->d_mv_col.p, c->n_steps, c->s_pad);
-        CU(launch_mv_digits(form, c->d_mv_D.as<float2>(), mv.tau, mv.colexp, c->n_steps, c->n_scen, c->s_pad, pitch,
-                            c->d_mv_dig[k].p, c->stream));
-        c->mv_dig_gen[k] = c->scen_gen;
-    }
-    const size_t tile = (size_t)mv_slices(form) * kMvP * mv_pitch(L.max_S) * 2;
-    const int panel = (int)std::max<size_t>(1, std::min<size_t>(std::max(1, L.n_tiles), kMvPanelBytes / tile));
-    CU(c->d_mv_E.ensure(tile * panel));
-    CU(c->d_mv_out.ensure((size_t)panel * kMvP * sizeof(MvOut)));
     c->mv_built = -1;
     return RSV_OK;
 }
@@ -647,11 +677,9 @@ rsv_status rsv::mv_prepare(rsv_ctx* c, int form) {
 rsv_status rsv::mv_launch(rsv_ctx* c, int form, int s0, int w, float* V0f, double* V0d, double* partial) {
     const Layout& L = c->lay;
     CfTables T;
-    const rsv_status st = cf_tables(c, T);
+    rsv_status st = cf_tables(c, T);
     if (st != RSV_OK) return st;
-    const int pitchE = mv_pitch(L.max_S), pitchD = mv_pitch(c->n_steps);
-    const size_t tile = (size_t)mv_slices(form) * kMvP * pitchE * 2;
-    const int panel = (int)std::max<size_t>(1, std::min<size_t>(std::max(1, L.n_tiles), kMvPanelBytes / tile));
+    const int panel = mv_panel_tiles(c, form, L.max_S, L.n_tiles);
     const MvScen mv = MvScen::at(c->d_mv_col.p, c->n_steps, c->s_pad);
     for (int t0 = 0; t0 < L.n_tiles; t0 += panel) {
         const int n = std::min(panel, L.n_tiles - t0);
@@ -664,7 +692,7 @@ rsv_status rsv::mv_launch(rsv_ctx* c, int form, int s0, int w, float* V0f, doubl
             b.amount = c->d_amount.as<double>();
             b.n_tiles = n;
             b.tab_pad = L.tab_pad;
-            b.pitch = pitchE;
+            b.pitch = mv_pitch(L.max_S);
             b.general_from = L.P_general > 0 ? std::max(0, L.grp_tiles[0] - t0) : n;
             b.cf = c->d_cf64.as<double>();
             b.cf_ld = c->cf_steps;
@@ -674,29 +702,18 @@ rsv_status rsv::mv_launch(rsv_ctx* c, int form, int s0, int w, float* V0f, doubl
             b.tilt_top = mv.tilt_top;
             b.digits = c->d_mv_E.p;
             b.out = c->d_mv_out.as<MvOut>();
-            CU(launch_mv_build(form, b, c->stream));
+            CU(launch_mv_build(mv_digits_of(form, c->mv_spread), b, c->stream));
             c->mv_built = t0;
         }
         MvArgs a{};
-        a.slots = slots;
+        a.steps = &slots->S;
         a.kinds = L.kinds.as<int32_t>() + t0;
-        a.out = c->d_mv_out.as<MvOut>();
-        a.colexp = mv.colexp + s0;
-        a.D = c->d_mv_D.as<float2>() + s0;
         a.amount = c->d_amount.as<double>();
         a.n_tiles = n;
-        a.n_chunks = (w + kMvM - 1) / kMvM;
-        a.s_pad = c->s_pad;
-        a.n_scen = w;
-        a.s0 = s0;
-        a.v0_ld = c->n_scen;
-        a.part_ld = c->s_pad;
         a.V0f = V0f;
         a.V0d = V0d;
         a.partial = partial ? partial + (size_t)t0 * c->s_pad : nullptr;
-        a.status = c->d_ctl.as<int32_t>() + 1;
-        CU(launch_mv_product(form, a, c->d_mv_dig[form == F_DEFL ? 1 : 0].p, c->d_mv_E.p, pitchD, pitchE, c->sm_count,
-                             c->stream));
+        if ((st = mv_multiply(c, form, a, L.max_S, s0, w)) != RSV_OK) return st;
     }
     return RSV_OK;
 }
@@ -770,7 +787,7 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
         return fail(c, RSV_E_ARG, "variant %d out of range", o->variant);
     }
     if (o->form == F_COMP && vi == nt && !extra && pay == PAY_END) {
-        mat = mv_applies(c);
+        mat = mv_applies(c, F_COMP, c->amt_lo, c->amt_hi);
         vi = 0;
     }
     if (split) vg = special_variant(vl, nv, false, PAY_END_GENERAL);
@@ -1054,8 +1071,8 @@ rsv_status compute_nested(rsv_ctx* c, const rsv_opts* o, const rsv_nested_spec* 
         // state j at node n] (FP64), in closed form from the survivor columns, a
         // node to a host part.
         if ((st = cf_tables(c, T)) != RSV_OK) return st;
-        const size_t cols = (size_t)L.n_tab * T.rows;
         const double* hm = c->h_cf_tab.data();
+        const size_t cols = c->h_cf_tab.size() / 6;
         const int32_t* hz = reinterpret_cast<const int32_t*>(hm + 2 * cols);
         const int32_t* hex = hz + cols;
         auto alive = [&](int table, int age, int m) {
@@ -1225,7 +1242,7 @@ rsv_status rsv_destroy(rsv_ctx* c) try {
                       &c->sur.d_comm, &c->sur.d_lnb, &c->d_tabf[0], &c->d_tabf[1], &c->d_tabf[2], &c->d_vf64,
                       &c->d_vf32, &c->d_vf2, &c->d_cf64, &c->d_cf32, &c->d_ml_rec,
                       &c->d_ml_amount, &c->sur.d_cnt, &c->sur.d_q2, &c->sur.d_idx, &c->sur.d_v2, &c->d_nest_bm,
-                      &c->d_mv_D, &c->d_mv_col, &c->d_mv_dig[0], &c->d_mv_dig[1], &c->d_mv_E, &c->d_mv_out,
+                      &c->d_mv_D, &c->d_mv_col, &c->d_mv_dig[0], &c->d_mv_dig[1], &c->d_mv_dig[2], &c->d_mv_E, &c->d_mv_out,
                       &c->d_defl_slots, &c->d_defl_kinds, &c->d_defl_tab, &c->d_defl_plane, &c->d_mlp_trace})
         b->release();
     c->mlp.release();
@@ -1447,7 +1464,7 @@ rsv_status rsv_load_scenarios(rsv_ctx* c, const double* v, int32_t n_scen, int32
     int32_t range[2];
     CU(cudaMemcpyAsync(range, mv.stat, sizeof range, cudaMemcpyDeviceToHost, c->stream));
     CU(cudaStreamSynchronize(c->stream));
-    c->mv_scen_ok = range[0] <= kMvSpread && range[1] <= kMvTilt;
+    c->mv_spread = range[1] <= kMvTilt ? range[0] : INT_MAX;
     ++c->scen_gen;
     c->n_scen = n_scen;
     c->n_steps = n_steps;

@@ -3,7 +3,7 @@ compensated and deflated forms): edges of its tiles, every reduced model and sta
 projections, varying cash flows, and the data that keeps the recurrence kernels.
 
 Tolerances.  Compensated: operands to 2^-48 of a row's largest entry, discount products
-within 2^6 of a column's largest, so 2^-42 an entry at the worst place, and FP32 truncations of an
+within 2^11 of a column's largest, so 2^-34 an entry at the worst place, and FP32 truncations of an
 accumulator 2^-24 below the result, at most 15 a block of 16 steps: 4,096 steps stay below
 2^-33; 5e-10 covers both.  Deflated: its stated bound 15 x 2^-24.
 Error metric: rel = |V_gpu - V_ref| / max(|V_ref|, 1e-9 * amount)."""
@@ -100,6 +100,22 @@ def test_long_level_projections(ctx, form, steps):
     check(form, pol, *value(ctx, form, pol, [tab], v), ref, ref_tot)
 
 
+@pytest.mark.parametrize("form", [COMP, DEFL])
+@pytest.mark.parametrize("bits", [3, 4, 5, 7, 8, 9, 10])
+def test_scenarios_far_from_their_mean(ctx, form, bits):
+    """Flat rates whose discount products end 2^bits apart from their mean's, single payments
+    where the discount product is smallest against its scenario's largest."""
+    tab = synth.gm_monthly_survival()
+    pol = every_product(60, bits, form)
+    pol["product"][:12], pol["term_m"][:12], pol["state0"][:12] = 2, 1, 0
+    pol["age1_m"][:12] = np.arange(240, 1440, 100)
+    pol["age1_m"][12:15], pol["product"][12:15], pol["state0"][12:15] = 1439, 0, 0
+    slope = np.linspace(-1, 1, 41)[:, None] * (bits - 0.01) * np.log(2.0) / 1200
+    v = np.exp(-0.0033 - slope + np.zeros((41, 1200)))
+    ref, ref_tot = oracle.reserves_batch(pol, tab, v)
+    check(form, pol, *value(ctx, form, pol, [tab], v), ref, ref_tot)
+
+
 def test_varying_cash_flows(ctx):
     """Rows that are level and rows that are not, deferred and annual payments."""
     tab = synth.gm_monthly_survival()
@@ -135,3 +151,35 @@ def test_data_out_of_range_keeps_the_recurrence(ctx, form, what):
         tab = synth.constant_force_table(0.8)
     a, b = value(ctx, form, pol, [tab], v), value(ctx, form, pol, [tab], v, variant=0)
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("n,n_scen", [(1, 1), (127, 31), (128, 128), (130, 129)])
+def test_lives_against_the_fp64_form(ctx, n, n_scen):
+    """Contracts on one to four lives with every k, both families, dead lives at valuation,
+    lives at and past the limiting age: the FP64 kernel applies the lives' transitions to
+    every chain."""
+    rng = np.random.default_rng(n)
+    rec = np.zeros(n, rsv.MLIFE_DTYPE)
+    rec["m"] = 1 + np.arange(n) % 4
+    rec["kind"] = (np.arange(n) // 4) % 2
+    rec["k"] = 1 + rng.integers(0, 100, n) % rec["m"]
+    rec["age_m"] = rng.integers(200, 1300, (n, 4))
+    rec["age_m"][::9, 0] = 1440
+    rec["age_m"][4::9, 0] = 1450
+    rec["table"] = rng.integers(0, 2, (n, 4))
+    rec["term_m"] = np.where(rec["kind"] == 1, rng.integers(1, 480, n), np.where(np.arange(n) % 3, 0, 200))
+    spare = np.where(rec["kind"] == 1, rec["k"] - 1, rec["m"] - rec["k"])   # lives that may be dead already
+    rec["dead0"] = np.where(spare > 0, rng.integers(0, 2, n), 0)
+    rec["amount"] = rng.lognormal(5.0, 2.0, n)
+    for i, t in enumerate([synth.gm_monthly_survival(), synth.gm_monthly_survival(A=0.0003, B=0.00002)]):
+        rsv.rsv_load_decrements(ctx, i, t)
+    rsv.rsv_load_scenarios(ctx, synth.vasicek_paths(n_scen, 1240, seed=n))
+    res = {}
+    for form in (rsv.RSV_FORM_F64, COMP):
+        V, tot = np.zeros((n, n_scen)), np.zeros(n_scen)
+        rsv.rsv_compute_mlife(ctx, rec, form, V0T, V0d=V, scen_total=tot)
+        res[form] = V, tot
+    V, tot = res[rsv.RSV_FORM_F64]
+    scale = np.maximum(np.abs(V), 1e-9 * rec["amount"][:, None])
+    assert np.max(np.abs(res[COMP][0] - V) / scale) <= TOL[COMP]
+    assert np.all(np.abs(res[COMP][1] - tot) <= TOL[COMP] * tot)
