@@ -10,7 +10,8 @@ namespace rsv {
 namespace {
 
 __global__ void cf_records_kernel(const CfTables T, const SlotRec* __restrict__ slots, const int32_t* __restrict__ kinds,
-                                  const double* __restrict__ amount, int n, int tab_pad, CfPol* __restrict__ out) {
+                                  const double* __restrict__ amount, int n, int per_kind, int tab_pad,
+                                  CfPol* __restrict__ out) {
     const int f = blockIdx.x * blockDim.x + threadIdx.x;
     if (f >= n) return;
     const SlotRec r = slots[f];
@@ -30,7 +31,7 @@ __global__ void cf_records_kernel(const CfTables T, const SlotRec* __restrict__ 
     p.pol = r.pol;
     p.amount = r.pol >= 0 ? amount[r.pol] : 0.0;
     p.bnd = r.bnd;
-    p.kind = kinds[f];
+    p.kind = kinds[f / per_kind];
     p.S = r.S;
     p.state0 = r.state0;
     out[f] = p;
@@ -95,9 +96,9 @@ __global__ void __launch_bounds__(1024) cf_finish_kernel(const double* __restric
 }  // namespace
 
 cudaError_t launch_cf_records(const CfTables& T, const SlotRec* slots, const int32_t* kinds, const double* amount, int n,
-                              int tab_pad, CfPol* out, cudaStream_t st) {
+                              int per_kind, int tab_pad, CfPol* out, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    cf_records_kernel<<<(n + 127) / 128, 128, 0, st>>>(T, slots, kinds, amount, n, tab_pad, out);
+    cf_records_kernel<<<(n + 127) / 128, 128, 0, st>>>(T, slots, kinds, amount, n, per_kind, tab_pad, out);
     return cudaGetLastError();
 }
 

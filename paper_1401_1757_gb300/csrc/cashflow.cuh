@@ -96,9 +96,9 @@ __device__ __forceinline__ double cf_boundary(const CfTables& T, const CfPol& p)
     return p.bnd * (p.state0 == 1 ? x : (p.state0 == 2 ? y : x + y * (1.0 - x)));
 }
 
-// Records of n one-policy tiles (slots, kinds as the layout of width 1 gives them).
+// Records of n layout slots, per_kind of them to a tile (a kind).
 cudaError_t launch_cf_records(const CfTables& T, const SlotRec* slots, const int32_t* kinds, const double* amount, int n,
-                              int tab_pad, CfPol* out, cudaStream_t st);
+                              int per_kind, int tab_pad, CfPol* out, cudaStream_t st);
 
 // The portfolio's cash flows: with A(t) = sum_p amount_p E_p(t) and M(t) the sum of
 // amount_p B_p over the policies with S = t,

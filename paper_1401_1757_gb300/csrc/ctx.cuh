@@ -222,8 +222,8 @@ struct rsv_ctx {
     int mv_spread = 0x7fffffff;   // of the scenario set (mv_max_spread)
     double tab_min[rsv::kMaxTables] = {};           // smallest survivor-column entry of a table
     double amt_lo = 0.0, amt_hi = 0.0;              // smallest non-zero and largest |amount|
-    DevBuf d_mv_D, d_mv_col, d_mv_dig[3], d_mv_E, d_mv_out;
-    unsigned long long scen_gen = 1, mv_dig_gen[3] = {0, 0, 0};
+    DevBuf d_mv_D, d_mv_col, d_mv_D64, d_mv_dig[4], d_mv_E, d_mv_out;
+    unsigned long long scen_gen = 1, mv_dig_gen[4] = {0, 0, 0, 0};
     int mv_built = -1;   // first tile of the panel whose digits are held, within one call
 
     Layout lay;
@@ -291,7 +291,7 @@ rsv_status cf_tables(rsv_ctx* c, CfTables& T);
 rsv_status stage_tables(rsv_ctx* c, int form, int pad, int n_tab, size_t& smem);
 // Whether the matrix product covers the loaded data; then, on the layout of width
 // kMvP: mv_prepare once a call, mv_launch for the scenario columns [s0, s0 + w) with the
-// output pointers at column s0 (partial: [n_tiles][s_pad]).
+// output pointers at column s0 (partial: [mv_part_rows][s_pad]).
 bool mv_applies(const rsv_ctx* c, int form, double amt_lo, double amt_hi);
 rsv_status mv_prepare(rsv_ctx* c, int form);
 // Its parts, for rows that come from elsewhere (m lives): the scenario set's digits, the tiles

@@ -64,13 +64,42 @@ __device__ __forceinline__ void mv_digits(float h0, float l0, float h1, float l1
     }
 }
 
+// The eight digits of a positive normal FP64 number a times 2^shift, in [0, 1], by integers:
+// a 2^63 rounded down, split into balanced bytes (the leading one 7 bits); `sh` = the
+// shift of the 53-bit mantissa.  0 for a = 0.
+__device__ __forceinline__ unsigned long long mv_fixed64(double a, int shift) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(a);
+    const int ex = (int)(bits >> 52);   // a >= 0
+    if (ex == 0) return 0;
+    const unsigned long long m = (bits & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+    const int sh = ex - 1023 + 11 + shift;
+    if (sh >= 0) return m << min(sh, 11);
+    return sh > -64 ? m >> -sh : 0;
+}
+// digit k of two numbers as a pair of BF16 values (exact: 8 bits and sign)
+__device__ __forceinline__ uint32_t mv_byte_pair(unsigned long long x, unsigned long long y, int k) {
+    constexpr unsigned long long kHalf = 0x0080808080808080ull;   // half of each lower byte
+    auto digit = [&](unsigned long long v) {
+        const uint32_t byte = (uint32_t)((v + kHalf) >> (56 - 8 * k)) & 0xFF;
+        const float d = __fsub_rn(__uint_as_float(0x4B000000u | byte), k ? 8388736.0f : 8388608.0f);
+        return __float_as_uint(__fmul_rn(d, pow2f(-7 - 8 * k)));
+    };
+    return digit(x) >> 16 | (digit(y) & 0xFFFF0000u);
+}
+
 // ---------------------------------------------------------- scenario side ----
 // Running products of 8 scenarios, the steps in 32 segments: a segment's product,
 // the products before it, then the running product, so that the serial chain is 1/16
 // of the steps.
 constexpr int kProdS = 8;
+__device__ __forceinline__ void put(double* p, double d) { *p = d; }
+__device__ __forceinline__ void put(float2* p, double d) {
+    const float h = __double2float_rn(d);
+    *p = make_float2(h, __double2float_rn(d - (double)h));
+}
+template <class T>
 __global__ void __launch_bounds__(kProdS * 32) mv_products_kernel(const double* __restrict__ v, int n_steps, int s_pad,
-                                                                  float2* __restrict__ D) {
+                                                                  T* __restrict__ D) {
     __shared__ double seg[32][kProdS];
     const int s = blockIdx.x * kProdS + threadIdx.x, k = threadIdx.y;
     const int len = (n_steps + 31) / 32, t0 = min(n_steps, k * len), t1 = min(n_steps, t0 + len);
@@ -84,8 +113,7 @@ __global__ void __launch_bounds__(kProdS * 32) mv_products_kernel(const double* 
 #pragma unroll 4
     for (int t = t0; t < t1; ++t) {
         d = __dmul_rn(d, v[(size_t)t * s_pad + s]);
-        const float h = __double2float_rn(d);
-        D[(size_t)t * s_pad + s] = make_float2(h, __double2float_rn(d - (double)h));
+        put(&D[(size_t)t * s_pad + s], d);
     }
 }
 
@@ -193,6 +221,27 @@ __global__ void __launch_bounds__(256) mv_digits_kernel(const float2* __restrict
     }
     __syncthreads();
     for (int i = threadIdx.x; i < NS * 32 * 32; i += 256) {
+        const int q = i & 31, r = (i >> 5) & 31, k = i >> 10;
+        out[(((size_t)k * s_pad + s0 + r) * pitch + t0) / 2 + q] = tile[k][r][q];
+    }
+}
+
+__global__ void __launch_bounds__(256) mv_digits64_kernel(const double* __restrict__ D, const int32_t* __restrict__ tau,
+                                                          const int32_t* __restrict__ colexp, int n_steps, int n_scen,
+                                                          int s_pad, int pitch, uint32_t* __restrict__ out) {
+    __shared__ uint32_t tile[8][32][33];
+    const int s0 = blockIdx.x * 32, t0 = blockIdx.y * 64, s = s0 + (threadIdx.x & 31);
+    const int c = colexp[s];
+    auto load = [&](int t) -> unsigned long long {
+        return t < n_steps && s < n_scen ? mv_fixed64(D[(size_t)t * s_pad + s], tau[t] - c) : 0;
+    };
+    for (int q = threadIdx.x >> 5; q < 32; q += 8) {
+        const unsigned long long x = load(t0 + 2 * q), y = load(t0 + 2 * q + 1);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) tile[k][threadIdx.x & 31][q] = mv_byte_pair(x, y, k);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < 8 * 32 * 32; i += 256) {
         const int q = i & 31, r = (i >> 5) & 31, k = i >> 10;
         out[(((size_t)k * s_pad + s0 + r) * pitch + t0) / 2 + q] = tile[k][r][q];
     }
@@ -385,6 +434,79 @@ __device__ __forceinline__ void mv_row(const MvBuild& b, const SlotRec& r, int r
     }
 }
 
+// ---- the FP64 form: the cash flows in FP64 (cashflow.cuh), the scale from their FP32 heads
+struct alignas(16) MvOut64 {   // in the place of MvOut
+    double sc, mat;
+    int32_t pol, S, pad[2];
+};
+static_assert(sizeof(MvOut64) == sizeof(MvOut), "record sizes");
+
+template <int KIND, bool CF>
+__device__ __forceinline__ void mv_row64(const MvBuild& b, const SlotRec& r, const CfPol& p, int row, int kt,
+                                         const float* __restrict__ tilt) {
+    const CfTables& T = b.T;
+    const MvLife x{p.a.i, p.a.last, df_of(KIND == K_JL && r.state0 == 2 ? 0.0 : p.a.inv)};
+    const MvLife y{p.b.i, p.b.last, df_of(KIND == K_JL ? (r.state0 == 1 ? 0.0 : p.b.inv * p.rho) : p.b.inv)};
+    const int S = r.pol >= 0 ? r.S : 0;
+    auto head = [&](int t) {   // per unit amount, as cf_expected
+        df e = mv_expected<KIND>(T, x, y, r.state0, t);
+        if constexpr (KIND == K_ANN || KIND == K_ASS) e = df_mul(e, x.c);
+        if constexpr (CF) e = df_mul(e, df_of(b.cf[(size_t)r.pol * b.cf_ld + t]));
+        return e;
+    };
+    int e;
+    if constexpr (!CF && (KIND == K_ANN || KIND == K_ANN2 || KIND == K_JL))
+        e = mv_row_exp(S > 0 ? __fmul_rn(head(0).h, b.tilt_top[S - 1]) : 0.0f, S);
+    else
+        e = mv_row_exp(mv_top(head, S, tilt), S);
+    uint32_t* base = static_cast<uint32_t*>(b.digits) + ((size_t)(row / kMvP) * 8 * kMvP + row % kMvP) * b.pitch / 2;
+    for (int t = 2 * (threadIdx.x & 31); t < kt; t += 64) {
+        unsigned long long v[2] = {0, 0};
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if (t + k < S) {
+                double f = cf_expected(T, p, t + k);
+                if constexpr (CF) f *= b.cf[(size_t)r.pol * b.cf_ld + t + k];
+                v[k] = mv_fixed64(f, (__float_as_int(tilt[t + k]) >> 23) - 127 - e);
+            }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) base[((size_t)k * kMvP * b.pitch + t) / 2] = mv_byte_pair(v[0], v[1], k);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        MvOut64 o;
+        o.sc = p.amount * __hiloint2double((e + 1023) << 20, 0);
+        o.mat = r.pol >= 0 && p.bnd != 0.0 ? p.amount * (S == 0 ? p.bnd : cf_boundary(T, p)) : 0.0;
+        o.pol = r.pol;
+        o.S = S;
+        o.pad[0] = o.pad[1] = 0;
+        reinterpret_cast<MvOut64*>(b.out)[row] = o;
+    }
+}
+
+__global__ void __launch_bounds__(256) mv_build64_kernel(const MvBuild b, const CfPol* __restrict__ pols) {
+    extern __shared__ float4 tilt4[];
+    float* tilt = reinterpret_cast<float*>(tilt4);
+    const int row = blockIdx.x * 8 + (threadIdx.x >> 5), tile = row / kMvP;
+    const int kt = max(64, (b.slots[(size_t)tile * kMvP].S + 63) / 64 * 64);
+    for (int t = threadIdx.x; t < kt; t += 256) tilt[t] = t < b.n_steps ? b.tilt[t] : 0.0f;
+    __syncthreads();
+    const SlotRec r = b.slots[row];
+    const CfPol p = pols[row];
+    auto run = [&](auto cf) {
+        constexpr bool CF = decltype(cf)::value;
+        switch (b.kinds[tile]) {
+        case K_ANN: return mv_row64<K_ANN, CF>(b, r, p, row, kt, tilt);
+        case K_ASS: return mv_row64<K_ASS, CF>(b, r, p, row, kt, tilt);
+        case K_JL: return mv_row64<K_JL, CF>(b, r, p, row, kt, tilt);
+        case K_ANN2: return mv_row64<K_ANN2, CF>(b, r, p, row, kt, tilt);
+        case K_ASS2: return mv_row64<K_ASS2, CF>(b, r, p, row, kt, tilt);
+        default: return mv_row64<K_LS2, CF>(b, r, p, row, kt, tilt);
+        }
+    };
+    if (tile >= b.general_from) run(std::true_type{});
+    else run(std::false_type{});
+}
+
 // ---- contracts on up to four lives (MvLives): the lives are independent, so a step's
 // expected cash flow is a polynomial in their survival and death probabilities.  A life
 // that is absent counts for nothing (an annuity counts it as dead, an assurance as alive).
@@ -512,29 +634,33 @@ __global__ void __launch_bounds__(256) mv_build_kernel(const MvBuild b) {
 // double-floats, scale, write V0 (32 consecutive scenarios of a policy a warp store) and
 // sum each scenario over the tile's policies.
 // Three digits: 6 products and 2 accumulators, so TMEM holds two tiles' and the epilogue
-// runs beside the next tile's products; four and six: 10 and 21 products, 4 accumulators.
+// runs beside the next tile's products; four and six: 10 and 21 products, 4 accumulators.  Eight (FP64): 36 products, an
+// accumulator for each level of half a tile's policies, added in FP64.
 template <int NS>
-struct MvShape;   // accumulators, tiles in TMEM, stages, steps of a block (64: 128-byte swizzled
-template <>       // rows); the products are (i, j), i + j < NS, of scenario digit i and policy
+struct MvShape;   // policies of an item, accumulators, items in TMEM, stages, steps of a block (64:
+template <>       // 128-byte swizzled rows); the products are (i, j), i + j < NS, of scenario digit i and policy
 struct MvShape<3> {   // digit j, in accumulator min(i + j, NA - 1)
-    static constexpr int NA = 2, NB = 2, ST = 3, KB = 64;
+    static constexpr int N = kMvP, NA = 2, NB = 2, ST = 3, KB = 64;
 };
 template <>
 struct MvShape<4> {
-    static constexpr int NA = 4, NB = 1, ST = 4, KB = 32;
+    static constexpr int N = kMvP, NA = 4, NB = 1, ST = 4, KB = 32;
 };
 template <>
 struct MvShape<6> {
-    static constexpr int NA = 4, NB = 1, ST = 3, KB = 32;
+    static constexpr int N = kMvP, NA = 4, NB = 1, ST = 3, KB = 32;
+};
+template <>
+struct MvShape<8> {
+    static constexpr int N = kMvP / 2, NA = 8, NB = 1, ST = 2, KB = 32;
 };
 constexpr int kMvEpi = 4 * kMvParts;                   // epilogue warps
 constexpr int kMvThreads = 32 * (kMvEpi + 2);
-constexpr int kMvHalf = kMvP / 2;                      // policies staged by one CTA of a pair
 
 // shared memory of a stage: NS slabs of scenario digits, then NS of policy digits
 template <int NS>
 struct MvStage {
-    static constexpr int kA = kMvM * MvShape<NS>::KB * 2, kB = kMvHalf * MvShape<NS>::KB * 2;
+    static constexpr int kA = kMvM * MvShape<NS>::KB * 2, kB = MvShape<NS>::N / 2 * MvShape<NS>::KB * 2;
     static constexpr int kBytes = NS * (kA + kB);
 };
 
@@ -545,7 +671,7 @@ __device__ __forceinline__ void mv_products(uint32_t d, uint64_t base, int off, 
     using G = MvStage<NS>;
     constexpr int acc = I + J < MvShape<NS>::NA ? I + J : MvShape<NS>::NA - 1;
     constexpr bool first = I == 0 && J == acc;   // of its accumulator
-    mma_f16_ss_pair(d + acc * kMvP, base + (uint64_t)((I * G::kA + off) >> 4),
+    mma_f16_ss_pair(d + acc * MvShape<NS>::N, base + (uint64_t)((I * G::kA + off) >> 4),
                     base + (uint64_t)((NS * G::kA + J * G::kB + off) >> 4), idesc, !first || more);
     if constexpr (I + J + 1 < NS) mv_products<NS, I, J + 1>(d, base, off, idesc, more);
     else if constexpr (I + 1 < NS) mv_products<NS, I + 1, 0>(d, base, off, idesc, more);
@@ -556,8 +682,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
     mv_product_kernel(const __grid_constant__ CUtensorMap mapD, const __grid_constant__ CUtensorMap mapE, const MvArgs a) {
     using Sh = MvShape<NS>;
     using G = MvStage<NS>;
-    constexpr int KB = Sh::KB;
-    constexpr uint32_t kIdesc = f16_idesc(NS != 3, 2 * kMvM, kMvP);   // both operands FP16, or both BF16
+    constexpr int KB = Sh::KB, N = Sh::N, kSub = kMvP / N;
+    constexpr uint32_t kIdesc = f16_idesc(NS != 3, 2 * kMvM, N);   // both operands FP16, or both BF16
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // (both CTAs of a pair place everything alike)
     unsigned char* ring = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -566,7 +692,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
     __shared__ uint64_t full[Sh::ST], empty[Sh::ST], acc_full[Sh::NB], acc_empty[Sh::NB], drained;
     __shared__ uint32_t tmem_slot;
     __shared__ MvOut recs[kMvP];
-    __shared__ float2 sums[kMvParts][kMvM];
+    __shared__ __align__(8) float2 sums[kMvParts][kMvM];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int rank = (int)cluster_rank();
     if (tid == 0) {
@@ -587,7 +713,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
     fence_after();
     const uint32_t tmem = tmem_slot;
     const int n_pairs = (a.n_chunks + 1) / 2, n_clusters = (int)gridDim.x / 2, cluster = (int)blockIdx.x / 2;
-    const long long n_items = (long long)a.n_tiles * n_pairs;
+    const long long n_items = (long long)a.n_tiles * kSub * n_pairs;   // part of a tile, pair of scenario tiles
     bool failed = false;
     auto wait_on = [&](uint64_t* bar, uint32_t parity) {   // a bounded wait; a timeout is recorded
         if (failed) return;
@@ -603,7 +729,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
         if (elect_one()) {
             uint32_t it = 0;
             for (long long item = cluster; item < n_items && !failed; item += n_clusters) {
-                const int tile = (int)(item / n_pairs), chunk = 2 * (int)(item - (long long)tile * n_pairs) + rank;
+                const int sub = (int)(item / n_pairs), chunk = 2 * (int)(item - (long long)sub * n_pairs) + rank;
+                const int tile = sub / kSub, col = (sub - tile * kSub) * N + rank * (N / 2);
                 const int nk = blocks_of(tile);
                 for (int kb = 0; kb < nk && !failed; ++kb, ++it) {
                     const int st = it % Sh::ST;
@@ -615,8 +742,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
 #pragma unroll
                     for (int k = 0; k < NS; ++k) {
                         tma_load_2d_pair(dst + k * G::kA, &mapD, kb * KB, k * a.s_pad + a.s0 + chunk * kMvM, bar);
-                        tma_load_2d_pair(dst + NS * G::kA + k * G::kB, &mapE, kb * KB, (tile * NS + k) * kMvP + rank * kMvHalf,
-                                         bar);
+                        tma_load_2d_pair(dst + NS * G::kA + k * G::kB, &mapE, kb * KB, (tile * NS + k) * kMvP + col, bar);
                     }
                 }
             }
@@ -633,10 +759,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
             uint32_t it = 0, n = 0;
             const uint64_t ring_desc = KB == 64 ? sw128_desc(ring) : sw64_desc(ring);
             for (long long item = cluster; item < n_items && !failed; item += n_clusters, ++n) {
-                const int nk = blocks_of((int)(item / n_pairs));
+                const int nk = blocks_of((int)(item / n_pairs) / kSub);
                 const int buf = n % Sh::NB;
                 if (n >= Sh::NB) wait_on(&acc_empty[buf], (n / Sh::NB - 1) & 1);
-                const uint32_t d = tmem + buf * (Sh::NA * kMvP);
+                const uint32_t d = tmem + buf * (Sh::NA * N);
                 for (int kb = 0; kb < nk && !failed; ++kb, ++it) {
                     const int st = it % Sh::ST;
                     wait_on(&full[st], (it / Sh::ST) & 1);
@@ -657,15 +783,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
         __syncwarp();
     } else {
         // ---- the epilogue: lanes = scenarios 32 (warp % 4) .., columns kCols (warp / 4) ..
-        constexpr int kCols = kMvP / (kMvEpi / 4);
+        constexpr int kCols = N / kMvParts;
         const int quarter = warp & 3, part = warp >> 2;
         uint32_t n = 0;
         uint32_t acc_free[Sh::NB];
         for (int i = 0; i < Sh::NB; ++i) acc_free[i] = of_rank0(&acc_empty[i]);
         for (long long item = cluster; item < n_items; item += n_clusters, ++n) {
-            const int tile = (int)(item / n_pairs), chunk = 2 * (int)(item - (long long)tile * n_pairs) + rank;
-            const int buf = n % Sh::NB;
-            if (tid < kMvP * 2) reinterpret_cast<float4*>(recs)[tid] = reinterpret_cast<const float4*>(a.out + (size_t)tile * kMvP)[tid];
+            const int sub = (int)(item / n_pairs), chunk = 2 * (int)(item - (long long)sub * n_pairs) + rank;
+            const int tile = sub / kSub, buf = n % Sh::NB;
+            if (tid < N * 2) reinterpret_cast<float4*>(recs)[tid] = reinterpret_cast<const float4*>(a.out + (size_t)sub * N)[tid];
             asm volatile("bar.sync 1, %0;" ::"n"(32 * kMvEpi) : "memory");
             bool ok = true;
             if (lane == 0 && !failed) ok = mbar_wait_bounded(&acc_full[buf], (n / Sh::NB) & 1, kMvPoll);
@@ -679,31 +805,66 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
             const bool inside = chunk < a.n_chunks, live = s < a.n_scen && !failed;   // an odd last pair's second tile is empty
             const int sl = inside ? s : 0;
             const float dsc = pow2f(a.colexp[sl] - (NS == 3 ? 30 : 0));
-            const uint32_t col0 = tmem + ((uint32_t)(quarter * 32) << 16) + buf * (Sh::NA * kMvP) + part * kCols;
+            const uint32_t col0 = tmem + ((uint32_t)(quarter * 32) << 16) + buf * (Sh::NA * N) + part * kCols;
             df tot{0.0f, 0.0f};
+            double tot64 = 0.0;
             // the columns of this warp, 16 at a time and without branches over them (padding
             // rows are 0), so that their chains overlap; MAT: maturity payments
             auto columns = [&](auto with_maturity) {
                 constexpr bool MAT = decltype(with_maturity)::value;
 #pragma unroll 1
                 for (int c = 0; c < kCols; c += 16) {
-                    uint32_t r[Sh::NA][16];
-#pragma unroll
-                    for (int k = 0; k < Sh::NA; ++k) tmem_ld16_async(col0 + k * kMvP + c, r[k]);
-#pragma unroll
-                    for (int k = 0; k < Sh::NA; ++k) tmem_wait_ld(r[k]);
-                    if (c == kCols - 16) {   // the accumulators are read
+                    auto release = [&] {   // the accumulators are read
+                        if (c != kCols - 16) return;
                         fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive_remote(acc_free[buf]);
+                    };
+                    if constexpr (NS == 8) {   // added in FP64, the smallest first
+                        double u[16];
+#pragma unroll
+                        for (int k = Sh::NA - 1; k >= 0; --k) {
+                            uint32_t r[16];
+                            tmem_ld16_async(col0 + k * N + c, r);
+                            tmem_wait_ld(r);
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) {
+                                const double x = (double)__uint_as_float(r[i]);
+                                u[i] = k == Sh::NA - 1 ? x : __dadd_rn(u[i], x);
+                            }
+                        }
+                        release();
+                        const double scale = __hiloint2double((a.colexp[sl] + 1023) << 20, 0);
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) {
+                            const MvOut64& q = reinterpret_cast<const MvOut64&>(recs[part * kCols + c + i]);
+                            double v = __dmul_rn(__dmul_rn(u[i], scale), q.sc);
+                            if constexpr (MAT) {
+                                const double d = q.S > 0 ? a.D64[(size_t)(q.S - 1) * a.s_pad + sl] : 1.0;
+                                v = __fma_rn(q.mat, d, v);
+                            }
+                            tot64 = __dadd_rn(tot64, v);
+                            if (live && q.pol >= 0) {
+                                const size_t o = (size_t)q.pol * a.v0_ld + s;
+                                if (a.V0f) a.V0f[o] = __double2float_rn(v);
+                                if (a.V0d) a.V0d[o] = v;
+                            }
+                        }
+                        continue;
                     }
+                    uint32_t r[NS == 8 ? 1 : Sh::NA][16];
+#pragma unroll
+                    for (int k = 0; k < (NS == 8 ? 0 : Sh::NA); ++k) tmem_ld16_async(col0 + k * N + c, r[k]);
+#pragma unroll
+                    for (int k = 0; k < (NS == 8 ? 0 : Sh::NA); ++k) tmem_wait_ld(r[k]);
+                    release();
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
                         const MvOut& q = recs[part * kCols + c + i];
                         // the accumulators' sum as a double-float
                         float h = __uint_as_float(r[0][i]), l = 0.0f;
 #pragma unroll
-                        for (int k = 1; k < Sh::NA; ++k) {
+                        for (int k = 1; k < (NS == 8 ? 1 : Sh::NA); ++k) {
                             const float b = __uint_as_float(r[k][i]), sum = __fadd_rn(h, b), bb = __fsub_rn(sum, h);
                             l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(sum, bb)), __fsub_rn(b, bb)));
                             h = sum;
@@ -736,16 +897,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
             if (kind == K_ASS || kind == K_ASS2 || kind == K_LS2) columns(std::true_type{});
             else columns(std::false_type{});
             // the parts' sums in part order; then the records and sums may be overwritten
-            sums[part][quarter * 32 + lane] = make_float2(tot.h, tot.l);
+            if constexpr (NS == 8) reinterpret_cast<double&>(sums[part][quarter * 32 + lane]) = tot64;
+            else sums[part][quarter * 32 + lane] = make_float2(tot.h, tot.l);
             asm volatile("bar.sync 1, %0;" ::"n"(32 * kMvEpi) : "memory");
             if (part == 0 && a.partial && inside && !failed) {
                 double x = 0.0;
 #pragma unroll
                 for (int k = 0; k < kMvParts; ++k) {
                     const float2 v = sums[k][quarter * 32 + lane];
-                    x += (double)v.x + (double)v.y;
+                    if constexpr (NS == 8) x += reinterpret_cast<const double&>(v);
+                    else x += (double)v.x + (double)v.y;
                 }
-                a.partial[(size_t)tile * a.part_ld + s] = x;
+                a.partial[(size_t)sub * a.part_ld + s] = x;
             }
         }
     }
@@ -764,20 +927,22 @@ cudaError_t product(const MvArgs& a, const void* digitsD, const void* digitsE, i
     if (!encode_map_16bit(&mD, CU_TENSOR_MAP_DATA_TYPE_UINT16, digitsD, pitchD, (uint64_t)NS * a.s_pad, pitchD, Sh::KB, kMvM,
                           swz) ||
         !encode_map_16bit(&mE, CU_TENSOR_MAP_DATA_TYPE_UINT16, digitsE, pitchE, (uint64_t)NS * kMvP * a.n_tiles, pitchE, Sh::KB,
-                          kMvHalf, swz))
+                          Sh::N / 2, swz))
         return cudaErrorNotSupported;
     constexpr size_t smem = (size_t)Sh::ST * MvStage<NS>::kBytes + 1024;
     auto k = mv_product_kernel<NS>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const long long items = (long long)a.n_tiles * ((a.n_chunks + 1) / 2);
+    const long long items = (long long)a.n_tiles * (kMvP / Sh::N) * ((a.n_chunks + 1) / 2);
     k<<<2 * (int)std::min<long long>(items, sm_count / 2), kMvThreads, smem, st>>>(mD, mE, a);
     return cudaGetLastError();
 }
 
 }  // namespace
 
-const char* mv_variant_name(int form) { return form == F_DEFL ? "deflated matrix f16x3 bf16x4" : "comp matrix bf16x6"; }
+const char* mv_variant_name(int form) {
+    return form == F_DEFL ? "deflated matrix f16x3 bf16x4" : (form == F_COMP ? "comp matrix bf16x6" : "f64 matrix bf16x8");
+}
 
 cudaError_t launch_mv_scenarios(const double* v64, int n_steps, int n_scen, int s_pad, float2* D, const MvScen& c,
                                 cudaStream_t st) {
@@ -803,6 +968,23 @@ cudaError_t launch_mv_digits(int ns, const float2* D, const int32_t* tau, const 
     return cudaGetLastError();
 }
 
+cudaError_t launch_mv_products64(const double* v64, int n_steps, int s_pad, double* D, cudaStream_t st) {
+    mv_products_kernel<<<s_pad / kProdS, dim3(kProdS, 32), 0, st>>>(v64, n_steps, s_pad, D);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mv_digits64(const double* D, const int32_t* tau, const int32_t* colexp, int n_steps, int n_scen, int s_pad,
+                               int pitch, void* digits, cudaStream_t st) {
+    mv_digits64_kernel<<<dim3(s_pad / 32, pitch / 64), 256, 0, st>>>(D, tau, colexp, n_steps, n_scen, s_pad, pitch,
+                                                                    static_cast<uint32_t*>(digits));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mv_build64(const MvBuild& b, const CfPol* pols, cudaStream_t st) {
+    mv_build64_kernel<<<b.n_tiles * (kMvP / 8), 256, (size_t)b.pitch * sizeof(float), st>>>(b, pols);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_mv_build(int ns, const MvBuild& b, cudaStream_t st) {
     const int grid = b.n_tiles * (kMvP / (8 * b.rows_per_warp));
     const size_t smem = (size_t)b.pitch * sizeof(float);
@@ -823,7 +1005,8 @@ cudaError_t launch_mv_product(int ns, const MvArgs& a, const void* digitsD, cons
     if (a.n_tiles <= 0 || a.n_chunks <= 0) return cudaSuccess;
     if (ns == 3) return product<3>(a, digitsD, digitsE, pitchD, pitchE, sm_count, st);
     if (ns == 4) return product<4>(a, digitsD, digitsE, pitchD, pitchE, sm_count, st);
-    return product<6>(a, digitsD, digitsE, pitchD, pitchE, sm_count, st);
+    if (ns == 6) return product<6>(a, digitsD, digitsE, pitchD, pitchE, sm_count, st);
+    return product<8>(a, digitsD, digitsE, pitchD, pitchE, sm_count, st);
 }
 
 }  // namespace rsv

@@ -12,14 +12,16 @@
 //   of the row's largest entry; stored times 2^15.
 //   Four and six: d2 and d3 the next 8 bits each (signed), the others BF16 values of the
 //   remainders, to 2^-33 and 2^-48.
+//   Eight (the FP64 form): seven more of 8 bits each (signed), to 2^-63.
 //
 // The products of digits i and j, i + j at most the last digit's number, are taken.  d1 d1'
 // products are multiples of 2^-14, so up to 1,000 of them add up exactly in FP32 (rows with
 // more steps give up one or two bits).  With four and six digits d1 d2', and d1 d3' and
 // d2 d2', 2^-8 and 2^-16 below, are multiples of 2^-22 and 2^-30 and have an exact
 // accumulator each; the rest shares one more, whose FP32 truncations (of a sum 2^-24,
-// with three digits 2^-8, below) are that much smaller.  The epilogue adds the
-// accumulators as double-floats.  A maturity payment is added there, from the discount
+// with three digits 2^-8, below) are that much smaller.  With eight every level has its
+// own.  The epilogue adds the accumulators as double-floats (FP64 form: in
+// FP64).  A maturity payment is added there, from the discount
 // products themselves, so that a row holds entries of one kind.
 //
 // Fixed point needs rows and columns of moderate range.  The discount products are
@@ -60,10 +62,15 @@ constexpr double kMvAmountMin = 0x1p-60, kMvAmountMax = 0x1p90;   // |amount|: V
 //     within the form's bound of 15 x 2^-24; at larger spreads the truncations of the low
 //     accumulator also grow past it (2e-6 measured at 7);
 //   four (deflated, to 8): below 2^-30 left out, 2^(spread - 28);
-//   six (compensated, to 10): about 2^-46 left out, 2^(spread - 44).
-inline int mv_max_spread(int form) { return form == F_DEFL ? 8 : 10; }
-inline int mv_digits_of(int form, int spread) { return form == F_DEFL ? (spread <= 4 ? 3 : 4) : 6; }
-inline int mv_digit_set(int ns) { return ns == 3 ? 0 : (ns == 4 ? 1 : 2); }   // index of a digit count
+//   six (compensated, to 10): about 2^-46 left out, 2^(spread - 44);
+//   eight (FP64, to 8): about 2^-61, 2^(spread - 59).
+inline int mv_max_spread(int form) { return form == F_COMP ? 10 : 8; }
+inline int mv_digits_of(int form, int spread) {
+    return form == F_F64 ? 8 : (form == F_COMP ? 6 : (spread <= 4 ? 3 : 4));
+}
+inline int mv_digit_set(int ns) { return ns == 8 ? 3 : (ns == 6 ? 2 : ns - 3); }   // index of a digit count
+// rows of scenario sums that the product writes: one a tile, FP64 one a half tile
+inline int mv_part_rows(int form, int n_tiles) { return form == F_F64 ? 2 * n_tiles : n_tiles; }
 inline int mv_pitch(int steps) { return steps < 1 ? 64 : (steps + 63) / 64 * 64; }
 
 // Scenario side, from the FP64 plane [n_steps][s_pad]: the discount products, and
@@ -128,19 +135,27 @@ constexpr int kMvRecWords = sizeof(SlotRec) / 4;
 cudaError_t launch_mv_build_lives(const CfTables& T, const MvLives* recs, const double* amount, int n_tiles, int pitch,
                                   int n_steps, const float* tilt, void* digits, MvOut* out, cudaStream_t st);
 
+// The FP64 form's: FP64 discount products, their eight digits, and the rows of the records that
+// launch_cf_records makes of the panel's slots.
+cudaError_t launch_mv_products64(const double* v64, int n_steps, int s_pad, double* D, cudaStream_t st);
+cudaError_t launch_mv_digits64(const double* D, const int32_t* tau, const int32_t* colexp, int n_steps, int n_scen, int s_pad,
+                               int pitch, void* digits, cudaStream_t st);
+cudaError_t launch_mv_build64(const MvBuild& b, const CfPol* pols, cudaStream_t st);
+
 struct MvArgs {
     const int32_t* steps;      // the steps of the panel's first record; one record is kMvRecWords
     const int32_t* kinds;      // of the tiles, or null: no maturity payments
     const MvOut* out;
     const int32_t* colexp;     // of the first column
     const float2* D;           // the discount products [n_steps][s_pad], at the first column
+    const double* D64;         // the same in FP64 (eight digits)
     const double* amount;
     int32_t n_tiles, n_chunks; // policy tiles of the panel, scenario tiles of the column block
     int32_t s_pad, n_scen, s0; // plane rows; valid columns of the block; the block's first column
     int32_t v0_ld, part_ld;
     float* V0f;                // at the block's first column
     double* V0d;
-    double* partial;           // [n_tiles][part_ld], at the panel's first tile and the block's first column
+    double* partial;           // [mv_part_rows][part_ld], at the panel's first tile and the block's first column
     int32_t* status;
 };
 // digitsE: launch_mv_build's, digitsD: launch_mv_digits', both of ns digits.

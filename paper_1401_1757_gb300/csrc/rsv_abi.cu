@@ -628,8 +628,15 @@ rsv_status rsv::mv_scenario_digits(rsv_ctx* c, int form) {
     if (c->mv_dig_gen[k] == c->scen_gen) return RSV_OK;   // with the scenario set, like its planes
     CU(c->d_mv_dig[k].ensure((size_t)ns * c->s_pad * pitch * 2));
     const MvScen mv = MvScen::at(c->d_mv_col.p, c->n_steps, c->s_pad);
-    CU(launch_mv_digits(ns, c->d_mv_D.as<float2>(), mv.tau, mv.colexp, c->n_steps, c->n_scen, c->s_pad, pitch,
-                        c->d_mv_dig[k].p, c->stream));
+    if (ns == 8) {
+        CU(c->d_mv_D64.ensure((size_t)c->n_steps * c->s_pad * sizeof(double)));
+        CU(launch_mv_products64(c->d_v64.as<double>(), c->n_steps, c->s_pad, c->d_mv_D64.as<double>(), c->stream));
+        CU(launch_mv_digits64(c->d_mv_D64.as<double>(), mv.tau, mv.colexp, c->n_steps, c->n_scen, c->s_pad, pitch,
+                              c->d_mv_dig[k].p, c->stream));
+    } else {
+        CU(launch_mv_digits(ns, c->d_mv_D.as<float2>(), mv.tau, mv.colexp, c->n_steps, c->n_scen, c->s_pad, pitch,
+                            c->d_mv_dig[k].p, c->stream));
+    }
     c->mv_dig_gen[k] = c->scen_gen;
     return RSV_OK;
 }
@@ -649,6 +656,7 @@ rsv_status rsv::mv_multiply(rsv_ctx* c, int form, MvArgs a, int max_S, int s0, i
     a.out = c->d_mv_out.as<MvOut>();
     a.colexp = MvScen::at(c->d_mv_col.p, c->n_steps, c->s_pad).colexp + s0;
     a.D = c->d_mv_D.as<float2>() + s0;
+    a.D64 = c->d_mv_D64.p ? c->d_mv_D64.as<double>() + s0 : nullptr;
     a.n_chunks = (w + kMvM - 1) / kMvM;
     a.s_pad = c->s_pad;
     a.n_scen = w;
@@ -702,7 +710,14 @@ rsv_status rsv::mv_launch(rsv_ctx* c, int form, int s0, int w, float* V0f, doubl
             b.tilt_top = mv.tilt_top;
             b.digits = c->d_mv_E.p;
             b.out = c->d_mv_out.as<MvOut>();
-            CU(launch_mv_build(mv_digits_of(form, c->mv_spread), b, c->stream));
+            if (form == F_F64) {
+                CU(c->d_cf_pol.ensure((size_t)panel * kMvP * sizeof(CfPol)));
+                CU(launch_cf_records(T, slots, b.kinds, b.amount, n * kMvP, kMvP, L.tab_pad, c->d_cf_pol.as<CfPol>(),
+                                     c->stream));
+                CU(launch_mv_build64(b, c->d_cf_pol.as<CfPol>(), c->stream));
+            } else {
+                CU(launch_mv_build(mv_digits_of(form, c->mv_spread), b, c->stream));
+            }
             c->mv_built = t0;
         }
         MvArgs a{};
@@ -712,7 +727,7 @@ rsv_status rsv::mv_launch(rsv_ctx* c, int form, int s0, int w, float* V0f, doubl
         a.n_tiles = n;
         a.V0f = V0f;
         a.V0d = V0d;
-        a.partial = partial ? partial + (size_t)t0 * c->s_pad : nullptr;
+        a.partial = partial ? partial + (size_t)mv_part_rows(form, t0) * c->s_pad : nullptr;
         if ((st = mv_multiply(c, form, a, L.max_S, s0, w)) != RSV_OK) return st;
     }
     return RSV_OK;
@@ -770,8 +785,8 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     // keep the fast kernel (tile group 0) and the others take the
     // general-cash-flow kernel (group 1).
     const bool split = cfl && pay == PAY_END && !extra && !scan && !summ;
-    // The matrix product (the last tunable variant of the compensated form) where it
-    // covers the data, unless another variant was tuned or asked for.
+    // The matrix product (the last tunable variant of the compensated and FP64 forms) where
+    // it covers the data, unless another variant was tuned or asked for.
     bool mat = false;
     int vi, vg = -1;
     if (extra || scan || summ) {
@@ -782,12 +797,12 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
         if (o->variant >= rsv_variant_count(o->form)) return fail(c, RSV_E_ARG, "variant %d out of range", o->variant);
         vi = o->variant;
     } else if (o->variant == -1) {
-        vi = c->tuned[o->form] >= 0 ? c->tuned[o->form] : (o->form == F_COMP ? nt : 0);
+        vi = c->tuned[o->form] >= 0 ? c->tuned[o->form] : (o->form == F_F32 ? 0 : nt);
     } else {
         return fail(c, RSV_E_ARG, "variant %d out of range", o->variant);
     }
-    if (o->form == F_COMP && vi == nt && !extra && pay == PAY_END) {
-        mat = mv_applies(c, F_COMP, c->amt_lo, c->amt_hi);
+    if (o->form != F_F32 && vi == nt && !extra && !scan && !summ && pay == PAY_END) {
+        mat = mv_applies(c, o->form, c->amt_lo, c->amt_hi);
         vi = 0;
     }
     if (split) vg = special_variant(vl, nv, false, PAY_END_GENERAL);
@@ -832,7 +847,8 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     CU(cudaMemsetAsync(c->d_ctl.p, 0, 2 * sizeof(int32_t), c->stream));
     if (pt) CU(cudaMemsetAsync(pt, 0, n_pt * sizeof(double), c->stream));
     if (traj) CU(cudaMemsetAsync(traj, 0, n_traj * sizeof(double), c->stream));
-    if (tot) CU(c->d_partial.ensure((size_t)std::max(1, L.n_tiles) * c->s_pad * sizeof(double)));
+    const int part_rows = mat ? mv_part_rows(o->form, L.n_tiles) : L.n_tiles;   // rows of scenario sums
+    if (tot) CU(c->d_partial.ensure((size_t)std::max(1, part_rows) * c->s_pad * sizeof(double)));
     if (tot && L.n_tiles == 0) CU(cudaMemsetAsync(tot, 0, NSc * sizeof(double), c->stream));
 
     RecurArgs a{};
@@ -947,7 +963,7 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
         c->ev_recorded = true;
     }
     if (L.n_tiles > 0) {
-        if (tot && (st = scenario_totals(c, a.partial, L.n_tiles, c->s_pad, NSc, tot)) != RSV_OK) return st;
+        if (tot && (st = scenario_totals(c, a.partial, part_rows, c->s_pad, NSc, tot)) != RSV_OK) return st;
         if (pt) {
             scale_kernel<<<c->sm_count * 4, 256, 0, c->stream>>>(pt, n_pt, 1.0 / NSc);
             CU(cudaGetLastError());
@@ -1052,7 +1068,7 @@ rsv_status compute_nested(rsv_ctx* c, const rsv_opts* o, const rsv_nested_spec* 
         double* due = flow + (T_max + 1);
         double* scale = due + (T_max + 1);
         CfPol* recs = c->d_cf_pol.as<CfPol>();
-        CU(launch_cf_records(T, L.slots.as<SlotRec>(), L.kinds.as<int32_t>(), c->d_amount.as<double>(), L.n_tiles, L.tab_pad,
+        CU(launch_cf_records(T, L.slots.as<SlotRec>(), L.kinds.as<int32_t>(), c->d_amount.as<double>(), L.n_tiles, 1, L.tab_pad,
                              recs, c->stream));
         CU(launch_cf_portfolio(T, recs, L.n_tiles, T_max, part, flow, due, reinterpret_cast<float2*>(flow2), scale, c->stream));
         const NestedRun run{sp->seed, sp->a, sp->b, sp->sigma, sp->r0, sp->outer_first, NO, NN, step, n_inner, T_max,
@@ -1242,7 +1258,7 @@ rsv_status rsv_destroy(rsv_ctx* c) try {
                       &c->sur.d_comm, &c->sur.d_lnb, &c->d_tabf[0], &c->d_tabf[1], &c->d_tabf[2], &c->d_vf64,
                       &c->d_vf32, &c->d_vf2, &c->d_cf64, &c->d_cf32, &c->d_ml_rec,
                       &c->d_ml_amount, &c->sur.d_cnt, &c->sur.d_q2, &c->sur.d_idx, &c->sur.d_v2, &c->d_nest_bm,
-                      &c->d_mv_D, &c->d_mv_col, &c->d_mv_dig[0], &c->d_mv_dig[1], &c->d_mv_dig[2], &c->d_mv_E, &c->d_mv_out,
+                      &c->d_mv_D, &c->d_mv_col, &c->d_mv_dig[0], &c->d_mv_dig[1], &c->d_mv_dig[2], &c->d_mv_dig[3], &c->d_mv_D64, &c->d_mv_E, &c->d_mv_out,
                       &c->d_defl_slots, &c->d_defl_kinds, &c->d_defl_tab, &c->d_defl_plane, &c->d_mlp_trace})
         b->release();
     c->mlp.release();
@@ -1497,17 +1513,17 @@ int32_t rsv_variant_count(int32_t form) {
     int n = 0;
     if (form == F_DEFL) return variants_defl(&n) ? n + 1 : 0;   // and the matrix product, the last
     const Variant* vl = variant_list(form, &n);
-    return vl ? tunable_count(vl, n) + (form == F_COMP ? 1 : 0) : 0;
+    return vl ? tunable_count(vl, n) + (form == F_F32 ? 0 : 1) : 0;
 }
 
 const char* rsv_variant_name(int32_t form, int32_t variant) {
     int n = 0;
     const int count = rsv_variant_count(form);
     if (variant < 0) return "";
-    if ((form == F_DEFL || form == F_COMP) && variant == count - 1) return mv_variant_name(form);
+    if (count > 0 && form != F_F32 && variant == count - 1) return mv_variant_name(form);
     if (form == F_DEFL) return variant < count ? variants_defl(&n)[variant].name : "";
     const Variant* v = variant_list(form, &n);   // the side-output and payment variants after the tunable ones
-    const int k = form == F_COMP && variant >= count ? variant - 1 : variant;
+    const int k = form != F_F32 && variant >= count ? variant - 1 : variant;
     return v && k < n ? v[k].name : "";
 }
 

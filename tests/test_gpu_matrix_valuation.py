@@ -5,7 +5,8 @@ projections, varying cash flows, and the data that keeps the recurrence kernels.
 Tolerances.  Compensated: operands to 2^-48 of a row's largest entry, discount products
 within 2^11 of a column's largest, so 2^-34 an entry at the worst place, and FP32 truncations of an
 accumulator 2^-24 below the result, at most 15 a block of 16 steps: 4,096 steps stay below
-2^-33; 5e-10 covers both.  Deflated: its stated bound 15 x 2^-24.
+2^-33; 5e-10 covers both.  Deflated: its stated bound 15 x 2^-24.  FP64: the form's 1e-12 (the
+same estimate with 2^-63, 2^-32 and 36 gives 2^-48).
 Error metric: rel = |V_gpu - V_ref| / max(|V_ref|, 1e-9 * amount)."""
 import numpy as np
 import pytest
@@ -16,8 +17,8 @@ import synth
 from paper_1401_1757_gb300 import rsv
 
 pytestmark = pytest.mark.gpu
-COMP, DEFL = rsv.RSV_FORM_F32_COMP, rsv.RSV_FORM_F32_DEFLATED
-TOL = {COMP: 5e-10, DEFL: 15 * 2.0 ** -24}
+COMP, DEFL, F64 = rsv.RSV_FORM_F32_COMP, rsv.RSV_FORM_F32_DEFLATED, rsv.RSV_FORM_F64
+TOL = {COMP: 5e-10, DEFL: 15 * 2.0 ** -24, F64: 1e-12}
 V0T = rsv.RSV_OUT_V0 | rsv.RSV_OUT_SCEN_TOTAL
 
 
@@ -55,7 +56,7 @@ def every_product(n, seed, form, **ages):
     return pol
 
 
-@pytest.mark.parametrize("form", [COMP, DEFL])
+@pytest.mark.parametrize("form", [COMP, DEFL, F64])
 @pytest.mark.parametrize("n_pol,n_scen", [(1, 1), (2, 31), (63, 33), (64, 127), (65, 128), (129, 129), (257, 300)])
 def test_tile_edges(ctx, form, n_pol, n_scen):
     tabs = [synth.gm_monthly_survival(), synth.gm_monthly_survival(A=0.0003, B=0.00002)]
@@ -68,7 +69,7 @@ def test_tile_edges(ctx, form, n_pol, n_scen):
     check(form, pol, *value(ctx, form, pol, tabs, v), ref, ref_tot)
 
 
-@pytest.mark.parametrize("form", [COMP, DEFL])
+@pytest.mark.parametrize("form", [COMP, DEFL, F64])
 @pytest.mark.parametrize("horizon", [1, 31, 32, 33, 64, 65, 0])
 def test_projection_lengths(ctx, form, horizon):
     """Around the 32-step blocks; without a horizon also policies at maturity and lives at
@@ -87,7 +88,7 @@ def test_projection_lengths(ctx, form, horizon):
         assert np.all(V[0] == pol["amount"][0])
 
 
-@pytest.mark.parametrize("form", [COMP, DEFL])
+@pytest.mark.parametrize("form", [COMP, DEFL, F64])
 @pytest.mark.parametrize("steps", [1000, 1001, 2001, 4001])
 def test_long_level_projections(ctx, form, steps):
     """No mortality and no interest to speak of: every entry near the row's largest, the sums
@@ -100,7 +101,7 @@ def test_long_level_projections(ctx, form, steps):
     check(form, pol, *value(ctx, form, pol, [tab], v), ref, ref_tot)
 
 
-@pytest.mark.parametrize("form", [COMP, DEFL])
+@pytest.mark.parametrize("form", [COMP, DEFL, F64])
 @pytest.mark.parametrize("bits", [3, 4, 5, 7, 8, 9, 10])
 def test_scenarios_far_from_their_mean(ctx, form, bits):
     """Flat rates whose discount products end 2^bits apart from their mean's, single payments
@@ -116,7 +117,8 @@ def test_scenarios_far_from_their_mean(ctx, form, bits):
     check(form, pol, *value(ctx, form, pol, [tab], v), ref, ref_tot)
 
 
-def test_varying_cash_flows(ctx):
+@pytest.mark.parametrize("form", [COMP, F64])
+def test_varying_cash_flows(ctx, form):
     """Rows that are level and rows that are not, deferred and annual payments."""
     tab = synth.gm_monthly_survival()
     pol = every_product(90, 8, COMP)
@@ -129,12 +131,12 @@ def test_varying_cash_flows(ctx):
     rsv.rsv_load_decrements(ctx, 0, tab)
     rsv.rsv_load_portfolio(ctx, pol)
     rsv.rsv_load_cashflows(ctx, cf)
-    V, tot = value(ctx, COMP, pol, [tab], v)
+    V, tot = value(ctx, form, pol, [tab], v)
     ref, ref_tot = oracle.reserves_batch(pol, tab, v, cf=cf)
-    check(COMP, pol, V, tot, ref, ref_tot)
+    check(form, pol, V, tot, ref, ref_tot)
 
 
-@pytest.mark.parametrize("form", [COMP, DEFL])
+@pytest.mark.parametrize("form", [COMP, DEFL, F64])
 @pytest.mark.parametrize("what", ["spread", "discount", "large", "small", "table"])
 def test_data_out_of_range_keeps_the_recurrence(ctx, form, what):
     tab, v = synth.gm_monthly_survival(), synth.vasicek_paths(33, 1200, seed=1)
