@@ -94,14 +94,15 @@ enum {
                               see below                                               */
 };
 
-/* The compensated and the deflated form run rsv_compute_reserves (V0 and totals,
- * payment at the end of the step, any cash-flow sequence that the form takes) as a
+/* The FP64, the compensated and the deflated form run rsv_compute_reserves (V0 and
+ * totals, payment at the end of the step, any cash-flow sequence that the form takes) as a
  * matrix product of the policies' expected cash flows and the scenarios' discount
- * products on the tensor cores, both split into exact 16-bit digits (compensated: 48
- * bits, error about 1e-12; deflated: 32 bits, within the bound below).  Data outside its
- * range keeps the recurrence kernels: scenarios whose discount products leave their
- * mean by more than a factor of about 2^10 (deflated 2^8), survival below 2^-100, amounts outside
- * 2^-60 .. 2^90.  It is the last of a form's tunable variants. */
+ * products on the tensor cores, both split into exact 16-bit digits (FP64: 63 bits;
+ * compensated: 48 bits, error about 1e-13; deflated: 32 bits, within the bound below).  Data
+ * outside its range keeps the recurrence kernels: scenarios whose discount products
+ * leave their mean by more than a factor of about 2^10 (FP64 and deflated 2^8), survival
+ * below 2^-100, amounts outside 2^-60 .. 2^90.  It is the last of a form's tunable
+ * variants. */
 
 /* RSV_FORM_F32_DEFLATED.  Eq. (generalForm) multiplied at step t by the
  * deflator G_t = D_t l_{x+t} / l_x (D_t = v_0 ... v_{t-1}, the discount-factor

@@ -306,7 +306,8 @@ rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     }
     CU(c->d_ctl.ensure(2 * sizeof(int32_t)));
     CU(cudaMemsetAsync(c->d_ctl.p, 0, 2 * sizeof(int32_t), c->stream));
-    if (tot) CU(c->d_partial.ensure((size_t)std::max(1, L.n_tiles) * s_pad * sizeof(double)));
+    const int part_rows = mat ? mv_part_rows(mv_digits_of(F_DEFL, c->mv_spread), L.n_tiles) : L.n_tiles;   // of scenario sums
+    if (tot) CU(c->d_partial.ensure((size_t)std::max(1, part_rows) * s_pad * sizeof(double)));
     if (tot && L.n_tiles == 0) CU(cudaMemsetAsync(tot, 0, NSc * sizeof(double), c->stream));
 
     // the deflator plane, rows of four steps, a whole number of staged blocks
@@ -389,7 +390,7 @@ rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
         CU(cudaEventRecord(c->ev1, c->stream));
     }
     c->ev_recorded = true;
-    if (tot && L.n_tiles > 0 && (st = scenario_totals(c, a.partial, L.n_tiles, s_pad, NSc, tot)) != RSV_OK) return st;
+    if (tot && L.n_tiles > 0 && (st = scenario_totals(c, a.partial, part_rows, s_pad, NSc, tot)) != RSV_OK) return st;
     if (!o->on_device) {
         if (hV0f && !copied_v0) CU(cudaMemcpyAsync(hV0f, V0f, n_v0 * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
         if (hV0d && !copied_v0) CU(cudaMemcpyAsync(hV0d, V0d, n_v0 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));

@@ -626,20 +626,25 @@ __global__ void __launch_bounds__(256) mv_build_kernel(const MvBuild b) {
 }
 
 // -------------------------------------------------------------- the product ----
-// Persistent pairs of CTAs over (policy tile, pair of scenario tiles) items.  A block of
-// steps of the digits is staged by TMA into a ring of stages: each CTA its 128 scenarios'
-// (A) and half of the tile's 128 policies' (B); one thread of rank 0 issues the digits'
-// products, m256 n128 k16 over both CTAs (cta_group::2).  In each CTA the scenarios are
+// Persistent pairs of CTAs over (policy tile or half tile, pair of scenario tiles) items.  A
+// block of steps of the digits is staged by TMA into a ring of stages: each CTA its 128
+// scenarios' (A) and half of the item's policies' (B); one thread of rank 0 issues the
+// digits' products, m256 k16 over both CTAs (cta_group::2).  In each CTA the scenarios are
 // on the lanes and the policies on the columns; sixteen warps add the accumulators as
 // double-floats, scale, write V0 (32 consecutive scenarios of a policy a warp store) and
-// sum each scenario over the tile's policies.
+// sum each scenario over the item's policies.
 // Three digits: 6 products and 2 accumulators, so TMEM holds two tiles' and the epilogue
-// runs beside the next tile's products; four and six: 10 and 21 products, 4 accumulators.  Eight (FP64): 36 products, an
-// accumulator for each level of half a tile's policies, added in FP64.
+// runs beside the next tile's products.  Four: 10 products, 4 accumulators (half tiles, two in
+// TMEM: 0.89 -> 0.95 ms for 100,000 policies x 1,000 scenarios).  Six and eight: 21 and 36
+// products, an accumulator for each level of half a tile's policies.  Such a product (n64)
+// lasts as long as the shared-memory reads of its A, so A is read once a scenario digit
+// and kept in the collector: 903 -> 755 us a launch of 50,000 x 1,000 with six.  Whole
+// tiles with the levels 3 to 5 in one accumulator took 690 us, at 13 times the error (totals of
+// annuities 1.8e-13 against the recurrence's 9e-14).
 template <int NS>
 struct MvShape;   // policies of an item, accumulators, items in TMEM, stages, steps of a block (64:
-template <>       // 128-byte swizzled rows); the products are (i, j), i + j < NS, of scenario digit i and policy
-struct MvShape<3> {   // digit j, in accumulator min(i + j, NA - 1)
+template <>       // 128-byte swizzled rows); the products are (i, j), i + j < NS, of scenario digit i
+struct MvShape<3> {   // and policy digit j, in accumulator min(i + j, NA - 1)
     static constexpr int N = kMvP, NA = 2, NB = 2, ST = 3, KB = 64;
 };
 template <>
@@ -648,7 +653,7 @@ struct MvShape<4> {
 };
 template <>
 struct MvShape<6> {
-    static constexpr int N = kMvP, NA = 4, NB = 1, ST = 3, KB = 32;
+    static constexpr int N = kMvP / 2, NA = 6, NB = 1, ST = 3, KB = 32;
 };
 template <>
 struct MvShape<8> {
@@ -660,7 +665,8 @@ constexpr int kMvThreads = 32 * (kMvEpi + 2);
 // shared memory of a stage: NS slabs of scenario digits, then NS of policy digits
 template <int NS>
 struct MvStage {
-    static constexpr int kA = kMvM * MvShape<NS>::KB * 2, kB = MvShape<NS>::N / 2 * MvShape<NS>::KB * 2;
+    using Sh = MvShape<NS>;
+    static constexpr int kA = kMvM * Sh::KB * 2, kB = Sh::N / 2 * Sh::KB * 2;
     static constexpr int kBytes = NS * (kA + kB);
 };
 
@@ -668,10 +674,13 @@ struct MvStage {
 // accumulators hold earlier blocks' sums.
 template <int NS, int I, int J>
 __device__ __forceinline__ void mv_products(uint32_t d, uint64_t base, int off, uint32_t idesc, bool more) {
+    using Sh = MvShape<NS>;
     using G = MvStage<NS>;
-    constexpr int acc = I + J < MvShape<NS>::NA ? I + J : MvShape<NS>::NA - 1;
+    constexpr int acc = I + J < Sh::NA ? I + J : Sh::NA - 1;
     constexpr bool first = I == 0 && J == acc;   // of its accumulator
-    mma_f16_ss_pair(d + acc * MvShape<NS>::N, base + (uint64_t)((I * G::kA + off) >> 4),
+    constexpr bool last = I + J + 1 == NS;
+    constexpr int coll = Sh::N == kMvP || (J == 0 && last) ? COLL_NONE : (J == 0 ? COLL_FILL : (last ? COLL_LAST : COLL_USE));
+    mma_f16_ss_pair<coll>(d + acc * Sh::N, base + (uint64_t)((I * G::kA + off) >> 4),
                     base + (uint64_t)((NS * G::kA + J * G::kB + off) >> 4), idesc, !first || more);
     if constexpr (I + J + 1 < NS) mv_products<NS, I, J + 1>(d, base, off, idesc, more);
     else if constexpr (I + 1 < NS) mv_products<NS, I + 1, 0>(d, base, off, idesc, more);
@@ -852,24 +861,32 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
                         }
                         continue;
                     }
-                    uint32_t r[NS == 8 ? 1 : Sh::NA][16];
+                    // the accumulators' sums as double-floats, the largest first
+                    float h[16], l[16];
+                    uint32_t r[2][16];
+                    tmem_ld16_async(col0 + c, r[0]);
 #pragma unroll
-                    for (int k = 0; k < (NS == 8 ? 0 : Sh::NA); ++k) tmem_ld16_async(col0 + k * N + c, r[k]);
+                    for (int k = 0; k < Sh::NA; ++k) {
+                        tmem_wait_ld(r[k & 1]);
+                        if (k + 1 < Sh::NA) tmem_ld16_async(col0 + (k + 1) * N + c, r[(k + 1) & 1]);
+                        else release();
 #pragma unroll
-                    for (int k = 0; k < (NS == 8 ? 0 : Sh::NA); ++k) tmem_wait_ld(r[k]);
-                    release();
+                        for (int i = 0; i < 16; ++i) {
+                            const float b = __uint_as_float(r[k & 1][i]);
+                            if (k == 0) {
+                                h[i] = b;
+                                l[i] = 0.0f;
+                            } else {
+                                const float sum = __fadd_rn(h[i], b), bb = __fsub_rn(sum, h[i]);
+                                l[i] = __fadd_rn(l[i], __fadd_rn(__fsub_rn(h[i], __fsub_rn(sum, bb)), __fsub_rn(b, bb)));
+                                h[i] = sum;
+                            }
+                        }
+                    }
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
                         const MvOut& q = recs[part * kCols + c + i];
-                        // the accumulators' sum as a double-float
-                        float h = __uint_as_float(r[0][i]), l = 0.0f;
-#pragma unroll
-                        for (int k = 1; k < (NS == 8 ? 1 : Sh::NA); ++k) {
-                            const float b = __uint_as_float(r[k][i]), sum = __fadd_rn(h, b), bb = __fsub_rn(sum, h);
-                            l = __fadd_rn(l, __fadd_rn(__fsub_rn(h, __fsub_rn(sum, bb)), __fsub_rn(b, bb)));
-                            h = sum;
-                        }
-                        df v = df_mul(df{__fmul_rn(h, dsc), __fmul_rn(l, dsc)}, df{q.sc_h, q.sc_l});
+                        df v = df_mul(df{__fmul_rn(h[i], dsc), __fmul_rn(l[i], dsc)}, df{q.sc_h, q.sc_l});
                         const int pol = q.pol;
                         bool due = false;
                         if constexpr (MAT) {   // a maturity payment, of the same sign, or 0

@@ -16,13 +16,12 @@
 //
 // The products of digits i and j, i + j at most the last digit's number, are taken.  d1 d1'
 // products are multiples of 2^-14, so up to 1,000 of them add up exactly in FP32 (rows with
-// more steps give up one or two bits).  With four and six digits d1 d2', and d1 d3' and
-// d2 d2', 2^-8 and 2^-16 below, are multiples of 2^-22 and 2^-30 and have an exact
-// accumulator each; the rest shares one more, whose FP32 truncations (of a sum 2^-24,
-// with three digits 2^-8, below) are that much smaller.  With eight every level has its
-// own.  The epilogue adds the accumulators as double-floats (FP64 form: in
-// FP64).  A maturity payment is added there, from the discount
-// products themselves, so that a row holds entries of one kind.
+// more steps give up one or two bits).  With four digits d1 d2', and d1 d3' and d2 d2', 2^-8
+// and 2^-16 below, are multiples of 2^-22 and 2^-30 and have an exact accumulator each; the
+// rest shares one more, whose FP32 truncations (of a sum 2^-24, with three digits 2^-8,
+// below) are that much smaller.  With six and eight every level has its own.  The epilogue
+// adds the accumulators as double-floats (FP64 form: in FP64).  A maturity payment is added
+// there, from the discount products themselves, so that a row holds entries of one kind.
 //
 // Fixed point needs rows and columns of moderate range.  The discount products are
 // tilted by a power of two per step, 2^tau(t) ~ 1 / (their geometric mean over the
@@ -31,13 +30,15 @@
 // entry.  A scenario set whose tilted products vary by too much along a scenario (see
 // mv_max_spread) keeps the recurrence kernels.
 //
-// Measured (one GB300, with the digits and the totals): the 100,000-policy mix under 1,000
-// scenarios, compensated 38.7 -> 1.56 ms (error 1e-8 -> 2e-11 at most; annuities alone
-// 1e-13 -> 2.4e-13 rms, assurances 4e-9 -> 2e-13), deflated 4.93 -> 0.62 ms (rms 3e-8 ->
-// 5e-9); 1,000,000 annuities, 600 steps, deflated 30.6 -> 4.3 ms.  It is the faster path
-// at every size measured: one policy and one scenario 53 -> 49 us compensated and
-// 158 -> 37 us deflated (host call included), 1,000 policies under 157 scenarios of the
-// mix 276 -> 102 us and 282 -> 63 us.
+// Measured (one GB300, with the digits and the totals), before: the recurrence.
+//   100,000 policies of every product, 1,000 scenarios: compensated 38.7 -> 1.70 ms
+//   (annuities 1e-13 -> 1.4e-14 rms, assurances 4e-9 -> 1.5e-14), deflated 4.93 -> 0.91 ms
+//   (rms 3e-8 -> 5e-9, with three digits 0.62 ms);
+//   1,000,000 annuities, 600 steps, 1,000 scenarios, deflated: 30.6 -> 4.3 ms;
+//   3,000 two-life policies, 333 scenarios, FP64: 5.17 -> 0.21 ms (1.4e-15 -> 1.3e-15).
+// It is the faster path at every size measured: one policy and one scenario 53 -> 49 us
+// compensated and 158 -> 37 us deflated (host call included), 1,000 policies under 157
+// scenarios of the mix 276 -> 102 us and 282 -> 63 us.
 #pragma once
 
 #include <cuda.h>
@@ -69,8 +70,8 @@ inline int mv_digits_of(int form, int spread) {
     return form == F_F64 ? 8 : (form == F_COMP ? 6 : (spread <= 4 ? 3 : 4));
 }
 inline int mv_digit_set(int ns) { return ns == 8 ? 3 : (ns == 6 ? 2 : ns - 3); }   // index of a digit count
-// rows of scenario sums that the product writes: one a tile, FP64 one a half tile
-inline int mv_part_rows(int form, int n_tiles) { return form == F_F64 ? 2 * n_tiles : n_tiles; }
+// rows of scenario sums that the product writes: one a tile, or one a half tile
+inline int mv_part_rows(int ns, int n_tiles) { return ns < 6 ? n_tiles : 2 * n_tiles; }
 inline int mv_pitch(int steps) { return steps < 1 ? 64 : (steps + 63) / 64 * 64; }
 
 // Scenario side, from the FP64 plane [n_steps][s_pad]: the discount products, and

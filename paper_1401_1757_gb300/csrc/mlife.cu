@@ -202,7 +202,8 @@ rsv_status mlife_matrix(rsv_ctx* c, const rsv_mlife_policy* pols, const std::vec
         if (V0d) { CU(c->d_o_v0d.ensure(n_v0 * sizeof(double))); V0d = c->d_o_v0d.as<double>(); }
         if (tot) { CU(c->d_o_tot.ensure(NSc * sizeof(double))); tot = c->d_o_tot.as<double>(); }
     }
-    if (tot) CU(c->d_partial.ensure((size_t)n_tiles * c->s_pad * sizeof(double)));
+    const int part_rows = mv_part_rows(6, n_tiles);
+    if (tot) CU(c->d_partial.ensure((size_t)part_rows * c->s_pad * sizeof(double)));
     CU(c->d_ml_rec.ensure(rows.size() * sizeof(MvLives)));
     CU(c->d_ml_amount.ensure(amount.size() * sizeof(double)));
     CU(c->d_ctl.ensure(2 * sizeof(int32_t)));
@@ -224,12 +225,12 @@ rsv_status mlife_matrix(rsv_ctx* c, const rsv_mlife_policy* pols, const std::vec
         a.amount = c->d_ml_amount.as<double>();
         a.V0f = V0f;
         a.V0d = V0d;
-        a.partial = tot ? c->d_partial.as<double>() + (size_t)t0 * c->s_pad : nullptr;
+        a.partial = tot ? c->d_partial.as<double>() + (size_t)mv_part_rows(6, t0) * c->s_pad : nullptr;
         if ((st = mv_multiply(c, F_COMP, a, max_S, 0, NSc)) != RSV_OK) return st;
     }
     CU(cudaEventRecord(c->ev1, c->stream));
     c->ev_recorded = true;
-    if (tot && (st = scenario_totals(c, c->d_partial.as<double>(), n_tiles, c->s_pad, NSc, tot)) != RSV_OK) return st;
+    if (tot && (st = scenario_totals(c, c->d_partial.as<double>(), part_rows, c->s_pad, NSc, tot)) != RSV_OK) return st;
     if (!o->on_device) {
         if (V0f) CU(cudaMemcpyAsync(out->V0, V0f, n_v0 * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
         if (V0d) CU(cudaMemcpyAsync(out->V0d, V0d, n_v0 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));

@@ -727,7 +727,7 @@ rsv_status rsv::mv_launch(rsv_ctx* c, int form, int s0, int w, float* V0f, doubl
         a.n_tiles = n;
         a.V0f = V0f;
         a.V0d = V0d;
-        a.partial = partial ? partial + (size_t)mv_part_rows(form, t0) * c->s_pad : nullptr;
+        a.partial = partial ? partial + (size_t)mv_part_rows(mv_digits_of(form, c->mv_spread), t0) * c->s_pad : nullptr;
         if ((st = mv_multiply(c, form, a, L.max_S, s0, w)) != RSV_OK) return st;
     }
     return RSV_OK;
@@ -847,7 +847,8 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     CU(cudaMemsetAsync(c->d_ctl.p, 0, 2 * sizeof(int32_t), c->stream));
     if (pt) CU(cudaMemsetAsync(pt, 0, n_pt * sizeof(double), c->stream));
     if (traj) CU(cudaMemsetAsync(traj, 0, n_traj * sizeof(double), c->stream));
-    const int part_rows = mat ? mv_part_rows(o->form, L.n_tiles) : L.n_tiles;   // rows of scenario sums
+    // rows of scenario sums
+    const int part_rows = mat ? mv_part_rows(mv_digits_of(o->form, c->mv_spread), L.n_tiles) : L.n_tiles;
     if (tot) CU(c->d_partial.ensure((size_t)std::max(1, part_rows) * c->s_pad * sizeof(double)));
     if (tot && L.n_tiles == 0) CU(cudaMemsetAsync(tot, 0, NSc * sizeof(double), c->stream));
 

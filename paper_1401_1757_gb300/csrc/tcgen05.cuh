@@ -130,12 +130,20 @@ __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* m
         "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
         : "memory");
 }
+// COLL: whether A stays in the collector buffer for the next products, or is taken from it
+enum { COLL_NONE, COLL_FILL, COLL_USE, COLL_LAST };
+template <int COLL = COLL_NONE>
 __device__ __forceinline__ void mma_f16_ss_pair(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(accum)
-        : "memory");
+#define RSV_MMA_PAIR(op)                                                   \
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"         \
+                 "tcgen05.mma.cta_group::2.kind::f16" op " [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem), \
+                 "l"(a), "l"(b), "r"(idesc), "r"(accum)                    \
+                 : "memory")
+    if constexpr (COLL == COLL_FILL) RSV_MMA_PAIR(".collector::a::fill");
+    else if constexpr (COLL == COLL_USE) RSV_MMA_PAIR(".collector::a::use");
+    else if constexpr (COLL == COLL_LAST) RSV_MMA_PAIR(".collector::a::lastuse");
+    else RSV_MMA_PAIR("");
+#undef RSV_MMA_PAIR
 }
 // arrives at the barrier's copies in both CTAs
 __device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
