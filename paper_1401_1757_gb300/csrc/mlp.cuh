@@ -30,14 +30,14 @@ struct Mlp {
     int cap = 0;                    // rows the activation buffers hold
     int step = 0;                   // Adam steps taken
     __nv_bfloat16* X = nullptr;     // batch features [cap][MLP_XW] (hi halves, then lo halves)
-    float* dW1 = nullptr;           // [MLP_XW][MLP_H] weight gradient of the tied first layer
     float* Z[4] = {};               // pre-activations
     __nv_bfloat16* A[4] = {};       // activations
-    float* A4f = nullptr;           // last hidden activations in FP32 (the head's input)
-    float* dZf[4] = {};
+    float* dZf[4] = {};             // written for traces only
     __nv_bfloat16* dZb[4] = {};
-    float *y = nullptr, *t = nullptr, *dy = nullptr, *sq = nullptr, *loss = nullptr;
-    float* part = nullptr;          // column-sum partials [cap / 128 + 1][MLP_H]
+    float *y = nullptr, *t = nullptr, *loss = nullptr;
+    float* wpart = nullptr;         // weight gradients of pieces of the batch
+    float* cpart = nullptr;         // dZ_1 .. dZ_3 summed over tiles of 64 rows [3][cap / 64 + 1][MLP_H]
+    float* hpart = nullptr;         // the head's sums over blocks of rows
     __nv_bfloat16* wt = nullptr;    // W_l^T (K-major) BF16 copies for the tcgen05 inference kernel
     bool wt_fresh = false;          // wt matches params (cleared whenever the BF16 weights are refreshed)
     bool use_tc = true;             // inference on tcgen05 (else the mma.sync kernels)
@@ -50,8 +50,8 @@ struct Mlp {
     void release();
     __nv_bfloat16* wb(int l) const;
     cudaError_t refresh_bf16(cudaStream_t st);
-    cudaError_t forward(const __nv_bfloat16* X, int B, float* y, const float* target, cudaStream_t st);
-    cudaError_t backward(const __nv_bfloat16* X, int B, cudaStream_t st);
+    cudaError_t forward(const __nv_bfloat16* X, int B, float* y, const float* target, cudaStream_t st, bool trace = false);
+    cudaError_t backward(const __nv_bfloat16* X, int B, cudaStream_t st, bool trace = false);
     cudaError_t adam_step(float lr, cudaStream_t st);
     // inference only: X [n][MLP_XW], n a multiple of 128, all four layers and
     // the head in one tcgen05 kernel (mlp_tc.cu)

@@ -5,7 +5,7 @@
 //
 // A is stored row-major ("K-major", [M][K]) or column-major ([K][M]); B is
 // stored [K][N] or [N][K].  Tiles are copied to shared memory as stored
-// (cp.async, double-buffered) and the transposition, where needed, happens in
+// (cp.async, a ring of four stages) and the transposition, where needed, happens in
 // ldmatrix(.trans), so the forward (X . W), input-gradient (dZ . W^T) and
 // weight-gradient (X^T . dZ) products all run without a transposed copy.
 // M, N and K must be multiples of 32; tiles past M or N are masked.
@@ -17,9 +17,8 @@
 namespace rsv {
 
 enum GemmEpi : int {
-    EPI_F32 = 0,        // Cf = acc
-    EPI_BIAS_GELU = 1,  // Z = acc + bias (FP32, optional), A = gelu(Z) (BF16)
-    EPI_GELU_BWD = 2    // G = acc * gelu'(Zin) (FP32 and BF16)
+    EPI_BIAS_GELU = 1,  // Z = acc + bias (FP32), A = gelu(Z) (BF16, optional)
+    EPI_GELU_BWD = 2    // G = acc * gelu'(Zin) (BF16, FP32 optional) and its column sums
 };
 
 struct GemmArgs {
@@ -27,11 +26,11 @@ struct GemmArgs {
     const __nv_bfloat16* B;
     int M, N, K;
     int lda, ldb;            // leading dimensions as stored
-    float* Cf;               // FP32 output [M][N] (EPI_F32, EPI_BIAS_GELU: Z, EPI_GELU_BWD: G)
+    float* Cf;               // FP32 output [M][N] (EPI_BIAS_GELU: Z, EPI_GELU_BWD: G)
     __nv_bfloat16* Cb;       // BF16 output [M][N] (activations or gradients)
     const float* bias;       // [N] (EPI_BIAS_GELU)
-    float* Af;               // FP32 activations [M][N] (EPI_BIAS_GELU, optional)
     const float* Zin;        // [M][N] pre-activations (EPI_GELU_BWD)
+    float* colpart;          // [M / 64][N] G's sums over the rows of a tile (EPI_GELU_BWD)
 };
 
 // GELU in the tanh form of Hendrycks & Gimpel (2016),
@@ -97,50 +96,50 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
 
 // 64 x 64 x 32 tiles, 4 warps (2 x 2), warp tile 32 x 32 (2 x 4 mma tiles).
 constexpr int GBM = 64, GBN = 64, GBK = 32, GTHREADS = 128;
+constexpr int GST = 4;   // stages in shared memory
 constexpr int PAD = 8;   // bf16 elements of row padding (16 B) against bank conflicts
 
-template <bool A_KMAJOR, bool B_KMAJOR, int EPI>
-__global__ void __launch_bounds__(GTHREADS) gemm_bf16_kernel(const GemmArgs g) {
+// acc = the tile (m0, n0) of A . B over k0 <= k < k1
+template <bool A_KMAJOR, bool B_KMAJOR>
+__device__ __forceinline__ void gemm_tile(const __nv_bfloat16* __restrict__ A, const __nv_bfloat16* __restrict__ B, int M, int N,
+                                          int lda, int ldb, int m0, int n0, int k0, int k1, float (&acc)[2][4][4]) {
     // shared tiles, as stored: A [GBM][GBK] or [GBK][GBM]; B [GBN][GBK] or [GBK][GBN]
     constexpr int A_ROWS = A_KMAJOR ? GBM : GBK, A_COLS = A_KMAJOR ? GBK : GBM;
     constexpr int B_ROWS = B_KMAJOR ? GBN : GBK, B_COLS = B_KMAJOR ? GBK : GBN;
-    __shared__ __align__(16) __nv_bfloat16 As[2][A_ROWS][A_COLS + PAD];
-    __shared__ __align__(16) __nv_bfloat16 Bs[2][B_ROWS][B_COLS + PAD];
+    __shared__ __align__(16) __nv_bfloat16 As[GST][A_ROWS][A_COLS + PAD];
+    __shared__ __align__(16) __nv_bfloat16 Bs[GST][B_ROWS][B_COLS + PAD];
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int m0 = blockIdx.y * GBM, n0 = blockIdx.x * GBN;
     const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
 
-    auto load_tile = [&](int buf, int k0) {
+    auto load_tile = [&](int buf, int k) {
         // A: 64 x 32 elements = 256 chunks of 8
 #pragma unroll
         for (int c = tid; c < (GBM * GBK) / 8; c += GTHREADS) {
             if constexpr (A_KMAJOR) {
                 const int r = c / (GBK / 8), col = (c % (GBK / 8)) * 8;
-                const bool ok = m0 + r < g.M;
-                cp_async16(&As[buf][r][col], g.A + (size_t)(ok ? m0 + r : 0) * g.lda + k0 + col, ok);
+                const bool ok = m0 + r < M;
+                cp_async16(&As[buf][r][col], A + (size_t)(ok ? m0 + r : 0) * lda + k + col, ok);
             } else {
                 const int r = c / (GBM / 8), col = (c % (GBM / 8)) * 8;
-                const bool ok = m0 + col < g.M;
-                cp_async16(&As[buf][r][col], g.A + (size_t)(k0 + r) * g.lda + (ok ? m0 + col : 0), ok);
+                const bool ok = m0 + col < M;
+                cp_async16(&As[buf][r][col], A + (size_t)(k + r) * lda + (ok ? m0 + col : 0), ok);
             }
         }
 #pragma unroll
         for (int c = tid; c < (GBN * GBK) / 8; c += GTHREADS) {
             if constexpr (B_KMAJOR) {
                 const int r = c / (GBK / 8), col = (c % (GBK / 8)) * 8;
-                const bool ok = n0 + r < g.N;
-                cp_async16(&Bs[buf][r][col], g.B + (size_t)(ok ? n0 + r : 0) * g.ldb + k0 + col, ok);
+                const bool ok = n0 + r < N;
+                cp_async16(&Bs[buf][r][col], B + (size_t)(ok ? n0 + r : 0) * ldb + k + col, ok);
             } else {
                 const int r = c / (GBN / 8), col = (c % (GBN / 8)) * 8;
-                const bool ok = n0 + col < g.N;
-                cp_async16(&Bs[buf][r][col], g.B + (size_t)(k0 + r) * g.ldb + (ok ? n0 + col : 0), ok);
+                const bool ok = n0 + col < N;
+                cp_async16(&Bs[buf][r][col], B + (size_t)(k + r) * ldb + (ok ? n0 + col : 0), ok);
             }
         }
-        cp_async_commit();
     };
 
-    float acc[2][4][4];
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -148,17 +147,18 @@ __global__ void __launch_bounds__(GTHREADS) gemm_bf16_kernel(const GemmArgs g) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) acc[i][j][k] = 0.0f;
 
-    const int nk = g.K / GBK;
-    load_tile(0, 0);
+    const int nk = (k1 - k0) / GBK;
+#pragma unroll
+    for (int kt = 0; kt < GST - 1; ++kt) {
+        if (kt < nk) load_tile(kt, k0 + kt * GBK);
+        cp_async_commit();   // a group an iteration, empty past the end
+    }
     for (int kt = 0; kt < nk; ++kt) {
-        const int buf = kt & 1;
-        if (kt + 1 < nk) {
-            load_tile(buf ^ 1, (kt + 1) * GBK);
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
-        __syncthreads();
+        const int buf = kt % GST;
+        cp_async_wait<GST - 2>();
+        __syncthreads();   // stage kt has arrived, and every warp has read stage kt - 1
+        if (kt + GST - 1 < nk) load_tile((kt + GST - 1) % GST, k0 + (kt + GST - 1) * GBK);
+        cp_async_commit();
 #pragma unroll
         for (int kk = 0; kk < GBK; kk += 16) {
             uint32_t af[2][4], bf[2][4];
@@ -189,38 +189,65 @@ __global__ void __launch_bounds__(GTHREADS) gemm_bf16_kernel(const GemmArgs g) {
                     mma_bf16(acc[mi][ni * 2 + 1], af[mi], bf[ni][2], bf[ni][3]);
                 }
         }
-        __syncthreads();
     }
+}
+
+template <bool A_KMAJOR, bool B_KMAJOR, int EPI>
+__global__ void __launch_bounds__(GTHREADS) gemm_bf16_kernel(const GemmArgs g) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int m0 = blockIdx.y * GBM, n0 = blockIdx.x * GBN;
+    const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
+    float acc[2][4][4];
+    gemm_tile<A_KMAJOR, B_KMAJOR>(g.A, g.B, g.M, g.N, g.lda, g.ldb, m0, n0, 0, g.K, acc);
 
     // epilogue: accumulator (row = lane/4 (+8), col = 2*(lane%4) + {0,1})
 #pragma unroll
-    for (int mi = 0; mi < 2; ++mi)
+    for (int nj = 0; nj < 4; ++nj) {
+        const int col = n0 + wn + nj * 8 + (lane & 3) * 2;
+        float s0 = 0.0f, s1 = 0.0f;
 #pragma unroll
-        for (int nj = 0; nj < 4; ++nj)
+        for (int mi = 0; mi < 2; ++mi)
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int row = m0 + wm + mi * 16 + (lane >> 2) + h * 8;
-                const int col = n0 + wn + nj * 8 + (lane & 3) * 2;
                 if (row >= g.M || col >= g.N) continue;
                 float v0 = acc[mi][nj][h * 2 + 0], v1 = acc[mi][nj][h * 2 + 1];
                 const size_t o = (size_t)row * g.N + col;
-                if constexpr (EPI == EPI_F32) {
-                    *reinterpret_cast<float2*>(g.Cf + o) = make_float2(v0, v1);
-                } else if constexpr (EPI == EPI_BIAS_GELU) {
+                if constexpr (EPI == EPI_BIAS_GELU) {
                     v0 += g.bias[col];
                     v1 += g.bias[col + 1];
-                    if (g.Cf) *reinterpret_cast<float2*>(g.Cf + o) = make_float2(v0, v1);
-                    const float a0 = gelu_f(v0), a1 = gelu_f(v1);
-                    *reinterpret_cast<__nv_bfloat162*>(g.Cb + o) = __floats2bfloat162_rn(a0, a1);
-                    if (g.Af) *reinterpret_cast<float2*>(g.Af + o) = make_float2(a0, a1);
+                    *reinterpret_cast<float2*>(g.Cf + o) = make_float2(v0, v1);
+                    if (g.Cb) *reinterpret_cast<__nv_bfloat162*>(g.Cb + o) = __floats2bfloat162_rn(gelu_f(v0), gelu_f(v1));
                 } else {
                     const float2 z = *reinterpret_cast<const float2*>(g.Zin + o);
                     v0 *= gelu_grad_f(z.x);
                     v1 *= gelu_grad_f(z.y);
                     if (g.Cf) *reinterpret_cast<float2*>(g.Cf + o) = make_float2(v0, v1);
                     *reinterpret_cast<__nv_bfloat162*>(g.Cb + o) = __floats2bfloat162_rn(v0, v1);
+                    s0 += v0;
+                    s1 += v1;
                 }
             }
+        if constexpr (EPI == EPI_GELU_BWD) {
+            // over the 32 rows of the warp, then of the two warps that share the columns
+            __shared__ float red[2][GBN];
+#pragma unroll
+            for (int o = 4; o < 32; o <<= 1) {
+                s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+                s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+            }
+            if (lane < 4) {
+                red[warp >> 1][wn + nj * 8 + lane * 2] = s0;
+                red[warp >> 1][wn + nj * 8 + lane * 2 + 1] = s1;
+            }
+            if (nj == 3) {
+                __syncthreads();
+                const int c = n0 + threadIdx.x;
+                if (threadIdx.x < GBN && c < g.N)
+                    g.colpart[(size_t)blockIdx.y * g.N + c] = red[0][threadIdx.x] + red[1][threadIdx.x];
+            }
+        }
+    }
 }
 
 }  // namespace rsv

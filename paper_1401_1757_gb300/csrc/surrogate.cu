@@ -355,19 +355,22 @@ __device__ float sur_ln_base(const PolSur& P, const SurTables& T, const SurQuery
     return (1.0f - f) * logf(b0) + f * logf(b1);
 }
 
+// Two features as exact hi + lo BF16 halves (pairs).
+__device__ __forceinline__ void sur_split(float a, float b, uint32_t& hi, uint32_t& lo) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    const float2 hf = __bfloat1622float2(h);
+    const __nv_bfloat162 l = __floats2bfloat162_rn(a - hf.x, b - hf.y);
+    hi = *reinterpret_cast<const uint32_t*>(&h);
+    lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+
 // A feature row as exact hi + lo BF16 halves (the first layer's weights are
 // tied across the halves, so it sees each feature to ~16 bits).
 // The row is written as eight 16-byte stores (rows are 128-byte aligned).
 __device__ __forceinline__ void sur_store_features(const float (&f)[MLP_IN], __nv_bfloat16* row) {
     uint32_t hi[MLP_IN / 2], lo[MLP_IN / 2];
 #pragma unroll
-    for (int k = 0; k < MLP_IN; k += 2) {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(f[k], f[k + 1]);
-        const float2 hf = __bfloat1622float2(h);
-        const __nv_bfloat162 l = __floats2bfloat162_rn(f[k] - hf.x, f[k + 1] - hf.y);
-        hi[k / 2] = *reinterpret_cast<const uint32_t*>(&h);
-        lo[k / 2] = *reinterpret_cast<const uint32_t*>(&l);
-    }
+    for (int k = 0; k < MLP_IN; k += 2) sur_split(f[k], f[k + 1], hi[k / 2], lo[k / 2]);
     uint4* dst = reinterpret_cast<uint4*>(row);
 #pragma unroll
     for (int q = 0; q < MLP_IN / 8; ++q) {
@@ -639,22 +642,27 @@ rsv_status mlp_upload(rsv_ctx* c, const float* host) {
     return RSV_OK;
 }
 
-// FP32 feature rows [n][MLP_IN] -> hi + lo BF16 rows [n][MLP_XW]
-__global__ void f32_to_bf16_rows(const float* __restrict__ x, long long rows, __nv_bfloat16* __restrict__ y) {
-    for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < rows; r += (long long)gridDim.x * blockDim.x) {
-        float f[MLP_IN];
-#pragma unroll
-        for (int k = 0; k < MLP_IN; ++k) f[k] = x[r * MLP_IN + k];
-        sur_store_features(f, y + r * MLP_XW);
+// FP32 feature rows [n][MLP_IN] -> hi + lo BF16 rows [n][MLP_XW], four features a thread; rows
+// n <= r < n_pad are 0
+__global__ void f32_to_bf16_rows(const float4* __restrict__ x, long long n, long long n_pad, __nv_bfloat16* __restrict__ y) {
+    constexpr int Q = MLP_IN / 4;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n_pad * Q; i += (long long)gridDim.x * blockDim.x) {
+        const long long r = i / Q;
+        const float4 f = r < n ? x[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        uint2 hi, lo;
+        sur_split(f.x, f.y, hi.x, lo.x);
+        sur_split(f.z, f.w, hi.y, lo.y);
+        uint2* dst = reinterpret_cast<uint2*>(y + r * MLP_XW);
+        dst[i % Q] = hi;
+        dst[Q + i % Q] = lo;
     }
 }
 
 rsv_status mlp_stage_inputs(rsv_ctx* c, const float* X, long long n, long long n_pad) {
     CU(c->mlp.ensure((int)n_pad));
     CU(c->sur.d_aux.ensure((size_t)n_pad * MLP_IN * 4));
-    CU(cudaMemsetAsync(c->sur.d_aux.p, 0, (size_t)n_pad * MLP_IN * 4, c->stream));
     CU(cudaMemcpyAsync(c->sur.d_aux.p, X, (size_t)n * MLP_IN * 4, cudaMemcpyHostToDevice, c->stream));
-    f32_to_bf16_rows<<<c->sm_count * 4, 256, 0, c->stream>>>(c->sur.d_aux.as<float>(), n_pad, c->mlp.X);
+    f32_to_bf16_rows<<<c->sm_count * 4, 256, 0, c->stream>>>(c->sur.d_aux.as<float4>(), n, n_pad, c->mlp.X);
     CU(cudaGetLastError());
     return RSV_OK;
 }
@@ -1003,8 +1011,8 @@ rsv_status rsv_mlp_trace(rsv_ctx* c, int32_t backend, const float* X, const floa
         CU(cudaMemcpyAsync(A, ta, 3 * L * 2, cudaMemcpyDeviceToHost, c->stream));
     } else {
         if (target) CU(cudaMemcpyAsync(c->mlp.t, target, (size_t)n * 4, cudaMemcpyHostToDevice, c->stream));
-        CU(c->mlp.forward(c->mlp.X, (int)n, c->mlp.y, target ? c->mlp.t : nullptr, c->stream));
-        if (target) CU(c->mlp.backward(c->mlp.X, (int)n, c->stream));
+        CU(c->mlp.forward(c->mlp.X, (int)n, c->mlp.y, target ? c->mlp.t : nullptr, c->stream, true));
+        if (target) CU(c->mlp.backward(c->mlp.X, (int)n, c->stream, true));
         for (int l = 0; l < 4; ++l) {
             CU(cudaMemcpyAsync(Z + l * L, c->mlp.Z[l], L * 4, cudaMemcpyDeviceToHost, c->stream));
             CU(cudaMemcpyAsync(A + l * L, c->mlp.A[l], L * 2, cudaMemcpyDeviceToHost, c->stream));
