@@ -195,12 +195,13 @@ struct rsv_ctx {
     unsigned long long tabf_gen = 1;
 
     std::vector<rsv_policy, rsv::DefaultInit<rsv_policy>> pols;   // resize leaves new records unset
+    std::vector<double, rsv::DefaultInit<double>> h_amount;       // their amounts
     unsigned long long pol_gen = 1;
     DevBuf d_amount;
     bool amount_dirty = true;
 
     int n_scen = 0, n_steps = 0, s_pad = 0;
-    DevBuf d_vstage, d_v64, d_v32, d_v2;
+    DevBuf d_vstage, d_vbad, d_v64, d_v32, d_v2;
 
     DevBuf d_tab[3];
     int tab_pad_of[3] = {-1, -1, -1};
@@ -223,7 +224,7 @@ struct rsv_ctx {
     double tab_min[rsv::kMaxTables] = {};           // smallest survivor-column entry of a table
     double amt_lo = 0.0, amt_hi = 0.0;              // smallest non-zero and largest |amount|
     DevBuf d_mv_D, d_mv_col, d_mv_D64, d_mv_dig[4], d_mv_E, d_mv_out;
-    unsigned long long scen_gen = 1, mv_dig_gen[4] = {0, 0, 0, 0};
+    unsigned long long scen_gen = 1, mv_range_gen = 0, mv_dig_gen[4] = {0, 0, 0, 0};
     int mv_built = -1;   // first tile of the panel whose digits are held, within one call
 
     Layout lay;
@@ -292,7 +293,7 @@ rsv_status stage_tables(rsv_ctx* c, int form, int pad, int n_tab, size_t& smem);
 // Whether the matrix product covers the loaded data; then, on the layout of width
 // kMvP: mv_prepare once a call, mv_launch for the scenario columns [s0, s0 + w) with the
 // output pointers at column s0 (partial: [mv_part_rows][s_pad]).
-bool mv_applies(const rsv_ctx* c, int form, double amt_lo, double amt_hi);
+rsv_status mv_applies(rsv_ctx* c, int form, double amt_lo, double amt_hi, bool& applies);
 rsv_status mv_prepare(rsv_ctx* c, int form);
 // Its parts, for rows that come from elsewhere (m lives): the scenario set's digits, the tiles
 // of a panel and their buffers (d_mv_E, d_mv_out), and the product of a built panel

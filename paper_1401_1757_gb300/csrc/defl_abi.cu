@@ -124,7 +124,11 @@ rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     } else {
         return fail(c, RSV_E_ARG, "variant %d out of range (the deflated form has no scan or summation)", o->variant);
     }
-    const bool mat = vi == nv && mv_applies(c, F_DEFL, c->amt_lo, c->amt_hi);
+    bool mat = false;
+    if (vi == nv) {
+        const rsv_status mst = mv_applies(c, F_DEFL, c->amt_lo, c->amt_hi, mat);
+        if (mst != RSV_OK) return mst;
+    }
     const bool by_index = o->variant >= 0 && o->variant < nv;
     if (vi == nv) vi = 0;
     // A variant whose staging ring does not fit beside the tables is replaced

@@ -174,6 +174,16 @@ __global__ void node_segments_kernel(const long long* __restrict__ noff, const d
     }
 }
 
+// The index of the first factor that is not finite and positive (bad starts at ~0).  The host's loop
+// over them took 0.35 ms for 600,000 (one compare and branch at a time), the copy and this 60 us.
+__global__ void check_factors_kernel(const double* __restrict__ v, size_t n, unsigned long long* __restrict__ bad) {
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+        if (!(isfinite(v[i]) && v[i] > 0.0)) {
+            atomicMin(bad, (unsigned long long)i);
+            return;   // the thread's later ones lie behind it
+        }
+}
+
 __global__ void scale_kernel(double* __restrict__ x, size_t n, double f) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
         x[i] *= f;
@@ -248,22 +258,30 @@ rsv_status prep_one(const rsv_ctx* c, int64_t i, int horizon, int max_steps, Pol
     return RSV_OK;
 }
 
+// Parts that n records' host work is split into.  A part is at least 8,192 records (some tens
+// of microseconds, the cost of waking a worker): 100,000 records loaded, laid out and
+// sorted in 0.65 ms, 1.3 ms when a part was 16,384 to 65,536.
+int host_parts(int64_t n) {
+    const int hw = (int)std::max(1u, std::thread::hardware_concurrency());
+    return (int)std::max<int64_t>(1, std::min<int64_t>(std::min(hw, 16), n / 8192));
+}
+
 // Validate every record and derive its reduced model, steps and boundary,
 // on several host threads for large portfolios.  The error reported is the
 // first bad record in portfolio order.
 rsv_status prep_policies(rsv_ctx* c, int horizon, int max_steps, std::vector<PolPrep>& out, int& tab_pad,
-                         int& n_tab, double& chain_steps) {
+                         int& n_tab, double& chain_steps, bool split, int& max_S, bool (&grp_two)[2]) {
     const int64_t n = (int64_t)c->pols.size();
     out.resize(n);
     struct Part {
-        int need = 1, n_tab = 1;
+        int need = 1, n_tab = 1, max_S = 0;
+        bool two[2] = {false, false};
         double steps = 0.0;
         int64_t bad = -1;
         rsv_status st = RSV_OK;
         char msg[160] = {0};
     };
-    const int hw = (int)std::max(1u, std::thread::hardware_concurrency());
-    const int T = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(hw, 16), n / 16384));
+    const int T = host_parts(n);
     std::vector<Part> part(T);
     auto run = [&](int k) {
         Part& pr = part[k];
@@ -275,18 +293,26 @@ rsv_status prep_policies(rsv_ctx* c, int horizon, int max_steps, std::vector<Pol
                 pr.bad = i;
                 return;
             }
-            pr.steps += out[i].S;
+            const PolPrep& q = out[i];
+            pr.steps += q.S;
+            pr.max_S = std::max(pr.max_S, q.S);
+            if (q.kind == K_ANN2 || q.kind == K_ASS2 || q.kind == K_LS2) pr.two[split && !c->cf_level[i] ? 1 : 0] = true;
         }
     };
     run_parts(T, run);
     int need = 1;
     n_tab = 1;
     chain_steps = 0;
+    max_S = 0;
+    grp_two[0] = grp_two[1] = false;
     for (const Part& pr : part) {   // parts in portfolio order: the first failure is the earliest record
         if (pr.st != RSV_OK) return fail(c, pr.st, "%s", pr.msg);
         need = std::max(need, pr.need);
         n_tab = std::max(n_tab, pr.n_tab);
         chain_steps += pr.steps;
+        max_S = std::max(max_S, pr.max_S);
+        grp_two[0] |= pr.two[0];
+        grp_two[1] |= pr.two[1];
     }
     for (int t = 0; t < n_tab; ++t) need = std::max(need, table_len(c, t));
     tab_pad = (need + 31) / 32 * 32;
@@ -307,7 +333,9 @@ rsv_status rsv::build_layout(rsv_ctx* c, int P, int horizon, int max_steps, int 
     std::vector<PolPrep>& pp = L.h_pp;
     int tab_pad, n_tab;
     double cs;
-    rsv_status st = prep_policies(c, horizon, max_steps, pp, tab_pad, n_tab, cs);
+    int max_S;
+    bool grp_two[2];
+    rsv_status st = prep_policies(c, horizon, max_steps, pp, tab_pad, n_tab, cs, split, max_S, grp_two);
     if (st != RSV_OK) return st;
     auto group = [&](const PolPrep& q) { return split && !c->cf_level[q.pol] ? 1 : 0; };
 
@@ -315,26 +343,26 @@ rsv_status rsv::build_layout(rsv_ctx* c, int P, int horizon, int max_steps, int 
     // three-state tiles, then joint and single-life annuities, then assurances
     static const int kind_rank[6] = {3, 5, 0, 2, 4, 1};   // by kind
     static const int rank_kind[6] = {K_JL, K_LS2, K_ANN2, K_ANN, K_ASS2, K_ASS};
-    // stable counting sort on the key: S <= kMaxAgeSteps
-    const int span = kMaxAgeSteps + 1, per_group = 6 * span;
-    const int nb = 2 * per_group;
+    // stable counting sort on the key: S <= max_S
+    const int span = max_S + 1, per_group = 6 * span;
+    const int nb = (split ? 2 : 1) * per_group;
     std::vector<int>& bucket_start = L.h_bucket;
     std::vector<int>& order = L.h_order;
-    bucket_start.assign(nb + 1, 0);
+    bucket_start.resize(nb + 1);
     order.resize(pp.size());
     auto key = [&](const PolPrep& q) {
-        return group(q) * per_group + kind_rank[q.kind] * span + (kMaxAgeSteps - q.S);
+        return group(q) * per_group + kind_rank[q.kind] * span + (max_S - q.S);
     };
     // in parallel for large portfolios: each part counts its contiguous range,
     // the parts' starts per bucket follow part order, and each part scatters
     // its range in order, so the sort stays stable
     const int64_t n_pp = (int64_t)pp.size();
-    const int hw_s = (int)std::max(1u, std::thread::hardware_concurrency());
-    const int TS = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(hw_s, 16), n_pp / 65536));
+    const int TS = host_parts(n_pp);
     std::vector<int>& cnt = L.h_cnt;
-    cnt.assign((size_t)TS * nb, 0);
+    cnt.resize((size_t)TS * nb);
     run_parts(TS, [&](int k) {
         int* h = cnt.data() + (size_t)k * nb;
+        std::fill(h, h + nb, 0);
         for (int64_t i = n_pp * k / TS, e = n_pp * (k + 1) / TS; i < e; ++i) ++h[key(pp[i])];
     });
     for (int b = 0, run = 0; b < nb; ++b) {
@@ -344,12 +372,12 @@ rsv_status rsv::build_layout(rsv_ctx* c, int P, int horizon, int max_steps, int 
             cnt[(size_t)k * nb + b] = run;
             run += v;
         }
-        bucket_start[b + 1] = run;
     }
     int run_lo[12], run_hi[12];   // sorted ranges of the (group, kind rank) runs
+    bucket_start[nb] = (int)n_pp;
     for (int r = 0; r < 12; ++r) {
-        run_lo[r] = bucket_start[r * span];
-        run_hi[r] = bucket_start[(r + 1) * span];
+        run_lo[r] = bucket_start[std::min(r * span, nb)];
+        run_hi[r] = bucket_start[std::min((r + 1) * span, nb)];
     }
     run_parts(TS, [&](int k) {
         int* h = cnt.data() + (size_t)k * nb;
@@ -443,9 +471,8 @@ rsv_status rsv::build_layout(rsv_ctx* c, int P, int horizon, int max_steps, int 
         }
     };
     {
-        const int hw = (int)std::max(1u, std::thread::hardware_concurrency());
         // by slots, not tiles: wide tiles (the deflated form's 60 policies) are few
-        const int T = (int)std::max<size_t>(1, std::min<size_t>((size_t)std::min(hw, 16), n_slots / 16384));
+        const int T = host_parts((int64_t)n_slots);
         run_parts(T, [&](int k) {
             fill((int)((long long)n_tiles * k / T), (int)((long long)n_tiles * (k + 1) / T));
         });
@@ -463,30 +490,10 @@ rsv_status rsv::build_layout(rsv_ctx* c, int P, int horizon, int max_steps, int 
     L.tab_pad = tab_pad;
     L.n_tab = n_tab;
     L.chain_steps = cs;
-    L.max_S = 0;
-    L.has_two = false;
-    L.grp_two[0] = L.grp_two[1] = false;
-    {
-        struct Scan {
-            int max_S = 0;
-            bool two[2] = {false, false};
-        };
-        std::vector<Scan> sc(TS);
-        run_parts(TS, [&](int k) {
-            Scan& r = sc[k];
-            for (int64_t i = n_pp * k / TS, e = n_pp * (k + 1) / TS; i < e; ++i) {
-                const PolPrep& q = pp[i];
-                r.max_S = std::max(r.max_S, q.S);
-                if (q.kind == K_ANN2 || q.kind == K_ASS2 || q.kind == K_LS2) r.two[group(q)] = true;
-            }
-        });
-        for (const Scan& r : sc) {
-            L.max_S = std::max(L.max_S, r.max_S);
-            L.grp_two[0] |= r.two[0];
-            L.grp_two[1] |= r.two[1];
-        }
-        L.has_two = L.grp_two[0] || L.grp_two[1];
-    }
+    L.max_S = max_S;
+    L.grp_two[0] = grp_two[0];
+    L.grp_two[1] = grp_two[1];
+    L.has_two = grp_two[0] || grp_two[1];
     return RSV_OK;
 }
 
@@ -604,8 +611,7 @@ namespace {
 
 rsv_status upload_amounts(rsv_ctx* c) {
     if (!c->amount_dirty) return RSV_OK;
-    std::vector<double> a(c->pols.size());
-    for (size_t i = 0; i < a.size(); ++i) a[i] = c->pols[i].amount;
+    const auto& a = c->h_amount;
     CU(c->d_amount.ensure(std::max<size_t>(1, a.size()) * sizeof(double)));
     if (!a.empty()) {
         CU(cudaMemcpyAsync(c->d_amount.p, a.data(), a.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));
@@ -616,11 +622,27 @@ rsv_status upload_amounts(rsv_ctx* c) {
 
 }  // namespace
 
-bool rsv::mv_applies(const rsv_ctx* c, int form, double amt_lo, double amt_hi) {
-    if (c->mv_spread > mv_max_spread(form) || !(amt_hi <= kMvAmountMax) || !(amt_lo >= kMvAmountMin)) return false;
+rsv_status rsv::mv_applies(rsv_ctx* c, int form, double amt_lo, double amt_hi, bool& applies) {
+    applies = false;
+    if (!(amt_hi <= kMvAmountMax) || !(amt_lo >= kMvAmountMin)) return RSV_OK;
     for (int t = 0; t < kMaxTables; ++t)
-        if (!c->tab[t].empty() && !(c->tab_min[t] >= kMvTableMin)) return false;
-    return true;
+        if (!c->tab[t].empty() && !(c->tab_min[t] >= kMvTableMin)) return RSV_OK;
+    if (c->mv_range_gen != c->scen_gen) {
+        // the discount products and their range, with the scenario set's first use here (a
+        // quarter of the load's time, which the other forms and the time scan need not pay)
+        const size_t np = (size_t)c->n_steps * c->s_pad;
+        CU(c->d_mv_D.ensure(np * sizeof(float2)));
+        CU(c->d_mv_col.ensure(MvScen::words(c->n_steps, c->s_pad) * sizeof(int32_t)));
+        const MvScen mv = MvScen::at(c->d_mv_col.p, c->n_steps, c->s_pad);
+        CU(launch_mv_scenarios(c->d_v64.as<double>(), c->n_steps, c->n_scen, c->s_pad, c->d_mv_D.as<float2>(), mv, c->stream));
+        int32_t range[2];
+        CU(cudaMemcpyAsync(range, mv.stat, sizeof range, cudaMemcpyDeviceToHost, c->stream));
+        CU(cudaStreamSynchronize(c->stream));
+        c->mv_spread = range[1] <= kMvTilt ? range[0] : INT_MAX;
+        c->mv_range_gen = c->scen_gen;
+    }
+    applies = c->mv_spread <= mv_max_spread(form);
+    return RSV_OK;
 }
 
 rsv_status rsv::mv_scenario_digits(rsv_ctx* c, int form) {
@@ -802,7 +824,8 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
         return fail(c, RSV_E_ARG, "variant %d out of range", o->variant);
     }
     if (o->form != F_F32 && vi == nt && !extra && !scan && !summ && pay == PAY_END) {
-        mat = mv_applies(c, o->form, c->amt_lo, c->amt_hi);
+        const rsv_status mst = mv_applies(c, o->form, c->amt_lo, c->amt_hi, mat);
+        if (mst != RSV_OK) return mst;
         vi = 0;
     }
     if (split) vg = special_variant(vl, nv, false, PAY_END_GENERAL);
@@ -1250,7 +1273,7 @@ rsv_status rsv_destroy(rsv_ctx* c) try {
     if (!c) return RSV_OK;
     cudaSetDevice(c->device);
     cudaStreamSynchronize(c->stream);
-    for (DevBuf* b : {&c->d_amount, &c->d_vstage, &c->d_v64, &c->d_v32, &c->d_v2, &c->d_tab[0], &c->d_tab[1],
+    for (DevBuf* b : {&c->d_amount, &c->d_vstage, &c->d_vbad, &c->d_v64, &c->d_v32, &c->d_v2, &c->d_tab[0], &c->d_tab[1],
                       &c->d_tab[2], &c->lay.slots, &c->lay.kinds, &c->d_ctl, &c->d_partial, &c->d_part2,
                       &c->d_o_v0f, &c->d_o_v0d, &c->d_o_tot, &c->d_o_pt, &c->d_o_traj, &c->d_cf_tab,
                       &c->d_cf_pol, &c->d_cf_sum, &c->d_nest_rn, &c->d_nest_d0, &c->d_nest_plane, &c->d_nest_mean,
@@ -1428,14 +1451,15 @@ rsv_status rsv_load_portfolio(rsv_ctx* c, const rsv_policy* pols, int64_t n) try
     if (n < 0 || n > 0x7fffffffLL || (n > 0 && !pols)) return fail(c, RSV_E_ARG, "bad portfolio size %lld", (long long)n);
     // copied by several host threads for large portfolios (no zero fill first)
     c->pols.resize((size_t)n);
-    const int hw = (int)std::max(1u, std::thread::hardware_concurrency());
-    const int T = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(hw, 16), n / 65536));
+    c->h_amount.resize((size_t)n);
+    const int T = host_parts(n);
     std::vector<double> amt_lo(T, INFINITY), amt_hi(T, 0.0);
     run_parts(T, [&](int k) {
         const int64_t lo = n * k / T, hi = n * (k + 1) / T;
         if (hi > lo) memcpy(c->pols.data() + lo, pols + lo, (size_t)(hi - lo) * sizeof(rsv_policy));
         double mn = INFINITY, mx = 0.0;
         for (int64_t i = lo; i < hi; ++i) {
+            c->h_amount[(size_t)i] = pols[i].amount;
             const double a = std::fabs(pols[i].amount);
             mx = std::max(mx, a);
             if (a > 0.0) mn = std::min(mn, a);
@@ -1457,31 +1481,31 @@ rsv_status rsv_load_scenarios(rsv_ctx* c, const double* v, int32_t n_scen, int32
     if (!v || n_scen < 1 || n_steps < 1 || (layout != 0 && layout != 1))
         return fail(c, RSV_E_ARG, "bad scenario arguments");
     const size_t n = (size_t)n_scen * n_steps;
-    for (size_t i = 0; i < n; ++i)
-        if (!(std::isfinite(v[i]) && v[i] > 0.0))
-            return fail(c, RSV_E_ASSUMPTION, "discount factor %zu = %g is not finite and positive", i, v[i]);
     cudaError_t e = cudaSetDevice(c->device);
     if (e != cudaSuccess) return fail(c, RSV_E_CUDA, "cudaSetDevice: %s", cudaGetErrorString(e));
     const int s_pad = (n_scen + 127) / 128 * 128;
     const size_t np = (size_t)n_steps * s_pad;
+    // staged and checked before anything of the loaded set changes
     CU(c->d_vstage.ensure(n * sizeof(double)));
+    CU(c->d_vbad.ensure(sizeof(unsigned long long)));
+    CU(cudaMemcpyAsync(c->d_vstage.p, v, n * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+    CU(cudaMemsetAsync(c->d_vbad.p, 0xff, sizeof(unsigned long long), c->stream));
+    check_factors_kernel<<<c->sm_count * 8, 256, 0, c->stream>>>(c->d_vstage.as<double>(), n,
+                                                                 c->d_vbad.as<unsigned long long>());
+    CU(cudaGetLastError());
+    unsigned long long bad;
+    CU(cudaMemcpyAsync(&bad, c->d_vbad.p, sizeof bad, cudaMemcpyDeviceToHost, c->stream));
+    CU(cudaStreamSynchronize(c->stream));
+    if (bad < n)
+        return fail(c, RSV_E_ASSUMPTION, "discount factor %zu = %g is not finite and positive", (size_t)bad, v[bad]);
     CU(c->d_v64.ensure(np * sizeof(double)));
     CU(c->d_v32.ensure(np * sizeof(float)));
     CU(c->d_v2.ensure(np * sizeof(float2)));
-    CU(cudaMemcpyAsync(c->d_vstage.p, v, n * sizeof(double), cudaMemcpyHostToDevice, c->stream));
     split_planes_kernel<<<c->sm_count * 8, 256, 0, c->stream>>>(c->d_vstage.as<double>(), layout, n_scen, n_steps,
                                                                 s_pad, c->d_v64.as<double>(), c->d_v32.as<float>(),
                                                                 c->d_v2.as<float2>());
     CU(cudaGetLastError());
-    // the discount products and their range for the matrix product
-    CU(c->d_mv_D.ensure(np * sizeof(float2)));
-    CU(c->d_mv_col.ensure(MvScen::words(n_steps, s_pad) * sizeof(int32_t)));
-    const MvScen mv = MvScen::at(c->d_mv_col.p, n_steps, s_pad);
-    CU(launch_mv_scenarios(c->d_v64.as<double>(), n_steps, n_scen, s_pad, c->d_mv_D.as<float2>(), mv, c->stream));
-    int32_t range[2];
-    CU(cudaMemcpyAsync(range, mv.stat, sizeof range, cudaMemcpyDeviceToHost, c->stream));
     CU(cudaStreamSynchronize(c->stream));
-    c->mv_spread = range[1] <= kMvTilt ? range[0] : INT_MAX;
     ++c->scen_gen;
     c->n_scen = n_scen;
     c->n_steps = n_steps;
