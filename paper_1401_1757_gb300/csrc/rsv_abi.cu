@@ -106,26 +106,49 @@ __global__ void split_planes_kernel(const double* __restrict__ v, int layout, in
     }
 }
 
-// Fixed-order two-level sum of the per-tile scenario sums (deterministic): 32 columns
-// and 8 interleaved row chains a block, so that the loads of a column are 8 deep; rows
-// [y G, (y + 1) G) of `in` into row y of `out` (row length out_ld, columns below n_col).
-// 1,000 rows of one scenario (the time scan): 36 us as serial chains of 256 rows, 11 us so;
-// 1,563 rows of 1,000: 38 -> 11 us.
+// Fixed-order two-level sum of the per-tile scenario sums (deterministic): 32 columns and 8
+// interleaved row chains a block, rows [y G, (y + 1) G) of `in` into row y of `part2`; the
+// block that finishes a column group last (done, which it leaves at 0) adds the rows of
+// part2 in the same manner.  Bound by latency: loads are eight deep a chain, and one launch
+// instead of two saves 3 us a call.  1,000 rows of one scenario (the time scan): 36 us as
+// serial chains of 256 rows, 8 us so; 1,563 rows of 1,000: 38 -> 12 us.
 constexpr int kSumRows = 8;
-__global__ void __launch_bounds__(32 * kSumRows) reduce_rows_kernel(const double* __restrict__ in, int n_rows, int s_pad, int G,
-                                                                    double* __restrict__ out, int out_ld, int n_col) {
-    __shared__ double part[kSumRows][32];
-    const int s = blockIdx.x * 32 + threadIdx.x;
-    const int t0 = blockIdx.y * G, t1 = min(n_rows, t0 + G);
+__device__ __forceinline__ double sum_rows(const double* __restrict__ in, int t0, int t1, int ld, int s, int n_col,
+                                           double (&part)[kSumRows][32]) {
     double acc = 0.0;
-#pragma unroll 4
-    for (int t = t0 + threadIdx.y; t < t1; t += kSumRows) acc += in[(size_t)t * s_pad + s];
+    if (s < n_col) {
+#pragma unroll 8
+        for (int t = t0 + threadIdx.y; t < t1; t += kSumRows) acc += __ldcg(in + (size_t)t * ld + s);
+    }
     part[threadIdx.y][threadIdx.x] = acc;
     __syncthreads();
-    if (threadIdx.y || s >= n_col) return;
 #pragma unroll
     for (int k = 1; k < kSumRows; ++k) acc += part[k][threadIdx.x];
-    out[(size_t)blockIdx.y * out_ld + s] = acc;
+    return acc;   // in the threads of chain 0
+}
+
+__global__ void __launch_bounds__(32 * kSumRows) reduce_rows_kernel(const double* __restrict__ in, int n_rows, int s_pad, int G,
+                                                                    double* part2, int* __restrict__ done,
+                                                                    double* __restrict__ out, int n_col) {
+    __shared__ double part[kSumRows][32];
+    __shared__ bool last;
+    const int s = blockIdx.x * 32 + threadIdx.x;
+    const int t0 = blockIdx.y * G, t1 = min(n_rows, t0 + G);
+    double x = sum_rows(in, t0, t1, s_pad, s, n_col, part);
+    if (gridDim.y > 1) {
+        if (threadIdx.y == 0 && s < n_col) {
+            part2[(size_t)blockIdx.y * s_pad + s] = x;
+            __threadfence();
+        }
+        __syncthreads();
+        if (threadIdx.x == 0 && threadIdx.y == 0) last = atomicAdd(done + blockIdx.x, 1) == (int)gridDim.y - 1;
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        x = sum_rows(part2, 0, gridDim.y, s_pad, s, n_col, part);
+        if (threadIdx.x == 0 && threadIdx.y == 0) done[blockIdx.x] = 0;
+    }
+    if (threadIdx.y == 0 && s < n_col) out[s] = x;
 }
 
 // L[k] = base[k] + sum over q in [seg[k], seg[k+1]) of w[q] V[q], one block per
@@ -568,17 +591,17 @@ rsv_status rsv::stage_tables(rsv_ctx* c, int form, int pad, int n_tab, size_t& s
 
 rsv_status rsv::scenario_totals(rsv_ctx* c, const double* partial, int n_rows, int s_pad, int n_scen, double* tot) {
     // one level up to 256 rows (32 a chain), else groups of 128
-    const int G = n_rows <= 256 ? n_rows : 128, groups = (n_rows + G - 1) / G;
-    const dim3 block(32, kSumRows);
-    if (groups == 1) {
-        reduce_rows_kernel<<<dim3(s_pad / 32, 1), block, 0, c->stream>>>(partial, n_rows, s_pad, G, tot, 0, n_scen);
-    } else {
+    const int G = n_rows <= 256 ? std::max(1, n_rows) : 128, groups = std::max(1, (n_rows + G - 1) / G), cols = (n_scen + 31) / 32;
+    if (groups > 1) {
         CU(c->d_part2.ensure((size_t)groups * s_pad * sizeof(double)));
-        double* part2 = c->d_part2.as<double>();
-        reduce_rows_kernel<<<dim3(s_pad / 32, groups), block, 0, c->stream>>>(partial, n_rows, s_pad, G, part2, s_pad, s_pad);
-        CU(cudaGetLastError());
-        reduce_rows_kernel<<<dim3(s_pad / 32, 1), block, 0, c->stream>>>(part2, groups, s_pad, groups, tot, 0, n_scen);
+        if (c->sum_done_cols < cols) {
+            CU(c->d_sum_done.ensure((size_t)cols * sizeof(int)));
+            CU(cudaMemsetAsync(c->d_sum_done.p, 0, (size_t)cols * sizeof(int), c->stream));
+            c->sum_done_cols = cols;
+        }
     }
+    reduce_rows_kernel<<<dim3(cols, groups), dim3(32, kSumRows), 0, c->stream>>>(partial, n_rows, s_pad, G, c->d_part2.as<double>(),
+                                                                                 c->d_sum_done.as<int>(), tot, n_scen);
     CU(cudaGetLastError());
     return RSV_OK;
 }
@@ -1274,7 +1297,7 @@ rsv_status rsv_destroy(rsv_ctx* c) try {
     cudaSetDevice(c->device);
     cudaStreamSynchronize(c->stream);
     for (DevBuf* b : {&c->d_amount, &c->d_vstage, &c->d_vbad, &c->d_v64, &c->d_v32, &c->d_v2, &c->d_tab[0], &c->d_tab[1],
-                      &c->d_tab[2], &c->lay.slots, &c->lay.kinds, &c->d_ctl, &c->d_partial, &c->d_part2,
+                      &c->d_tab[2], &c->lay.slots, &c->lay.kinds, &c->d_ctl, &c->d_partial, &c->d_part2, &c->d_sum_done,
                       &c->d_o_v0f, &c->d_o_v0d, &c->d_o_tot, &c->d_o_pt, &c->d_o_traj, &c->d_cf_tab,
                       &c->d_cf_pol, &c->d_cf_sum, &c->d_nest_rn, &c->d_nest_d0, &c->d_nest_plane, &c->d_nest_mean,
                       &c->d_nest_kth, &c->d_nest_all, &c->d_pols, &c->sur.d_flag, &c->sur.d_q, &c->sur.d_lab,
