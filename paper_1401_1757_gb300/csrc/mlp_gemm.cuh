@@ -94,6 +94,13 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// Lets the next kernel of the stream be launched, and waits until the one before it has
+// finished and its writes are seen (both at once if it was launched as an ordinary kernel).
+__device__ __forceinline__ void grid_dependency_wait() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // 64 x 64 x 32 tiles, 4 warps (2 x 2), warp tile 32 x 32 (2 x 4 mma tiles).
 constexpr int GBM = 64, GBN = 64, GBK = 32, GTHREADS = 128;
 constexpr int GST = 4;   // stages in shared memory
@@ -194,6 +201,7 @@ __device__ __forceinline__ void gemm_tile(const __nv_bfloat16* __restrict__ A, c
 
 template <bool A_KMAJOR, bool B_KMAJOR, int EPI>
 __global__ void __launch_bounds__(GTHREADS) gemm_bf16_kernel(const GemmArgs g) {
+    grid_dependency_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int m0 = blockIdx.y * GBM, n0 = blockIdx.x * GBN;
     const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
