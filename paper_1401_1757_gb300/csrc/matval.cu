@@ -7,6 +7,7 @@
 #include <climits>
 #include <cmath>
 
+#include "launch_next.cuh"
 #include "matval.cuh"
 #include "tcgen05.cuh"
 
@@ -484,6 +485,7 @@ __device__ __forceinline__ void mv_row64(const MvBuild& b, const SlotRec& r, con
 }
 
 __global__ void __launch_bounds__(256) mv_build64_kernel(const MvBuild b, const CfPol* __restrict__ pols) {
+    grid_dependency_wait();
     extern __shared__ float4 tilt4[];
     float* tilt = reinterpret_cast<float*>(tilt4);
     const int row = blockIdx.x * 8 + (threadIdx.x >> 5), tile = row / kMvP;
@@ -570,6 +572,7 @@ __global__ void __launch_bounds__(256) mv_build_lives_kernel(const CfTables T, c
                                                              const double* __restrict__ amount, int pitch, int n_steps,
                                                              const float* __restrict__ tilt_g, void* digits,
                                                              MvOut* __restrict__ out) {
+    grid_dependency_wait();
     extern __shared__ float4 tilt4[];
     float* tilt = reinterpret_cast<float*>(tilt4);
     const int row = blockIdx.x * 8 + (threadIdx.x >> 5), tile = row / kMvP;
@@ -601,6 +604,7 @@ __global__ void __launch_bounds__(256) mv_build_lives_kernel(const CfTables T, c
 
 template <int NS>
 __global__ void __launch_bounds__(256) mv_build_kernel(const MvBuild b) {
+    grid_dependency_wait();
     extern __shared__ float4 tilt4[];   // 2^-tau(t)
     float* tilt = reinterpret_cast<float*>(tilt4);
     const int rows = 8 * b.rows_per_warp, row0 = blockIdx.x * rows, tile = row0 / kMvP;
@@ -720,6 +724,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
     fence_before();
     cluster_sync();
     fence_after();
+    grid_dependency_wait();   // for the rows of the builder
     const uint32_t tmem = tmem_slot;
     const int n_pairs = (a.n_chunks + 1) / 2, n_clusters = (int)gridDim.x / 2, cluster = (int)blockIdx.x / 2;
     const long long n_items = (long long)a.n_tiles * kSub * n_pairs;   // part of a tile, pair of scenario tiles
@@ -951,8 +956,7 @@ cudaError_t product(const MvArgs& a, const void* digitsD, const void* digitsE, i
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const long long items = (long long)a.n_tiles * (kMvP / Sh::N) * ((a.n_chunks + 1) / 2);
-    k<<<2 * (int)std::min<long long>(items, sm_count / 2), kMvThreads, smem, st>>>(mD, mE, a);
-    return cudaGetLastError();
+    return launch_next(k, dim3(2 * (int)std::min<long long>(items, sm_count / 2)), kMvThreads, smem, st, mD, mE, a);
 }
 
 }  // namespace
