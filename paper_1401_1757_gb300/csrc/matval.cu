@@ -645,6 +645,11 @@ __global__ void __launch_bounds__(256) mv_build_kernel(const MvBuild b) {
 // and kept in the collector: 903 -> 755 us a launch of 50,000 x 1,000 with six.  Whole
 // tiles with the levels 3 to 5 in one accumulator took 690 us, at 13 times the error (totals of
 // annuities 1.8e-13 against the recurrence's 9e-14).
+// With one item in TMEM the products stand still until its accumulators are read, so before
+// the release the low ones are only summed and the rest follows after it; in the FP64
+// form all of this had been conversions and sums on the FP64 pipe, longer than the products
+// (100,000 x 1,000 of every product: four digits 0.90 -> 0.88 ms, six 1.68 -> 1.62 ms; 3,000 x 333
+// in FP64: 0.203 -> 0.148 ms).
 template <int NS>
 struct MvShape;   // policies of an item, accumulators, items in TMEM, stages, steps of a block (64:
 template <>       // 128-byte swizzled rows); the products are (i, j), i + j < NS, of scenario digit i
@@ -688,6 +693,19 @@ __device__ __forceinline__ void mv_products(uint32_t d, uint64_t base, int off, 
                     base + (uint64_t)((NS * G::kA + J * G::kB + off) >> 4), idesc, !first || more);
     if constexpr (I + J + 1 < NS) mv_products<NS, I, J + 1>(d, base, off, idesc, more);
     else if constexpr (I + 1 < NS) mv_products<NS, I + 1, 0>(d, base, off, idesc, more);
+}
+
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+    const float t = __fadd_rn(a, b), bb = __fsub_rn(t, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, bb)), __fsub_rn(b, bb));
+    s = t;
+}
+// x 2^e, by the bits (the conversion instruction runs at the FP64 rate); 0 below 2^-126
+__device__ __forceinline__ double scaled_double(float x, int e) {
+    const uint32_t b = __float_as_uint(x), m = b & 0x7FFFFFFFu;
+    const bool zero = m < 0x00800000u;
+    const uint32_t hi = (b & 0x80000000u) | ((m >> 3) + ((uint32_t)(896 + e) << 20));
+    return __hiloint2double(zero ? 0 : (int)hi, zero ? 0 : (int)(b << 29));
 }
 
 template <int NS>
@@ -820,99 +838,155 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
             const int sl = inside ? s : 0;
             const float dsc = pow2f(a.colexp[sl] - (NS == 3 ? 30 : 0));
             const uint32_t col0 = tmem + ((uint32_t)(quarter * 32) << 16) + buf * (Sh::NA * N) + part * kCols;
+            auto load2 = [&](int k0, int k1, int c, float (&y)[16], float (&z)[16]) {   // two accumulators' 16 columns
+                uint32_t r[2][16];
+                tmem_ld16_async(col0 + k0 * N + c, r[0]);
+                tmem_ld16_async(col0 + k1 * N + c, r[1]);
+                tmem_wait_ld(r[0]);
+                tmem_wait_ld(r[1]);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    y[i] = __uint_as_float(r[0][i]);
+                    z[i] = __uint_as_float(r[1][i]);
+                }
+            };
             df tot{0.0f, 0.0f};
             double tot64 = 0.0;
-            // the columns of this warp, 16 at a time and without branches over them (padding
-            // rows are 0), so that their chains overlap; MAT: maturity payments
+            auto release = [&] {   // the accumulators are read
+                fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_remote(acc_free[buf]);
+            };
+            // the columns of this warp, without branches over them (padding rows are 0), so that
+            // their chains overlap; MAT: maturity payments
             auto columns = [&](auto with_maturity) {
                 constexpr bool MAT = decltype(with_maturity)::value;
+                auto emit = [&](const MvOut& q, float h, float l) {   // of a policy's sum h + l
+                    df v = df_mul(df{__fmul_rn(h, dsc), __fmul_rn(l, dsc)}, df{q.sc_h, q.sc_l});
+                    const int pol = q.pol;
+                    bool due = false;
+                    if constexpr (MAT) {   // a maturity payment, of the same sign, or 0
+                        const float2 d = a.D[(size_t)max(q.S - 1, 0) * a.s_pad + sl];
+                        due = q.S == 0;
+                        const df m = df_mul(df{q.mat_h, q.mat_l}, due ? df{1.0f, 0.0f} : df{d.x, d.y});
+                        const float sum = __fadd_rn(v.h, m.h), bb = __fsub_rn(sum, v.h);
+                        const float e = __fadd_rn(__fsub_rn(v.h, __fsub_rn(sum, bb)), __fsub_rn(m.h, bb));
+                        v = df{sum, __fadd_rn(e, __fadd_rn(v.l, m.l))};
+                        due = due && q.mat_h != 0.0f;
+                    }
+                    // the sum over the policies
+                    const float sum = __fadd_rn(tot.h, v.h), bb = __fsub_rn(sum, tot.h);
+                    const float e = __fadd_rn(__fsub_rn(tot.h, __fsub_rn(sum, bb)), __fsub_rn(v.h, bb));
+                    tot = df{sum, __fadd_rn(tot.l, __fadd_rn(e, v.l))};
+                    const size_t o = (size_t)pol * a.v0_ld + s;
+                    if (live && pol >= 0) {
+                        if (a.V0f) a.V0f[o] = __fadd_rn(v.h, v.l);
+                        if (a.V0d) a.V0d[o] = due ? a.amount[pol] : (double)v.h + (double)v.l;
+                    }
+                };
+                // Columns whose accumulators are added before they are released: as little as
+                // fits the registers, since with one item in TMEM the products stand still until then.
+                constexpr int kHold = NS == 4 ? kCols : 16;
 #pragma unroll 1
-                for (int c = 0; c < kCols; c += 16) {
-                    auto release = [&] {   // the accumulators are read
-                        if (c != kCols - 16) return;
-                        fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive_remote(acc_free[buf]);
-                    };
-                    if constexpr (NS == 8) {   // added in FP64, the smallest first
-                        double u[16];
+                for (int c0 = 0; c0 < kCols; c0 += kHold) {
+                    if constexpr (NS == 8) {
+                        // u = a0 + w + v + x: the levels from 2^-32 of the first as plain FP32
+                        // sums (2^-56), the others' errors kept; the rest after the release
+                        float p[16], w[16], v[16], x[16];
+                        {
+                            float y[16], z[16];
+                            load2(7, 6, c0, y, z);
 #pragma unroll
-                        for (int k = Sh::NA - 1; k >= 0; --k) {
-                            uint32_t r[16];
-                            tmem_ld16_async(col0 + k * N + c, r);
-                            tmem_wait_ld(r);
+                            for (int i = 0; i < 16; ++i) x[i] = __fadd_rn(y[i], z[i]);
+                            load2(5, 4, c0, y, z);
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) x[i] = __fadd_rn(z[i], __fadd_rn(y[i], x[i]));
+                            load2(3, 2, c0, y, z);
 #pragma unroll
                             for (int i = 0; i < 16; ++i) {
-                                const double x = (double)__uint_as_float(r[i]);
-                                u[i] = k == Sh::NA - 1 ? x : __dadd_rn(u[i], x);
+                                two_sum(y[i], x[i], v[i], x[i]);
+                                w[i] = z[i];
+                            }
+                            load2(1, 0, c0, y, p);
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) {
+                                float e;
+                                two_sum(y[i], w[i], w[i], e);
+                                x[i] = __fadd_rn(x[i], e);
                             }
                         }
                         release();
-                        const double scale = __hiloint2double((a.colexp[sl] + 1023) << 20, 0);
+                        const int ce = a.colexp[sl];
 #pragma unroll
                         for (int i = 0; i < 16; ++i) {
-                            const MvOut64& q = reinterpret_cast<const MvOut64&>(recs[part * kCols + c + i]);
-                            double v = __dmul_rn(__dmul_rn(u[i], scale), q.sc);
+                            const MvOut64& q = reinterpret_cast<const MvOut64&>(recs[part * kCols + c0 + i]);
+                            float e;
+                            two_sum(p[i], w[i], p[i], w[i]);
+                            two_sum(w[i], v[i], w[i], e);
+                            x[i] = __fadd_rn(x[i], e);
+                            // of the FP64 pipe (1/64 of the FP32 rate) only what needs 53 bits
+                            double t = __dadd_rn(scaled_double(w[i], ce), scaled_double(x[i], ce));
+                            t = __dmul_rn(__dadd_rn(scaled_double(p[i], ce), t), q.sc);
                             if constexpr (MAT) {
                                 const double d = q.S > 0 ? a.D64[(size_t)(q.S - 1) * a.s_pad + sl] : 1.0;
-                                v = __fma_rn(q.mat, d, v);
+                                t = __fma_rn(q.mat, d, t);
                             }
-                            tot64 = __dadd_rn(tot64, v);
+                            tot64 = __dadd_rn(tot64, t);
                             if (live && q.pol >= 0) {
                                 const size_t o = (size_t)q.pol * a.v0_ld + s;
-                                if (a.V0f) a.V0f[o] = __double2float_rn(v);
-                                if (a.V0d) a.V0d[o] = v;
+                                if (a.V0f) a.V0f[o] = __double2float_rn(t);
+                                if (a.V0d) a.V0d[o] = t;
                             }
                         }
                         continue;
                     }
-                    // the accumulators' sums as double-floats, the largest first
-                    float h[16], l[16];
-                    uint32_t r[2][16];
-                    tmem_ld16_async(col0 + c, r[0]);
+                    // the accumulators' sum as a double-float: the errors of adding the first
+                    // ones are kept; those from 2^-24 (four digits: 2^-16) of the first are
+                    // added as they are, 2^-48 (2^-40)
+                    float h[kHold], l[kHold];
 #pragma unroll
-                    for (int k = 0; k < Sh::NA; ++k) {
-                        tmem_wait_ld(r[k & 1]);
-                        if (k + 1 < Sh::NA) tmem_ld16_async(col0 + (k + 1) * N + c, r[(k + 1) & 1]);
-                        else release();
+                    for (int c = 0; c < kHold; c += 16) {
+                        float y[16], z[16], x[16];
+                        if constexpr (NS == 6) {
+                            load2(5, 4, c0 + c, y, z);
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            const float b = __uint_as_float(r[k & 1][i]);
-                            if (k == 0) {
-                                h[i] = b;
-                                l[i] = 0.0f;
-                            } else {
-                                const float sum = __fadd_rn(h[i], b), bb = __fsub_rn(sum, h[i]);
-                                l[i] = __fadd_rn(l[i], __fadd_rn(__fsub_rn(h[i], __fsub_rn(sum, bb)), __fsub_rn(b, bb)));
-                                h[i] = sum;
+                            for (int i = 0; i < 16; ++i) x[i] = __fadd_rn(y[i], z[i]);
+                            load2(3, 2, c0 + c, y, z);
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) l[c + i] = __fadd_rn(y[i], x[i]);
+                            load2(1, 0, c0 + c, y, x);
+                            release();
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) {
+                                float e1, e2;
+                                two_sum(x[i], y[i], x[i], e1);
+                                two_sum(x[i], z[i], h[c + i], e2);
+                                l[c + i] = __fadd_rn(l[c + i], __fadd_rn(e1, e2));
                             }
+                        } else if constexpr (NS == 4) {
+                            load2(3, 2, c0 + c, y, z);
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) x[i] = __fadd_rn(y[i], z[i]);
+                            load2(1, 0, c0 + c, y, z);
+                            if (c0 + c == kCols - 16) release();
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) {
+                                two_sum(z[i], y[i], h[c + i], l[c + i]);
+                                l[c + i] = __fadd_rn(l[c + i], x[i]);
+                            }
+                        } else {
+                            uint32_t r[2][16];
+                            tmem_ld16_async(col0 + c0, r[0]);
+                            tmem_ld16_async(col0 + N + c0, r[1]);
+                            tmem_wait_ld(r[0]);
+                            tmem_wait_ld(r[1]);
+                            if (c0 == kCols - 16) release();
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) two_sum(__uint_as_float(r[0][i]), __uint_as_float(r[1][i]), h[i], l[i]);
                         }
                     }
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const MvOut& q = recs[part * kCols + c + i];
-                        df v = df_mul(df{__fmul_rn(h[i], dsc), __fmul_rn(l[i], dsc)}, df{q.sc_h, q.sc_l});
-                        const int pol = q.pol;
-                        bool due = false;
-                        if constexpr (MAT) {   // a maturity payment, of the same sign, or 0
-                            const float2 d = a.D[(size_t)max(q.S - 1, 0) * a.s_pad + sl];
-                            due = q.S == 0;
-                            const df m = df_mul(df{q.mat_h, q.mat_l}, due ? df{1.0f, 0.0f} : df{d.x, d.y});
-                            const float sum = __fadd_rn(v.h, m.h), bb = __fsub_rn(sum, v.h);
-                            const float e = __fadd_rn(__fsub_rn(v.h, __fsub_rn(sum, bb)), __fsub_rn(m.h, bb));
-                            v = df{sum, __fadd_rn(e, __fadd_rn(v.l, m.l))};
-                            due = due && q.mat_h != 0.0f;
-                        }
-                        // the sum over the policies
-                        const float sum = __fadd_rn(tot.h, v.h), bb = __fsub_rn(sum, tot.h);
-                        const float e = __fadd_rn(__fsub_rn(tot.h, __fsub_rn(sum, bb)), __fsub_rn(v.h, bb));
-                        tot = df{sum, __fadd_rn(tot.l, __fadd_rn(e, v.l))};
-                        const size_t o = (size_t)pol * a.v0_ld + s;
-                        if (live && pol >= 0) {
-                            if (a.V0f) a.V0f[o] = __fadd_rn(v.h, v.l);
-                            if (a.V0d) a.V0d[o] = due ? a.amount[pol] : (double)v.h + (double)v.l;
-                        }
-                    }
+                    for (int i = 0; i < kHold; ++i) emit(recs[part * kCols + c0 + i], h[i], l[i]);
                 }
             };
             const int kind = a.kinds ? a.kinds[tile] : K_ANN;

@@ -20,8 +20,9 @@
 // and 2^-16 below, are multiples of 2^-22 and 2^-30 and have an exact accumulator each; the
 // rest shares one more, whose FP32 truncations (of a sum 2^-24, with three digits 2^-8,
 // below) are that much smaller.  With six and eight every level has its own.  The epilogue
-// adds the accumulators as double-floats (FP64 form: in FP64).  A maturity payment is added
-// there, from the discount products themselves, so that a row holds entries of one kind.
+// adds the accumulators: the first ones with their rounding errors, the low ones as they
+// are (to 2^-40, 2^-48 and 2^-56 with four, six and eight digits).  A maturity payment is
+// added there, from the discount products themselves, so that a row holds entries of one kind.
 //
 // Fixed point needs rows and columns of moderate range.  The discount products are
 // tilted by a power of two per step, 2^tau(t) ~ 1 / (their geometric mean over the
@@ -31,11 +32,11 @@
 // mv_max_spread) keeps the recurrence kernels.
 //
 // Measured (one GB300, with the digits and the totals), before: the recurrence.
-//   100,000 policies of every product, 1,000 scenarios: compensated 38.7 -> 1.70 ms
-//   (annuities 1e-13 -> 1.4e-14 rms, assurances 4e-9 -> 1.5e-14), deflated 4.93 -> 0.91 ms
+//   100,000 policies of every product, 1,000 scenarios: compensated 38.7 -> 1.62 ms
+//   (annuities 1e-13 -> 1.5e-14 rms, assurances 4e-9 -> 1.7e-14), deflated 4.93 -> 0.89 ms
 //   (rms 3e-8 -> 5e-9, with three digits 0.62 ms);
 //   1,000,000 annuities, 600 steps, 1,000 scenarios, deflated: 30.6 -> 4.3 ms;
-//   3,000 two-life policies, 333 scenarios, FP64: 5.17 -> 0.21 ms (1.4e-15 -> 1.3e-15).
+//   3,000 two-life policies, 333 scenarios, FP64: 5.17 -> 0.15 ms (1.4e-15 -> 1.3e-15).
 // It is the faster path at every size measured: one policy and one scenario 53 -> 49 us
 // compensated and 158 -> 37 us deflated (host call included), 1,000 policies under 157
 // scenarios of the mix 276 -> 102 us and 282 -> 63 us.
