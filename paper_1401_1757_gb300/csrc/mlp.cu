@@ -70,15 +70,14 @@ __global__ void __launch_bounds__(256) head_train_kernel(const float* __restrict
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     float w[8], dw[8] = {}, db[8] = {}, sdy = 0.0f, sq = 0.0f;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) w[j] = w5[lane * 4 + (j & 3) + (j >> 2) * 128];
+    for (int j = 0; j < 8; ++j) w[j] = w5[lane + 32 * j];
     const int r0 = blockIdx.x * kHeadRows;
     for (int r = r0 + warp; r < min(B, r0 + kHeadRows); r += 8) {
-        const float4* row = reinterpret_cast<const float4*>(Z4 + (size_t)r * MLP_H);
-        const float4 q[2] = {row[lane], row[lane + 32]};
-        const float z[8] = {q[0].x, q[0].y, q[0].z, q[0].w, q[1].x, q[1].y, q[1].z, q[1].w};
-        float a[8], g[8], s = 0.0f;
+        float z[8], a[8], s = 0.0f;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < 8; ++j) z[j] = Z4[(size_t)r * MLP_H + lane + 32 * j];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {   // in head_fwd_kernel's order: the same y
             a[j] = gelu_f(z[j]);
             s += a[j] * w[j];
         }
@@ -91,22 +90,17 @@ __global__ void __launch_bounds__(256) head_train_kernel(const float* __restrict
         sq += e * e;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            g[j] = dy * w[j] * gelu_grad_f(z[j]);
+            const float g = dy * w[j] * gelu_grad_f(z[j]);
+            const size_t o = (size_t)r * MLP_H + lane + 32 * j;
             dw[j] += dy * a[j];
-            db[j] += g[j];
-        }
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const size_t o = (size_t)r * MLP_H + h * 128 + lane * 4;
-            const __nv_bfloat162 p[2] = {__floats2bfloat162_rn(g[4 * h], g[4 * h + 1]),
-                                         __floats2bfloat162_rn(g[4 * h + 2], g[4 * h + 3])};
-            *reinterpret_cast<uint2*>(dZb + o) = *reinterpret_cast<const uint2*>(p);
-            if (dZf) *reinterpret_cast<float4*>(dZf + o) = make_float4(g[4 * h], g[4 * h + 1], g[4 * h + 2], g[4 * h + 3]);
+            db[j] += g;
+            dZb[o] = __float2bfloat16_rn(g);
+            if (dZf) dZf[o] = g;
         }
     }
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-        const int k = lane * 4 + (j & 3) + (j >> 2) * 128;
+        const int k = lane + 32 * j;
         red[warp][k] = dw[j];
         red[warp][MLP_H + k] = db[j];
     }
