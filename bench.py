@@ -102,8 +102,36 @@ def algorithmic_flops(pol, n_scen, horizon=0):
     return float(sum(ALGO_FLOPS[p] * cs[p] for p in cs) * n_scen)
 
 
-def issued_flops(pol, form, n_scen, horizon=0, variant_name=""):
+def is_matrix(variant_name):
+    """The valuation as a matrix product of split operands on the tensor cores."""
+    return " matrix " in variant_name
+
+
+def matrix_digits(form, v):
+    """The digits that the matrix product splits its operands in (csrc/matval.cuh): in the
+    deflated form three up to a spread of 4 of the scenario set, then four."""
+    if form != "f32defl":
+        return {"f32comp": 6, "f64": 8}[form]
+    D = np.cumprod(v, axis=1)
+    e = np.frexp(D * np.exp2(-np.round(np.log2(D).mean(axis=0))))[1]
+    return 3 if int((e.max(axis=1) - e.min(axis=1)).max()) <= 4 else 4
+
+
+def matrix_launches(pol, form, v, horizon):
+    """Kernels of a matrix valuation: a builder and a product for each 1 GiB of the cash flows' digits
+    and the totals' reduction."""
+    d = matrix_digits(form, v)
+    S = int(projection_steps(pol, horizon=horizon).max())
+    tile = d * 128 * ((S + 63) // 64 * 64) * 2
+    tiles = sum(-(-int((pol["product"] == p).sum()) // 128) for p in np.unique(pol["product"]))
+    return 2 * -(-tiles // max(1, (1 << 30) // tile)) + 1
+
+
+def issued_flops(pol, form, n_scen, horizon=0, variant_name="", v=None):
     cs = chain_steps_by_product(pol, horizon)
+    if is_matrix(variant_name):   # the products of digits i and j, i + j below their number
+        d = matrix_digits(form, v)
+        return float(d * (d + 1) * sum(cs.values()) * n_scen)
     per = dict(ISSUED_FLOPS[form])
     if form == "f32defl":
         if variant_name.endswith(" tm2"):   # one fold per 32 steps: 2 x 30 + the spans' add (2) + join and fold (7)
@@ -125,9 +153,11 @@ def kernel_source_hash(form=HEAD):
     return h.hexdigest()[:16]
 
 
-def measured_traffic(form, workload_key):
+def measured_traffic(form, workload_key, variant=""):
     """DRAM bytes per launch of a form's kernel on a workload, from the
     committed ncu summary, if it was taken on the current kernel source."""
+    if is_matrix(variant):   # no capture of its kernels at this size
+        return None
     path = os.path.join(ROOT, "profiles", "recur_traffic.json")
     try:
         d = json.load(open(path))
@@ -286,8 +316,7 @@ def bench_nested(rsv, torch, tab, steps, warmup, n_outer=None, sur_epochs=10, su
 def bench_cashflows(rsv, torch, ctx, fid, level_ms, steps, warmup, flush):
     """The main workload with the paper's payment mix (Section 5: about 80%
     monthly and 20% annual payments, 5% escalating at 3%, 4.25% or 5% on each
-    anniversary), expanded on the device and valued by the general-cash-flow
-    kernel; against the level cash flows of the timed step."""
+    anniversary), expanded on the device, in the default variant; against the level cash flows of the timed step."""
     n_pol, n_scen, n_steps = C2["n_pol"], C2["n_scen"], C2["n_steps"]
     sch = synth.payment_schedules(n_pol, seed=0)
     rsv.rsv_load_schedules(ctx, sch, n_steps)
@@ -306,7 +335,7 @@ def bench_cashflows(rsv, torch, ctx, fid, level_ms, steps, warmup, flush):
     return {"workload": C2_WORKLOAD + "; payment schedules: 80% monthly / 20% annual, 5% escalating",
             "kernel_ms": t, "valuations_s": n_pol * n_scen / (t / 1e3), "level_kernel_ms": level_ms,
             "cost_vs_level": t / level_ms,
-            "variant": "general cash flows (unshifted states, c_t per policy and step)"}
+            "variant": rsv.rsv_variant_name(fid, rsv.rsv_variant_count(fid) - 1) + ", general cash flows c_t"}
 
 
 # Operations per chain-step of the m-life kernel (m lives; FMA = 2): each of
@@ -367,8 +396,11 @@ def bench_mlife(rsv, torch, tab, n_pol=20_000, reps=3):
             rsv.rsv_compute_mlife(ctx, pol, fid, rsv.RSV_OUT_V0, on_device=True, V0=V0)
             ms.append(rsv.rsv_last_kernel_ms(ctx))
         t = statistics.mean(ms) / 1e3
-        flops = sum(mlife_flops(form, int(pol["m"][i]), pol["kind"][i] == 1, int(pol["k"][i])) * int(S[i])
-                    for i in range(n_pol)) * C2["n_scen"]
+        if form == "f32comp":   # the matrix product: 21 products of 16-bit digits a month
+            flops = 42.0 * float(S.sum()) * C2["n_scen"]
+        else:
+            flops = sum(mlife_flops(form, int(pol["m"][i]), pol["kind"][i] == 1, int(pol["k"][i])) * int(S[i])
+                        for i in range(n_pol)) * C2["n_scen"]
         res[form] = {"ms": t * 1e3, "valuations_s": n_pol * C2["n_scen"] / t, "flops_per_launch": flops,
                      "achieved_tflops": flops / t / 1e12}
     rsv.rsv_destroy(ctx)
@@ -605,7 +637,7 @@ def time_form(rsv, torch, ctx, form, V0, tot, horizon, steps, warmup, flush, str
     if tune:
         best, tune_ms = rsv.rsv_tune(ctx, fid, horizon=horizon, reps=1)
     else:
-        best = 0
+        best = 0 if form == "f32" else rsv.rsv_variant_count(fid) - 1   # the default
     world = part.world if part else 1
     for _ in range(warmup):
         rsv.rsv_compute_reserves(ctx, fid, outs, horizon=horizon, on_device=True, V0=V0, scen_total=tot)
@@ -679,7 +711,7 @@ def bench_forms(rsv, torch, ctx, pol, tab, v, forms, horizon, steps, warmup, flu
         r["chain_steps_s"] = world * cs / t
         kt = r["kernel_ms"] / 1e3
         r["algorithmic_tflops"] = algorithmic_flops(pol, n_scen, horizon) / kt / 1e12
-        r["issued_tflops"] = issued_flops(pol, form, n_scen, horizon, r["variant"]) / kt / 1e12
+        r["issued_tflops"] = issued_flops(pol, form, n_scen, horizon, r["variant"], v) / kt / 1e12
         results[form] = r
     del V0
     if n_sample > 0:
@@ -943,26 +975,31 @@ def main():
         extras["cpu_oracle_full"] = cpu_full_configs(tab, args.cpu_runs, args.cpu_full)
     for f, r in results.items():
         pk = peaks["fp64_fma_tflops"] if f == "f64" else peaks["fp32_fma_tflops"]
+        if is_matrix(r["variant"]):
+            mp = measured_peaks()
+            r["issued_frac_of_measured_peak"] = r["issued_tflops"] / mp["bf16_tflops"] if mp else None
+            continue
         r["algorithmic_frac_of_measured_peak"] = r["algorithmic_tflops"] / pk
         r["issued_frac_of_measured_peak"] = r["issued_tflops"] / pk
     if "mlife" in extras:
         m = extras["mlife"]
-        m["f32comp"]["frac_of_measured_fp32_fma_peak"] = m["f32comp"]["achieved_tflops"] / peaks["fp32_fma_tflops"]
+        mp = measured_peaks()
+        m["f32comp"]["frac_of_measured_bf16_burst_peak"] = m["f32comp"]["achieved_tflops"] / mp["bf16_tflops"] if mp else None
         m["f64"]["frac_of_measured_fp64_fma_peak"] = m["f64"]["achieved_tflops"] / peaks["fp64_fma_tflops"]
     if "config2" in extras:
         for f, r in extras["config2"].items():
-            if isinstance(r, dict) and "algorithmic_tflops" in r:
+            if isinstance(r, dict) and "algorithmic_tflops" in r and not is_matrix(r["variant"]):
                 pk = peaks["fp64_fma_tflops"] if f == "f64" else peaks["fp32_fma_tflops"]
                 r["algorithmic_frac_of_measured_peak"] = r["algorithmic_tflops"] / pk
 
     h = results[head]
     n_scen = v.shape[0]
     flops = algorithmic_flops(pol, n_scen, horizon)
-    ifl = issued_flops(pol, head, n_scen, horizon, h["variant"])
+    ifl = issued_flops(pol, head, n_scen, horizon, h["variant"], v)
     kt = h["kernel_ms"] / 1e3
     roof = {"bound": "alu", "achieved": flops / kt / 1e12, "peak": FP32_PEAK_TFLOPS, "unit": "TFLOP/s",
             "frac": flops / kt / 1e12 / FP32_PEAK_TFLOPS,
-            "traffic": measured_traffic(head, "c5A") if full else None,
+            "traffic": measured_traffic(head, "c5A", h["variant"]) if full else None,
             "kernel": f"defl_kernel ({h['variant']}) with its deflator-plane pass" if head == "f32defl" else
                       f"recur_kernel ({h['variant']})",
             "flops_per_launch": flops,
@@ -971,6 +1008,17 @@ def main():
             "frac_of_measured_fma_peak": flops / kt / 1e12 / peaks["fp32_fma_tflops"],
             "issued_flops_per_launch": ifl, "issued_frac": ifl / kt / 1e12 / FP32_PEAK_TFLOPS,
             "issued_count": "FP32 operations the kernel issues per chain-step (FMA 2, others 1)"}
+    if is_matrix(h["variant"]):
+        mp = measured_peaks()
+        roof.update({"bound": "tensor", "achieved": ifl / kt / 1e12, "peak": mp["bf16_tflops"] if mp else None,
+                     "frac": ifl / kt / 1e12 / mp["bf16_tflops"] if mp else None,
+                     "kernel": f"mv_build_kernel and mv_product_kernel ({h['variant']})",
+                     "count": f"16-bit products of {matrix_digits(head, v)} digits: 2 flop each, every chain-step",
+                     "peak_note": "measured cuBLAS BF16 burst rate",
+                     "algorithmic_tflops": flops / kt / 1e12})
+        for k in ("frac_of_measured_fma_peak", "issued_flops_per_launch", "issued_frac", "issued_count"):
+            roof.pop(k)
+        roof["flops_per_launch"] = ifl
     line = {
         "metric": METRIC, "value": h["valuations_s"], "unit": "valuations/s", "n_gpus": world,
         "steps": h["steps"], "warmup": args.warmup, "ms_per_step": h["ms_per_step"], "higher_is_better": True,
@@ -983,7 +1031,8 @@ def main():
         "roofline": roof,
         "cpu_baseline": cpu,
         "e2e": e2e,
-        "gpu_launches": (4 if head == "f32defl" else 3) * h["steps"],
+        "gpu_launches": (matrix_launches(pol, head, v, horizon) if is_matrix(h["variant"]) else
+                         4 if head == "f32defl" else 3) * h["steps"],
         "clocks": clocks,
         "forms": results,
         "measured_alu_peaks": peaks,
