@@ -101,8 +101,9 @@ enum {
  * compensated: 48 bits, error about 1e-13; deflated: 32 bits, within the bound below).  Data
  * outside its range keeps the recurrence kernels: scenarios whose discount products
  * leave their mean by more than a factor of about 2^10 (FP64 and deflated 2^8), survival
- * below 2^-100, amounts outside 2^-60 .. 2^90.  It is the last of a form's tunable
- * variants. */
+ * below 2^-100, amounts outside 2^-60 .. 2^90, cash-flow multipliers whose products with
+ * survival and mean discount leave 2^-100 .. 2^100 (compensated and deflated: with the
+ * amounts, 2^-90 .. 2^110).  It is the last of a form's tunable variants. */
 
 /* RSV_FORM_F32_DEFLATED.  Eq. (generalForm) multiplied at step t by the
  * deflator G_t = D_t l_{x+t} / l_x (D_t = v_0 ... v_{t-1}, the discount-factor

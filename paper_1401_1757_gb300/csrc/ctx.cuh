@@ -216,11 +216,13 @@ struct rsv_ctx {
     DevBuf d_cf64, d_cf32;                          //   FP64 rows and their FP32 copy
     std::vector<unsigned char> cf_level;            //   per policy: 1 = the row is all ones
     unsigned long long cf_gen = 1;
+    double cf_lo = 1.0, cf_hi = 1.0;                //   smallest multiplier that is not 0 and largest
     DevBuf d_ml_rec, d_ml_amount;                   // m-life records of the last call
 
     // the valuation as a matrix product (matval.cuh): whether the scenario set, the tables and
     // the amounts are in its range, the discount products and their digits per digit count
     int mv_spread = 0x7fffffff;   // of the scenario set (mv_max_spread)
+    int mv_tilt = 0x7fffffff;     // its largest |tau|
     double tab_min[rsv::kMaxTables] = {};           // smallest survivor-column entry of a table
     double amt_lo = 0.0, amt_hi = 0.0;              // smallest non-zero and largest |amount|
     DevBuf d_mv_D, d_mv_col, d_mv_D64, d_mv_dig[4], d_mv_E, d_mv_out;
@@ -294,7 +296,8 @@ rsv_status stage_tables(rsv_ctx* c, int form, int pad, int n_tab, size_t& smem);
 // Whether the matrix product covers the loaded data; then, on the layout of width
 // kMvP: mv_prepare once a call, mv_launch for the scenario columns [s0, s0 + w) with the
 // output pointers at column s0 (partial: [mv_part_rows][s_pad]).
-rsv_status mv_applies(rsv_ctx* c, int form, double amt_lo, double amt_hi, bool& applies);
+// cf: the rows take the loaded cash-flow multipliers.
+rsv_status mv_applies(rsv_ctx* c, int form, double amt_lo, double amt_hi, bool cf, bool& applies);
 rsv_status mv_prepare(rsv_ctx* c, int form);
 // Its parts, for rows that come from elsewhere (m lives): the scenario set's digits, the tiles
 // of a panel and their buffers (d_mv_E, d_mv_out), and the product of a built panel

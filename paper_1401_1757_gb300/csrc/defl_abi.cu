@@ -126,7 +126,7 @@ rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     }
     bool mat = false;
     if (vi == nv) {
-        const rsv_status mst = mv_applies(c, F_DEFL, c->amt_lo, c->amt_hi, mat);
+        const rsv_status mst = mv_applies(c, F_DEFL, c->amt_lo, c->amt_hi, false, mat);
         if (mst != RSV_OK) return mst;
     }
     const bool by_index = o->variant >= 0 && o->variant < nv;

@@ -53,8 +53,12 @@ constexpr int kMvM = 128;          // scenarios per tile (MMA M)
 constexpr int kMvParts = 4;        // column groups of the epilogue
 constexpr int kMvTilt = 60;        // largest |tau|
 constexpr size_t kMvPanelBytes = size_t(1) << 30;            // cash-flow digits held at a time
-constexpr double kMvTableMin = 0x1p-100;                    // survivor columns in FP32 head and tail
-constexpr double kMvAmountMin = 0x1p-60, kMvAmountMax = 0x1p90;   // |amount|: V in FP32 head and tail
+// A row's entries, survivor-column entry times cash-flow multiplier times tilt, are formed in FP32
+// head and tail (in the FP64 form their heads, for the row's scale), and a row's scale times its
+// amount is one too; beyond these an exponent would be clamped or a tail lost.
+constexpr double kMvEntryMin = 0x1p-100, kMvEntryMax = 0x1p100;
+constexpr double kMvScaleMin = 0x1p-90, kMvScaleMax = 0x1p110;
+constexpr double kMvAmountMin = 0x1p-60, kMvAmountMax = 0x1p90;   // |amount|
 
 // The spread of a scenario set: the largest difference of the binary exponents of a scenario's
 // tilted discount products (Vasicek paths, sd of the rate 2.2%: 3 to 5 over 50 years, 5 to 7

@@ -318,7 +318,7 @@ extern "C" rsv_status rsv_compute_mlife(rsv_ctx* c, const rsv_mlife_policy* pols
         if (v > 0.0) amt_lo = std::min(amt_lo, v);
     }
     bool mat = false;
-    if (o->form == F_COMP && n > 0 && (st = mv_applies(c, F_COMP, amt_lo, amt_hi, mat)) != RSV_OK) return st;
+    if (o->form == F_COMP && n > 0 && (st = mv_applies(c, F_COMP, amt_lo, amt_hi, false, mat)) != RSV_OK) return st;
     if (mat) return mlife_matrix(c, pols, recs, ms, o, out);
     if ((st = stage_tables(c, o->form, pad, n_tab, smem)) != RSV_OK) return st;
 

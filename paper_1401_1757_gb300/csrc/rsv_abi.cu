@@ -68,17 +68,27 @@ __global__ void schedule_kernel(const rsv_schedule* __restrict__ sch, int64_t n_
     }
 }
 
-// Per policy: 1 if its cash-flow row is all ones (level), one warp per row.
+// Per policy: 1 if its cash-flow row is all ones (level), one warp per row; and the smallest
+// that is not 0 and the largest of all multipliers (range[0], which starts at ~0, and
+// range[1], at 0), as their bits, which sort like the numbers (>= 0).
 __global__ void cf_level_kernel(const double* __restrict__ cf, int64_t n_pol, int n_steps,
-                                unsigned char* __restrict__ level) {
+                                unsigned char* __restrict__ level, unsigned long long* __restrict__ range) {
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x / 32);
+    double lo = INFINITY, hi = 0.0;
     for (int64_t p = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; p < n_pol; p += warps) {
         bool one = true;
-        for (int t = lane; t < n_steps; t += 32) one &= cf[(size_t)p * n_steps + t] == 1.0;
+        for (int t = lane; t < n_steps; t += 32) {
+            const double x = cf[(size_t)p * n_steps + t];
+            one &= x == 1.0;
+            if (x > 0.0) lo = fmin(lo, x);
+            hi = x >= 0.0 ? fmax(hi, x) : INFINITY;   // a schedule may overflow to NaN
+        }
         one = __all_sync(0xffffffffu, one);
         if (lane == 0) level[p] = one ? 1 : 0;
     }
+    atomicMin(&range[0], (unsigned long long)__double_as_longlong(lo));
+    atomicMax(&range[1], (unsigned long long)__double_as_longlong(hi));
 }
 
 const Variant* variant_list(int form, int* n) {
@@ -645,11 +655,20 @@ rsv_status upload_amounts(rsv_ctx* c) {
 
 }  // namespace
 
-rsv_status rsv::mv_applies(rsv_ctx* c, int form, double amt_lo, double amt_hi, bool& applies) {
+rsv_status rsv::mv_applies(rsv_ctx* c, int form, double amt_lo, double amt_hi, bool cf, bool& applies) {
     applies = false;
     if (!(amt_hi <= kMvAmountMax) || !(amt_lo >= kMvAmountMin)) return RSV_OK;
+    // the smallest and largest entries of a row, but for the tilt
+    double lo = 1.0, hi = 1.0;
+    if (cf && c->cf_pol > 0) {
+        lo = std::min(lo, c->cf_lo);
+        hi = std::max(hi, c->cf_hi);
+    }
+    double tab_min = 1.0;
     for (int t = 0; t < kMaxTables; ++t)
-        if (!c->tab[t].empty() && !(c->tab_min[t] >= kMvTableMin)) return RSV_OK;
+        if (!c->tab[t].empty()) tab_min = std::min(tab_min, c->tab_min[t]);
+    lo *= tab_min;
+    if (!(lo >= kMvEntryMin) || !(hi <= kMvEntryMax)) return RSV_OK;
     if (c->mv_range_gen != c->scen_gen) {
         // the discount products and their range, with the scenario set's first use here (a
         // quarter of the load's time, which the other forms and the time scan need not pay)
@@ -662,9 +681,14 @@ rsv_status rsv::mv_applies(rsv_ctx* c, int form, double amt_lo, double amt_hi, b
         CU(cudaMemcpyAsync(range, mv.stat, sizeof range, cudaMemcpyDeviceToHost, c->stream));
         CU(cudaStreamSynchronize(c->stream));
         c->mv_spread = range[1] <= kMvTilt ? range[0] : INT_MAX;
+        c->mv_tilt = range[1];
         c->mv_range_gen = c->scen_gen;
     }
-    applies = c->mv_spread <= mv_max_spread(form);
+    if (c->mv_spread > mv_max_spread(form)) return RSV_OK;
+    lo = std::ldexp(lo, -c->mv_tilt);
+    hi = std::ldexp(hi, c->mv_tilt);
+    applies = lo >= kMvEntryMin && hi <= kMvEntryMax &&
+              (form == F_F64 || (amt_lo * lo >= kMvScaleMin && amt_hi * hi <= kMvScaleMax));
     return RSV_OK;
 }
 
@@ -847,7 +871,7 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
         return fail(c, RSV_E_ARG, "variant %d out of range", o->variant);
     }
     if (o->form != F_F32 && vi == nt && !extra && !scan && !summ && pay == PAY_END) {
-        const rsv_status mst = mv_applies(c, o->form, c->amt_lo, c->amt_hi, mat);
+        const rsv_status mst = mv_applies(c, o->form, c->amt_lo, c->amt_hi, true, mat);
         if (mst != RSV_OK) return mst;
         vi = 0;
     }
@@ -1397,13 +1421,20 @@ rsv_status rsv_load_scenarios_fraction(rsv_ctx* c, const double* v, int32_t n_sc
 
 // The level flags of freshly written rows (device FP64) and the new generation.
 static rsv_status finish_cashflows(rsv_ctx* c, int64_t n_pol, int32_t n_steps) {
-    CU(c->d_vstage.ensure((size_t)n_pol));
-    cf_level_kernel<<<c->sm_count * 8, 256, 0, c->stream>>>(c->d_cf64.as<double>(), n_pol, n_steps,
-                                                            c->d_vstage.as<unsigned char>());
+    unsigned long long range[2];
+    CU(c->d_vstage.ensure(sizeof range + (size_t)n_pol));
+    unsigned char* level = c->d_vstage.as<unsigned char>() + sizeof range;
+    CU(cudaMemsetAsync(c->d_vstage.p, 0xff, sizeof range[0], c->stream));
+    CU(cudaMemsetAsync(c->d_vstage.as<unsigned long long>() + 1, 0, sizeof range[1], c->stream));
+    cf_level_kernel<<<c->sm_count * 8, 256, 0, c->stream>>>(c->d_cf64.as<double>(), n_pol, n_steps, level,
+                                                            c->d_vstage.as<unsigned long long>());
     CU(cudaGetLastError());
     c->cf_level.resize((size_t)n_pol);
-    CU(cudaMemcpyAsync(c->cf_level.data(), c->d_vstage.p, (size_t)n_pol, cudaMemcpyDeviceToHost, c->stream));
+    CU(cudaMemcpyAsync(c->cf_level.data(), level, (size_t)n_pol, cudaMemcpyDeviceToHost, c->stream));
+    CU(cudaMemcpyAsync(range, c->d_vstage.p, sizeof range, cudaMemcpyDeviceToHost, c->stream));
     CU(cudaStreamSynchronize(c->stream));
+    memcpy(&c->cf_lo, &range[0], sizeof c->cf_lo);
+    memcpy(&c->cf_hi, &range[1], sizeof c->cf_hi);
     c->cf_pol = n_pol;
     c->cf_steps = n_steps;
     ++c->cf_gen;
