@@ -317,11 +317,12 @@ __device__ __forceinline__ float mv_top(const Flow& flow, int S, const float* __
     for (int d = 16; d > 0; d >>= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, d));
     return top;
 }
-// the row's binary exponent: entries below 1; one bit less for each doubling of the steps
-// beyond 1,000, so that the leading digits' sum stays exact
+// the row's binary exponent: entries below 1; in the FP64 form one bit less for each doubling
+// of the steps beyond 1,000, so that the leading digits' sum over the segments stays exact
+template <int NS>
 __device__ __forceinline__ int mv_row_exp(float top, int S) {
     const int e = top > 0.0f ? ((__float_as_int(top) >> 23) & 255) - 126 : 0;
-    return e + (S > 1000) + (S > 2000) + (S > 4000);
+    return NS == 8 ? e + (S > 1000) + (S > 2000) + (S > 4000) : e;
 }
 // digits of flow(t) tilted and times 2^-e, t < live, and zeros up to kt
 template <int NS, class Flow>
@@ -397,9 +398,9 @@ __device__ __forceinline__ void mv_row(const MvBuild& b, const SlotRec& r, int r
         // A level annuity's cash flows do not increase, so its first one times the largest
         // tilt bounds them (it is the largest unless the tilt increases later, by
         // negative rates); the others are looked through.
-        e = mv_row_exp(S > 0 ? __fmul_rn(flow(0).h, b.tilt_top[S - 1]) : 0.0f, S);
+        e = mv_row_exp<NS>(S > 0 ? __fmul_rn(flow(0).h, b.tilt_top[S - 1]) : 0.0f, S);
     } else {
-        e = mv_row_exp(mv_top(flow, S, tilt), S);
+        e = mv_row_exp<NS>(mv_top(flow, S, tilt), S);
     }
     if constexpr (!CF && (KIND == K_ANN || KIND == K_ASS)) {   // straight from the column
         const int live = KIND == K_ANN ? min(S, x.last) : min(S, x.last + 1);
@@ -457,9 +458,9 @@ __device__ __forceinline__ void mv_row64(const MvBuild& b, const SlotRec& r, con
     };
     int e;
     if constexpr (!CF && (KIND == K_ANN || KIND == K_ANN2 || KIND == K_JL))
-        e = mv_row_exp(S > 0 ? __fmul_rn(head(0).h, b.tilt_top[S - 1]) : 0.0f, S);
+        e = mv_row_exp<8>(S > 0 ? __fmul_rn(head(0).h, b.tilt_top[S - 1]) : 0.0f, S);
     else
-        e = mv_row_exp(mv_top(head, S, tilt), S);
+        e = mv_row_exp<8>(mv_top(head, S, tilt), S);
     uint32_t* base = static_cast<uint32_t*>(b.digits) + ((size_t)(row / kMvP) * 8 * kMvP + row % kMvP) * b.pitch / 2;
     for (int t = 2 * (threadIdx.x & 31); t < kt; t += 64) {
         unsigned long long v[2] = {0, 0};
@@ -593,7 +594,7 @@ __global__ void __launch_bounds__(256) mv_build_lives_kernel(const CfTables T, c
     }
     const int S = r.pol >= 0 ? r.S : 0;
     auto flow = [&](int t) { return mv_lives_flow(T, r, l, one, t); };
-    const int e = mv_row_exp(mv_top(flow, S, tilt), S);
+    const int e = mv_row_exp<NS>(mv_top(flow, S, tilt), S);
     mv_write_row<NS>(flow, S, e, kt, tilt, digits, row, pitch);
     if ((threadIdx.x & 31) == 0) {
         int ex;
@@ -650,23 +651,28 @@ __global__ void __launch_bounds__(256) mv_build_kernel(const MvBuild b) {
 // form all of this had been conversions and sums on the FP64 pipe, longer than the products
 // (100,000 x 1,000 of every product: four digits 0.90 -> 0.88 ms, six 1.68 -> 1.62 ms; 3,000 x 333
 // in FP64: 0.203 -> 0.148 ms).
+// An accumulator sums at most SEG steps (a segment), so that the levels that must be exact
+// are (matval.cuh); a longer item's segments are added up by the epilogue, whose sums so far wait
+// in local memory (in registers they would not fit beside an accumulator's columns).  A segment's
+// end costs about 2,000 cycles: 100,000 x 1,000 of every product with six digits 1.62 -> 1.74 ms,
+// 3,000 x 333 in FP64 0.146 -> 0.154 ms.
 template <int NS>
-struct MvShape;   // policies of an item, accumulators, items in TMEM, stages, steps of a block (64:
-template <>       // 128-byte swizzled rows); the products are (i, j), i + j < NS, of scenario digit i
-struct MvShape<3> {   // and policy digit j, in accumulator min(i + j, NA - 1)
-    static constexpr int N = kMvP, NA = 2, NB = 2, ST = 3, KB = 64;
+struct MvShape;   // policies of an item, accumulators, segments in TMEM, stages, steps of a block (64:
+template <>       // 128-byte swizzled rows) and of a segment; the products are (i, j), i + j < NS, of
+struct MvShape<3> {   // scenario digit i and policy digit j, in accumulator min(i + j, NA - 1)
+    static constexpr int N = kMvP, NA = 2, NB = 2, ST = 3, KB = 64, SEG = 1024;
 };
 template <>
 struct MvShape<4> {
-    static constexpr int N = kMvP, NA = 4, NB = 1, ST = 4, KB = 32;
+    static constexpr int N = kMvP, NA = 4, NB = 1, ST = 4, KB = 32, SEG = 1024;
 };
 template <>
 struct MvShape<6> {
-    static constexpr int N = kMvP / 2, NA = 6, NB = 1, ST = 3, KB = 32;
+    static constexpr int N = kMvP / 2, NA = 6, NB = 1, ST = 3, KB = 32, SEG = 256;
 };
 template <>
 struct MvShape<8> {
-    static constexpr int N = kMvP / 2, NA = 8, NB = 1, ST = 2, KB = 32;
+    static constexpr int N = kMvP / 2, NA = 8, NB = 1, ST = 2, KB = 32, SEG = 256;
 };
 constexpr int kMvEpi = 4 * kMvParts;                   // epilogue warps
 constexpr int kMvThreads = 32 * (kMvEpi + 2);
@@ -713,7 +719,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
     mv_product_kernel(const __grid_constant__ CUtensorMap mapD, const __grid_constant__ CUtensorMap mapE, const MvArgs a) {
     using Sh = MvShape<NS>;
     using G = MvStage<NS>;
-    constexpr int KB = Sh::KB, N = Sh::N, kSub = kMvP / N;
+    constexpr int KB = Sh::KB, N = Sh::N, kSub = kMvP / N, kSeg = Sh::SEG / KB;   // kSeg: blocks of a segment
     constexpr uint32_t kIdesc = f16_idesc(NS != 3, 2 * kMvM, N);   // both operands FP16, or both BF16
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // (both CTAs of a pair place everything alike)
@@ -790,22 +796,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
         if (rank == 0 && elect_one()) {
             uint32_t it = 0, n = 0;
             const uint64_t ring_desc = KB == 64 ? sw128_desc(ring) : sw64_desc(ring);
-            for (long long item = cluster; item < n_items && !failed; item += n_clusters, ++n) {
+            for (long long item = cluster; item < n_items && !failed; item += n_clusters) {
                 const int nk = blocks_of((int)(item / n_pairs) / kSub);
-                const int buf = n % Sh::NB;
-                if (n >= Sh::NB) wait_on(&acc_empty[buf], (n / Sh::NB - 1) & 1);
-                const uint32_t d = tmem + buf * (Sh::NA * N);
-                for (int kb = 0; kb < nk && !failed; ++kb, ++it) {
-                    const int st = it % Sh::ST;
-                    wait_on(&full[st], (it / Sh::ST) & 1);
-                    if (failed) break;
-                    fence_after();
-                    const uint64_t base = ring_desc + (uint64_t)((st * G::kBytes) >> 4);
+                for (int k0 = 0; k0 < nk && !failed; k0 += kSeg, ++n) {
+                    const int buf = n % Sh::NB;
+                    if (n >= Sh::NB) wait_on(&acc_empty[buf], (n / Sh::NB - 1) & 1);
+                    const uint32_t d = tmem + buf * (Sh::NA * N);
+                    for (int kb = k0; kb < min(nk, k0 + kSeg) && !failed; ++kb, ++it) {
+                        const int st = it % Sh::ST;
+                        wait_on(&full[st], (it / Sh::ST) & 1);
+                        if (failed) break;
+                        fence_after();
+                        const uint64_t base = ring_desc + (uint64_t)((st * G::kBytes) >> 4);
 #pragma unroll
-                    for (int k16 = 0; k16 < KB / 16; ++k16) mv_products<NS, 0, 0>(d, base, k16 * 32, kIdesc, kb + k16 > 0);
-                    mma_commit_pair(&empty[st]);
+                        for (int k16 = 0; k16 < KB / 16; ++k16)
+                            mv_products<NS, 0, 0>(d, base, k16 * 32, kIdesc, kb - k0 + k16 > 0);
+                        mma_commit_pair(&empty[st]);
+                    }
+                    if (!failed) mma_commit_pair(&acc_full[buf]);
                 }
-                if (!failed) mma_commit_pair(&acc_full[buf]);
             }
             if (failed) {   // let the products in flight finish before the memory is released
                 mma_commit_pair(&drained);
@@ -820,178 +829,216 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
         uint32_t n = 0;
         uint32_t acc_free[Sh::NB];
         for (int i = 0; i < Sh::NB; ++i) acc_free[i] = of_rank0(&acc_empty[i]);
-        for (long long item = cluster; item < n_items; item += n_clusters, ++n) {
+        volatile float run[NS == 8 ? 3 : 2][kCols];   // the item's earlier segments
+        for (long long item = cluster; item < n_items; item += n_clusters) {
             const int sub = (int)(item / n_pairs), chunk = 2 * (int)(item - (long long)sub * n_pairs) + rank;
-            const int tile = sub / kSub, buf = n % Sh::NB;
+            const int tile = sub / kSub, nk = blocks_of(tile);
             if (tid < N * 2) reinterpret_cast<float4*>(recs)[tid] = reinterpret_cast<const float4*>(a.out + (size_t)sub * N)[tid];
             asm volatile("bar.sync 1, %0;" ::"n"(32 * kMvEpi) : "memory");
-            bool ok = true;
-            if (lane == 0 && !failed) ok = mbar_wait_bounded(&acc_full[buf], (n / Sh::NB) & 1, kMvPoll);
-            ok = __shfl_sync(0xffffffffu, ok, 0);
-            if (!ok && !failed) {   // recorded; the later waits are skipped and nothing is written
-                failed = true;
-                if (lane == 0) atomicExch(a.status, DEV_TIMEOUT);
-            }
-            fence_after();
             const int s = chunk * kMvM + quarter * 32 + lane;
-            const bool inside = chunk < a.n_chunks, live = s < a.n_scen && !failed;   // an odd last pair's second tile is empty
+            const bool inside = chunk < a.n_chunks;   // an odd last pair's second tile is empty
             const int sl = inside ? s : 0;
             const float dsc = pow2f(a.colexp[sl] - (NS == 3 ? 30 : 0));
-            const uint32_t col0 = tmem + ((uint32_t)(quarter * 32) << 16) + buf * (Sh::NA * N) + part * kCols;
-            auto load2 = [&](int k0, int k1, int c, float (&y)[16], float (&z)[16]) {   // two accumulators' 16 columns
-                uint32_t r[2][16];
-                tmem_ld16_async(col0 + k0 * N + c, r[0]);
-                tmem_ld16_async(col0 + k1 * N + c, r[1]);
-                tmem_wait_ld(r[0]);
-                tmem_wait_ld(r[1]);
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    y[i] = __uint_as_float(r[0][i]);
-                    z[i] = __uint_as_float(r[1][i]);
-                }
-            };
             df tot{0.0f, 0.0f};
             double tot64 = 0.0;
-            auto release = [&] {   // the accumulators are read
-                fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive_remote(acc_free[buf]);
-            };
-            // the columns of this warp, without branches over them (padding rows are 0), so that
-            // their chains overlap; MAT: maturity payments
-            auto columns = [&](auto with_maturity) {
-                constexpr bool MAT = decltype(with_maturity)::value;
-                auto emit = [&](const MvOut& q, float h, float l) {   // of a policy's sum h + l
-                    df v = df_mul(df{__fmul_rn(h, dsc), __fmul_rn(l, dsc)}, df{q.sc_h, q.sc_l});
-                    const int pol = q.pol;
-                    bool due = false;
-                    if constexpr (MAT) {   // a maturity payment, of the same sign, or 0
-                        const float2 d = a.D[(size_t)max(q.S - 1, 0) * a.s_pad + sl];
-                        due = q.S == 0;
-                        const df m = df_mul(df{q.mat_h, q.mat_l}, due ? df{1.0f, 0.0f} : df{d.x, d.y});
-                        const float sum = __fadd_rn(v.h, m.h), bb = __fsub_rn(sum, v.h);
-                        const float e = __fadd_rn(__fsub_rn(v.h, __fsub_rn(sum, bb)), __fsub_rn(m.h, bb));
-                        v = df{sum, __fadd_rn(e, __fadd_rn(v.l, m.l))};
-                        due = due && q.mat_h != 0.0f;
-                    }
-                    // the sum over the policies
-                    const float sum = __fadd_rn(tot.h, v.h), bb = __fsub_rn(sum, tot.h);
-                    const float e = __fadd_rn(__fsub_rn(tot.h, __fsub_rn(sum, bb)), __fsub_rn(v.h, bb));
-                    tot = df{sum, __fadd_rn(tot.l, __fadd_rn(e, v.l))};
-                    const size_t o = (size_t)pol * a.v0_ld + s;
-                    if (live && pol >= 0) {
-                        if (a.V0f) a.V0f[o] = __fadd_rn(v.h, v.l);
-                        if (a.V0d) a.V0d[o] = due ? a.amount[pol] : (double)v.h + (double)v.l;
+            for (int k0 = 0; k0 < nk; k0 += kSeg, ++n) {
+                const int buf = n % Sh::NB;
+                const bool last = k0 + kSeg >= nk;
+                bool ok = true;
+                if (lane == 0 && !failed) ok = mbar_wait_bounded(&acc_full[buf], (n / Sh::NB) & 1, kMvPoll);
+                ok = __shfl_sync(0xffffffffu, ok, 0);
+                if (!ok && !failed) {   // recorded; the later waits are skipped and nothing is written
+                    failed = true;
+                    if (lane == 0) atomicExch(a.status, DEV_TIMEOUT);
+                }
+                fence_after();
+                const bool live = s < a.n_scen && !failed;
+                const uint32_t col0 = tmem + ((uint32_t)(quarter * 32) << 16) + buf * (Sh::NA * N) + part * kCols;
+                auto load2 = [&](int k0, int k1, int c, float (&y)[16], float (&z)[16]) {   // two accumulators' 16 columns
+                    uint32_t r[2][16];
+                    tmem_ld16_async(col0 + k0 * N + c, r[0]);
+                    tmem_ld16_async(col0 + k1 * N + c, r[1]);
+                    tmem_wait_ld(r[0]);
+                    tmem_wait_ld(r[1]);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        y[i] = __uint_as_float(r[0][i]);
+                        z[i] = __uint_as_float(r[1][i]);
                     }
                 };
-                // Columns whose accumulators are added before they are released: as little as
-                // fits the registers, since with one item in TMEM the products stand still until then.
-                constexpr int kHold = NS == 4 ? kCols : 16;
+                auto release = [&] {   // the accumulators are read
+                    fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_remote(acc_free[buf]);
+                };
+                // the columns of this warp, without branches over them (padding rows are 0), so that
+                // their chains overlap; MAT: maturity payments
+                auto columns = [&](auto with_maturity) {
+                    constexpr bool MAT = decltype(with_maturity)::value;
+                    auto emit = [&](const MvOut& q, float h, float l) {   // of a policy's sum h + l
+                        df v = df_mul(df{__fmul_rn(h, dsc), __fmul_rn(l, dsc)}, df{q.sc_h, q.sc_l});
+                        const int pol = q.pol;
+                        bool due = false;
+                        if constexpr (MAT) {   // a maturity payment, of the same sign, or 0
+                            const float2 d = a.D[(size_t)max(q.S - 1, 0) * a.s_pad + sl];
+                            due = q.S == 0;
+                            const df m = df_mul(df{q.mat_h, q.mat_l}, due ? df{1.0f, 0.0f} : df{d.x, d.y});
+                            const float sum = __fadd_rn(v.h, m.h), bb = __fsub_rn(sum, v.h);
+                            const float e = __fadd_rn(__fsub_rn(v.h, __fsub_rn(sum, bb)), __fsub_rn(m.h, bb));
+                            v = df{sum, __fadd_rn(e, __fadd_rn(v.l, m.l))};
+                            due = due && q.mat_h != 0.0f;
+                        }
+                        // the sum over the policies
+                        const float sum = __fadd_rn(tot.h, v.h), bb = __fsub_rn(sum, tot.h);
+                        const float e = __fadd_rn(__fsub_rn(tot.h, __fsub_rn(sum, bb)), __fsub_rn(v.h, bb));
+                        tot = df{sum, __fadd_rn(tot.l, __fadd_rn(e, v.l))};
+                        const size_t o = (size_t)pol * a.v0_ld + s;
+                        if (live && pol >= 0) {
+                            if (a.V0f) a.V0f[o] = __fadd_rn(v.h, v.l);
+                            if (a.V0d) a.V0d[o] = due ? a.amount[pol] : (double)v.h + (double)v.l;
+                        }
+                    };
+                    // Columns whose accumulators are added before they are released: as little as
+                    // fits the registers, since with one item in TMEM the products stand still until then.
+                    constexpr int kHold = NS == 4 ? kCols : 16;
 #pragma unroll 1
-                for (int c0 = 0; c0 < kCols; c0 += kHold) {
-                    if constexpr (NS == 8) {
-                        // u = a0 + w + v + x: the levels from 2^-32 of the first as plain FP32
-                        // sums (2^-56), the others' errors kept; the rest after the release
-                        float p[16], w[16], v[16], x[16];
-                        {
-                            float y[16], z[16];
-                            load2(7, 6, c0, y, z);
+                    for (int c0 = 0; c0 < kCols; c0 += kHold) {
+                        if constexpr (NS == 8) {
+                            // u = a0 + w + v + x: the levels from 2^-32 of the first as plain FP32
+                            // sums (2^-56), the others' errors kept; the rest after the release
+                            float p[16], w[16], v[16], x[16];
+                            {
+                                float y[16], z[16];
+                                load2(7, 6, c0, y, z);
 #pragma unroll
-                            for (int i = 0; i < 16; ++i) x[i] = __fadd_rn(y[i], z[i]);
-                            load2(5, 4, c0, y, z);
+                                for (int i = 0; i < 16; ++i) x[i] = __fadd_rn(y[i], z[i]);
+                                load2(5, 4, c0, y, z);
 #pragma unroll
-                            for (int i = 0; i < 16; ++i) x[i] = __fadd_rn(z[i], __fadd_rn(y[i], x[i]));
-                            load2(3, 2, c0, y, z);
+                                for (int i = 0; i < 16; ++i) x[i] = __fadd_rn(z[i], __fadd_rn(y[i], x[i]));
+                                load2(3, 2, c0, y, z);
 #pragma unroll
-                            for (int i = 0; i < 16; ++i) {
-                                two_sum(y[i], x[i], v[i], x[i]);
-                                w[i] = z[i];
+                                for (int i = 0; i < 16; ++i) {
+                                    two_sum(y[i], x[i], v[i], x[i]);
+                                    w[i] = z[i];
+                                }
+                                load2(1, 0, c0, y, p);
+#pragma unroll
+                                for (int i = 0; i < 16; ++i) {
+                                    float e;
+                                    two_sum(y[i], w[i], w[i], e);
+                                    x[i] = __fadd_rn(x[i], e);
+                                }
                             }
-                            load2(1, 0, c0, y, p);
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) {
-                                float e;
-                                two_sum(y[i], w[i], w[i], e);
-                                x[i] = __fadd_rn(x[i], e);
-                            }
-                        }
-                        release();
-                        const int ce = a.colexp[sl];
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) {
-                            const MvOut64& q = reinterpret_cast<const MvOut64&>(recs[part * kCols + c0 + i]);
-                            float e;
-                            two_sum(p[i], w[i], p[i], w[i]);
-                            two_sum(w[i], v[i], w[i], e);
-                            x[i] = __fadd_rn(x[i], e);
-                            // of the FP64 pipe (1/64 of the FP32 rate) only what needs 53 bits
-                            double t = __dadd_rn(scaled_double(w[i], ce), scaled_double(x[i], ce));
-                            t = __dmul_rn(__dadd_rn(scaled_double(p[i], ce), t), q.sc);
-                            if constexpr (MAT) {
-                                const double d = q.S > 0 ? a.D64[(size_t)(q.S - 1) * a.s_pad + sl] : 1.0;
-                                t = __fma_rn(q.mat, d, t);
-                            }
-                            tot64 = __dadd_rn(tot64, t);
-                            if (live && q.pol >= 0) {
-                                const size_t o = (size_t)q.pol * a.v0_ld + s;
-                                if (a.V0f) a.V0f[o] = __double2float_rn(t);
-                                if (a.V0d) a.V0d[o] = t;
-                            }
-                        }
-                        continue;
-                    }
-                    // the accumulators' sum as a double-float: the errors of adding the first
-                    // ones are kept; those from 2^-24 (four digits: 2^-16) of the first are
-                    // added as they are, 2^-48 (2^-40)
-                    float h[kHold], l[kHold];
-#pragma unroll
-                    for (int c = 0; c < kHold; c += 16) {
-                        float y[16], z[16], x[16];
-                        if constexpr (NS == 6) {
-                            load2(5, 4, c0 + c, y, z);
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) x[i] = __fadd_rn(y[i], z[i]);
-                            load2(3, 2, c0 + c, y, z);
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) l[c + i] = __fadd_rn(y[i], x[i]);
-                            load2(1, 0, c0 + c, y, x);
                             release();
+                            const int ce = a.colexp[sl];
 #pragma unroll
                             for (int i = 0; i < 16; ++i) {
-                                float e1, e2;
-                                two_sum(x[i], y[i], x[i], e1);
-                                two_sum(x[i], z[i], h[c + i], e2);
-                                l[c + i] = __fadd_rn(l[c + i], __fadd_rn(e1, e2));
+                                const MvOut64& q = reinterpret_cast<const MvOut64&>(recs[part * kCols + c0 + i]);
+                                float e;
+                                if (k0 > 0 || !last) {   // several segments: the first levels' sum is exact
+                                    two_sum(w[i], v[i], w[i], v[i]);
+                                    x[i] = __fadd_rn(x[i], v[i]);
+                                    v[i] = 0.0f;
+                                    if (k0 > 0) {
+                                        p[i] = __fadd_rn(p[i], run[0][c0 + i]);
+                                        two_sum(w[i], run[1][c0 + i], w[i], e);
+                                        x[i] = __fadd_rn(__fadd_rn(x[i], e), run[2][c0 + i]);
+                                    }
+                                    if (!last) {
+                                        run[0][c0 + i] = p[i];
+                                        run[1][c0 + i] = w[i];
+                                        run[2][c0 + i] = x[i];
+                                        continue;
+                                    }
+                                }
+                                two_sum(p[i], w[i], p[i], w[i]);
+                                two_sum(w[i], v[i], w[i], e);
+                                x[i] = __fadd_rn(x[i], e);
+                                // of the FP64 pipe (1/64 of the FP32 rate) only what needs 53 bits
+                                double t = __dadd_rn(scaled_double(w[i], ce), scaled_double(x[i], ce));
+                                t = __dmul_rn(__dadd_rn(scaled_double(p[i], ce), t), q.sc);
+                                if constexpr (MAT) {
+                                    const double d = q.S > 0 ? a.D64[(size_t)(q.S - 1) * a.s_pad + sl] : 1.0;
+                                    t = __fma_rn(q.mat, d, t);
+                                }
+                                tot64 = __dadd_rn(tot64, t);
+                                if (live && q.pol >= 0) {
+                                    const size_t o = (size_t)q.pol * a.v0_ld + s;
+                                    if (a.V0f) a.V0f[o] = __double2float_rn(t);
+                                    if (a.V0d) a.V0d[o] = t;
+                                }
                             }
-                        } else if constexpr (NS == 4) {
-                            load2(3, 2, c0 + c, y, z);
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) x[i] = __fadd_rn(y[i], z[i]);
-                            load2(1, 0, c0 + c, y, z);
-                            if (c0 + c == kCols - 16) release();
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) {
-                                two_sum(z[i], y[i], h[c + i], l[c + i]);
-                                l[c + i] = __fadd_rn(l[c + i], x[i]);
-                            }
-                        } else {
-                            uint32_t r[2][16];
-                            tmem_ld16_async(col0 + c0, r[0]);
-                            tmem_ld16_async(col0 + N + c0, r[1]);
-                            tmem_wait_ld(r[0]);
-                            tmem_wait_ld(r[1]);
-                            if (c0 == kCols - 16) release();
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) two_sum(__uint_as_float(r[0][i]), __uint_as_float(r[1][i]), h[i], l[i]);
+                            continue;
                         }
-                    }
+                        // the accumulators' sum as a double-float: the errors of adding the first
+                        // ones are kept; those from 2^-24 (four digits: 2^-16) of the first are
+                        // added as they are, 2^-48 (2^-40)
+                        float h[kHold], l[kHold];
 #pragma unroll
-                    for (int i = 0; i < kHold; ++i) emit(recs[part * kCols + c0 + i], h[i], l[i]);
-                }
-            };
-            const int kind = a.kinds ? a.kinds[tile] : K_ANN;
-            if (kind == K_ASS || kind == K_ASS2 || kind == K_LS2) columns(std::true_type{});
-            else columns(std::false_type{});
+                        for (int c = 0; c < kHold; c += 16) {
+                            float y[16], z[16], x[16];
+                            if constexpr (NS == 6) {
+                                load2(5, 4, c0 + c, y, z);
+#pragma unroll
+                                for (int i = 0; i < 16; ++i) x[i] = __fadd_rn(y[i], z[i]);
+                                load2(3, 2, c0 + c, y, z);
+#pragma unroll
+                                for (int i = 0; i < 16; ++i) l[c + i] = __fadd_rn(y[i], x[i]);
+                                load2(1, 0, c0 + c, y, x);
+                                release();
+#pragma unroll
+                                for (int i = 0; i < 16; ++i) {
+                                    float e1, e2;
+                                    two_sum(x[i], y[i], x[i], e1);
+                                    two_sum(x[i], z[i], h[c + i], e2);
+                                    l[c + i] = __fadd_rn(l[c + i], __fadd_rn(e1, e2));
+                                }
+                            } else if constexpr (NS == 4) {
+                                load2(3, 2, c0 + c, y, z);
+#pragma unroll
+                                for (int i = 0; i < 16; ++i) x[i] = __fadd_rn(y[i], z[i]);
+                                load2(1, 0, c0 + c, y, z);
+                                if (c0 + c == kCols - 16) release();
+#pragma unroll
+                                for (int i = 0; i < 16; ++i) {
+                                    two_sum(z[i], y[i], h[c + i], l[c + i]);
+                                    l[c + i] = __fadd_rn(l[c + i], x[i]);
+                                }
+                            } else {
+                                uint32_t r[2][16];
+                                tmem_ld16_async(col0 + c0, r[0]);
+                                tmem_ld16_async(col0 + N + c0, r[1]);
+                                tmem_wait_ld(r[0]);
+                                tmem_wait_ld(r[1]);
+                                if (c0 == kCols - 16) release();
+#pragma unroll
+                                for (int i = 0; i < 16; ++i) two_sum(__uint_as_float(r[0][i]), __uint_as_float(r[1][i]), h[i], l[i]);
+                            }
+                        }
+                        if (k0 > 0) {
+#pragma unroll
+                            for (int i = 0; i < kHold; ++i) {
+                                float e;
+                                two_sum(h[i], run[0][c0 + i], h[i], e);
+                                l[i] = __fadd_rn(__fadd_rn(l[i], e), run[1][c0 + i]);
+                            }
+                        }
+                        if (!last) {
+#pragma unroll
+                            for (int i = 0; i < kHold; ++i) {
+                                run[0][c0 + i] = h[i];
+                                run[1][c0 + i] = l[i];
+                            }
+                            continue;
+                        }
+#pragma unroll
+                        for (int i = 0; i < kHold; ++i) emit(recs[part * kCols + c0 + i], h[i], l[i]);
+                    }
+                };
+                const int kind = a.kinds ? a.kinds[tile] : K_ANN;
+                if (kind == K_ASS || kind == K_ASS2 || kind == K_LS2) columns(std::true_type{});
+                else columns(std::false_type{});
+            }
             // the parts' sums in part order; then the records and sums may be overwritten
             if constexpr (NS == 8) reinterpret_cast<double&>(sums[part][quarter * 32 + lane]) = tot64;
             else sums[part][quarter * 32 + lane] = make_float2(tot.h, tot.l);

@@ -14,13 +14,18 @@
 //   remainders, to 2^-33 and 2^-48.
 //   Eight (the FP64 form): seven more of 8 bits each (signed), to 2^-63.
 //
-// The products of digits i and j, i + j at most the last digit's number, are taken.  d1 d1'
-// products are multiples of 2^-14, so up to 1,000 of them add up exactly in FP32 (rows with
-// more steps give up one or two bits).  With four digits d1 d2', and d1 d3' and d2 d2', 2^-8
-// and 2^-16 below, are multiples of 2^-22 and 2^-30 and have an exact accumulator each; the
-// rest shares one more, whose FP32 truncations (of a sum 2^-24, with three digits 2^-8,
-// below) are that much smaller.  With six and eight every level has its own.  The epilogue
-// adds the accumulators: the first ones with their rounding errors, the low ones as they
+// The products of digits i and j, i + j at most the last digit's number, are taken.  A digit is
+// at most 2^7 units in size and a product 2^14, so that FP32 adds up 1,024 products of a level
+// exactly whatever their signs.  Operands that hardly change (no interest and no mortality to
+// speak of) have digits of one sign from step to step, so this is the bound that counts: with
+// six and eight digits an accumulator of level i + j sums at most 256 steps, a segment, which
+// makes the levels 0 to 2 (eight digits: to 3) exact and leaves truncations below 2^-40 (2^-47) of
+// the sum at the very worst; one accumulator over 1,000 steps was off by 4e-9 on such operands.
+// The epilogue adds up the segments in double-floats (eight digits: three floats).  With three
+// and four digits a segment is 1,024 steps, so that level 0 is exact; the truncations of the
+// others, at most 2^-24 of a sum 2^-7 below for each block of 16 steps and pair of digits,
+// stay within 2^-22.
+// The epilogue adds the accumulators: the first ones with their rounding errors, the low ones as they
 // are (to 2^-40, 2^-48 and 2^-56 with four, six and eight digits).  A maturity payment is
 // added there, from the discount products themselves, so that a row holds entries of one kind.
 //
@@ -32,10 +37,10 @@
 // mv_max_spread) keeps the recurrence kernels.
 //
 // Measured (one GB300, with the digits and the totals), before: the recurrence.
-//   100,000 policies of every product, 1,000 scenarios: compensated 38.7 -> 1.62 ms
-//   (annuities 1e-13 -> 1.5e-14 rms, assurances 4e-9 -> 1.7e-14), deflated 4.93 -> 0.89 ms
+//   100,000 policies of every product, 1,000 scenarios: compensated 38.7 -> 1.74 ms
+//   (annuities 1e-13 -> 1.5e-14 rms, assurances 4e-9 -> 1.7e-14), deflated 4.93 -> 0.88 ms
 //   (rms 3e-8 -> 5e-9, with three digits 0.62 ms);
-//   1,000,000 annuities, 600 steps, 1,000 scenarios, deflated: 30.6 -> 4.3 ms;
+//   1,000,000 annuities, 600 steps, 1,000 scenarios, deflated: 30.6 -> 4.1 ms;
 //   3,000 two-life policies, 333 scenarios, FP64: 5.17 -> 0.15 ms (1.4e-15 -> 1.3e-15).
 // It is the faster path at every size measured: one policy and one scenario 53 -> 49 us
 // compensated and 158 -> 37 us deflated (host call included), 1,000 policies under 157

@@ -119,8 +119,10 @@ __device__ __forceinline__ uint32_t of_rank0(const void* p) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(smem_u32(p)));
     return r;
 }
+// After fence_before: orders what was done in tensor memory and no other memory, so that it does not
+// wait for the thread's stores (with .release 1,500 cycles more until the waiting thread saw it).
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t bar) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 // into this CTA's shared memory, completing on a barrier of either CTA
 __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
