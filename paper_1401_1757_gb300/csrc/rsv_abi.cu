@@ -487,8 +487,10 @@ rsv_status rsv::build_layout(rsv_ctx* c, int P, int horizon, int max_steps, int 
                 SlotRec sl;
                 if (k < len) {
                     const PolPrep& q = pp[order[st0 + k]];
-                    sl.idx1 = q.table1 * tab_pad + q.idx_age1;
-                    sl.idx2 = q.table2 * tab_pad + q.idx_age2;
+                    // an age of tab_pad has no step left to read a table for (age + S <= tab_pad); as
+                    // the last entry the index keeps its table
+                    sl.idx1 = q.table1 * tab_pad + std::min(q.idx_age1, tab_pad - 1);
+                    sl.idx2 = q.table2 * tab_pad + std::min(q.idx_age2, tab_pad - 1);
                     sl.S = q.S;
                     sl.pol = q.pol;
                     sl.rho_h = (float)q.rho;
