@@ -64,23 +64,18 @@ class PartPool {
             ctx_ = ctx;
             T_ = T;
             done_ = 0;
+            err_ = nullptr;
             next_.store((uint64_t)g << 32);
         }
         cv_.notify_all();
-        std::exception_ptr err;
         in_part() = true;
-        for (int k; (k = claim(g, T)) >= 0;) {
-            try {
-                fn(ctx, k);
-            } catch (...) {   // the other parts still run; the first error is rethrown
-                if (!err) err = std::current_exception();
-            }
-            count(g);
-        }
+        work(g, T, fn, ctx);
         in_part() = false;
+        std::exception_ptr err;
         {
             std::unique_lock<std::mutex> l(m_);
             done_cv_.wait(l, [&] { return done_ == T; });
+            std::swap(err, err_);
         }
         if (err) std::rethrow_exception(err);
         return true;
@@ -106,9 +101,20 @@ class PartPool {
             if (next_.compare_exchange_weak(v, v + 1)) return (int)(uint32_t)v;
         }
     }
-    void count(uint32_t g) {
-        std::lock_guard<std::mutex> l(m_);
-        if (g == gen_ && ++done_ == T_) done_cv_.notify_all();
+    // The parts of job g that are left.  A part that throws, on whichever thread, counts as run:
+    // the others still run, and the caller rethrows the first error.
+    void work(uint32_t g, int T, void (*fn)(void*, int), void* ctx) {
+        for (int k; (k = claim(g, T)) >= 0;) {
+            std::exception_ptr err;
+            try {
+                fn(ctx, k);
+            } catch (...) {
+                err = std::current_exception();
+            }
+            std::lock_guard<std::mutex> l(m_);   // the job is not over before this part is counted
+            if (err && !err_) err_ = err;
+            if (++done_ == T_) done_cv_.notify_all();
+        }
     }
     void start_workers(int want) {
         const int hw = (int)std::max(1u, std::thread::hardware_concurrency());
@@ -135,10 +141,7 @@ class PartPool {
                 ctx = ctx_;
                 T = T_;
             }
-            for (int k; (k = claim(g, T)) >= 0;) {
-                fn(ctx, k);
-                count(g);
-            }
+            work(g, T, fn, ctx);
         }
     }
     std::mutex use_, m_;
@@ -148,13 +151,14 @@ class PartPool {
     void (*fn_)(void*, int) = nullptr;
     void* ctx_ = nullptr;
     int T_ = 0, done_ = 0;
+    std::exception_ptr err_;   // the running job's first
     uint32_t gen_ = 0;
     bool stop_ = false;
 };
 
 // Run part(k) for k = 0 .. T-1 on the pool's workers and this thread (or, if
 // the pool is busy, on T - 1 helper threads and this one; parts whose thread
-// cannot start run here).
+// cannot start run here).  Every part runs; the first exception of one is rethrown here.
 template <class F>
 inline void run_parts(int T, F&& part) {
     if (T <= 1) {
@@ -165,19 +169,30 @@ inline void run_parts(int T, F&& part) {
     if (PartPool::get().run(T, [](void* c, int k) { (*static_cast<P*>(c))(k); },
                             const_cast<void*>(static_cast<const void*>(&part))))
         return;
+    std::exception_ptr err;
+    std::mutex m;
+    auto run = [&](int k) {
+        try {
+            part(k);
+        } catch (...) {
+            std::lock_guard<std::mutex> l(m);
+            if (!err) err = std::current_exception();
+        }
+    };
     std::vector<std::thread> th;
     int started = 1;
     try {
         th.reserve(T - 1);
         for (int k = 1; k < T; ++k) {
-            th.emplace_back(part, k);
+            th.emplace_back(run, k);
             ++started;
         }
     } catch (...) {   // no more threads: the rest runs serially below
     }
-    part(0);
-    for (int k = started; k < T; ++k) part(k);
+    run(0);
+    for (int k = started; k < T; ++k) run(k);
     for (auto& t : th) t.join();
+    if (err) std::rethrow_exception(err);
 }
 
 }  // namespace rsv
