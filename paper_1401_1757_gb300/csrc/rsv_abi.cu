@@ -1505,11 +1505,14 @@ rsv_status rsv_clear_cashflows(rsv_ctx* c) try {
 rsv_status rsv_load_portfolio(rsv_ctx* c, const rsv_policy* pols, int64_t n) try {
     if (!c) return RSV_E_ARG;
     if (n < 0 || n > 0x7fffffffLL || (n > 0 && !pols)) return fail(c, RSV_E_ARG, "bad portfolio size %lld", (long long)n);
+    // whatever may throw comes before anything of the loaded book changes
+    const int T = host_parts(n);
+    std::vector<double> amt_lo(T, INFINITY), amt_hi(T, 0.0);
+    c->pols.reserve((size_t)n);
+    c->h_amount.reserve((size_t)n);
     // copied by several host threads for large portfolios (no zero fill first)
     c->pols.resize((size_t)n);
     c->h_amount.resize((size_t)n);
-    const int T = host_parts(n);
-    std::vector<double> amt_lo(T, INFINITY), amt_hi(T, 0.0);
     run_parts(T, [&](int k) {
         const int64_t lo = n * k / T, hi = n * (k + 1) / T;
         if (hi > lo) memcpy(c->pols.data() + lo, pols + lo, (size_t)(hi - lo) * sizeof(rsv_policy));
