@@ -227,6 +227,7 @@ struct rsv_ctx {
     double amt_lo = 0.0, amt_hi = 0.0;              // smallest non-zero and largest |amount|
     DevBuf d_mv_D, d_mv_col, d_mv_D64, d_mv_dig[4], d_mv_E, d_mv_out;
     unsigned long long scen_gen = 1, mv_range_gen = 0, mv_dig_gen[4] = {0, 0, 0, 0};
+    unsigned long long mv_used[4] = {0, 0, 0, 0};   // per form: the last scenario set whose range it asked for
     int mv_built = -1;   // first tile of the panel whose digits are held, within one call
 
     Layout lay;
@@ -302,6 +303,8 @@ rsv_status mv_prepare(rsv_ctx* c, int form);
 // Its parts, for rows that come from elsewhere (m lives): the scenario set's digits, the tiles
 // of a panel and their buffers (d_mv_E, d_mv_out), and the product of a built panel
 // (a: steps, kinds, amount, n_tiles and the outputs set).
+rsv_status mv_range(rsv_ctx* c);
+rsv_status mv_digit_buffers(rsv_ctx* c, int form);
 rsv_status mv_scenario_digits(rsv_ctx* c, int form);
 int mv_panel_tiles(const rsv_ctx* c, int form, int max_S, int n_tiles);
 rsv_status mv_panel_buffers(rsv_ctx* c, int form, int max_S, int tiles);

@@ -657,6 +657,24 @@ rsv_status upload_amounts(rsv_ctx* c) {
 
 }  // namespace
 
+// The scenario set's discount products and their range (one synchronisation): with its first use
+// (a quarter of the load's time, which the other forms and the time scan need not pay) or, if
+// the set before it was valued as a matrix product, with the load.
+rsv_status rsv::mv_range(rsv_ctx* c) {
+    const size_t np = (size_t)c->n_steps * c->s_pad;
+    CU(c->d_mv_D.ensure(np * sizeof(float2)));
+    CU(c->d_mv_col.ensure(MvScen::words(c->n_steps, c->s_pad) * sizeof(int32_t)));
+    const MvScen mv = MvScen::at(c->d_mv_col.p, c->n_steps, c->s_pad);
+    CU(launch_mv_scenarios(c->d_v64.as<double>(), c->n_steps, c->n_scen, c->s_pad, c->d_mv_D.as<float2>(), mv, c->stream));
+    int32_t range[2];
+    CU(cudaMemcpyAsync(range, mv.stat, sizeof range, cudaMemcpyDeviceToHost, c->stream));
+    CU(cudaStreamSynchronize(c->stream));
+    c->mv_spread = range[1] <= kMvTilt ? range[0] : INT_MAX;
+    c->mv_tilt = range[1];
+    c->mv_range_gen = c->scen_gen;
+    return RSV_OK;
+}
+
 rsv_status rsv::mv_applies(rsv_ctx* c, int form, double amt_lo, double amt_hi, bool cf, bool& applies) {
     applies = false;
     if (!(amt_hi <= kMvAmountMax) || !(amt_lo >= kMvAmountMin)) return RSV_OK;
@@ -672,20 +690,10 @@ rsv_status rsv::mv_applies(rsv_ctx* c, int form, double amt_lo, double amt_hi, b
     lo *= tab_min;
     if (!(lo >= kMvEntryMin) || !(hi <= kMvEntryMax)) return RSV_OK;
     if (c->mv_range_gen != c->scen_gen) {
-        // the discount products and their range, with the scenario set's first use here (a
-        // quarter of the load's time, which the other forms and the time scan need not pay)
-        const size_t np = (size_t)c->n_steps * c->s_pad;
-        CU(c->d_mv_D.ensure(np * sizeof(float2)));
-        CU(c->d_mv_col.ensure(MvScen::words(c->n_steps, c->s_pad) * sizeof(int32_t)));
-        const MvScen mv = MvScen::at(c->d_mv_col.p, c->n_steps, c->s_pad);
-        CU(launch_mv_scenarios(c->d_v64.as<double>(), c->n_steps, c->n_scen, c->s_pad, c->d_mv_D.as<float2>(), mv, c->stream));
-        int32_t range[2];
-        CU(cudaMemcpyAsync(range, mv.stat, sizeof range, cudaMemcpyDeviceToHost, c->stream));
-        CU(cudaStreamSynchronize(c->stream));
-        c->mv_spread = range[1] <= kMvTilt ? range[0] : INT_MAX;
-        c->mv_tilt = range[1];
-        c->mv_range_gen = c->scen_gen;
+        const rsv_status st = mv_range(c);
+        if (st != RSV_OK) return st;
     }
+    c->mv_used[form] = c->scen_gen;
     if (c->mv_spread > mv_max_spread(form)) return RSV_OK;
     lo = std::ldexp(lo, -c->mv_tilt);
     hi = std::ldexp(hi, c->mv_tilt);
@@ -694,13 +702,21 @@ rsv_status rsv::mv_applies(rsv_ctx* c, int form, double amt_lo, double amt_hi, b
     return RSV_OK;
 }
 
+// Buffers of the scenario set's digits: a set of the same shape needs no others.
+rsv_status rsv::mv_digit_buffers(rsv_ctx* c, int form) {
+    const int ns = mv_digits_of(form, c->mv_spread);
+    CU(c->d_mv_dig[mv_digit_set(ns)].ensure((size_t)ns * c->s_pad * mv_pitch(c->n_steps) * 2));
+    if (ns == 8) CU(c->d_mv_D64.ensure((size_t)c->n_steps * c->s_pad * sizeof(double)));
+    return RSV_OK;
+}
+
 rsv_status rsv::mv_scenario_digits(rsv_ctx* c, int form) {
     const int ns = mv_digits_of(form, c->mv_spread), k = mv_digit_set(ns), pitch = mv_pitch(c->n_steps);
     if (c->mv_dig_gen[k] == c->scen_gen) return RSV_OK;   // with the scenario set, like its planes
-    CU(c->d_mv_dig[k].ensure((size_t)ns * c->s_pad * pitch * 2));
+    const rsv_status st = mv_digit_buffers(c, form);
+    if (st != RSV_OK) return st;
     const MvScen mv = MvScen::at(c->d_mv_col.p, c->n_steps, c->s_pad);
     if (ns == 8) {
-        CU(c->d_mv_D64.ensure((size_t)c->n_steps * c->s_pad * sizeof(double)));
         CU(launch_mv_products64(c->d_v64.as<double>(), c->n_steps, c->s_pad, c->d_mv_D64.as<double>(), c->stream));
         CU(launch_mv_digits64(c->d_mv_D64.as<double>(), mv.tau, mv.colexp, c->n_steps, c->n_scen, c->s_pad, pitch,
                               c->d_mv_dig[k].p, c->stream));
@@ -708,7 +724,10 @@ rsv_status rsv::mv_scenario_digits(rsv_ctx* c, int form) {
         CU(launch_mv_digits(ns, c->d_mv_D.as<float2>(), mv.tau, mv.colexp, c->n_steps, c->n_scen, c->s_pad, pitch,
                             c->d_mv_dig[k].p, c->stream));
     }
-    c->mv_dig_gen[k] = c->scen_gen;
+    // captured into a graph they are made by its launches, and a call outside it makes its own
+    cudaStreamCaptureStatus capture;
+    CU(cudaStreamIsCapturing(c->stream, &capture));
+    if (capture == cudaStreamCaptureStatusNone) c->mv_dig_gen[k] = c->scen_gen;
     return RSV_OK;
 }
 
@@ -718,7 +737,11 @@ int rsv::mv_panel_tiles(const rsv_ctx* c, int form, int max_S, int n_tiles) {
 }
 
 rsv_status rsv::mv_panel_buffers(rsv_ctx* c, int form, int max_S, int tiles) {
-    CU(c->d_mv_E.ensure((size_t)mv_digits_of(form, c->mv_spread) * kMvP * mv_pitch(max_S) * 2 * tiles));
+    // the deflated form's for four digits, so that a set of another spread needs no others
+    const size_t digit = (size_t)kMvP * mv_pitch(max_S) * 2;
+    size_t bytes = mv_digits_of(form, c->mv_spread) * digit * tiles;
+    if (form == F_DEFL) bytes = std::max(bytes, 4 * digit * std::min<size_t>(tiles, kMvPanelBytes / (4 * digit)));
+    CU(c->d_mv_E.ensure(bytes));
     CU(c->d_mv_out.ensure((size_t)tiles * kMvP * sizeof(MvOut)));
     return RSV_OK;
 }
@@ -1564,12 +1587,22 @@ rsv_status rsv_load_scenarios(rsv_ctx* c, const double* v, int32_t n_scen, int32
                                                                 s_pad, c->d_v64.as<double>(), c->d_v32.as<float>(),
                                                                 c->d_v2.as<float2>());
     CU(cudaGetLastError());
-    CU(cudaStreamSynchronize(c->stream));
-    ++c->scen_gen;
+    const unsigned long long before = c->scen_gen++;
     c->n_scen = n_scen;
     c->n_steps = n_steps;
     c->s_pad = s_pad;
     c->lay.gen = ~0ull;   // scenario length changes validation
+    // A set that takes the place of one valued as a matrix product: the next call on it
+    // neither waits nor allocates, so that it can be captured as the last one could.
+    bool again = false;
+    for (int form = 0; form < 4; ++form) again |= c->mv_used[form] == before;
+    if (again) {
+        rsv_status st = mv_range(c);
+        for (int form = 0; form < 4 && st == RSV_OK; ++form)
+            if (c->mv_used[form] == before && c->mv_spread <= mv_max_spread(form)) st = mv_digit_buffers(c, form);
+        return st;
+    }
+    CU(cudaStreamSynchronize(c->stream));
     return RSV_OK;
 } catch (...) {
     return rsv::host_error(c);
