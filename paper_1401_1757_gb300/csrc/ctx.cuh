@@ -33,6 +33,7 @@ struct DevBuf {
         n = 0;
         cudaError_t e = cudaMalloc(&p, bytes ? bytes : 16);
         if (e == cudaSuccess) n = bytes;
+        else cudaGetLastError();   // reported here, not by a later launch
         return e;
     }
     void release() {
@@ -311,7 +312,20 @@ rsv_status mv_panel_buffers(rsv_ctx* c, int form, int max_S, int tiles);
 rsv_status mv_multiply(rsv_ctx* c, int form, MvArgs a, int max_S, int s0, int w);
 rsv_status mv_launch(rsv_ctx* c, int form, int s0, int w, float* V0f, double* V0d, double* partial);
 // rsv_compute_reserves in the deflated form (defl_abi.cu); opts checked by the caller
-rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out);
+// (matrix: the matrix product may be taken)
+rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out, bool matrix);
+// What the matrix product holds of device memory, and its release.
+bool mv_holds(const rsv_ctx* c);
+void mv_release(rsv_ctx* c);
+// call(true), which may take the matrix product; where that leaves too little device memory its
+// buffers are given back and call(false) goes without it.
+template <class F>
+rsv_status mv_or_without(rsv_ctx* c, const F& call) {
+    const rsv_status st = call(true);
+    if (st != RSV_E_NOMEM || !mv_holds(c)) return st;
+    mv_release(c);
+    return call(false);
+}
 // The deflated kernels' staged life tables (defl_abi.cu): their shape from the
 // layout's kinds (RSV_E_ARG for a product the form does not take), then the
 // FP64 life tables {l_k} (l_0 = 2^100) and the staged FP32 arrays.

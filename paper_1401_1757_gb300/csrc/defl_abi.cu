@@ -106,7 +106,7 @@ rsv_status defl_table_stage(rsv_ctx* c, DeflTabs& T) {
     return RSV_OK;
 }
 
-rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
+rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out, bool matrix) {
     const int outs = o->outputs;
     if (outs & (RSV_OUT_PT_MEAN | RSV_OUT_TRAJ))
         return fail(c, RSV_E_ARG, "the deflated form outputs V0 and the totals; per-step outputs need another form");
@@ -125,7 +125,7 @@ rsv_status compute_deflated(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
         return fail(c, RSV_E_ARG, "variant %d out of range (the deflated form has no scan or summation)", o->variant);
     }
     bool mat = false;
-    if (vi == nv) {
+    if (vi == nv && matrix) {
         const rsv_status mst = mv_applies(c, F_DEFL, c->amt_lo, c->amt_hi, false, mat);
         if (mst != RSV_OK) return mst;
     }

@@ -245,9 +245,7 @@ rsv_status mlife_matrix(rsv_ctx* c, const rsv_mlife_policy* pols, const std::vec
 
 using namespace rsv;
 
-extern "C" rsv_status rsv_compute_mlife(rsv_ctx* c, const rsv_mlife_policy* pols, int64_t n, const rsv_opts* o,
-                                        rsv_out* out) try {
-    if (!c) return RSV_E_ARG;
+static rsv_status mlife_as(rsv_ctx* c, const rsv_mlife_policy* pols, int64_t n, const rsv_opts* o, rsv_out* out, bool matrix) {
     if (!o || !out || n < 0 || n > 0x7fffffffLL || (n > 0 && !pols)) return fail(c, RSV_E_ARG, "bad m-life arguments");
     if (o->form < F_F64 || o->form > F_COMP) return fail(c, RSV_E_ARG, "bad form %d", o->form);
     if ((o->outputs & ~(RSV_OUT_V0 | RSV_OUT_SCEN_TOTAL)) || o->horizon != 0 || o->payment != 0 ||
@@ -318,7 +316,7 @@ extern "C" rsv_status rsv_compute_mlife(rsv_ctx* c, const rsv_mlife_policy* pols
         if (v > 0.0) amt_lo = std::min(amt_lo, v);
     }
     bool mat = false;
-    if (o->form == F_COMP && n > 0 && (st = mv_applies(c, F_COMP, amt_lo, amt_hi, false, mat)) != RSV_OK) return st;
+    if (matrix && o->form == F_COMP && n > 0 && (st = mv_applies(c, F_COMP, amt_lo, amt_hi, false, mat)) != RSV_OK) return st;
     if (mat) return mlife_matrix(c, pols, recs, ms, o, out);
     if ((st = stage_tables(c, o->form, pad, n_tab, smem)) != RSV_OK) return st;
 
@@ -411,6 +409,12 @@ extern "C" rsv_status rsv_compute_mlife(rsv_ctx* c, const rsv_mlife_policy* pols
         return rsv_synchronize(c);
     }
     return RSV_OK;
+}
+
+extern "C" rsv_status rsv_compute_mlife(rsv_ctx* c, const rsv_mlife_policy* pols, int64_t n, const rsv_opts* o,
+                                        rsv_out* out) try {
+    if (!c) return RSV_E_ARG;
+    return mv_or_without(c, [&](bool matrix) { return mlife_as(c, pols, n, o, out, matrix); });
 } catch (...) {
     return rsv::host_error(c);
 }

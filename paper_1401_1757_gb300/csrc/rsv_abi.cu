@@ -746,6 +746,23 @@ rsv_status rsv::mv_panel_buffers(rsv_ctx* c, int form, int max_S, int tiles) {
     return RSV_OK;
 }
 
+bool rsv::mv_holds(const rsv_ctx* c) {
+    bool any = false;
+    for (const DevBuf* b : {&c->d_mv_D, &c->d_mv_col, &c->d_mv_D64, &c->d_mv_dig[0], &c->d_mv_dig[1], &c->d_mv_dig[2],
+                            &c->d_mv_dig[3], &c->d_mv_E, &c->d_mv_out})
+        any |= b->p != nullptr;
+    return any;
+}
+
+void rsv::mv_release(rsv_ctx* c) {
+    for (DevBuf* b : {&c->d_mv_D, &c->d_mv_col, &c->d_mv_D64, &c->d_mv_dig[0], &c->d_mv_dig[1], &c->d_mv_dig[2],
+                      &c->d_mv_dig[3], &c->d_mv_E, &c->d_mv_out})
+        b->release();
+    c->mv_range_gen = 0;
+    c->mv_spread = INT_MAX;
+    for (unsigned long long& g : c->mv_dig_gen) g = 0;
+}
+
 rsv_status rsv::mv_multiply(rsv_ctx* c, int form, MvArgs a, int max_S, int s0, int w) {
     a.out = c->d_mv_out.as<MvOut>();
     a.colexp = MvScen::at(c->d_mv_col.p, c->n_steps, c->s_pad).colexp + s0;
@@ -829,8 +846,7 @@ rsv_status rsv::mv_launch(rsv_ctx* c, int form, int s0, int w, float* V0f, doubl
 
 namespace {
 
-rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
-    if (!c) return RSV_E_ARG;
+rsv_status compute_as(rsv_ctx* c, const rsv_opts* o, rsv_out* out, bool matrix) {
     if (!o || !out) return fail(c, RSV_E_ARG, "opts and out must not be NULL");
     if (o->form < F_F64 || o->form > F_DEFL) return fail(c, RSV_E_ARG, "bad form %d", o->form);
     if (o->horizon < 0 || (o->on_device != 0 && o->on_device != 1))
@@ -846,7 +862,7 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
     if ((outs & RSV_OUT_SCEN_TOTAL) && !out->scen_total) return fail(c, RSV_E_ARG, "scen_total NULL");
     if ((outs & RSV_OUT_PT_MEAN) && !out->pt_mean) return fail(c, RSV_E_ARG, "pt_mean NULL");
     if ((outs & RSV_OUT_TRAJ) && !out->traj) return fail(c, RSV_E_ARG, "traj NULL");
-    if (o->form == F_DEFL) return compute_deflated(c, o, out);
+    if (o->form == F_DEFL) return compute_deflated(c, o, out, matrix);
 
     const int64_t n_pol = (int64_t)c->pols.size();
     const int T = c->n_steps, NSc = c->n_scen;
@@ -896,8 +912,10 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
         return fail(c, RSV_E_ARG, "variant %d out of range", o->variant);
     }
     if (o->form != F_F32 && vi == nt && !extra && !scan && !summ && pay == PAY_END) {
-        const rsv_status mst = mv_applies(c, o->form, c->amt_lo, c->amt_hi, true, mat);
-        if (mst != RSV_OK) return mst;
+        if (matrix) {
+            const rsv_status mst = mv_applies(c, o->form, c->amt_lo, c->amt_hi, true, mat);
+            if (mst != RSV_OK) return mst;
+        }
         vi = 0;
     }
     if (split) vg = special_variant(vl, nv, false, PAY_END_GENERAL);
@@ -1074,6 +1092,11 @@ rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
         return rsv_synchronize(c);
     }
     return RSV_OK;
+}
+
+rsv_status compute(rsv_ctx* c, const rsv_opts* o, rsv_out* out) {
+    if (!c) return RSV_E_ARG;
+    return mv_or_without(c, [&](bool matrix) { return compute_as(c, o, out, matrix); });
 }
 
 // The nested run: outer paths, then every (node, outer path, inner path) by its mode.
@@ -1600,7 +1623,8 @@ rsv_status rsv_load_scenarios(rsv_ctx* c, const double* v, int32_t n_scen, int32
         rsv_status st = mv_range(c);
         for (int form = 0; form < 4 && st == RSV_OK; ++form)
             if (c->mv_used[form] == before && c->mv_spread <= mv_max_spread(form)) st = mv_digit_buffers(c, form);
-        return st;
+        if (st != RSV_E_NOMEM) return st;
+        mv_release(c);   // the set is loaded all the same
     }
     CU(cudaStreamSynchronize(c->stream));
     return RSV_OK;
@@ -1621,7 +1645,7 @@ rsv_status rsv_compute_nested(rsv_ctx* c, const rsv_opts* o, const rsv_nested_sp
     if (!c) return RSV_E_ARG;
     cudaError_t e = cudaSetDevice(c->device);
     if (e != cudaSuccess) return fail(c, RSV_E_CUDA, "cudaSetDevice: %s", cudaGetErrorString(e));
-    return compute_nested(c, o, sp, out);
+    return mv_or_without(c, [&](bool) { return compute_nested(c, o, sp, out); });
 } catch (...) {
     return rsv::host_error(c);
 }
