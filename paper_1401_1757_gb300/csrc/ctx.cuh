@@ -233,8 +233,7 @@ struct rsv_ctx {
 
     Layout lay;
     DevBuf d_ctl;       // [0] queue head, [1] status
-    DevBuf d_partial, d_part2, d_sum_done;
-    int sum_done_cols = 0;          // zeroed counters in d_sum_done
+    DevBuf d_partial, d_part2, d_sum_done;   // d_sum_done: counters, 0 between calls
     DevBuf d_o_v0f, d_o_v0d, d_o_tot, d_o_pt, d_o_traj;   // staging for host outputs
     DevBuf d_nest_rn, d_nest_d0, d_nest_plane, d_nest_mean, d_nest_kth, d_nest_all;
     DevBuf d_nest_bm;            // tables of the inner-path generators (staged once)

@@ -606,10 +606,9 @@ rsv_status rsv::scenario_totals(rsv_ctx* c, const double* partial, int n_rows, i
     const int G = n_rows <= 256 ? std::max(1, n_rows) : 128, groups = std::max(1, (n_rows + G - 1) / G), cols = (n_scen + 31) / 32;
     if (groups > 1) {
         CU(c->d_part2.ensure((size_t)groups * s_pad * sizeof(double)));
-        if (c->sum_done_cols < cols) {
+        if (c->d_sum_done.n < (size_t)cols * sizeof(int)) {   // 0 bytes after an allocation that failed
             CU(c->d_sum_done.ensure((size_t)cols * sizeof(int)));
             CU(cudaMemsetAsync(c->d_sum_done.p, 0, (size_t)cols * sizeof(int), c->stream));
-            c->sum_done_cols = cols;
         }
     }
     reduce_rows_kernel<<<dim3(cols, groups), dim3(32, kSumRows), 0, c->stream>>>(partial, n_rows, s_pad, G, c->d_part2.as<double>(),
