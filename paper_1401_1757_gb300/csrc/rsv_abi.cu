@@ -1450,6 +1450,7 @@ rsv_status rsv_load_scenarios_fraction(rsv_ctx* c, const double* v, int32_t n_sc
     const int s_pad = (n_scen + 127) / 128 * 128;
     const size_t np = (size_t)n_steps * s_pad;
     CU(c->d_vstage.ensure(n * sizeof(double)));
+    c->vf_scen = 0;   // until the planes hold the new ones
     CU(c->d_vf64.ensure(np * sizeof(double)));
     CU(c->d_vf32.ensure(np * sizeof(float)));
     CU(c->d_vf2.ensure(np * sizeof(float2)));
@@ -1602,6 +1603,7 @@ rsv_status rsv_load_scenarios(rsv_ctx* c, const double* v, int32_t n_scen, int32
     CU(cudaStreamSynchronize(c->stream));
     if (bad < n)
         return fail(c, RSV_E_ASSUMPTION, "discount factor %zu = %g is not finite and positive", (size_t)bad, v[bad]);
+    c->n_scen = 0;   // until the planes hold the new one; growing them frees the old
     CU(c->d_v64.ensure(np * sizeof(double)));
     CU(c->d_v32.ensure(np * sizeof(float)));
     CU(c->d_v2.ensure(np * sizeof(float2)));
