@@ -262,23 +262,28 @@ __global__ void tied_w1_kernel(const float* __restrict__ w1, __nv_bfloat16* __re
 
 cudaError_t Mlp::ensure(int batch) {
     if (batch <= cap) return cudaSuccess;
+    cap = 0;   // until every buffer has grown
     const size_t B = (size_t)batch;
     const size_t P = mlp_n_params();
     cudaError_t e;
 #define ALLOC(ptr, bytes)                                       \
     do {                                                        \
         if (ptr) cudaFree(ptr);                                 \
+        ptr = nullptr;                                          \
         e = cudaMalloc((void**)&ptr, (bytes));                  \
-        if (e != cudaSuccess) return e;                         \
+        if (e != cudaSuccess) {                                 \
+            cudaGetLastError();                                 \
+            return e;                                           \
+        }                                                       \
     } while (0)
-    if (!params) {
-        ALLOC(params, P * 4);
+    if (!params) {   // the last of them
         ALLOC(grads, P * 4);
         ALLOC(adam_m, P * 4);
         ALLOC(adam_v, P * 4);
         ALLOC(wbf, (size_t)MLP_XW * MLP_H * 2 + 3 * (size_t)MLP_H * MLP_H * 2);
         cudaMemset(adam_m, 0, P * 4);
         cudaMemset(adam_v, 0, P * 4);
+        ALLOC(params, P * 4);
     }
     ALLOC(X, B * MLP_XW * 2);
     for (int l = 0; l < 4; ++l) {
