@@ -935,25 +935,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
                             for (int i = 0; i < 16; ++i) {
                                 const MvOut64& q = reinterpret_cast<const MvOut64&>(recs[part * kCols + c0 + i]);
                                 float e;
-                                if (k0 > 0 || !last) {   // several segments: the first levels' sum is exact
-                                    two_sum(w[i], v[i], w[i], v[i]);
-                                    x[i] = __fadd_rn(x[i], v[i]);
-                                    v[i] = 0.0f;
-                                    if (k0 > 0) {
-                                        p[i] = __fadd_rn(p[i], run[0][c0 + i]);
-                                        two_sum(w[i], run[1][c0 + i], w[i], e);
-                                        x[i] = __fadd_rn(__fadd_rn(x[i], e), run[2][c0 + i]);
-                                    }
-                                    if (!last) {
-                                        run[0][c0 + i] = p[i];
-                                        run[1][c0 + i] = w[i];
-                                        run[2][c0 + i] = x[i];
-                                        continue;
-                                    }
+                                two_sum(w[i], v[i], w[i], v[i]);
+                                x[i] = __fadd_rn(x[i], v[i]);
+                                if (k0 > 0) {   // the first levels' sum is exact
+                                    p[i] = __fadd_rn(p[i], run[0][c0 + i]);
+                                    two_sum(w[i], run[1][c0 + i], w[i], e);
+                                    x[i] = __fadd_rn(__fadd_rn(x[i], e), run[2][c0 + i]);
+                                }
+                                if (!last) {
+                                    run[0][c0 + i] = p[i];
+                                    run[1][c0 + i] = w[i];
+                                    run[2][c0 + i] = x[i];
+                                    continue;
                                 }
                                 two_sum(p[i], w[i], p[i], w[i]);
-                                two_sum(w[i], v[i], w[i], e);
-                                x[i] = __fadd_rn(x[i], e);
                                 // of the FP64 pipe (1/64 of the FP32 rate) only what needs 53 bits
                                 double t = __dadd_rn(scaled_double(w[i], ce), scaled_double(x[i], ce));
                                 t = __dmul_rn(__dadd_rn(scaled_double(p[i], ce), t), q.sc);
