@@ -246,7 +246,9 @@ cudaError_t launch_scan(const RecurArgs& a, int sm_count, size_t smem, cudaStrea
     const size_t cols = (size_t)a.n_scen * a.n_steps * sizeof(double);
     const int v_bytes = cols <= 32 * 1024 && smem + cols <= 100 * 1024 ? (int)cols : 0;
     smem += v_bytes;
-    cudaError_t e = cudaFuncSetAttribute(scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the limit, not this launch's size: another thread may set it for its own between here and the launch
+    constexpr int kMost = 200 * 1024;   // tables at their largest; with columns at most half of it
+    cudaError_t e = cudaFuncSetAttribute(scan_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
     if (e != cudaSuccess) return e;
     int bps = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, scan_kernel, 256, smem)) != cudaSuccess) return e;
