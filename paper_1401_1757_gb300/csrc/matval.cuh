@@ -57,6 +57,7 @@ constexpr int kMvP = 128;          // policies per tile (MMA N)
 constexpr int kMvM = 128;          // scenarios per tile (MMA M)
 constexpr int kMvParts = 4;        // column groups of the epilogue
 constexpr int kMvTilt = 60;        // largest |tau|
+constexpr int kMvMaxSteps = 64 * 65535;   // of a scenario set: blocks of 64 along a grid's second dimension
 constexpr size_t kMvPanelBytes = size_t(1) << 30;            // cash-flow digits held at a time
 // A row's entries, survivor-column entry times cash-flow multiplier times tilt, are formed in FP32
 // head and tail (in the FP64 form their heads, for the row's scale), and a row's scale times its

@@ -676,6 +676,7 @@ rsv_status rsv::mv_range(rsv_ctx* c) {
 
 rsv_status rsv::mv_applies(rsv_ctx* c, int form, double amt_lo, double amt_hi, bool cf, bool& applies) {
     applies = false;
+    if (c->n_steps > kMvMaxSteps) return RSV_OK;
     if (!(amt_hi <= kMvAmountMax) || !(amt_lo >= kMvAmountMin)) return RSV_OK;
     // the smallest and largest entries of a row, but for the tilt
     double lo = 1.0, hi = 1.0;
