@@ -641,7 +641,7 @@ __global__ void __launch_bounds__(256) mv_build_kernel(const MvBuild b) {
 // Three digits: 6 products and 2 accumulators, so TMEM holds two tiles' and the epilogue
 // runs beside the next tile's products.  Four: 10 products, 4 accumulators (half tiles, two in
 // TMEM: 0.89 -> 0.95 ms for 100,000 policies x 1,000 scenarios).  Six and eight: 21 and 36
-// products, an accumulator for each level of half a tile's policies.  Such a product (n64)
+// products, seven and eight accumulators of half a tile's policies.  Such a product (n64)
 // lasts as long as the shared-memory reads of its A, so A is read once a scenario digit
 // and kept in the collector: 903 -> 755 us a launch of 50,000 x 1,000 with six.  Whole
 // tiles with the levels 3 to 5 in one accumulator took 690 us, at 13 times the error (totals of
@@ -654,12 +654,13 @@ __global__ void __launch_bounds__(256) mv_build_kernel(const MvBuild b) {
 // An accumulator sums at most SEG steps (a segment), so that the levels that must be exact
 // are (matval.cuh); a longer item's segments are added up by the epilogue, whose sums so far wait
 // in local memory (in registers they would not fit beside an accumulator's columns).  A segment's
-// end costs about 2,000 cycles: 100,000 x 1,000 of every product with six digits 1.62 -> 1.74 ms,
-// 3,000 x 333 in FP64 0.146 -> 0.154 ms.
+// end costs about 2,000 cycles.  Six digits, 100,000 x 1,000 of every product: 1.67 ms; 1.74 with
+// segments of 256 steps and a level an accumulator, 1.62 over whole projections, inexact.  FP64,
+// 3,000 x 333: 0.148, 0.154 and 0.146 ms.
 template <int NS>
 struct MvShape;   // policies of an item, accumulators, segments in TMEM, stages, steps of a block (64:
 template <>       // 128-byte swizzled rows) and of a segment; the products are (i, j), i + j < NS, of
-struct MvShape<3> {   // scenario digit i and policy digit j, in accumulator min(i + j, NA - 1)
+struct MvShape<3> {   // scenario digit i and policy digit j, in accumulator mv_acc
     static constexpr int N = kMvP, NA = 2, NB = 2, ST = 3, KB = 64, SEG = 1024;
 };
 template <>
@@ -668,12 +669,29 @@ struct MvShape<4> {
 };
 template <>
 struct MvShape<6> {
-    static constexpr int N = kMvP / 2, NA = 6, NB = 1, ST = 3, KB = 32, SEG = 256;
+    static constexpr int N = kMvP / 2, NA = 7, NB = 1, ST = 3, KB = 32, SEG = 512;
 };
 template <>
 struct MvShape<8> {
-    static constexpr int N = kMvP / 2, NA = 8, NB = 1, ST = 2, KB = 32, SEG = 256;
+    static constexpr int N = kMvP / 2, NA = 8, NB = 1, ST = 2, KB = 32, SEG = 512;
 };
+// The accumulator of the product (i, j).  Three and four digits: one for each of the first levels.
+// Six and eight: levels 0 and 1; 2 and 3, of three and four products, in two each, so that none
+// takes more than two of an exact level; the rest in one (eight: 4, and the rest).
+template <int NS>
+__host__ __device__ constexpr int mv_acc(int i, int j) {
+    const int level = i + j, inner = i > 0 && j > 0;
+    if (NS < 6 || level < 2) return level < MvShape<NS>::NA ? level : MvShape<NS>::NA - 1;
+    if (level < 4) return 2 * level - 2 + inner;
+    return NS == 8 && level > 4 ? 7 : 6;
+}
+template <int NS>
+__host__ __device__ constexpr bool mv_acc_first(int i, int j) {   // no product before (i, j) goes there
+    for (int a = 0; a <= i; ++a)
+        for (int b = 0; a + b < NS && (a < i || b < j); ++b)
+            if (mv_acc<NS>(a, b) == mv_acc<NS>(i, j)) return false;
+    return true;
+}
 constexpr int kMvEpi = 4 * kMvParts;                   // epilogue warps
 constexpr int kMvThreads = 32 * (kMvEpi + 2);
 
@@ -691,8 +709,8 @@ template <int NS, int I, int J>
 __device__ __forceinline__ void mv_products(uint32_t d, uint64_t base, int off, uint32_t idesc, bool more) {
     using Sh = MvShape<NS>;
     using G = MvStage<NS>;
-    constexpr int acc = I + J < Sh::NA ? I + J : Sh::NA - 1;
-    constexpr bool first = I == 0 && J == acc;   // of its accumulator
+    constexpr int acc = mv_acc<NS>(I, J);
+    constexpr bool first = mv_acc_first<NS>(I, J);
     constexpr bool last = I + J + 1 == NS;
     constexpr int coll = Sh::N == kMvP || (J == 0 && last) ? COLL_NONE : (J == 0 ? COLL_FILL : (last ? COLL_LAST : COLL_USE));
     mma_f16_ss_pair<coll>(d + acc * Sh::N, base + (uint64_t)((I * G::kA + off) >> 4),
@@ -904,8 +922,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
 #pragma unroll 1
                     for (int c0 = 0; c0 < kCols; c0 += kHold) {
                         if constexpr (NS == 8) {
-                            // u = a0 + w + v + x: the levels from 2^-32 of the first as plain FP32
-                            // sums (2^-56), the others' errors kept; the rest after the release
+                            // u = p + w + v + x: the levels 0 (p), 1 and 2 (w) and 3 (v) with
+                            // their sums' errors, the lower ones as plain FP32 sums (2^-56) (x);
+                            // the rest after the release
                             float p[16], w[16], v[16], x[16];
                             {
                                 float y[16], z[16];
@@ -914,12 +933,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
                                 for (int i = 0; i < 16; ++i) x[i] = __fadd_rn(y[i], z[i]);
                                 load2(5, 4, c0, y, z);
 #pragma unroll
-                                for (int i = 0; i < 16; ++i) x[i] = __fadd_rn(z[i], __fadd_rn(y[i], x[i]));
+                                for (int i = 0; i < 16; ++i) {
+                                    float e;
+                                    two_sum(y[i], z[i], v[i], e);
+                                    x[i] = __fadd_rn(x[i], e);
+                                }
                                 load2(3, 2, c0, y, z);
 #pragma unroll
                                 for (int i = 0; i < 16; ++i) {
-                                    two_sum(y[i], x[i], v[i], x[i]);
-                                    w[i] = z[i];
+                                    float e;
+                                    two_sum(y[i], z[i], w[i], e);
+                                    x[i] = __fadd_rn(x[i], e);
                                 }
                                 load2(1, 0, c0, y, p);
 #pragma unroll
@@ -973,12 +997,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
                         for (int c = 0; c < kHold; c += 16) {
                             float y[16], z[16], x[16];
                             if constexpr (NS == 6) {
-                                load2(5, 4, c0 + c, y, z);
+                                load2(6, 5, c0 + c, y, z);
 #pragma unroll
-                                for (int i = 0; i < 16; ++i) x[i] = __fadd_rn(y[i], z[i]);
-                                load2(3, 2, c0 + c, y, z);
+                                for (int i = 0; i < 16; ++i) l[c + i] = __fadd_rn(y[i], z[i]);
+                                load2(4, 3, c0 + c, y, z);
 #pragma unroll
-                                for (int i = 0; i < 16; ++i) l[c + i] = __fadd_rn(y[i], x[i]);
+                                for (int i = 0; i < 16; ++i) l[c + i] = __fadd_rn(l[c + i], y[i]);
+                                uint32_t r[16];
+                                tmem_ld16_async(col0 + 2 * N + c0 + c, r);
+                                tmem_wait_ld(r);
+#pragma unroll
+                                for (int i = 0; i < 16; ++i) {
+                                    float e;
+                                    two_sum(__uint_as_float(r[i]), z[i], z[i], e);
+                                    l[c + i] = __fadd_rn(l[c + i], e);
+                                }
                                 load2(1, 0, c0 + c, y, x);
                                 release();
 #pragma unroll

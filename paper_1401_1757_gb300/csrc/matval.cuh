@@ -17,17 +17,17 @@
 // The products of digits i and j, i + j at most the last digit's number, are taken.  A digit is
 // at most 2^7 units in size and a product 2^14, so that FP32 adds up 1,024 products of a level
 // exactly whatever their signs.  Operands that hardly change (no interest and no mortality to
-// speak of) have digits of one sign from step to step, so this is the bound that counts: with
-// six and eight digits an accumulator of level i + j sums at most 256 steps, a segment, which
-// makes the levels 0 to 2 (eight digits: to 3) exact and leaves truncations below 2^-40 (2^-47) of
-// the sum at the very worst; one accumulator over 1,000 steps was off by 4e-9 on such operands.
-// The epilogue adds up the segments in double-floats (eight digits: three floats).  With three
-// and four digits a segment is 1,024 steps, so that level 0 is exact; the truncations of the
-// others, at most 2^-24 of a sum 2^-7 below for each block of 16 steps and pair of digits,
-// stay within 2^-22.
-// The epilogue adds the accumulators: the first ones with their rounding errors, the low ones as they
-// are (to 2^-40, 2^-48 and 2^-56 with four, six and eight digits).  A maturity payment is
-// added there, from the discount products themselves, so that a row holds entries of one kind.
+// speak of) have digits of one sign from step to step, so this is the bound that counts: one
+// accumulator a level over 1,000 steps was off by 4e-9 on such operands.  With six and eight
+// digits an accumulator takes one or two products of a level and sums at most 512 steps, a segment,
+// which makes the levels 0 to 2 (eight digits: to 3) exact and leaves truncations below 2^-40
+// (2^-46) of the sum at the very worst.  With three and four digits a segment is 1,024 steps, so
+// that level 0 is exact; the truncations of the others, at most 2^-24 of a sum 2^-7 below for each
+// block of 16 steps and pair of digits, stay within 2^-22.
+// The epilogue adds the accumulators: the first ones with their rounding errors, the low ones as
+// they are (to 2^-40, 2^-48 and 2^-56 with four, six and eight digits), and the segments as
+// double-floats (eight digits: three floats).  A maturity payment is added there, from the
+// discount products themselves, so that a row holds entries of one kind.
 //
 // Fixed point needs rows and columns of moderate range.  The discount products are
 // tilted by a power of two per step, 2^tau(t) ~ 1 / (their geometric mean over the
@@ -37,8 +37,8 @@
 // mv_max_spread) keeps the recurrence kernels.
 //
 // Measured (one GB300, with the digits and the totals), before: the recurrence.
-//   100,000 policies of every product, 1,000 scenarios: compensated 38.7 -> 1.74 ms
-//   (annuities 1e-13 -> 1.5e-14 rms, assurances 4e-9 -> 1.7e-14), deflated 4.93 -> 0.88 ms
+//   100,000 policies of every product, 1,000 scenarios: compensated 38.7 -> 1.67 ms
+//   (annuities 1.5e-13 -> 6e-15 rms, assurances 2e-9 -> 1.2e-14), deflated 4.93 -> 0.88 ms
 //   (rms 3e-8 -> 5e-9, with three digits 0.62 ms);
 //   1,000,000 annuities, 600 steps, 1,000 scenarios, deflated: 30.6 -> 4.1 ms;
 //   3,000 two-life policies, 333 scenarios, FP64: 5.17 -> 0.15 ms (1.4e-15 -> 1.3e-15).
