@@ -901,14 +901,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMvThreads, 1)
                             const float2 d = a.D[(size_t)max(q.S - 1, 0) * a.s_pad + sl];
                             due = q.S == 0;
                             const df m = df_mul(df{q.mat_h, q.mat_l}, due ? df{1.0f, 0.0f} : df{d.x, d.y});
-                            const float sum = __fadd_rn(v.h, m.h), bb = __fsub_rn(sum, v.h);
-                            const float e = __fadd_rn(__fsub_rn(v.h, __fsub_rn(sum, bb)), __fsub_rn(m.h, bb));
+                            float sum, e;
+                            two_sum(v.h, m.h, sum, e);
                             v = df{sum, __fadd_rn(e, __fadd_rn(v.l, m.l))};
                             due = due && q.mat_h != 0.0f;
                         }
                         // the sum over the policies
-                        const float sum = __fadd_rn(tot.h, v.h), bb = __fsub_rn(sum, tot.h);
-                        const float e = __fadd_rn(__fsub_rn(tot.h, __fsub_rn(sum, bb)), __fsub_rn(v.h, bb));
+                        float sum, e;
+                        two_sum(tot.h, v.h, sum, e);
                         tot = df{sum, __fadd_rn(tot.l, __fadd_rn(e, v.l))};
                         const size_t o = (size_t)pol * a.v0_ld + s;
                         if (live && pol >= 0) {

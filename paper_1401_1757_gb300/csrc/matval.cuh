@@ -5,7 +5,9 @@
 // (Eq. basicReserveSummation; cashflow.cuh): a product of the policies' expected cash
 // flows [policy][step] and the scenarios' discount products [step][scenario].  The
 // recurrence kernels run it chain by chain on the FP32 pipe; here it runs as 16-bit
-// matrix instructions with FP32 accumulation, on operands split into exact digits:
+// matrix instructions with FP32 accumulation, on operands split into exact digits (the splitting
+// of Ozaki, Ogita, Oishi & Rump, "Error-free transformations of matrix multiplication by using
+// fast routines of matrix multiplication", Numer. Algorithms 59, 2012):
 //
 //   a = d1 + d2 + ...  with a in [0, 1]; d1: a to 7 bits.
 //   Three digits: d2 and d3 the FP16 values (11 bits and sign) of the remainders, to 2^-32
@@ -125,7 +127,7 @@ struct MvBuild {
     const double* cf;          // their multipliers [n_pol][cf_ld], or null
     int32_t cf_ld;
     int32_t n_steps;           // of the scenario set
-    int32_t rows_per_warp;     // 1 to 16: more once there are tiles enough to fill the chip
+    int32_t rows_per_warp;     // 1, or 4 once there are tiles enough to fill the chip
     const float* tilt;
     const float* tilt_top;
     void* digits;

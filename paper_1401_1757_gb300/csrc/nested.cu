@@ -21,7 +21,7 @@
 // month's discount factor: below.  Outer path o:
 // (k, o, 0, 2 << 24); inner path (o, n, i): (k, i, n, (3 << 24) | o).
 // Vasicek exact monthly step of (r, integral of r) (Glasserman 2004 3.3.1);
-// v = exp(-integral), FP64, stored in the form's plane format.
+// v = exp(-integral) goes into the path's discount product at once.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
